@@ -213,8 +213,10 @@ KERNEL_OF_STAGE = {
     (True, "edge_bwd_l0"): ("k_edge_bwd_grp<64,3,2,16,1>", "potential_bf16.cu"),
     (True, "edge_bwd"): ("k_edge_bwd_grp<64,3,2,16,0>", "potential_bf16.cu"),
     (True, "edge_fwd"): ("k_edge_fwd_bf16<64,16>", "potential_bf16.cu"),
-    (False, "edge_bwd"): ("k_edge_bwd<64,16>", "potential_f32.cu"),
-    (False, "edge_fwd"): ("k_edge_fwd<64,16>", "potential_f32.cu"),
+    # FP32: the layer-0 forward stage is the pair index, the filters of every layer and the layer's gather
+    (False, "edge_fwd_l0"): ("k_pair_filter<64,16>", "potential_f32.cu"),
+    (False, "edge_bwd"): ("k_gather_bwd<64,3,0>", "potential_f32.cu"),
+    (False, "edge_fwd"): ("k_gather_fwd<64>", "potential_f32.cu"),
 }
 
 
@@ -247,7 +249,9 @@ def roofline_of(D, prec, stages_big, E_big, ba):
     dom = max((k for k in stages_big if k.startswith("edge_")), key=lambda k: stages_big[k])
     K, F = ba.n_radial, ba.n_feat
     if prec == D.FP32:
-        flop_edge = 2 * (2 * K * F + 2 * F * F) if dom.startswith("edge_bwd") else 2 * (K * F + F * F)
+        # w and dw/dd of every layer, 4 F (K + F) flop per unordered pair and layer; the other stages are
+        # gathers: g . dw/dd and w * mbar (8 F) or w * u (2 F) per directed pair
+        flop_edge = {"edge_fwd_l0": ba.n_layers * 2 * F * (K + F)}.get(dom, 8 * F if dom.startswith("edge_bwd") else 2 * F)
         peak, bound, src, kind = FP32_SIMT_TFLOPS, "alu", "derived: 152 SMs x 128 FP32 lanes x 2 x 2.07 GHz", "FP32 SIMT"
     else:
         # the algorithmic edge-GEMM work per pair and layer, K padded to 16: one pass 2F(16 + F) forward,

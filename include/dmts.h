@@ -303,7 +303,8 @@ DMTS_API int dmts_get_bwd_tiles(dmts_ctx* ctx, int which);
  *   [0] quantisation, cell list and neighbour list,
  *   [1] species embedding (no work: h^0 and u^0 depend only on species and
  *       parameters and are built once per parameter upload),
- *   [2 + l] forward edge pass of layer l (l < n_layers),
+ *   [2 + l] forward edge pass of layer l (l < n_layers); in DMTS_FP32 mode
+ *       layer 0 includes the pairs' filters of every layer,
  *   [2 + n_layers + l] per-atom MLPs after it,
  *   [2 + 2 n_layers + l] backward edge pass of layer l,
  *   [2 + 3 n_layers + l] per-atom adjoint MLPs after it (0 for l = 0),

@@ -189,6 +189,7 @@ struct Model {
     int cps_fwd = 0, cps_bwd = 0;      // tensor-core kernels: persistent CTAs per SM (0: as many as fit)
     int bwd_tiles = 0;                 // tensor-core backward: 128-pair tiles in flight per CTA (0: default)
     float* carry = nullptr;            // tensor-core path: per-tile partial sums of split rows
+    PairFilter filt{};                 // FP32 mode: filter rows of the pairs
     SumScratch esum{};                 // scratch of the per-system energy sum
 };
 
@@ -320,8 +321,48 @@ int check_model(const dmts_model_desc* d, const char* name) {
 
 void free_model_nbr(Model& m) {
     dfree(m.nbr_tmp); dfree(m.col); dfree(m.recv); dfree(m.vl_rows); dfree(m.carry);
+    dfree(m.filt.w); dfree(m.filt.pairs); dfree(m.filt.pid); dfree(m.filt.count);
     m.nbr_tmp = m.col = m.recv = m.vl_rows = nullptr;
     m.carry = nullptr;
+    m.filt = PairFilter{};
+}
+
+// Filter rows of the FP32 mode (PairFilter): for every unordered pair and
+// layer if that takes at most kFilterBytes (about 800,000 atoms of water with
+// the big model; 0.5 GB at 12,288) and the memory is there, otherwise for the
+// directed pairs of as many atoms as fit in kFilterChunkBytes at a time,
+// halved until the allocation succeeds. Checked builds use small limits, so
+// that both forms run on small systems.
+#ifdef DMTS_CHECK
+constexpr size_t kFilterBytes = (size_t)64 << 20, kFilterChunkBytes = (size_t)16 << 20;
+#else
+constexpr size_t kFilterBytes = (size_t)32 << 30, kFilterChunkBytes = (size_t)8 << 30;
+#endif
+
+cudaError_t alloc_filters(Model& m) {
+    PairFilter& f = m.filt;
+    const size_t row = 2 * sizeof(float) * m.F;               // w and dw/dd of one layer
+    const long long half = m.e_cap / 2 + 1;
+    cudaError_t e;
+    if (half * row * m.L <= kFilterBytes) {
+        e = dalloc(&f.w, half * (row / sizeof(float)) * m.L);
+        if (e == cudaSuccess) e = dalloc(&f.pairs, (size_t)half);
+        if (e == cudaSuccess) e = dalloc(&f.pid, (size_t)m.e_cap);
+        if (e == cudaSuccess) e = dalloc(&f.count, 1);
+        if (e == cudaSuccess) e = cudaMemset(f.count, 0, sizeof(int));
+        f.cap = half;
+        if (e == cudaSuccess) return e;
+        cudaGetLastError();
+        dfree(f.w); dfree(f.pairs); dfree(f.pid); dfree(f.count);
+        f = PairFilter{};
+    }
+    long long atoms = std::max<long long>(1, (long long)(kFilterChunkBytes / row) / m.row_cap);
+    for (;; atoms /= 2) {
+        f.chunk_atoms = (int)atoms;
+        f.cap = atoms * m.row_cap;
+        if ((e = dalloc(&f.w, f.cap * (row / sizeof(float)))) == cudaSuccess || atoms == 1) return e;
+        cudaGetLastError();
+    }
 }
 
 cudaError_t alloc_model_nbr(dmts_ctx* c, Model& m) {
@@ -332,6 +373,7 @@ cudaError_t alloc_model_nbr(dmts_ctx* c, Model& m) {
     if (c->skin > 0 && (e = dalloc(&m.vl_rows, (size_t)c->N * m.vl_cap)) != cudaSuccess) return e;
     const size_t tiles = (size_t)((m.e_cap + 127) / 128);
     if ((e = dalloc(&m.carry, tiles * 2 * (size_t)(m.F + 16))) != cudaSuccess) return e;
+    if (m.precision == DMTS_FP32 && (e = alloc_filters(m)) != cudaSuccess) return e;
     return cudaSuccess;
 }
 
@@ -553,13 +595,8 @@ int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells) {
     CUDA_TRY(dalloc(&m.esum.ctr, kSumMaxSplit));
     CUDA_TRY(cudaMemset(m.esum.ctr, 0, sizeof(unsigned int) * kSumMaxSplit));
     CUDA_TRY(dalloc(&m.W, (size_t)9 * c->n_sys));
-    // FP32: atoms per CTA (bounded by shared memory); BF16: atoms per chunk of
-    // the persistent kernels
-    int mf = max_atoms_per_cta_f32(m.F, m.K, false);
-    int mb = max_atoms_per_cta_f32(m.F, m.K, true);
-    int want = m.F == 64 ? 16 : 32;
-    m.apc_fwd = std::max(8, std::min(want, mf));
-    m.apc_bwd = std::max(8, std::min(want, mb));
+    // FP32: atoms per CTA of the gathers (eight warps, one atom each at a time)
+    m.apc_fwd = m.apc_bwd = 8;
     return DMTS_OK;
 }
 
@@ -634,6 +671,7 @@ PotArgs pot_args(dmts_ctx* c, Model& m) {
     a.at = m.at;
     a.carry = m.carry;
     a.carry_w = m.F + 16;
+    a.filter = m.filt;
     a.h = m.h;
     a.h_in = m.h;
     a.gh = m.gh;
@@ -1140,11 +1178,11 @@ int autotune_models(dmts_ctx* c) {
         double best_tf = 1e30, best_tb = 1e30;
         int best_f = gf, best_b = gb, best_t = m.bwd_tiles;
         for (int tiles : tiles_c) {
-            const int lim_f = tc ? bf16_max_ctas_per_sm(m.F, false) : max_atoms_per_cta_f32(m.F, m.K, false);
-            const int lim_b = tc ? bf16_max_ctas_per_sm(m.F, true, tiles) : max_atoms_per_cta_f32(m.F, m.K, true);
+            const int lim_f = tc ? bf16_max_ctas_per_sm(m.F, false) : kMaxAtomsPerCtaF32;
+            const int lim_b = tc ? bf16_max_ctas_per_sm(m.F, true, tiles) : kMaxAtomsPerCtaF32;
             std::vector<int> cand;
             if (tc) for (int k = 1; k <= std::max(lim_f, lim_b); ++k) cand.push_back(k);
-            else cand = m.F == 64 ? std::vector<int>{8, 16, 24} : std::vector<int>{16, 32, 48};
+            else cand = {8, 16};
             m.bwd_tiles = tiles;
             for (int A : cand) {
                 gf = std::min(A, lim_f);
@@ -1388,13 +1426,13 @@ int dmts_create(const dmts_model_desc* small, const dmts_model_desc* big, const 
     if (small) {
         rc = init_model(c, c->m[0], small, c->skin <= 0 || c->vl_src == 0);
         if (rc) { std::string k = g_err; dmts_destroy(c); g_err = k; return rc; }
-        c->m[0].apc_fwd = std::min(c->m[0].apc_fwd, (int)opt.get("atoms_per_cta_small", c->m[0].apc_fwd));
-        c->m[0].apc_bwd = std::min(c->m[0].apc_bwd, (int)opt.get("atoms_per_cta_small", c->m[0].apc_bwd));
+        c->m[0].apc_fwd = std::min(kMaxAtomsPerCtaF32, (int)opt.get("atoms_per_cta_small", c->m[0].apc_fwd));
+        c->m[0].apc_bwd = std::min(kMaxAtomsPerCtaF32, (int)opt.get("atoms_per_cta_small", c->m[0].apc_bwd));
     }
     rc = init_model(c, c->m[1], big, c->skin <= 0 || c->vl_src == 1);
     if (rc) { std::string k = g_err; dmts_destroy(c); g_err = k; return rc; }
-    c->m[1].apc_fwd = std::min(c->m[1].apc_fwd, (int)opt.get("atoms_per_cta_big", c->m[1].apc_fwd));
-    c->m[1].apc_bwd = std::min(c->m[1].apc_bwd, (int)opt.get("atoms_per_cta_big", c->m[1].apc_bwd));
+    c->m[1].apc_fwd = std::min(kMaxAtomsPerCtaF32, (int)opt.get("atoms_per_cta_big", c->m[1].apc_fwd));
+    c->m[1].apc_bwd = std::min(kMaxAtomsPerCtaF32, (int)opt.get("atoms_per_cta_big", c->m[1].apc_bwd));
     for (int w = 0; w < 2; ++w) {
         if (c->m[w].present && opt_row_cap >= 1.0) {
             // smaller initial row capacity (exercises the overflow-and-retry path)
@@ -1966,8 +2004,8 @@ int dmts_set_tuning(dmts_ctx* c, int which, int fwd, int bwd, int bwd_tiles) {
         m.cps_fwd = std::min(fwd, bf16_max_ctas_per_sm(m.F, false));
         m.cps_bwd = std::min(bwd, bf16_max_ctas_per_sm(m.F, true, m.bwd_tiles));
     } else {
-        m.apc_fwd = std::min(fwd, max_atoms_per_cta_f32(m.F, m.K, false));
-        m.apc_bwd = std::min(bwd, max_atoms_per_cta_f32(m.F, m.K, true));
+        m.apc_fwd = std::min(fwd, kMaxAtomsPerCtaF32);
+        m.apc_bwd = std::min(bwd, kMaxAtomsPerCtaF32);
     }
     c->tuned = true;                          // the tuner keeps the caller's choice
     if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }

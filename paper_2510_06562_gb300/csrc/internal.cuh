@@ -41,6 +41,7 @@ __device__ __forceinline__ I checked_index(I i, long long n, int* flags, int lin
 
 constexpr int kMaxLayers = 4;
 constexpr int kThreads = 256;          // threads per CTA of the edge kernels
+constexpr int kSmCount = 152;          // SMs of a GB300 (grid sizes only)
 constexpr int kMaxMolAtoms = 1024;     // atoms per non-periodic system
 
 // Offsets (in floats) of every parameter block inside the flat vector.
@@ -229,9 +230,23 @@ struct CellPlace {
     int flag_cell;
 };
 
+// FP32 mode: filter rows w and dw/dd (F floats each), one of each per
+// unordered pair and layer (chunk_atoms == 0), w at [2 l cap + p], dw/dd cap
+// rows later; or, where those would take too much memory, of the directed
+// pairs of chunk_atoms atoms and one layer at a time, recomputed by each pass.
+struct PairFilter {
+    float* w;
+    long long cap;           // rows per array
+    int2* pairs;             // [cap] the unordered pairs (i, j), i < j
+    int* pid;                // [e_cap] each directed pair's entry
+    int* count;              // entries in use (zero between evaluations)
+    int chunk_atoms;
+};
+
 // Arguments of the potential's kernels (one model, one layer).
 struct PotArgs {
-    int* check;              // checked builds: flags array receiving index violations
+    int* check;              // the flags array (checked builds record index violations there)
+    PairFilter filter;       // FP32 mode
     const float* P;          // FP32 parameters, flat order
     ModelOffsets off;
     int layer;
@@ -314,9 +329,10 @@ void launch_vl_filter(const NbrArgs& a, cudaStream_t s);
 
 // potential_f32.cu
 void launch_embed(const PotArgs& a, int F, cudaStream_t s);
+// (the forward launch of layer 0 also computes the pairs' filters of every layer)
 void launch_edge_fwd_f32(const PotArgs& a, int F, int K, cudaStream_t s);
 void launch_edge_bwd_f32(const PotArgs& a, int F, int K, cudaStream_t s);
-int max_atoms_per_cta_f32(int F, int K, bool bwd);
+constexpr int kMaxAtomsPerCtaF32 = 256;
 
 // potential_bf16.cu (tensor cores; status receives 1 if a bounded wait gave up)
 void launch_edge_fwd_bf16(const PotArgs& a, int F, int K, int* status, cudaStream_t s);

@@ -1,55 +1,48 @@
 // FP32 SIMT path of the potential: forward message passing and the force
-// adjoint, with the per-edge filter MLP recomputed (never stored).
+// adjoint.
 //
-// Work decomposition: CTA b owns the atoms [b*A, (b+1)*A) and therefore the
-// contiguous CSR edge range of their rows. It walks that range in tiles of
-// TE edges; within a tile the filter MLP is a register-blocked GEMM (each of
-// the 256 threads owns 4 edges x 4 features), and the per-row sums are taken
-// in edge order by one thread per feature, so results are deterministic and
-// atomic-free. The per-atom sums (messages, or the adjoint ubar) are written
-// to global memory for the per-atom MLP kernels.
+// The filter w_ij = fc(d) phi(d) and its derivative dw/dd depend on the pair's
+// distance only: they are the same for (i, j) and (j, i) and do not depend on
+// the features. So an evaluation computes both once per unordered pair and
+// layer (k_pair_filter, register-blocked GEMMs over tiles of 128 pairs), and
+// the passes over the directed pairs are gathers over each atom's own row:
+//   forward   m_i = sum_j w_ij * u_j
+//   backward  F_i = sum_j dE/dd_ij rhat_ij,  dE/dd_ij = g_ij . dw/dd_ij,
+//             g_ij = mbar_i * u_j + mbar_j * u_i,  ubar_i = sum_j w_ij * mbar_j
+// one warp per atom, the row's pairs in a fixed order, no atomics on results:
+// deterministic and independent of the launch shape.
 //
-// Adjoint (F = -dE/dx): with g_ij = mbar_i * u_j + mbar_j * u_i (the filter
-// depends on d only, so w_ij = w_ji), dE/dd_ij = fc' (g . phi) +
-// fc sum_k [(g W2^T)_k SiLU'(a_k)] (e' W1)_k, and F_i = sum_j dE/dd_ij rhat_ij
-// over row i; the adjoint of u is ubar_i = sum_j w_ij * mbar_j, again a sum
-// over row i. Both are gathers over the atom's own row.
+// Against recomputing the filter per directed pair in each pass (20,480 and
+// 10,240 flop per directed pair and layer), this is 20,480 flop per unordered
+// pair and layer in all, and w, dw/dd travel through memory (512 bytes per
+// unordered pair and layer at F = 64, written once, read three times). Big
+// model, 12,288-atom water, one evaluation: 3.48 -> 0.69 ms (edge passes 3.36
+// -> 0.57 ms); 192 atoms: 0.61 -> 0.16 ms.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
+#include "f32x2.cuh"
 #include "internal.cuh"
 
 namespace dmts {
 
 namespace {
 
-template <int K>
-__device__ __forceinline__ void basis_fwd(float d, float pi_over_rc, float pref, float* e, float& fc) {
-    float s1, c1;
-    sincospif(d * (pi_over_rc * 0.31830988618379067f), &s1, &c1);
-    float inv_d = 1.0f / d;
-    float sk = s1, skm1 = 0.f;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        e[k] = pref * sk * inv_d;
-        float sn = 2.f * c1 * sk - skm1;
-        skm1 = sk;
-        sk = sn;
-    }
-    fc = 0.5f * (c1 + 1.0f);
-}
-
-template <int K>
-__device__ __forceinline__ void basis_bwd(float d, float pi_over_rc, float pref, float* e, float* de,
-                                          float& fc, float& dfc) {
+// Bessel functions e_k(d) = pref sin(k pi d / rc) / d, k < K <= KP (zero from
+// K on), their derivatives, the cosine cutoff and its derivative.
+template <int KP>
+__device__ __forceinline__ void basis_pair(float d, int K, float pi_over_rc, float pref, float* e, float* de,
+                                           float& fc, float& dfc) {
     float s1, c1;
     sincospif(d * (pi_over_rc * 0.31830988618379067f), &s1, &c1);
     float inv_d = 1.0f / d;
     float sk = s1, skm1 = 0.f, ck = c1, ckm1 = 1.f;
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
+    for (int k = 0; k < KP; ++k) {
         float kw = (float)(k + 1) * pi_over_rc;
-        e[k] = pref * sk * inv_d;
-        de[k] = pref * (kw * ck - sk * inv_d) * inv_d;
+        e[k] = k < K ? pref * sk * inv_d : 0.f;
+        de[k] = k < K ? pref * (kw * ck - sk * inv_d) * inv_d : 0.f;
         float sn = 2.f * c1 * sk - skm1;
         float cn = 2.f * c1 * ck - ckm1;
         skm1 = sk; sk = sn;
@@ -57,41 +50,6 @@ __device__ __forceinline__ void basis_bwd(float d, float pi_over_rc, float pref,
     }
     fc = 0.5f * (c1 + 1.0f);
     dfc = -0.5f * pi_over_rc * s1;
-}
-
-__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
-__device__ __forceinline__ float4 ldg4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
-__device__ __forceinline__ float f4(const float4& v, int c) {
-    return c == 0 ? v.x : (c == 1 ? v.y : (c == 2 ? v.z : v.w));
-}
-
-// ------------------------------------------------------------ shared layout
-template <int F, int K>
-struct Tile {
-    static constexpr int TE = 4096 / F;          // edges per tile (EPT = 4)
-    static constexpr int FG = F / 4;             // feature groups
-    static constexpr int EG = kThreads / FG;     // edge groups
-    static constexpr int PS = F + 4;             // row stride of the message tile
-    static_assert(EG * 4 == TE, "tile shape");
-};
-
-template <int F, int K>
-constexpr int fwd_smem_floats(int A) {
-    using T = Tile<F, K>;
-    return K * F + F + F * F + F + K * T::TE + F * T::TE + T::TE * T::PS + 4 * T::TE + A * F;
-}
-
-template <int F, int K>
-constexpr int bwd_smem_floats(int A) {
-    using T = Tile<F, K>;
-    return K * F + F + F * F + F + F * F        // W1 b1 W2 b2 W2T
-           + 2 * K * T::TE                      // BT DT
-           + 2 * F * T::TE                      // ST GT
-           + T::TE * T::PS                      // P
-           + 10 * T::TE                         // fc dfc se rh(4) j row pad
-           + 2 * T::TE * T::FG                  // red1 red2
-           + A * F + A * 4 + A * 8;             // acc force virial
 }
 
 // ------------------------------------------------------------ embedding
@@ -112,522 +70,522 @@ __global__ void k_embed(PotArgs a) {
             __float2bfloat16_rn(acc);
 }
 
-// ------------------------------------------------------------ forward edge pass
-template <int F, int K>
-__global__ void __launch_bounds__(kThreads) k_edge_fwd(PotArgs a) {
-    using T = Tile<F, K>;
-    constexpr int TE = T::TE, FG = T::FG, PS = T::PS;
-    extern __shared__ float4 smem4[];
-    float* sW1 = reinterpret_cast<float*>(smem4);
-    float* sb1 = sW1 + K * F;
-    float* sW2 = sb1 + F;
-    float* sb2 = sW2 + F * F;
-    float* sBT = sb2 + F;
-    float* sST = sBT + K * TE;
-    float* sP = sST + F * TE;
-    float* sfc = sP + TE * PS;
-    int* sj = reinterpret_cast<int*>(sfc + TE);
-    int* srow = sj + TE;
-    float* srep = reinterpret_cast<float*>(srow + TE);
-    float* sAcc = srep + TE;
-    const int A = a.atoms_per_cta;
-    const int tid = threadIdx.x;
-    const int l = a.layer;
-    const int a0 = blockIdx.x * A;
-    const int a1 = min(a.n_atoms, a0 + A);
-    const int nA = a1 - a0;
-    if (nA <= 0) return;
+// ------------------------------------------------------------ unordered pairs
+// The unordered pairs of the list, one entry (i, j), j > i, each, and for
+// every directed pair e the number pid[e] of its entry. A row's columns
+// ascend, so its pairs with j > i are a suffix. A block takes a range of
+// entries for its 32 atoms with one atomic (the order of the ranges varies
+// from run to run and no result depends on it); the entry's number goes to
+// its own directed pair and, found by bisection in row j, to the reverse one.
+constexpr int kIdxWarps = 8, kIdxRows = 4;     // rows per warp
 
-    for (int t = tid; t < K * F; t += kThreads) sW1[t] = __ldg(a.P + a.off.W1[l] + t);
-    for (int t = tid; t < F * F; t += kThreads) sW2[t] = __ldg(a.P + a.off.W2[l] + t);
-    for (int t = tid; t < F; t += kThreads) {
-        sb1[t] = __ldg(a.P + a.off.b1[l] + t);
-        sb2[t] = __ldg(a.P + a.off.b2[l] + t);
+__global__ void __launch_bounds__(kIdxWarps * 32) k_pair_index(PotArgs a, PairFilter pf) {
+    __shared__ int w_sum[kIdxWarps];
+    __shared__ int blk;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int r0 = (blockIdx.x * kIdxWarps + w) * kIdxRows;
+    int first[kIdxRows], cnt[kIdxRows], total = 0;       // first pair with j > i, and their number
+#pragma unroll
+    for (int q = 0; q < kIdxRows; ++q) {
+        const int i = r0 + q;
+        int n_up = 0;
+        long long end = 0;
+        if (i < a.n_atoms) {
+            const long long beg = min((long long)a.row_ptr[i], a.e_cap);
+            end = min((long long)a.row_ptr[i + 1], a.e_cap);
+            for (long long e = beg + lane; e < end; e += 32) n_up += a.col[e] > i ? 1 : 0;
+        }
+        n_up = __reduce_add_sync(0xffffffffu, n_up);
+        first[q] = (int)end - n_up;
+        cnt[q] = n_up;
+        total += n_up;
     }
-    for (int t = tid; t < A * F; t += kThreads) sAcc[t] = 0.f;
-    // layer 0 also sums the pair repulsion, 1/2 phi(d_ij) per directed pair
-    if (l == 0)
-        for (int t = tid; t < nA; t += kThreads) a.erep[a0 + t] = 0.f;
-
-    const long long e_beg = min((long long)a.row_ptr[a0], a.e_cap);
-    const long long e_end = min((long long)a.row_ptr[a1], a.e_cap);
-    const int fg = tid % FG, eg = tid / FG;
-    const int f0 = fg * 4, e0 = eg * 4;
-    int cur = -1;
-    float run = 0.f;
+    if (lane == 0) w_sum[w] = total;
     __syncthreads();
-
-    for (long long t0 = e_beg; t0 < e_end; t0 += TE) {
-        if (tid < TE) {
-            long long e = t0 + tid;
-            float eb[K];
-            if (e < e_end) {
-                int j = DMTS_IDX(a.col[e], a.n_atoms, a.check), i = DMTS_IDX(a.recv[e], a.n_atoms, a.check);
-                uint4 qi = a.q[i], qj = a.q[j];
-                float3 r = edge_vec(qi, qj, a.frame[qi.w].qscale);
-                float d = sqrtf(r.x * r.x + r.y * r.y + r.z * r.z);
-                float fc;
-                basis_fwd<K>(d, a.pi_over_rc, a.bessel_pref, eb, fc);
-                sfc[tid] = fc;
-                sj[tid] = j;
-                srow[tid] = i - a0;
-                srep[tid] = l == 0 ? 0.5f * rep_phi(d, a.rep_a, a.rep_inv_rho, a.rep_rc, a.rep_pi_over_rc, nullptr) : 0.f;
-            } else {
-#pragma unroll
-                for (int k = 0; k < K; ++k) eb[k] = 0.f;
-                sfc[tid] = 0.f;
-                sj[tid] = a0;
-                srow[tid] = -1;
-                srep[tid] = 0.f;
-            }
-#pragma unroll
-            for (int k = 0; k < K; ++k) sBT[k * TE + tid] = eb[k];
-        }
-        __syncthreads();
-        // GEMM 1: hidden = SiLU(e W1 + b1), stored transposed
-        {
-            float acc[4][4];
-            float4 b = ld4(sb1 + f0);
-#pragma unroll
-            for (int r = 0; r < 4; ++r) { acc[r][0] = b.x; acc[r][1] = b.y; acc[r][2] = b.z; acc[r][3] = b.w; }
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                float4 bv = ld4(sBT + k * TE + e0);
-                float4 wv = ld4(sW1 + k * F + f0);
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[r][c] += f4(bv, r) * f4(wv, c);
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                float sg, s[4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) s[r] = silu_f(acc[r][c], sg);
-                st4(sST + (f0 + c) * TE + e0, make_float4(s[0], s[1], s[2], s[3]));
-            }
-        }
-        __syncthreads();
-        // GEMM 2: phi = hidden W2 + b2; message = fc * phi * u_j
-        {
-            float acc[4][4];
-            float4 b = ld4(sb2 + f0);
-#pragma unroll
-            for (int r = 0; r < 4; ++r) { acc[r][0] = b.x; acc[r][1] = b.y; acc[r][2] = b.z; acc[r][3] = b.w; }
-#pragma unroll 4
-            for (int k = 0; k < F; ++k) {
-                float4 sv = ld4(sST + k * TE + e0);
-                float4 wv = ld4(sW2 + k * F + f0);
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[r][c] += f4(sv, r) * f4(wv, c);
-            }
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                int e = e0 + r;
-                float fc = sfc[e];
-                float4 uj = ldg4(a.u + (size_t)sj[e] * F + f0);
-                st4(sP + e * PS + f0, make_float4(fc * acc[r][0] * uj.x, fc * acc[r][1] * uj.y,
-                                                  fc * acc[r][2] * uj.z, fc * acc[r][3] * uj.w));
-            }
-        }
-        __syncthreads();
-        // segmented row sums, in edge order (thread F: repulsion energy)
-        if (tid < F) {
-            for (int e = 0; e < TE; ++e) {
-                int r = srow[e];
-                if (r < 0) break;
-                if (r != cur) {
-                    if (cur >= 0) sAcc[cur * F + tid] = run;
-                    cur = r;
-                    run = 0.f;
-                }
-                run += sP[e * PS + tid];
-            }
-        } else if (tid == F && l == 0) {
-            for (int e = 0; e < TE; ++e) {
-                int r = srow[e];
-                if (r < 0) break;
-                if (r != cur) {
-                    if (cur >= 0) a.erep[a0 + cur] = run;
-                    cur = r;
-                    run = 0.f;
-                }
-                run += srep[e];
-            }
-        }
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        int sum = 0;
+        for (int k = 0; k < kIdxWarps; ++k) sum += w_sum[k];
+        blk = sum ? atomicAdd(pf.count, sum) : 0;
     }
-    if (tid < F && cur >= 0) sAcc[cur * F + tid] = run;
-    if (tid == F && l == 0 && cur >= 0) a.erep[a0 + cur] = run;
-
     __syncthreads();
-    for (int t = tid; t < nA * F; t += kThreads) a.msg_out[(size_t)a0 * F + t] = sAcc[t];
+    int base = blk;
+    for (int k = 0; k < w; ++k) base += w_sum[k];
+    for (int t = lane; t < total; t += 32) {
+        int q = 0, o = t;
+#pragma unroll
+        for (int k = 0; k < kIdxRows - 1; ++k)
+            if (q == k && o >= cnt[k]) { o -= cnt[k]; ++q; }
+        int e = 0;
+#pragma unroll
+        for (int k = 0; k < kIdxRows; ++k)
+            if (q == k) e = first[k] + o;
+        const int i = r0 + q, j = DMTS_IDX(a.col[e], a.n_atoms, a.check), p = base + t;
+        if (p >= pf.cap) continue;                       // a truncated (overflowed) list: the call is redone
+        pf.pairs[p] = make_int2(i, j);
+        pf.pid[e] = p;
+        int lo = (int)min((long long)a.row_ptr[j], a.e_cap);
+        const int hi = (int)min((long long)a.row_ptr[j + 1], a.e_cap);
+        int n = hi - lo;
+        while (n > 0) {                                  // first column of row j that is >= i
+            const int h = n >> 1;
+            if (a.col[lo + h] < i) { lo += h + 1; n -= h + 1; }
+            else n = h;
+        }
+        if (lo < hi && a.col[lo] == i) pf.pid[lo] = p;
+    }
 }
 
-// ------------------------------------------------------------ backward edge pass
-template <int F, int K>
-__global__ void __launch_bounds__(kThreads) k_edge_bwd(PotArgs a) {
-    using T = Tile<F, K>;
-    constexpr int TE = T::TE, FG = T::FG, PS = T::PS;
-    extern __shared__ float4 smem4[];
-    float* sW1 = reinterpret_cast<float*>(smem4);
-    float* sb1 = sW1 + K * F;
-    float* sW2 = sb1 + F;
-    float* sb2 = sW2 + F * F;
-    float* sW2T = sb2 + F;
-    float* sBT = sW2T + F * F;
-    float* sDT = sBT + K * TE;
-    float* sST = sDT + K * TE;
-    float* sGT = sST + F * TE;
-    float* sP = sGT + F * TE;
-    float* sfc = sP + TE * PS;
-    float* sdfc = sfc + TE;
-    float* sse = sdfc + TE;
-    float* srh = sse + TE;                       // [TE][4] rhat, d
-    int* sj = reinterpret_cast<int*>(srh + 4 * TE);
-    int* srow = sj + TE;
-    float* red1 = reinterpret_cast<float*>(srow + TE) + TE;  // one pad block
-    float* red2 = red1 + TE * FG;
-    float* sAcc = red2 + TE * FG;                // [A][F] ubar
-    float* sF = sAcc + a.atoms_per_cta * F;      // [A][4]
-    float* sV = sF + a.atoms_per_cta * 4;        // [A][8]
-    const int A = a.atoms_per_cta;
-    const int tid = threadIdx.x;
-    const int l = a.layer;
-    const int a0 = blockIdx.x * A;
-    const int a1 = min(a.n_atoms, a0 + A);
-    const int nA = a1 - a0;
-    if (nA <= 0) return;
-    const bool need_ubar = (l > 0);
+// ------------------------------------------------------------ filter of every pair
+// w = fc phi and dw/dd = fc' phi + fc (SiLU'(a) (e' W1)) W2, with
+// a = e W1 + b1 and phi = SiLU(a) W2 + b2, for tiles of 128 pairs.
+//
+// Bound by FP32 FMA issue: 2 (2 KP F + 2 F F) flop per pair and layer against
+// 512 bytes written (F = 64): 639,638 directed pairs, two layers, 13.1 GFLOP in
+// 296 us (ncu: FMA pipe 63 %, DRAM 12 %). Each thread owns 8 pairs x 4 features of both
+// products that share a weight matrix (64 accumulators), as packed f32x2
+// operations over two pairs: one FFMA2 for two FMAs leaves issue slots for the
+// operand loads (five 16-byte shared loads per 64 FMAs). The hidden layer is
+// kept [feature][pair] with a row stride of 132 floats: the four hidden
+// features of a thread are F / 4 apart, so that the eight lanes of a 16-byte
+// store phase fall into distinct banks, while its four output features are
+// adjacent, so that a row of w is written as whole 128-byte lines.
+template <int F, int KP>
+struct FiltTile {
+    static constexpr int FG = F / 4;                     // feature groups of 4
+    static constexpr int TP = 128;                       // pairs per tile
+    static constexpr int NT = TP / 8 * FG;               // threads: 8 pairs x 4 features each
+    static constexpr int TS = TP + 4;
+    float W1[KP * F];                                    // [k][4 fg + c] = W1[k][fg + FG c]
+    float b1[F];                                         // permuted alike
+    float W2[F * F];
+    float b2[F];
+    float B[KP * TS], D[KP * TS];                        // basis and derivative, [k][pair]
+    float S[F * TS], Q[F * TS];                          // SiLU(a), SiLU'(a) (e' W1), [feature][pair]
+    float fc[2][TP], dfc[2][TP];                         // two tiles in turn
+};
 
-    for (int t = tid; t < K * F; t += kThreads) sW1[t] = __ldg(a.P + a.off.W1[l] + t);
-    for (int t = tid; t < F * F; t += kThreads) {
-        float w = __ldg(a.P + a.off.W2[l] + t);
-        sW2[t] = w;
-        sW2T[(t % F) * F + t / F] = w;
-    }
-    for (int t = tid; t < F; t += kThreads) {
-        sb1[t] = __ldg(a.P + a.off.b1[l] + t);
-        sb2[t] = __ldg(a.P + a.off.b2[l] + t);
-    }
-    for (int t = tid; t < A * F; t += kThreads) sAcc[t] = 0.f;
-    for (int t = tid; t < A * 12; t += kThreads) sF[t] = 0.f;   // sF and sV are adjacent
-
-    const long long e_beg = min((long long)a.row_ptr[a0], a.e_cap);
-    const long long e_end = min((long long)a.row_ptr[a1], a.e_cap);
-    const int fg = tid % FG, eg = tid / FG;
-    const int f0 = fg * 4, e0 = eg * 4;
-    // running sums: threads [128, 128+F) for ubar, threads [0, 9) for force/virial
-    int cur = -1;
-    float run = 0.f;
-    __syncthreads();
-
-    for (long long t0 = e_beg; t0 < e_end; t0 += TE) {
-        if (tid < TE) {
-            long long e = t0 + tid;
-            float eb[K], db[K];
-            if (e < e_end) {
-                int j = DMTS_IDX(a.col[e], a.n_atoms, a.check), i = DMTS_IDX(a.recv[e], a.n_atoms, a.check);
-                uint4 qi = a.q[i], qj = a.q[j];
-                float3 r = edge_vec(qi, qj, a.frame[qi.w].qscale);
-                float d = sqrtf(r.x * r.x + r.y * r.y + r.z * r.z);
-                float fc, dfc;
-                basis_bwd<K>(d, a.pi_over_rc, a.bessel_pref, eb, db, fc, dfc);
-                float inv = 1.0f / d;
-                sfc[tid] = fc;
-                sdfc[tid] = dfc;
-                st4(srh + 4 * tid, make_float4(r.x * inv, r.y * inv, r.z * inv, d));
-                sj[tid] = j;
-                srow[tid] = i - a0;
-            } else {
+// acc[p][c] += A[k][p0 + 2p, + 1] W[k][f0 + c] for two operands that share W
+template <int KIN, int TS, int WS, int UNROLL>
+__device__ __forceinline__ void gemm_pair(const float* A0, const float* A1, const float* W, f2::f32x2 (&x)[4][4],
+                                          f2::f32x2 (&y)[4][4]) {
+#pragma unroll UNROLL
+    for (int k = 0; k < KIN; ++k) {
+        const ulonglong2 s01 = *reinterpret_cast<const ulonglong2*>(A0 + k * TS);
+        const ulonglong2 s23 = *reinterpret_cast<const ulonglong2*>(A0 + k * TS + 4);
+        const ulonglong2 q01 = *reinterpret_cast<const ulonglong2*>(A1 + k * TS);
+        const ulonglong2 q23 = *reinterpret_cast<const ulonglong2*>(A1 + k * TS + 4);
+        const float4 w4 = *reinterpret_cast<const float4*>(W + k * WS);
+        const f2::f32x2 s[4] = {s01.x, s01.y, s23.x, s23.y}, q[4] = {q01.x, q01.y, q23.x, q23.y};
+        const f2::f32x2 w[4] = {f2::splat(w4.x), f2::splat(w4.y), f2::splat(w4.z), f2::splat(w4.w)};
 #pragma unroll
-                for (int k = 0; k < K; ++k) { eb[k] = 0.f; db[k] = 0.f; }
-                sfc[tid] = 0.f;
-                sdfc[tid] = 0.f;
-                st4(srh + 4 * tid, make_float4(0.f, 0.f, 0.f, 0.f));
-                sj[tid] = a0;
-                srow[tid] = -1;
-            }
-#pragma unroll
-            for (int k = 0; k < K; ++k) { sBT[k * TE + tid] = eb[k]; sDT[k * TE + tid] = db[k]; }
-        }
-        __syncthreads();
-        // GEMM 1 (+ its derivative companion): a = e W1 + b1, T = e' W1
-        float sp[4][4], tt[4][4];
-        {
-            float acc[4][4];
-            float4 b = ld4(sb1 + f0);
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                acc[r][0] = b.x; acc[r][1] = b.y; acc[r][2] = b.z; acc[r][3] = b.w;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) tt[r][c] = 0.f;
-            }
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                float4 bv = ld4(sBT + k * TE + e0);
-                float4 dv = ld4(sDT + k * TE + e0);
-                float4 wv = ld4(sW1 + k * F + f0);
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        acc[r][c] += f4(bv, r) * f4(wv, c);
-                        tt[r][c] += f4(dv, r) * f4(wv, c);
-                    }
-            }
+        for (int p = 0; p < 4; ++p)
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                float s[4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    float sg;
-                    s[r] = silu_f(acc[r][c], sg);
-                    sp[r][c] = sg * (1.f + acc[r][c] * (1.f - sg));
-                }
-                st4(sST + (f0 + c) * TE + e0, make_float4(s[0], s[1], s[2], s[3]));
+                x[p][c] = f2::fma(s[p], w[c], x[p][c]);
+                y[p][c] = f2::fma(q[p], w[c], y[p][c]);
             }
+    }
+}
+
+template <int F, int KP>
+__global__ void __launch_bounds__(FiltTile<F, KP>::NT, F == 64 ? 2 : 4) k_pair_filter(PotArgs a, PairFilter pf, int K,
+                                                                                      int l0, int l1, int a0, int a1) {
+    using T = FiltTile<F, KP>;
+    constexpr int TP = T::TP, TS = T::TS, FG = T::FG, NT = T::NT;
+    extern __shared__ float4 smem4[];
+    T& S = *reinterpret_cast<T*>(smem4);
+    const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+    const int fg = (F == 64 ? (wp & 1) * 8 : 0) + (lane & 7);
+    const int p0 = 8 * ((F == 64 ? wp >> 1 : wp) * 4 + (lane >> 3));
+    const int f0 = 4 * fg;
+    // the pairs: the unordered ones, or (chunked) the directed pairs of atoms a0 .. a1
+    const bool half = pf.chunk_atoms == 0;
+    const long long e_beg = half ? 0 : min((long long)a.row_ptr[a0], a.e_cap);
+    const long long n_pairs = half ? min((long long)*pf.count, pf.cap)
+                                   : min(min((long long)a.row_ptr[a1], a.e_cap) - e_beg, pf.cap);
+    const long long tiles = (n_pairs + TP - 1) / TP, units = tiles * (l1 - l0);
+    int cur = -1, buf = 0;
+    for (long long unit = blockIdx.x; unit < units; unit += gridDim.x, buf ^= 1) {
+        const int l = l0 + (int)(unit / tiles);
+        const long long t0 = (unit - (l - l0) * tiles) * TP;
+        if (l != cur) {                                  // this layer's weights
+            __syncthreads();
+            for (int t = tid; t < KP * F; t += NT) {
+                const int k = t / F, r = t % F, f = (r >> 2) + FG * (r & 3);
+                S.W1[t] = k < K ? __ldg(a.P + a.off.W1[l] + k * F + f) : 0.f;
+            }
+            for (int t = tid; t < F * F; t += NT) S.W2[t] = __ldg(a.P + a.off.W2[l] + t);
+            for (int t = tid; t < F; t += NT) {
+                S.b1[t] = __ldg(a.P + a.off.b1[l] + (t >> 2) + FG * (t & 3));
+                S.b2[t] = __ldg(a.P + a.off.b2[l] + t);
+            }
+            cur = l;
         }
-        __syncthreads();
-        // GEMM 2: phi = s W2 + b2; g = mbar_i u_j + mbar_j u_i; partial g.phi;
-        // G^T for GEMM 3; ubar message w * mbar_j
-        {
-            float acc[4][4];
-            float4 b = ld4(sb2 + f0);
-#pragma unroll
-            for (int r = 0; r < 4; ++r) { acc[r][0] = b.x; acc[r][1] = b.y; acc[r][2] = b.z; acc[r][3] = b.w; }
-#pragma unroll 4
-            for (int k = 0; k < F; ++k) {
-                float4 sv = ld4(sST + k * TE + e0);
-                float4 wv = ld4(sW2 + k * F + f0);
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[r][c] += f4(sv, r) * f4(wv, c);
-            }
-            float g[4][4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                int e = e0 + r;
-                int j = sj[e];
-                int rr = srow[e];
-                int i = rr < 0 ? a0 : a0 + rr;
-                float4 uj = ldg4(a.u + (size_t)j * F + f0);
-                float4 mj = ldg4(a.mbar + (size_t)j * F + f0);
-                float4 ui = ldg4(a.u + (size_t)i * F + f0);
-                float4 mi = ldg4(a.mbar + (size_t)i * F + f0);
-                g[r][0] = mi.x * uj.x + mj.x * ui.x;
-                g[r][1] = mi.y * uj.y + mj.y * ui.y;
-                g[r][2] = mi.z * uj.z + mj.z * ui.z;
-                g[r][3] = mi.w * uj.w + mj.w * ui.w;
-                float dot = g[r][0] * acc[r][0] + g[r][1] * acc[r][1] + g[r][2] * acc[r][2] + g[r][3] * acc[r][3];
-                red1[e * FG + fg] = dot;
-                if (need_ubar) {
-                    float fc = sfc[e];
-                    st4(sP + e * PS + f0, make_float4(fc * acc[r][0] * mj.x, fc * acc[r][1] * mj.y,
-                                                      fc * acc[r][2] * mj.z, fc * acc[r][3] * mj.w));
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                st4(sGT + (f0 + c) * TE + e0, make_float4(g[0][c], g[1][c], g[2][c], g[3][c]));
-        }
-        __syncthreads();
-        // GEMM 3: abar = G W2^T; partial sum_k abar_k SiLU'(a_k) T_k
-        {
-            float acc[4][4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
-#pragma unroll 4
-            for (int k = 0; k < F; ++k) {
-                float4 gv = ld4(sGT + k * TE + e0);
-                float4 wv = ld4(sW2T + k * F + f0);
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[r][c] += f4(gv, r) * f4(wv, c);
-            }
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                float p = 0.f;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) p += acc[r][c] * sp[r][c] * tt[r][c];
-                red2[(e0 + r) * FG + fg] = p;
-            }
-        }
-        __syncthreads();
-        // per-edge dE/dd, and the ubar row sums (threads 128..128+F)
-        if (tid < TE) {
-            float s1 = 0.f, s2 = 0.f;
-#pragma unroll
-            for (int k = 0; k < FG; ++k) { s1 += red1[tid * FG + k]; s2 += red2[tid * FG + k]; }
-            float se = sdfc[tid] * s1 + sfc[tid] * s2;
-            if (l == 0 && srow[tid] >= 0) {
-                float dphi;
-                (void)rep_phi(srh[4 * tid + 3], a.rep_a, a.rep_inv_rho, a.rep_rc, a.rep_pi_over_rc, &dphi);
-                se += dphi;
-            }
-            sse[tid] = se;
-        } else if (need_ubar && tid >= 128 && tid < 128 + F) {
-            int ff = tid - 128;
-            for (int e = 0; e < TE; ++e) {
-                int r = srow[e];
-                if (r < 0) break;
-                if (r != cur) {
-                    if (cur >= 0) sAcc[cur * F + ff] = run;
-                    cur = r;
-                    run = 0.f;
-                }
-                run += sP[e * PS + ff];
-            }
-        }
-        __syncthreads();
-        // force (3) and virial (6) row sums, in edge order
-        if (tid < 9) {
-            for (int e = 0; e < TE; ++e) {
-                int r = srow[e];
-                if (r < 0) break;
-                if (r != cur) {
-                    if (cur >= 0) {
-                        if (tid < 3) sF[cur * 4 + tid] = run;
-                        else sV[cur * 8 + tid - 3] = run;
-                    }
-                    cur = r;
-                    run = 0.f;
-                }
-                float4 rh = ld4(srh + 4 * e);
-                float s = sse[e];
-                float val;
-                if (tid < 3) {
-                    val = s * f4(rh, tid);
+        if (tid < TP) {
+            float eb[KP], db[KP], fc = 0.f, dfc = 0.f;
+            const long long p = t0 + tid;
+            if (p < n_pairs) {
+                int i, j;
+                if (half) {
+                    const int2 ij = pf.pairs[p];
+                    i = DMTS_IDX(ij.x, a.n_atoms, a.check);
+                    j = DMTS_IDX(ij.y, a.n_atoms, a.check);
                 } else {
-                    // W_ab = -1/2 sum_directed s d rhat_a rhat_b; components xx yy zz xy xz yz
-                    const int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};
-                    int c = tid - 3;
-                    val = -0.5f * s * rh.w * f4(rh, ia[c]) * f4(rh, ib[c]);
+                    i = DMTS_IDX(a.recv[e_beg + p], a.n_atoms, a.check);
+                    j = DMTS_IDX(a.col[e_beg + p], a.n_atoms, a.check);
                 }
-                run += val;
+                const uint4 qi = a.q[i], qj = a.q[j];
+                const float3 r = edge_vec(qi, qj, a.frame[qi.w].qscale);
+                const float d = sqrtf(r.x * r.x + r.y * r.y + r.z * r.z);
+                basis_pair<KP>(d, K, a.pi_over_rc, a.bessel_pref, eb, db, fc, dfc);
+            } else {
+#pragma unroll
+                for (int k = 0; k < KP; ++k) eb[k] = db[k] = 0.f;
+            }
+#pragma unroll
+            for (int k = 0; k < KP; ++k) {
+                S.B[k * TS + tid] = eb[k];
+                S.D[k * TS + tid] = db[k];
+            }
+            S.fc[buf][tid] = fc;
+            S.dfc[buf][tid] = dfc;
+        }
+        __syncthreads();
+        f2::f32x2 x[4][4], y[4][4];
+        {
+            const float4 b = *reinterpret_cast<const float4*>(S.b1 + f0);
+            const float bc[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    x[p][c] = f2::splat(bc[c]);
+                    y[p][c] = 0ull;
+                }
+            gemm_pair<KP, TS, F, KP>(S.B + p0, S.D + p0, S.W1 + f0, x, y);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {                // hidden feature fg + FG c of the thread's 8 pairs
+                float s[8], q[8];
+#pragma unroll
+                for (int p = 0; p < 8; ++p) {
+                    const float v = (p & 1) ? f2::hi(x[p >> 1][c]) : f2::lo(x[p >> 1][c]);
+                    const float t = (p & 1) ? f2::hi(y[p >> 1][c]) : f2::lo(y[p >> 1][c]);
+                    const float sg = __fdividef(1.0f, 1.0f + __expf(-v));
+                    s[p] = v * sg;
+                    q[p] = sg * (1.f + v * (1.f - sg)) * t;
+                }
+                float* ds = S.S + (fg + FG * c) * TS + p0;
+                float* dq = S.Q + (fg + FG * c) * TS + p0;
+                *reinterpret_cast<float4*>(ds) = make_float4(s[0], s[1], s[2], s[3]);
+                *reinterpret_cast<float4*>(ds + 4) = make_float4(s[4], s[5], s[6], s[7]);
+                *reinterpret_cast<float4*>(dq) = make_float4(q[0], q[1], q[2], q[3]);
+                *reinterpret_cast<float4*>(dq + 4) = make_float4(q[4], q[5], q[6], q[7]);
             }
         }
         __syncthreads();
+        {
+            const float4 b = *reinterpret_cast<const float4*>(S.b2 + f0);
+            const float bc[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    x[p][c] = f2::splat(bc[c]);
+                    y[p][c] = 0ull;
+                }
+            gemm_pair<F, TS, F, 4>(S.S + p0, S.Q + p0, S.W2 + f0, x, y);
+            const size_t row0 = (size_t)(half ? l : 0) * 2 * pf.cap;
+#pragma unroll
+            for (int p = 0; p < 8; ++p) {
+                const long long r = t0 + p0 + p;
+                if (r >= n_pairs) break;
+                const float fc = S.fc[buf][p0 + p], dfc = S.dfc[buf][p0 + p];
+                float ph[4], ps[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    ph[c] = (p & 1) ? f2::hi(x[p >> 1][c]) : f2::lo(x[p >> 1][c]);
+                    ps[c] = (p & 1) ? f2::hi(y[p >> 1][c]) : f2::lo(y[p >> 1][c]);
+                }
+                float* w = pf.w + (row0 + r) * F + f0;
+                *reinterpret_cast<float4*>(w) = make_float4(fc * ph[0], fc * ph[1], fc * ph[2], fc * ph[3]);
+                *reinterpret_cast<float4*>(w + (size_t)pf.cap * F) =
+                    make_float4(dfc * ph[0] + fc * ps[0], dfc * ph[1] + fc * ps[1], dfc * ph[2] + fc * ps[2],
+                                dfc * ph[3] + fc * ps[3]);
+            }
+        }
+        // the next tile's basis, SiLU and fc tiles: B and D were last read before the
+        // second barrier, fc alternates, S and Q are written after the next first barrier
     }
-    if (cur >= 0) {
-        if (tid < 3) sF[cur * 4 + tid] = run;
-        else if (tid < 9) sV[cur * 8 + tid - 3] = run;
-        else if (tid >= 128 && tid < 128 + F) sAcc[cur * F + tid - 128] = run;
-    }
-    __syncthreads();
-    // forces / virial of the CTA's atoms
-    for (int t = tid; t < nA * 3; t += kThreads) {
-        int r = t / 3, c = t % 3;
-        size_t o = (size_t)c * a.n_atoms + a0 + r;
-        a.force[o] = a.accumulate ? a.force[o] + sF[r * 4 + c] : sF[r * 4 + c];
-    }
-    for (int t = tid; t < nA * 6; t += kThreads) {
-        int r = t / 6, c = t % 6;
-        size_t o = (size_t)(a0 + r) * 6 + c;
-        a.vir6[o] = a.accumulate ? a.vir6[o] + sV[r * 8 + c] : sV[r * 8 + c];
-    }
-    if (need_ubar)
-        for (int t = tid; t < nA * F; t += kThreads) a.msg_out[(size_t)a0 * F + t] = sAcc[t];
 }
 
-template <int F, int K>
-void set_smem_attrs() {
-    smem_opt_in((const void*)k_edge_fwd<F, K>, 227 * 1024);
-    smem_opt_in((const void*)k_edge_bwd<F, K>, 227 * 1024);
-}
+// ------------------------------------------------------------ gathers
+// One warp per atom; a row of F floats is read by F / 4 lanes, 16 bytes each,
+// so one warp instruction reads 2 (F = 64) or 4 (F = 32) whole rows. Bound by
+// the bytes of the gathered rows through L2: w and u_j forward (512 bytes per
+// directed pair at F = 64), dw/dd, u_j, mbar_j and, above layer 0, w backward
+// (768 or 1,024 bytes).
 
-template <int F, int K>
-void fwd_launch(const PotArgs& a, cudaStream_t s) {
-    set_smem_attrs<F, K>();
-    int grid = (a.n_atoms + a.atoms_per_cta - 1) / a.atoms_per_cta;
-    size_t smem = sizeof(float) * fwd_smem_floats<F, K>(a.atoms_per_cta);
-    k_edge_fwd<F, K><<<grid, kThreads, smem, s>>>(a);
-}
-
-template <int F, int K>
-void bwd_launch(const PotArgs& a, cudaStream_t s) {
-    set_smem_attrs<F, K>();
-    int grid = (a.n_atoms + a.atoms_per_cta - 1) / a.atoms_per_cta;
-    size_t smem = sizeof(float) * bwd_smem_floats<F, K>(a.atoms_per_cta);
-    k_edge_bwd<F, K><<<grid, kThreads, smem, s>>>(a);
+// Filter row of directed pair e, or -1 if there is none: after an overflow
+// (the call will be redone) a pair may lack its entry, and a stale number is
+// recognised by the pair stored there.
+__device__ __forceinline__ long long filter_row(const PotArgs& a, const PairFilter& pf, long long e, long long e_beg,
+                                                int i, int j, bool overflow) {
+    if (pf.chunk_atoms) return e - e_beg < pf.cap ? e - e_beg : -1;
+    const int p = pf.pid[e];
+    if (!overflow) return DMTS_IDX(p, pf.cap, a.check);
+    if (p < 0 || p >= pf.cap) return -1;
+    const int2 ij = pf.pairs[p];
+    return ij.x == min(i, j) && ij.y == max(i, j) ? p : -1;
 }
 
 template <int F>
-int max_atoms(int K, bool bwd) {
-    // largest A whose shared memory fits
-    int best = 0;
-    for (int A = 8; A <= 256; A += 8) {
-        long long fl;
-        long long region;
-        switch (K) {
-            default: return 0;
-#define DMTS_K(KK)                                                                   \
-    case KK:                                                                         \
-        fl = bwd ? bwd_smem_floats<F, KK>(A) : fwd_smem_floats<F, KK>(A);            \
-        break;
-            DMTS_K(1) DMTS_K(2) DMTS_K(3) DMTS_K(4) DMTS_K(5) DMTS_K(6) DMTS_K(7) DMTS_K(8)
-            DMTS_K(9) DMTS_K(10) DMTS_K(11) DMTS_K(12) DMTS_K(13) DMTS_K(14) DMTS_K(15) DMTS_K(16)
-#undef DMTS_K
+__global__ void __launch_bounds__(kThreads) k_gather_fwd(PotArgs a, PairFilter pf, int a0, int a1) {
+    constexpr int LPR = F / 4, RPI = 32 / LPR;
+    const int lane = threadIdx.x & 31, sub = lane / LPR, ch = lane % LPR;
+    const bool overflow = a.check[kFlagOverflow] != 0;
+    const bool rep_on = a.layer == 0 && a.energy;
+    const float* W = pf.w + (size_t)(pf.chunk_atoms ? 0 : a.layer) * 2 * pf.cap * F + 4 * ch;
+    const float* U = a.u + 4 * ch;
+    const long long e_beg = min((long long)a.row_ptr[a0], a.e_cap);
+    const int last = min(a1, a0 + (int)(blockIdx.x + 1) * a.atoms_per_cta);
+    for (int i = a0 + blockIdx.x * a.atoms_per_cta + (threadIdx.x >> 5); i < last; i += kThreads / 32) {
+        const long long beg = min((long long)a.row_ptr[i], a.e_cap), end = min((long long)a.row_ptr[i + 1], a.e_cap);
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        float rep = 0.f;
+        const uint4 qi = a.q[i];
+        const float qscale = a.frame[qi.w].qscale;
+        for (long long b = beg; b < end; b += 32) {
+            const long long e = b + lane;
+            int j = 0;
+            long long p = -1;
+            if (e < end) {
+                j = DMTS_IDX(a.col[e], a.n_atoms, a.check);
+                p = filter_row(a, pf, e, e_beg, i, j, overflow);
+                if (rep_on) {                            // 1/2 phi(d_ij) per directed pair
+                    const float3 r = edge_vec(qi, a.q[j], qscale);
+                    const float d = sqrtf(r.x * r.x + r.y * r.y + r.z * r.z);
+                    rep += 0.5f * rep_phi(d, a.rep_a, a.rep_inv_rho, a.rep_rc, a.rep_pi_over_rc, nullptr);
+                }
+            }
+            const int n = (int)min(32ll, end - b);
+#pragma unroll 4
+            for (int k = 0; k < n; k += RPI) {
+                const long long pk = __shfl_sync(0xffffffffu, p, k + sub);
+                const int jk = __shfl_sync(0xffffffffu, j, k + sub);
+                if (pk >= 0) {
+                    const float4 w = __ldg(reinterpret_cast<const float4*>(W + pk * F));
+                    const float4 u = __ldg(reinterpret_cast<const float4*>(U + (size_t)jk * F));
+                    acc.x += w.x * u.x;
+                    acc.y += w.y * u.y;
+                    acc.z += w.z * u.z;
+                    acc.w += w.w * u.w;
+                }
+            }
         }
-        (void)region;
-        region = 0;
-        if (fl * 4 <= 227 * 1024) best = A;
+#pragma unroll
+        for (int o = LPR; o < 32; o <<= 1) {
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+            acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o);
+            acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
+        }
+        if (sub == 0) *reinterpret_cast<float4*>(a.msg_out + (size_t)i * F + 4 * ch) = acc;
+        if (rep_on) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) rep += __shfl_xor_sync(0xffffffffu, rep, o);
+            if (lane == 0) a.erep[i] = rep;
+        }
     }
-    return best;
+    // every reader of the pair count has finished: zero for the next index
+    if (a.layer == 0 && !pf.chunk_atoms && blockIdx.x == 0 && threadIdx.x == 0) *pf.count = 0;
+}
+
+// NV = 9: forces and the per-atom virial; NV = 3: forces only.
+// L0: layer 0, whose u does not depend on the positions (no ubar).
+// The dot products g . dw/dd of a chunk of 32 pairs are partial sums in
+// registers, one per row instruction, reduced over the lanes of a row by
+// halving exchanges (LPR - 1 shuffles for LPR sums) that leave the sum of
+// pair RPI ch + sub in lane (sub, ch), the lane that holds its geometry.
+template <int F, int NV, bool L0>
+__global__ void __launch_bounds__(kThreads) k_gather_bwd(PotArgs a, PairFilter pf, int a0, int a1) {
+    constexpr int LPR = F / 4, RPI = 32 / LPR;
+    const int lane = threadIdx.x & 31, sub = lane / LPR, ch = lane % LPR;
+    const bool overflow = a.check[kFlagOverflow] != 0;
+    const float* W = pf.w + (size_t)(pf.chunk_atoms ? 0 : a.layer) * 2 * pf.cap * F + 4 * ch;
+    const float* DW = W + (size_t)pf.cap * F;
+    const float* U = a.u + 4 * ch;
+    const float* MB = a.mbar + 4 * ch;
+    const long long e_beg = min((long long)a.row_ptr[a0], a.e_cap);
+    const int last = min(a1, a0 + (int)(blockIdx.x + 1) * a.atoms_per_cta);
+    for (int i = a0 + blockIdx.x * a.atoms_per_cta + (threadIdx.x >> 5); i < last; i += kThreads / 32) {
+        const long long beg = min((long long)a.row_ptr[i], a.e_cap), end = min((long long)a.row_ptr[i + 1], a.e_cap);
+        const uint4 qi = a.q[i];
+        const float qscale = a.frame[qi.w].qscale;
+        const float4 ui = __ldg(reinterpret_cast<const float4*>(U + (size_t)i * F));
+        const float4 mi = __ldg(reinterpret_cast<const float4*>(MB + (size_t)i * F));
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        float fv[NV];
+#pragma unroll
+        for (int c = 0; c < NV; ++c) fv[c] = 0.f;
+        for (long long b = beg; b < end; b += 32) {
+            const long long e = b + RPI * ch + sub;       // this lane's pair of the chunk
+            int j = 0;
+            long long p = -1;
+            float rx = 0.f, ry = 0.f, rz = 0.f, d = 1.f;
+            if (e < end) {
+                j = DMTS_IDX(a.col[e], a.n_atoms, a.check);
+                p = filter_row(a, pf, e, e_beg, i, j, overflow);
+                const float3 r = edge_vec(qi, a.q[j], qscale);
+                d = sqrtf(r.x * r.x + r.y * r.y + r.z * r.z);
+                const float inv = 1.0f / d;
+                rx = r.x * inv; ry = r.y * inv; rz = r.z * inv;
+            }
+            const int n = (int)min(32ll, end - b);
+            float s[LPR];
+#pragma unroll
+            for (int k = 0; k < LPR; ++k) {
+                s[k] = 0.f;
+                if (RPI * k < n) {                        // warp-uniform
+                    const long long pk = __shfl_sync(0xffffffffu, p, sub * LPR + k);
+                    const int jk = __shfl_sync(0xffffffffu, j, sub * LPR + k);
+                    if (pk >= 0) {
+                        const float4 dw = __ldg(reinterpret_cast<const float4*>(DW + pk * F));
+                        const float4 uj = __ldg(reinterpret_cast<const float4*>(U + (size_t)jk * F));
+                        const float4 mj = __ldg(reinterpret_cast<const float4*>(MB + (size_t)jk * F));
+                        float t = (mi.x * uj.x + mj.x * ui.x) * dw.x;
+                        t += (mi.y * uj.y + mj.y * ui.y) * dw.y;
+                        t += (mi.z * uj.z + mj.z * ui.z) * dw.z;
+                        t += (mi.w * uj.w + mj.w * ui.w) * dw.w;
+                        s[k] = t;
+                        if (!L0) {
+                            const float4 w = __ldg(reinterpret_cast<const float4*>(W + pk * F));
+                            acc.x += w.x * mj.x;
+                            acc.y += w.y * mj.y;
+                            acc.z += w.z * mj.z;
+                            acc.w += w.w * mj.w;
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int m = LPR / 2; m > 0; m >>= 1) {
+                const bool up = (ch & m) != 0;
+#pragma unroll
+                for (int k = 0; k < m; ++k) {
+                    const float give = up ? s[k] : s[k + m], keep = up ? s[k + m] : s[k];
+                    s[k] = keep + __shfl_xor_sync(0xffffffffu, give, m);
+                }
+            }
+            if (e < end) {
+                float se = s[0];                          // dE/dd of this lane's pair
+                if (L0) {
+                    float dphi;
+                    (void)rep_phi(d, a.rep_a, a.rep_inv_rho, a.rep_rc, a.rep_pi_over_rc, &dphi);
+                    se += dphi;
+                }
+                fv[0] += se * rx;
+                fv[1] += se * ry;
+                fv[2] += se * rz;
+                if constexpr (NV == 9) {
+                    const float hv = -0.5f * se * d;      // W_ab = -1/2 sum_directed s d rhat_a rhat_b
+                    fv[3] += hv * rx * rx; fv[4] += hv * ry * ry; fv[5] += hv * rz * rz;
+                    fv[6] += hv * rx * ry; fv[7] += hv * rx * rz; fv[8] += hv * ry * rz;
+                }
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < NV; ++c)
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) fv[c] += __shfl_xor_sync(0xffffffffu, fv[c], o);
+        if (lane == 0) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                float* f = a.force + (size_t)c * a.n_atoms + i;
+                *f = a.accumulate ? *f + fv[c] : fv[c];
+            }
+            if constexpr (NV == 9)
+#pragma unroll
+                for (int c = 0; c < 6; ++c) {
+                    float* v = a.vir6 + (size_t)i * 6 + c;
+                    *v = a.accumulate ? *v + fv[3 + c] : fv[3 + c];
+                }
+        }
+        if (!L0) {
+#pragma unroll
+            for (int o = LPR; o < 32; o <<= 1) {
+                acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+                acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+                acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o);
+                acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
+            }
+            if (sub == 0) *reinterpret_cast<float4*>(a.msg_out + (size_t)i * F + 4 * ch) = acc;
+        }
+    }
+}
+
+// ------------------------------------------------------------ launches
+// Filters of layers l0 .. l1 - 1 for the unordered pairs, or (chunked) the
+// directed pairs of atoms a0 .. a1 - 1. Persistent: two CTAs of 256 threads
+// per SM at F = 64, four of 128 at F = 32 (shared memory and registers).
+template <int F, int KP>
+void filter_go(const PotArgs& a, int K, int l0, int l1, int a0, int a1, cudaStream_t s) {
+    using T = FiltTile<F, KP>;
+    smem_opt_in((const void*)k_pair_filter<F, KP>, (int)sizeof(T));
+    const long long tiles = (a.filter.cap + T::TP - 1) / T::TP * (l1 - l0);
+    const int grid = (int)std::min<long long>(tiles, (long long)kSmCount * (F == 64 ? 2 : 4));
+    k_pair_filter<F, KP><<<std::max(1, grid), T::NT, sizeof(T), s>>>(a, a.filter, K, l0, l1, a0, a1);
+    count_launch();
+}
+
+template <int F>
+void filters(const PotArgs& a, int K, int l0, int l1, int a0, int a1, cudaStream_t s) {
+    if (K <= 8) filter_go<F, 8>(a, K, l0, l1, a0, a1, s);
+    else filter_go<F, 16>(a, K, l0, l1, a0, a1, s);
+}
+
+inline int gather_blocks(const PotArgs& a, int a0, int a1) { return (a1 - a0 + a.atoms_per_cta - 1) / a.atoms_per_cta; }
+
+template <int F>
+void fwd_go(const PotArgs& a, int K, cudaStream_t s) {
+    if (!a.filter.chunk_atoms) {
+        if (a.layer == 0) {                              // the filters of every layer at once
+            k_pair_index<<<(a.n_atoms + kIdxWarps * kIdxRows - 1) / (kIdxWarps * kIdxRows), kIdxWarps * 32, 0, s>>>(
+                a, a.filter);
+            count_launch();
+            filters<F>(a, K, 0, a.n_layers, 0, a.n_atoms, s);
+        }
+        k_gather_fwd<F><<<gather_blocks(a, 0, a.n_atoms), kThreads, 0, s>>>(a, a.filter, 0, a.n_atoms);
+        count_launch();
+        return;
+    }
+    for (int a0 = 0; a0 < a.n_atoms; a0 += a.filter.chunk_atoms) {
+        const int a1 = std::min(a.n_atoms, a0 + a.filter.chunk_atoms);
+        filters<F>(a, K, a.layer, a.layer + 1, a0, a1, s);
+        k_gather_fwd<F><<<gather_blocks(a, a0, a1), kThreads, 0, s>>>(a, a.filter, a0, a1);
+        count_launch();
+    }
+}
+
+template <int F, int NV>
+void gather_bwd(const PotArgs& a, int a0, int a1, cudaStream_t s) {
+    const int grid = gather_blocks(a, a0, a1);
+    if (a.layer == 0) k_gather_bwd<F, NV, true><<<grid, kThreads, 0, s>>>(a, a.filter, a0, a1);
+    else k_gather_bwd<F, NV, false><<<grid, kThreads, 0, s>>>(a, a.filter, a0, a1);
+    count_launch();
+}
+
+template <int F>
+void bwd_go(const PotArgs& a, int K, cudaStream_t s) {
+    const int step = a.filter.chunk_atoms ? a.filter.chunk_atoms : a.n_atoms;
+    for (int a0 = 0; a0 < a.n_atoms; a0 += step) {
+        const int a1 = std::min(a.n_atoms, a0 + step);
+        if (a.filter.chunk_atoms) filters<F>(a, K, a.layer, a.layer + 1, a0, a1, s);
+        if (a.virial) gather_bwd<F, 9>(a, a0, a1, s);
+        else gather_bwd<F, 3>(a, a0, a1, s);
+    }
 }
 
 }  // namespace
-
-#define DMTS_DISPATCH(FN, F_, K_, ...)                                                       \
-    do {                                                                                     \
-        bool ok_ = false;                                                                    \
-        if (F_ == 64) {                                                                      \
-            switch (K_) {                                                                    \
-                case 1: FN<64, 1>(__VA_ARGS__); ok_ = true; break;                           \
-                case 2: FN<64, 2>(__VA_ARGS__); ok_ = true; break;                           \
-                case 3: FN<64, 3>(__VA_ARGS__); ok_ = true; break;                           \
-                case 4: FN<64, 4>(__VA_ARGS__); ok_ = true; break;                           \
-                case 5: FN<64, 5>(__VA_ARGS__); ok_ = true; break;                           \
-                case 6: FN<64, 6>(__VA_ARGS__); ok_ = true; break;                           \
-                case 7: FN<64, 7>(__VA_ARGS__); ok_ = true; break;                           \
-                case 8: FN<64, 8>(__VA_ARGS__); ok_ = true; break;                           \
-                case 9: FN<64, 9>(__VA_ARGS__); ok_ = true; break;                           \
-                case 10: FN<64, 10>(__VA_ARGS__); ok_ = true; break;                         \
-                case 11: FN<64, 11>(__VA_ARGS__); ok_ = true; break;                         \
-                case 12: FN<64, 12>(__VA_ARGS__); ok_ = true; break;                         \
-                case 13: FN<64, 13>(__VA_ARGS__); ok_ = true; break;                         \
-                case 14: FN<64, 14>(__VA_ARGS__); ok_ = true; break;                         \
-                case 15: FN<64, 15>(__VA_ARGS__); ok_ = true; break;                         \
-                case 16: FN<64, 16>(__VA_ARGS__); ok_ = true; break;                         \
-            }                                                                                \
-        } else if (F_ == 32) {                                                               \
-            switch (K_) {                                                                    \
-                case 1: FN<32, 1>(__VA_ARGS__); ok_ = true; break;                           \
-                case 2: FN<32, 2>(__VA_ARGS__); ok_ = true; break;                           \
-                case 3: FN<32, 3>(__VA_ARGS__); ok_ = true; break;                           \
-                case 4: FN<32, 4>(__VA_ARGS__); ok_ = true; break;                           \
-                case 5: FN<32, 5>(__VA_ARGS__); ok_ = true; break;                           \
-                case 6: FN<32, 6>(__VA_ARGS__); ok_ = true; break;                           \
-                case 7: FN<32, 7>(__VA_ARGS__); ok_ = true; break;                           \
-                case 8: FN<32, 8>(__VA_ARGS__); ok_ = true; break;                           \
-                case 9: FN<32, 9>(__VA_ARGS__); ok_ = true; break;                           \
-                case 10: FN<32, 10>(__VA_ARGS__); ok_ = true; break;                         \
-                case 11: FN<32, 11>(__VA_ARGS__); ok_ = true; break;                         \
-                case 12: FN<32, 12>(__VA_ARGS__); ok_ = true; break;                         \
-                case 13: FN<32, 13>(__VA_ARGS__); ok_ = true; break;                         \
-                case 14: FN<32, 14>(__VA_ARGS__); ok_ = true; break;                         \
-                case 15: FN<32, 15>(__VA_ARGS__); ok_ = true; break;                         \
-                case 16: FN<32, 16>(__VA_ARGS__); ok_ = true; break;                         \
-            }                                                                                \
-        }                                                                                    \
-        (void)sizeof(ok_);                                                                   \
-    } while (0)
 
 void launch_embed(const PotArgs& a, int F, cudaStream_t s) {
     if (a.n_atoms == 0) return;
@@ -639,20 +597,14 @@ void launch_embed(const PotArgs& a, int F, cudaStream_t s) {
 
 void launch_edge_fwd_f32(const PotArgs& a, int F, int K, cudaStream_t s) {
     if (a.n_atoms == 0) return;
-    DMTS_DISPATCH(fwd_launch, F, K, a, s);
-    count_launch();
+    if (F == 64) fwd_go<64>(a, K, s);
+    else fwd_go<32>(a, K, s);
 }
 
 void launch_edge_bwd_f32(const PotArgs& a, int F, int K, cudaStream_t s) {
     if (a.n_atoms == 0) return;
-    DMTS_DISPATCH(bwd_launch, F, K, a, s);
-    count_launch();
-}
-
-int max_atoms_per_cta_f32(int F, int K, bool bwd) {
-    if (F == 64) return max_atoms<64>(K, bwd);
-    if (F == 32) return max_atoms<32>(K, bwd);
-    return 0;
+    if (F == 64) bwd_go<64>(a, K, s);
+    else bwd_go<32>(a, K, s);
 }
 
 // ------------------------------------------------------------ reductions
