@@ -251,7 +251,7 @@ def roofline_of(D, prec, stages_big, E_big, ba):
     if prec == D.FP32:
         # w and dw/dd of every layer, 4 F (K + F) flop per unordered pair and layer; the other stages are
         # gathers: g . dw/dd and w * mbar (8 F) or w * u (2 F) per directed pair
-        flop_edge = {"edge_fwd_l0": ba.n_layers * 2 * F * (K + F)}.get(dom, 8 * F if dom.startswith("edge_bwd") else 2 * F)
+        flop_edge = {"edge_fwd_l0": getattr(ba, "n_layers", 1) * 2 * F * (K + F)}.get(dom, 8 * F if dom.startswith("edge_bwd") else 2 * F)
         peak, bound, src, kind = FP32_SIMT_TFLOPS, "alu", "derived: 152 SMs x 128 FP32 lanes x 2 x 2.07 GHz", "FP32 SIMT"
     else:
         # the algorithmic edge-GEMM work per pair and layer, K padded to 16: one pass 2F(16 + F) forward,
