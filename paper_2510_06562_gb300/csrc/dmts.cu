@@ -203,6 +203,7 @@ struct dmts_ctx {
     std::vector<int> h_off;
     std::vector<double> h_box;
     int *d_off = nullptr, *d_species = nullptr, *d_sys = nullptr;
+    int* d_first_of = nullptr;   // [N] the first atom of each atom's species
     double *d_box = nullptr, *d_mass = nullptr, *d_inv_m = nullptr;
     double *d_x = nullptr, *d_v = nullptr;
     uint4* d_q = nullptr;
@@ -321,7 +322,7 @@ int check_model(const dmts_model_desc* d, const char* name) {
 
 void free_model_nbr(Model& m) {
     dfree(m.nbr_tmp); dfree(m.col); dfree(m.recv); dfree(m.vl_rows); dfree(m.carry);
-    dfree(m.filt.w); dfree(m.filt.pairs); dfree(m.filt.pid); dfree(m.filt.count);
+    dfree(m.filt.w); dfree(m.filt.se); dfree(m.filt.pairs); dfree(m.filt.pid); dfree(m.filt.count);
     m.nbr_tmp = m.col = m.recv = m.vl_rows = nullptr;
     m.carry = nullptr;
     m.filt = PairFilter{};
@@ -346,6 +347,7 @@ cudaError_t alloc_filters(Model& m) {
     cudaError_t e;
     if (half * row * m.L <= kFilterBytes) {
         e = dalloc(&f.w, half * (row / sizeof(float)) * m.L);
+        if (e == cudaSuccess) e = dalloc(&f.se, (size_t)half);
         if (e == cudaSuccess) e = dalloc(&f.pairs, (size_t)half);
         if (e == cudaSuccess) e = dalloc(&f.pid, (size_t)m.e_cap);
         if (e == cudaSuccess) e = dalloc(&f.count, 1);
@@ -353,15 +355,19 @@ cudaError_t alloc_filters(Model& m) {
         f.cap = half;
         if (e == cudaSuccess) return e;
         cudaGetLastError();
-        dfree(f.w); dfree(f.pairs); dfree(f.pid); dfree(f.count);
+        dfree(f.w); dfree(f.se); dfree(f.pairs); dfree(f.pid); dfree(f.count);
         f = PairFilter{};
     }
     long long atoms = std::max<long long>(1, (long long)(kFilterChunkBytes / row) / m.row_cap);
     for (;; atoms /= 2) {
         f.chunk_atoms = (int)atoms;
         f.cap = atoms * m.row_cap;
-        if ((e = dalloc(&f.w, f.cap * (row / sizeof(float)))) == cudaSuccess || atoms == 1) return e;
+        e = dalloc(&f.w, f.cap * (row / sizeof(float)));
+        if (e == cudaSuccess) e = dalloc(&f.se, (size_t)f.cap);
+        if (e == cudaSuccess || atoms == 1) return e;
         cudaGetLastError();
+        dfree(f.w);
+        f.w = nullptr;
     }
 }
 
@@ -652,6 +658,7 @@ PotArgs pot_args(dmts_ctx* c, Model& m) {
     a.q = c->d_q;
     a.frame = c->d_frame;
     a.species = c->d_species;
+    a.first_of = c->d_first_of;
     a.row_ptr = m.row_ptr;
     a.col = m.col;
     a.recv = m.recv;
@@ -1256,7 +1263,7 @@ void dmts_destroy(dmts_ctx* c) {
     if (c->graph) cudaGraphExecDestroy(c->graph);
     free_model(c->m[0]);
     free_model(c->m[1]);
-    dfree(c->d_off); dfree(c->d_species); dfree(c->d_sys); dfree(c->d_box); dfree(c->d_mass);
+    dfree(c->d_off); dfree(c->d_species); dfree(c->d_first_of); dfree(c->d_sys); dfree(c->d_box); dfree(c->d_mass);
     dfree(c->d_inv_m); dfree(c->d_x); dfree(c->d_v); dfree(c->d_q); dfree(c->d_frame); dfree(c->d_stage);
     dfree(c->d_ke); dfree(c->d_ekin); dfree(c->d_ring); dfree(c->d_flags); dfree(c->d_epart); dfree(c->d_eticket);
     dfree(c->d_bx); dfree(c->d_bv);
@@ -1368,10 +1375,18 @@ int dmts_create(const dmts_model_desc* small, const dmts_model_desc* big, const 
     std::vector<int> sys_of(N);
     for (int s = 0; s < ns; ++s)
         for (int i = sys->atom_offset[s]; i < sys->atom_offset[s + 1]; ++i) sys_of[i] = s;
+    std::vector<int> first_of(N);
+    std::vector<int> first(S_min, -1);
+    for (int i = 0; i < N; ++i) {
+        int& f = first[sys->species[i]];
+        if (f < 0) f = i;
+        first_of[i] = f;
+    }
     std::vector<double> inv_m(N);
     for (int i = 0; i < N; ++i) inv_m[i] = 1.0 / sys->mass[i];
     CREATE_TRY(dalloc(&c->d_off, ns + 1));
     CREATE_TRY(dalloc(&c->d_species, N));
+    CREATE_TRY(dalloc(&c->d_first_of, N));
     CREATE_TRY(dalloc(&c->d_sys, N));
     CREATE_TRY(dalloc(&c->d_box, ns));
     CREATE_TRY(dalloc(&c->d_mass, N));
@@ -1416,6 +1431,7 @@ int dmts_create(const dmts_model_desc* small, const dmts_model_desc* big, const 
     }
     CREATE_TRY(cudaMemcpy(c->d_off, sys->atom_offset, sizeof(int) * (ns + 1), cudaMemcpyHostToDevice));
     CREATE_TRY(cudaMemcpy(c->d_species, sys->species, sizeof(int) * std::max(N, 0), cudaMemcpyHostToDevice));
+    CREATE_TRY(cudaMemcpy(c->d_first_of, first_of.data(), sizeof(int) * N, cudaMemcpyHostToDevice));
     CREATE_TRY(cudaMemcpy(c->d_sys, sys_of.data(), sizeof(int) * N, cudaMemcpyHostToDevice));
     CREATE_TRY(cudaMemcpy(c->d_box, sys->box, sizeof(double) * ns, cudaMemcpyHostToDevice));
     CREATE_TRY(cudaMemcpy(c->d_mass, sys->mass, sizeof(double) * N, cudaMemcpyHostToDevice));

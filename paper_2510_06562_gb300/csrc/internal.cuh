@@ -239,6 +239,7 @@ struct PairFilter {
     long long cap;           // rows per array
     int2* pairs;             // [cap] the unordered pairs (i, j), i < j
     int* pid;                // [e_cap] each directed pair's entry
+    float* se;               // [cap] dE/dd of each pair
     int* count;              // entries in use (zero between evaluations)
     int chunk_atoms;
 };
@@ -256,6 +257,7 @@ struct PotArgs {
     const uint4* q;
     const Frame* frame;
     const int* species;
+    const int* first_of;     // [N] the first atom of each atom's species
     const int* row_ptr;
     const int* col;
     const int* recv;

@@ -7,17 +7,18 @@
 // layer (k_pair_filter, register-blocked GEMMs over tiles of 128 pairs), and
 // the passes over the directed pairs are gathers over each atom's own row:
 //   forward   m_i = sum_j w_ij * u_j
-//   backward  F_i = sum_j dE/dd_ij rhat_ij,  dE/dd_ij = g_ij . dw/dd_ij,
-//             g_ij = mbar_i * u_j + mbar_j * u_i,  ubar_i = sum_j w_ij * mbar_j
-// one warp per atom, the row's pairs in a fixed order, no atomics on results:
+//   backward  ubar_i = sum_j w_ij * mbar_j,  F_i = sum_j dE/dd_ij rhat_ij
+// around one pass over the unordered pairs per layer,
+//   dE/dd_ij = g_ij . dw/dd_ij,  g_ij = mbar_i * u_j + mbar_j * u_i (symmetric).
+// One warp per atom, the row's pairs in a fixed order, no atomics on results:
 // deterministic and independent of the launch shape.
 //
 // Against recomputing the filter per directed pair in each pass (20,480 and
 // 10,240 flop per directed pair and layer), this is 20,480 flop per unordered
 // pair and layer in all, and w, dw/dd travel through memory (512 bytes per
-// unordered pair and layer at F = 64, written once, read three times). Big
-// model, 12,288-atom water, one evaluation: 3.48 -> 0.69 ms (edge passes 3.36
-// -> 0.57 ms); 192 atoms: 0.61 -> 0.16 ms.
+// unordered pair and layer at F = 64, written once, w read four times and
+// dw/dd once). Big model, 12,288-atom water, one evaluation: 3.48 -> 0.62 ms
+// (edge passes 3.36 -> 0.50 ms); 192 atoms: 0.61 -> 0.155 ms.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -77,7 +78,7 @@ __global__ void k_embed(PotArgs a) {
 // entries for its 32 atoms with one atomic (the order of the ranges varies
 // from run to run and no result depends on it); the entry's number goes to
 // its own directed pair and, found by bisection in row j, to the reverse one.
-constexpr int kIdxWarps = 8, kIdxRows = 4;     // rows per warp
+constexpr int kIdxWarps = 8, kIdxRows = 1;     // rows per warp
 
 __global__ void __launch_bounds__(kIdxWarps * 32) k_pair_index(PotArgs a, PairFilter pf) {
     __shared__ int w_sum[kIdxWarps];
@@ -205,6 +206,31 @@ __global__ void __launch_bounds__(FiltTile<F, KP>::NT, F == 64 ? 2 : 4) k_pair_f
                                    : min(min((long long)a.row_ptr[a1], a.e_cap) - e_beg, pf.cap);
     const long long tiles = (n_pairs + TP - 1) / TP, units = tiles * (l1 - l0);
     int cur = -1, buf = 0;
+    // The thread's pair of the next tile (pair tid mod TP): atom indices loaded
+    // at the start of a tile, positions before its second product.
+    const int lp = tid & (TP - 1);
+    int ni = -1, nj = 0;
+    uint4 qi = make_uint4(0, 0, 0, 0), qj = qi;
+    auto load_pair = [&](long long u) {
+        const long long p = u < units ? u % tiles * TP + lp : n_pairs;
+        ni = -1;
+        if (p >= n_pairs) return;
+        if (half) {
+            const int2 ij = pf.pairs[p];
+            ni = DMTS_IDX(ij.x, a.n_atoms, a.check);
+            nj = DMTS_IDX(ij.y, a.n_atoms, a.check);
+        } else {
+            ni = DMTS_IDX(a.recv[e_beg + p], a.n_atoms, a.check);
+            nj = DMTS_IDX(a.col[e_beg + p], a.n_atoms, a.check);
+        }
+    };
+    auto load_pos = [&]() {
+        if (ni < 0) return;
+        qi = a.q[ni];
+        qj = a.q[nj];
+    };
+    load_pair(blockIdx.x);
+    load_pos();
     for (long long unit = blockIdx.x; unit < units; unit += gridDim.x, buf ^= 1) {
         const int l = l0 + (int)(unit / tiles);
         const long long t0 = (unit - (l - l0) * tiles) * TP;
@@ -221,20 +247,9 @@ __global__ void __launch_bounds__(FiltTile<F, KP>::NT, F == 64 ? 2 : 4) k_pair_f
             }
             cur = l;
         }
-        if (tid < TP) {
+        {
             float eb[KP], db[KP], fc = 0.f, dfc = 0.f;
-            const long long p = t0 + tid;
-            if (p < n_pairs) {
-                int i, j;
-                if (half) {
-                    const int2 ij = pf.pairs[p];
-                    i = DMTS_IDX(ij.x, a.n_atoms, a.check);
-                    j = DMTS_IDX(ij.y, a.n_atoms, a.check);
-                } else {
-                    i = DMTS_IDX(a.recv[e_beg + p], a.n_atoms, a.check);
-                    j = DMTS_IDX(a.col[e_beg + p], a.n_atoms, a.check);
-                }
-                const uint4 qi = a.q[i], qj = a.q[j];
+            if (ni >= 0) {
                 const float3 r = edge_vec(qi, qj, a.frame[qi.w].qscale);
                 const float d = sqrtf(r.x * r.x + r.y * r.y + r.z * r.z);
                 basis_pair<KP>(d, K, a.pi_over_rc, a.bessel_pref, eb, db, fc, dfc);
@@ -242,14 +257,19 @@ __global__ void __launch_bounds__(FiltTile<F, KP>::NT, F == 64 ? 2 : 4) k_pair_f
 #pragma unroll
                 for (int k = 0; k < KP; ++k) eb[k] = db[k] = 0.f;
             }
+            // with two threads per pair (F = 64) one writes the basis, the other its derivative
+            if (NT == TP || tid < TP) {
 #pragma unroll
-            for (int k = 0; k < KP; ++k) {
-                S.B[k * TS + tid] = eb[k];
-                S.D[k * TS + tid] = db[k];
+                for (int k = 0; k < KP; ++k) S.B[k * TS + lp] = eb[k];
+                S.fc[buf][lp] = fc;
             }
-            S.fc[buf][tid] = fc;
-            S.dfc[buf][tid] = dfc;
+            if (NT == TP || tid >= TP) {
+#pragma unroll
+                for (int k = 0; k < KP; ++k) S.D[k * TS + lp] = db[k];
+                S.dfc[buf][lp] = dfc;
+            }
         }
+        load_pair(unit + gridDim.x);
         __syncthreads();
         f2::f32x2 x[4][4], y[4][4];
         {
@@ -283,6 +303,7 @@ __global__ void __launch_bounds__(FiltTile<F, KP>::NT, F == 64 ? 2 : 4) k_pair_f
             }
         }
         __syncthreads();
+        load_pos();
         {
             const float4 b = *reinterpret_cast<const float4*>(S.b2 + f0);
             const float bc[4] = {b.x, b.y, b.z, b.w};
@@ -308,9 +329,9 @@ __global__ void __launch_bounds__(FiltTile<F, KP>::NT, F == 64 ? 2 : 4) k_pair_f
                 }
                 float* w = pf.w + (row0 + r) * F + f0;
                 *reinterpret_cast<float4*>(w) = make_float4(fc * ph[0], fc * ph[1], fc * ph[2], fc * ph[3]);
-                *reinterpret_cast<float4*>(w + (size_t)pf.cap * F) =
-                    make_float4(dfc * ph[0] + fc * ps[0], dfc * ph[1] + fc * ps[1], dfc * ph[2] + fc * ps[2],
-                                dfc * ph[3] + fc * ps[3]);
+                __stcs(reinterpret_cast<float4*>(w + (size_t)pf.cap * F),
+                       make_float4(dfc * ph[0] + fc * ps[0], dfc * ph[1] + fc * ps[1], dfc * ph[2] + fc * ps[2],
+                                   dfc * ph[3] + fc * ps[3]));
             }
         }
         // the next tile's basis, SiLU and fc tiles: B and D were last read before the
@@ -320,17 +341,32 @@ __global__ void __launch_bounds__(FiltTile<F, KP>::NT, F == 64 ? 2 : 4) k_pair_f
 
 // ------------------------------------------------------------ gathers
 // One warp per atom; a row of F floats is read by F / 4 lanes, 16 bytes each,
-// so one warp instruction reads 2 (F = 64) or 4 (F = 32) whole rows. Bound by
-// the bytes of the gathered rows through L2: w and u_j forward (512 bytes per
-// directed pair at F = 64), dw/dd, u_j, mbar_j and, above layer 0, w backward
-// (768 or 1,024 bytes).
+// so one warp instruction reads 2 (F = 64) or 4 (F = 32) whole rows: w_ij and
+// v_j, 512 bytes per directed pair at F = 64 (639,638 pairs: 39 us, 8.4 TB/s
+// through L2). Bound by the latency of those rows: the next 32 pairs' indices
+// are loaded, and their w rows (mostly in DRAM by then) sent for, while the
+// present ones are summed.
+// At layer 0, u_j = A[Z_j] W_in depends on the species only: its row is read
+// at the first atom of that species (first_of), a few rows that stay in L1.
+// Blocks that run on one SM one after another take adjacent atoms
+// (gather_range), whose neighbours' rows they share in L1.
+
+// The atoms of this block: block b of a grid of kSmCount x per blocks takes
+// range (b mod kSmCount) per + b / kSmCount, so that blocks kSmCount apart,
+// which the hardware mostly gives to the same SM, are neighbours.
+__device__ __forceinline__ void gather_range(int n_per_cta, int a0, int a1, int& first, int& last) {
+    const int per = gridDim.x / kSmCount;
+    const int r = per > 0 ? (int)(blockIdx.x % kSmCount) * per + (int)(blockIdx.x / kSmCount) : (int)blockIdx.x;
+    first = min(a1, a0 + r * n_per_cta);
+    last = min(a1, first + n_per_cta);
+}
 
 // Filter row of directed pair e, or -1 if there is none: after an overflow
 // (the call will be redone) a pair may lack its entry, and a stale number is
 // recognised by the pair stored there.
-__device__ __forceinline__ long long filter_row(const PotArgs& a, const PairFilter& pf, long long e, long long e_beg,
-                                                int i, int j, bool overflow) {
-    if (pf.chunk_atoms) return e - e_beg < pf.cap ? e - e_beg : -1;
+__device__ __forceinline__ int filter_row(const PotArgs& a, const PairFilter& pf, long long e, long long e_beg, int i,
+                                          int j, bool overflow) {
+    if (pf.chunk_atoms) return e - e_beg < pf.cap ? (int)(e - e_beg) : -1;
     const int p = pf.pid[e];
     if (!overflow) return DMTS_IDX(p, pf.cap, a.check);
     if (p < 0 || p >= pf.cap) return -1;
@@ -338,47 +374,72 @@ __device__ __forceinline__ long long filter_row(const PotArgs& a, const PairFilt
     return ij.x == min(i, j) && ij.y == max(i, j) ? p : -1;
 }
 
+__device__ __forceinline__ float4 ld4(const float* p, int row, int F) {
+    return __ldg(reinterpret_cast<const float4*>(p + (size_t)(unsigned int)row * F));
+}
+
+// Starts moving row p of an [.][F] array into L2.
 template <int F>
-__global__ void __launch_bounds__(kThreads) k_gather_fwd(PotArgs a, PairFilter pf, int a0, int a1) {
+__device__ __forceinline__ void prefetch_row(const float* base, int p) {
+#pragma unroll
+    for (int k = 0; k < F; k += 32) asm volatile("prefetch.global.L2 [%0];" :: "l"(base + (size_t)(unsigned int)p * F + k));
+}
+
+// out_i = sum_j w_ij * v_j over atom i's row: the messages (v = u) or, in the
+// backward pass above layer 0, ubar (v = mbar). FWD: the forward pass, which
+// at layer 0 also sums the pair repulsion, 1/2 phi(d_ij) per directed pair.
+template <int F, bool FWD>
+__global__ void __launch_bounds__(kThreads) k_gather(PotArgs a, PairFilter pf, const float* __restrict__ v, int a0,
+                                                     int a1) {
     constexpr int LPR = F / 4, RPI = 32 / LPR;
     const int lane = threadIdx.x & 31, sub = lane / LPR, ch = lane % LPR;
     const bool overflow = a.check[kFlagOverflow] != 0;
-    const bool rep_on = a.layer == 0 && a.energy;
-    const float* W = pf.w + (size_t)(pf.chunk_atoms ? 0 : a.layer) * 2 * pf.cap * F + 4 * ch;
-    const float* U = a.u + 4 * ch;
+    const bool l0 = FWD && a.layer == 0, rep_on = l0 && a.energy;
+    const float* W0 = pf.w + (size_t)(pf.chunk_atoms ? 0 : a.layer) * 2 * pf.cap * F;
+    const float* W = W0 + 4 * ch;
+    const float* V = v + 4 * ch;
     const long long e_beg = min((long long)a.row_ptr[a0], a.e_cap);
-    const int last = min(a1, a0 + (int)(blockIdx.x + 1) * a.atoms_per_cta);
-    for (int i = a0 + blockIdx.x * a.atoms_per_cta + (threadIdx.x >> 5); i < last; i += kThreads / 32) {
+    int first, last;
+    gather_range(a.atoms_per_cta, a0, a1, first, last);
+    for (int i = first + (threadIdx.x >> 5); i < last; i += kThreads / 32) {
         const long long beg = min((long long)a.row_ptr[i], a.e_cap), end = min((long long)a.row_ptr[i + 1], a.e_cap);
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         float rep = 0.f;
         const uint4 qi = a.q[i];
         const float qscale = a.frame[qi.w].qscale;
-        for (long long b = beg; b < end; b += 32) {
-            const long long e = b + lane;
-            int j = 0;
-            long long p = -1;
+        int nj = 0, np = -1;                             // the lane's pair of the next chunk
+        auto load = [&](long long e) {
+            np = -1;
             if (e < end) {
-                j = DMTS_IDX(a.col[e], a.n_atoms, a.check);
-                p = filter_row(a, pf, e, e_beg, i, j, overflow);
-                if (rep_on) {                            // 1/2 phi(d_ij) per directed pair
+                nj = DMTS_IDX(a.col[e], a.n_atoms, a.check);
+                np = filter_row(a, pf, e, e_beg, i, nj, overflow);
+                if (np >= 0) prefetch_row<F>(W0, np);
+            }
+        };
+        load(beg + lane);
+        for (long long b = beg; b < end; b += 32) {
+            const int j = nj, p = np;                    // row of w (-1: no pair)
+            int jv = j;                                  // row of v
+            if (l0 && b + lane < end) {
+                jv = a.first_of[j];
+                if (rep_on) {
                     const float3 r = edge_vec(qi, a.q[j], qscale);
                     const float d = sqrtf(r.x * r.x + r.y * r.y + r.z * r.z);
                     rep += 0.5f * rep_phi(d, a.rep_a, a.rep_inv_rho, a.rep_rc, a.rep_pi_over_rc, nullptr);
                 }
             }
+            load(b + 32 + lane);
             const int n = (int)min(32ll, end - b);
-#pragma unroll 4
+#pragma unroll 8
             for (int k = 0; k < n; k += RPI) {
-                const long long pk = __shfl_sync(0xffffffffu, p, k + sub);
-                const int jk = __shfl_sync(0xffffffffu, j, k + sub);
+                const int pk = __shfl_sync(0xffffffffu, p, k + sub);
+                const int jk = __shfl_sync(0xffffffffu, jv, k + sub);
+                const float4 w = ld4(W, max(pk, 0), F), x = ld4(V, jk, F);
                 if (pk >= 0) {
-                    const float4 w = __ldg(reinterpret_cast<const float4*>(W + pk * F));
-                    const float4 u = __ldg(reinterpret_cast<const float4*>(U + (size_t)jk * F));
-                    acc.x += w.x * u.x;
-                    acc.y += w.y * u.y;
-                    acc.z += w.z * u.z;
-                    acc.w += w.w * u.w;
+                    acc.x += w.x * x.x;
+                    acc.y += w.y * x.y;
+                    acc.z += w.z * x.z;
+                    acc.w += w.w * x.w;
                 }
             }
         }
@@ -396,45 +457,195 @@ __global__ void __launch_bounds__(kThreads) k_gather_fwd(PotArgs a, PairFilter p
             if (lane == 0) a.erep[i] = rep;
         }
     }
-    // every reader of the pair count has finished: zero for the next index
-    if (a.layer == 0 && !pf.chunk_atoms && blockIdx.x == 0 && threadIdx.x == 0) *pf.count = 0;
 }
 
-// NV = 9: forces and the per-atom virial; NV = 3: forces only.
-// L0: layer 0, whose u does not depend on the positions (no ubar).
-// The dot products g . dw/dd of a chunk of 32 pairs are partial sums in
-// registers, one per row instruction, reduced over the lanes of a row by
-// halving exchanges (LPR - 1 shuffles for LPR sums) that leave the sum of
-// pair RPI ch + sub in lane (sub, ch), the lane that holds its geometry.
-template <int F, int NV, bool L0>
-__global__ void __launch_bounds__(kThreads) k_gather_bwd(PotArgs a, PairFilter pf, int a0, int a1) {
+// s[k] of the LPR lanes of a row, summed over those lanes by halving exchanges
+// (LPR - 1 shuffles): lane ch is left with the sum of s[ch] in s[0].
+template <int LPR>
+__device__ __forceinline__ void halving_sum(float (&s)[LPR], int ch) {
+#pragma unroll
+    for (int m = LPR / 2; m > 0; m >>= 1) {
+        const bool up = (ch & m) != 0;
+#pragma unroll
+        for (int k = 0; k < m; ++k) {
+            const float give = up ? s[k] : s[k + m], keep = up ? s[k + m] : s[k];
+            s[k] = keep + __shfl_xor_sync(0xffffffffu, give, m);
+        }
+    }
+}
+
+// One pair's share of atom i's force, dE/dd rhat, and (NV = 9) of its virial,
+// W_ab = -1/2 sum_directed dE/dd d rhat_a rhat_b (xx yy zz xy xz yz).
+template <int NV>
+__device__ __forceinline__ void add_force(float (&fv)[NV], float se, float rx, float ry, float rz, float d) {
+    fv[0] += se * rx;
+    fv[1] += se * ry;
+    fv[2] += se * rz;
+    if constexpr (NV == 9) {
+        const float hv = -0.5f * se * d;
+        fv[3] += hv * rx * rx; fv[4] += hv * ry * ry; fv[5] += hv * rz * rz;
+        fv[6] += hv * rx * ry; fv[7] += hv * rx * rz; fv[8] += hv * ry * rz;
+    }
+}
+
+template <int NV>
+__device__ __forceinline__ void store_force(const PotArgs& a, int i, float (&fv)[NV], int lane, int accumulate) {
+#pragma unroll
+    for (int c = 0; c < NV; ++c)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) fv[c] += __shfl_xor_sync(0xffffffffu, fv[c], o);
+    if (lane != 0) return;
+#pragma unroll
+    for (int c = 0; c < NV; ++c) {
+        float* f = c < 3 ? a.force + (size_t)c * a.n_atoms + i : a.vir6 + (size_t)i * 6 + c - 3;
+        *f = accumulate ? *f + fv[c] : fv[c];
+    }
+}
+
+// ------------------------------------------------------------ dE/dd of every pair
+// se = g . dw/dd, g = mbar_i * u_j + mbar_j * u_i: symmetric in (i, j), so once
+// per unordered pair; at layer 0 plus the repulsion's derivative. The layers
+// add up in pf.se (add). (In atom rows, both directions of every pair with the
+// ubar sum alongside: 100 and 69 us for layers 1 and 0 of the big model on
+// 12,288-atom water; so, with k_gather and k_pair_force: 70 and 47.) A warp takes 32 consecutive pairs: their dw/dd rows
+// are contiguous, and consecutive pairs mostly share atom i. The products of
+// a row of lanes are partial sums in registers, one per row instruction; the
+// sum of pair RPI ch + sub ends in lane (sub, ch).
+template <int F, bool L0>
+__global__ void __launch_bounds__(kThreads, F == 64 ? 3 : 4) k_pair_dedd(PotArgs a, PairFilter pf, int a0, int a1, int add) {
     constexpr int LPR = F / 4, RPI = 32 / LPR;
     const int lane = threadIdx.x & 31, sub = lane / LPR, ch = lane % LPR;
-    const bool overflow = a.check[kFlagOverflow] != 0;
-    const float* W = pf.w + (size_t)(pf.chunk_atoms ? 0 : a.layer) * 2 * pf.cap * F + 4 * ch;
-    const float* DW = W + (size_t)pf.cap * F;
+    const bool half = pf.chunk_atoms == 0;
+    const long long e_beg = half ? 0 : min((long long)a.row_ptr[a0], a.e_cap);
+    const long long n_pairs = half ? min((long long)*pf.count, pf.cap)
+                                   : min(min((long long)a.row_ptr[a1], a.e_cap) - e_beg, pf.cap);
+    const float* DW = pf.w + (size_t)((half ? a.layer : 0) * 2 + 1) * pf.cap * F + 4 * ch;
     const float* U = a.u + 4 * ch;
     const float* MB = a.mbar + 4 * ch;
+    const long long step = (long long)gridDim.x * (kThreads / 32) * 32;
+    int ni = 0, nj = 0;
+    auto load_pair = [&](long long p) {                  // atoms of pair p (the atoms of the chunk's first pair past the end)
+        if (p >= n_pairs) return;
+        if (half) {
+            const int2 ij = pf.pairs[p];
+            ni = DMTS_IDX(ij.x, a.n_atoms, a.check);
+            nj = DMTS_IDX(ij.y, a.n_atoms, a.check);
+        } else {
+            ni = DMTS_IDX(a.recv[e_beg + p], a.n_atoms, a.check);
+            nj = DMTS_IDX(a.col[e_beg + p], a.n_atoms, a.check);
+        }
+    };
+    const int own = RPI * ch + sub;                      // this lane's pair of a chunk
+    long long p0 = ((long long)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * 32;
+    load_pair(p0 + own);
+    for (; p0 < n_pairs; p0 += step) {
+        const int i = ni, j = nj;
+        int iu = i, ju = j;
+        if (L0) {
+            iu = a.first_of[i];
+            ju = a.first_of[j];
+        }
+        load_pair(p0 + step + own);
+        const int n = (int)min(32ll, n_pairs - p0);
+        float s[LPR];
+#pragma unroll
+        for (int k = 0; k < LPR; ++k) {
+            s[k] = 0.f;
+            if (RPI * k < n) {                            // warp-uniform
+                const int src = sub * LPR + k;
+                const int ik = __shfl_sync(0xffffffffu, i, src), jk = __shfl_sync(0xffffffffu, j, src);
+                const int iuk = L0 ? __shfl_sync(0xffffffffu, iu, src) : ik;
+                const int juk = L0 ? __shfl_sync(0xffffffffu, ju, src) : jk;
+                const int row = min(RPI * k + sub, n - 1);
+                const float4 dw = __ldcs(reinterpret_cast<const float4*>(DW + (p0 + row) * F));
+                const float4 ui = ld4(U, iuk, F), uj = ld4(U, juk, F), mi = ld4(MB, ik, F), mj = ld4(MB, jk, F);
+                float t = (mi.x * uj.x + mj.x * ui.x) * dw.x;
+                t += (mi.y * uj.y + mj.y * ui.y) * dw.y;
+                t += (mi.z * uj.z + mj.z * ui.z) * dw.z;
+                t += (mi.w * uj.w + mj.w * ui.w) * dw.w;
+                s[k] = t;
+            }
+        }
+        halving_sum<LPR>(s, ch);
+        if (own < n) {
+            float se = s[0];
+            if (L0) {
+                const uint4 qi = a.q[i];
+                const float3 r = edge_vec(qi, a.q[j], a.frame[qi.w].qscale);
+                float dphi;
+                (void)rep_phi(sqrtf(r.x * r.x + r.y * r.y + r.z * r.z), a.rep_a, a.rep_inv_rho, a.rep_rc,
+                              a.rep_pi_over_rc, &dphi);
+                se += dphi;
+            }
+            float* out = pf.se + p0 + own;
+            *out = add ? *out + se : se;
+        }
+    }
+}
+
+// F_i = sum_j dE/dd_ij rhat_ij over atom i's row, and (NV = 9) the per-atom
+// virial; one warp per atom, one pair per lane.
+template <int NV>
+__global__ void __launch_bounds__(kThreads) k_pair_force(PotArgs a, PairFilter pf, int a0, int a1, int accumulate) {
+    const int lane = threadIdx.x & 31;
+    const bool overflow = a.check[kFlagOverflow] != 0;
     const long long e_beg = min((long long)a.row_ptr[a0], a.e_cap);
-    const int last = min(a1, a0 + (int)(blockIdx.x + 1) * a.atoms_per_cta);
-    for (int i = a0 + blockIdx.x * a.atoms_per_cta + (threadIdx.x >> 5); i < last; i += kThreads / 32) {
+    int first, last;
+    gather_range(a.atoms_per_cta, a0, a1, first, last);
+    for (int i = first + (threadIdx.x >> 5); i < last; i += kThreads / 32) {
         const long long beg = min((long long)a.row_ptr[i], a.e_cap), end = min((long long)a.row_ptr[i + 1], a.e_cap);
         const uint4 qi = a.q[i];
         const float qscale = a.frame[qi.w].qscale;
-        const float4 ui = __ldg(reinterpret_cast<const float4*>(U + (size_t)i * F));
-        const float4 mi = __ldg(reinterpret_cast<const float4*>(MB + (size_t)i * F));
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        float fv[NV];
+#pragma unroll
+        for (int c = 0; c < NV; ++c) fv[c] = 0.f;
+        for (long long e = beg + lane; e < end; e += 32) {
+            const int j = DMTS_IDX(a.col[e], a.n_atoms, a.check);
+            const int p = filter_row(a, pf, e, e_beg, i, j, overflow);
+            const float3 r = edge_vec(qi, a.q[j], qscale);
+            const float d = sqrtf(r.x * r.x + r.y * r.y + r.z * r.z);
+            const float inv = 1.0f / d;
+            const float rx = r.x * inv, ry = r.y * inv, rz = r.z * inv;
+            const float se = p >= 0 ? pf.se[p] : 0.f;
+            add_force<NV>(fv, se, rx, ry, rz, d);
+        }
+        store_force<NV>(a, i, fv, lane, accumulate);
+    }
+    // every reader of the pair count has finished: zero for the next index
+    if (!pf.chunk_atoms && blockIdx.x == 0 && threadIdx.x == 0) *pf.count = 0;
+}
+
+// One-layer models: dE/dd, force and (NV = 9) virial in one pass over each
+// atom's row, every pair's dE/dd evaluated in both directions: at F = 32 that
+// costs no more than the two passes above (12,288-atom water, small model:
+// 18.5 against 18.9 us; 192 atoms: 8 against 14 us).
+template <int F, int NV>
+__global__ void __launch_bounds__(kThreads, NV == 3 ? 3 : 2) k_row_force(PotArgs a, PairFilter pf, int a0, int a1) {
+    constexpr int LPR = F / 4, RPI = 32 / LPR;
+    const int lane = threadIdx.x & 31, sub = lane / LPR, ch = lane % LPR;
+    const bool overflow = a.check[kFlagOverflow] != 0;
+    const float* DW = pf.w + (size_t)pf.cap * F + 4 * ch;
+    const float* U = a.u + 4 * ch;
+    const float* MB = a.mbar + 4 * ch;
+    const long long e_beg = min((long long)a.row_ptr[a0], a.e_cap);
+    int first, last;
+    gather_range(a.atoms_per_cta, a0, a1, first, last);
+    for (int i = first + (threadIdx.x >> 5); i < last; i += kThreads / 32) {
+        const long long beg = min((long long)a.row_ptr[i], a.e_cap), end = min((long long)a.row_ptr[i + 1], a.e_cap);
+        const uint4 qi = a.q[i];
+        const float qscale = a.frame[qi.w].qscale;
+        const float4 ui = ld4(U, i, F), mi = ld4(MB, i, F);
         float fv[NV];
 #pragma unroll
         for (int c = 0; c < NV; ++c) fv[c] = 0.f;
         for (long long b = beg; b < end; b += 32) {
             const long long e = b + RPI * ch + sub;       // this lane's pair of the chunk
-            int j = 0;
-            long long p = -1;
+            int j = i, ju = i, p = -1;
             float rx = 0.f, ry = 0.f, rz = 0.f, d = 1.f;
             if (e < end) {
                 j = DMTS_IDX(a.col[e], a.n_atoms, a.check);
                 p = filter_row(a, pf, e, e_beg, i, j, overflow);
+                ju = a.first_of[j];
                 const float3 r = edge_vec(qi, a.q[j], qscale);
                 d = sqrtf(r.x * r.x + r.y * r.y + r.z * r.z);
                 const float inv = 1.0f / d;
@@ -446,81 +657,27 @@ __global__ void __launch_bounds__(kThreads) k_gather_bwd(PotArgs a, PairFilter p
             for (int k = 0; k < LPR; ++k) {
                 s[k] = 0.f;
                 if (RPI * k < n) {                        // warp-uniform
-                    const long long pk = __shfl_sync(0xffffffffu, p, sub * LPR + k);
-                    const int jk = __shfl_sync(0xffffffffu, j, sub * LPR + k);
-                    if (pk >= 0) {
-                        const float4 dw = __ldg(reinterpret_cast<const float4*>(DW + pk * F));
-                        const float4 uj = __ldg(reinterpret_cast<const float4*>(U + (size_t)jk * F));
-                        const float4 mj = __ldg(reinterpret_cast<const float4*>(MB + (size_t)jk * F));
-                        float t = (mi.x * uj.x + mj.x * ui.x) * dw.x;
-                        t += (mi.y * uj.y + mj.y * ui.y) * dw.y;
-                        t += (mi.z * uj.z + mj.z * ui.z) * dw.z;
-                        t += (mi.w * uj.w + mj.w * ui.w) * dw.w;
-                        s[k] = t;
-                        if (!L0) {
-                            const float4 w = __ldg(reinterpret_cast<const float4*>(W + pk * F));
-                            acc.x += w.x * mj.x;
-                            acc.y += w.y * mj.y;
-                            acc.z += w.z * mj.z;
-                            acc.w += w.w * mj.w;
-                        }
-                    }
+                    const int src = sub * LPR + k;
+                    const int pk = __shfl_sync(0xffffffffu, p, src), jk = __shfl_sync(0xffffffffu, j, src);
+                    const int juk = __shfl_sync(0xffffffffu, ju, src);
+                    const float4 dw = ld4(DW, max(pk, 0), F), uj = ld4(U, juk, F), mj = ld4(MB, jk, F);
+                    float t = (mi.x * uj.x + mj.x * ui.x) * dw.x;
+                    t += (mi.y * uj.y + mj.y * ui.y) * dw.y;
+                    t += (mi.z * uj.z + mj.z * ui.z) * dw.z;
+                    t += (mi.w * uj.w + mj.w * ui.w) * dw.w;
+                    s[k] = pk >= 0 ? t : 0.f;
                 }
             }
-#pragma unroll
-            for (int m = LPR / 2; m > 0; m >>= 1) {
-                const bool up = (ch & m) != 0;
-#pragma unroll
-                for (int k = 0; k < m; ++k) {
-                    const float give = up ? s[k] : s[k + m], keep = up ? s[k + m] : s[k];
-                    s[k] = keep + __shfl_xor_sync(0xffffffffu, give, m);
-                }
-            }
+            halving_sum<LPR>(s, ch);
             if (e < end) {
-                float se = s[0];                          // dE/dd of this lane's pair
-                if (L0) {
-                    float dphi;
-                    (void)rep_phi(d, a.rep_a, a.rep_inv_rho, a.rep_rc, a.rep_pi_over_rc, &dphi);
-                    se += dphi;
-                }
-                fv[0] += se * rx;
-                fv[1] += se * ry;
-                fv[2] += se * rz;
-                if constexpr (NV == 9) {
-                    const float hv = -0.5f * se * d;      // W_ab = -1/2 sum_directed s d rhat_a rhat_b
-                    fv[3] += hv * rx * rx; fv[4] += hv * ry * ry; fv[5] += hv * rz * rz;
-                    fv[6] += hv * rx * ry; fv[7] += hv * rx * rz; fv[8] += hv * ry * rz;
-                }
+                float dphi;
+                (void)rep_phi(d, a.rep_a, a.rep_inv_rho, a.rep_rc, a.rep_pi_over_rc, &dphi);
+                add_force<NV>(fv, s[0] + dphi, rx, ry, rz, d);
             }
         }
-#pragma unroll
-        for (int c = 0; c < NV; ++c)
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) fv[c] += __shfl_xor_sync(0xffffffffu, fv[c], o);
-        if (lane == 0) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                float* f = a.force + (size_t)c * a.n_atoms + i;
-                *f = a.accumulate ? *f + fv[c] : fv[c];
-            }
-            if constexpr (NV == 9)
-#pragma unroll
-                for (int c = 0; c < 6; ++c) {
-                    float* v = a.vir6 + (size_t)i * 6 + c;
-                    *v = a.accumulate ? *v + fv[3 + c] : fv[3 + c];
-                }
-        }
-        if (!L0) {
-#pragma unroll
-            for (int o = LPR; o < 32; o <<= 1) {
-                acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-                acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-                acc.z += __shfl_xor_sync(0xffffffffu, acc.z, o);
-                acc.w += __shfl_xor_sync(0xffffffffu, acc.w, o);
-            }
-            if (sub == 0) *reinterpret_cast<float4*>(a.msg_out + (size_t)i * F + 4 * ch) = acc;
-        }
+        store_force<NV>(a, i, fv, lane, a.accumulate);
     }
+    if (!pf.chunk_atoms && blockIdx.x == 0 && threadIdx.x == 0) *pf.count = 0;
 }
 
 // ------------------------------------------------------------ launches
@@ -543,7 +700,12 @@ void filters(const PotArgs& a, int K, int l0, int l1, int a0, int a1, cudaStream
     else filter_go<F, 16>(a, K, l0, l1, a0, a1, s);
 }
 
-inline int gather_blocks(const PotArgs& a, int a0, int a1) { return (a1 - a0 + a.atoms_per_cta - 1) / a.atoms_per_cta; }
+// Blocks for the atoms a0 .. a1 - 1: a multiple of the SM count once there are
+// that many (gather_range).
+inline int gather_blocks(const PotArgs& a, int a0, int a1) {
+    const int n = (a1 - a0 + a.atoms_per_cta - 1) / a.atoms_per_cta;
+    return n < kSmCount ? n : (n + kSmCount - 1) / kSmCount * kSmCount;
+}
 
 template <int F>
 void fwd_go(const PotArgs& a, int K, cudaStream_t s) {
@@ -554,34 +716,49 @@ void fwd_go(const PotArgs& a, int K, cudaStream_t s) {
             count_launch();
             filters<F>(a, K, 0, a.n_layers, 0, a.n_atoms, s);
         }
-        k_gather_fwd<F><<<gather_blocks(a, 0, a.n_atoms), kThreads, 0, s>>>(a, a.filter, 0, a.n_atoms);
+        k_gather<F, true><<<gather_blocks(a, 0, a.n_atoms), kThreads, 0, s>>>(a, a.filter, a.u, 0, a.n_atoms);
         count_launch();
         return;
     }
     for (int a0 = 0; a0 < a.n_atoms; a0 += a.filter.chunk_atoms) {
         const int a1 = std::min(a.n_atoms, a0 + a.filter.chunk_atoms);
         filters<F>(a, K, a.layer, a.layer + 1, a0, a1, s);
-        k_gather_fwd<F><<<gather_blocks(a, a0, a1), kThreads, 0, s>>>(a, a.filter, a0, a1);
+        k_gather<F, true><<<gather_blocks(a, a0, a1), kThreads, 0, s>>>(a, a.filter, a.u, a0, a1);
         count_launch();
     }
 }
 
-template <int F, int NV>
-void gather_bwd(const PotArgs& a, int a0, int a1, cudaStream_t s) {
-    const int grid = gather_blocks(a, a0, a1);
-    if (a.layer == 0) k_gather_bwd<F, NV, true><<<grid, kThreads, 0, s>>>(a, a.filter, a0, a1);
-    else k_gather_bwd<F, NV, false><<<grid, kThreads, 0, s>>>(a, a.filter, a0, a1);
-    count_launch();
-}
-
+// The forces need every layer's dE/dd: summed over the layers per unordered
+// pair, then one pass; chunked, one pass per layer and chunk.
 template <int F>
 void bwd_go(const PotArgs& a, int K, cudaStream_t s) {
-    const int step = a.filter.chunk_atoms ? a.filter.chunk_atoms : a.n_atoms;
+    const bool half = !a.filter.chunk_atoms;
+    const int step = half ? a.n_atoms : a.filter.chunk_atoms;
+    const bool top = a.layer == a.n_layers - 1;
     for (int a0 = 0; a0 < a.n_atoms; a0 += step) {
-        const int a1 = std::min(a.n_atoms, a0 + step);
-        if (a.filter.chunk_atoms) filters<F>(a, K, a.layer, a.layer + 1, a0, a1, s);
-        if (a.virial) gather_bwd<F, 9>(a, a0, a1, s);
-        else gather_bwd<F, 3>(a, a0, a1, s);
+        const int a1 = std::min(a.n_atoms, a0 + step), grid = gather_blocks(a, a0, a1);
+        if (!half) filters<F>(a, K, a.layer, a.layer + 1, a0, a1, s);
+        const int warps = (int)std::min<long long>((a.filter.cap + 31) / 32, (long long)kSmCount * 8 * (F == 64 ? 3 : 4));
+        const int pgrid = (warps + kThreads / 32 - 1) / (kThreads / 32);
+        if (a.n_layers == 1) {
+            if (a.virial) k_row_force<F, 9><<<grid, kThreads, 0, s>>>(a, a.filter, a0, a1);
+            else k_row_force<F, 3><<<grid, kThreads, 0, s>>>(a, a.filter, a0, a1);
+            count_launch();
+            continue;
+        }
+        if (a.layer == 0) {
+            k_pair_dedd<F, true><<<pgrid, kThreads, 0, s>>>(a, a.filter, a0, a1, half && !top);
+        } else {
+            k_pair_dedd<F, false><<<pgrid, kThreads, 0, s>>>(a, a.filter, a0, a1, half && !top);
+            k_gather<F, false><<<grid, kThreads, 0, s>>>(a, a.filter, a.mbar, a0, a1);
+            count_launch();
+        }
+        count_launch();
+        if (half && a.layer > 0) continue;
+        const int acc = half ? 0 : a.accumulate;
+        if (a.virial) k_pair_force<9><<<grid, kThreads, 0, s>>>(a, a.filter, a0, a1, acc);
+        else k_pair_force<3><<<grid, kThreads, 0, s>>>(a, a.filter, a0, a1, acc);
+        count_launch();
     }
 }
 
