@@ -341,9 +341,12 @@ DMTS_API int dmts_force_matching_grad(dmts_ctx* ctx, int n_frames, const double*
  * ((eV/atom)^-2 against (eV/A)^-2 for the force term; 0 gives
  * dmts_force_matching_grad). Arguments as dmts_force_matching_grad, plus
  * e_ref [M] reference energies (host or device); same support, FP32
- * adjoints, restored state and invalidated forces. The frames are enqueued
- * without host synchronisation between them; a neighbour overflow in any
- * frame grows the capacities and redoes the batch. */
+ * adjoints, restored state and invalidated forces. The frames run in batches
+ * of about 131,072 atoms, as independent systems of an inner context that the
+ * first call with several frames creates (kept until dmts_destroy; with no
+ * memory for it they run one at a time), without host synchronisation between
+ * batches; a neighbour overflow in any frame grows the capacities and redoes
+ * the call. */
 DMTS_API int dmts_distill_grad(dmts_ctx* ctx, int n_frames, const double* frames, const double* f_ref,
                                const double* e_ref, double lambda_e, double* loss_out, double* grad_out);
 

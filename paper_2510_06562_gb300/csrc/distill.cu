@@ -77,19 +77,52 @@ __device__ __forceinline__ void basis_pair(float d, float pi_over_rc, float pref
 }
 
 // ------------------------------------------------------------ residual g
-// g_i = c (F_i - F_ref,i) (SoA), c = 2 / (3 N M); per-atom squared residual
-// (FP64) for the loss.
-__global__ void k_fm_residual(int n, const float* __restrict__ f, const double* __restrict__ f_ref_aos, double c,
-                              float* __restrict__ g, double* __restrict__ sq) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+// g_i = c (F_i - F_ref,i) (SoA), c = 2 / (3 N M), and the force term of the
+// loss, c/2 sum |F_i - F_ref,i|^2 (FP64): every block leaves its sum in part,
+// the last one to finish adds them in block order (one order for any
+// schedule) and resets the ticket.
+constexpr int kResT = 256;
+__global__ void __launch_bounds__(kResT) k_fm_residual(int n, const float* __restrict__ f,
+                                                       const double* __restrict__ f_ref_aos, double c,
+                                                       float* __restrict__ g, double* __restrict__ part,
+                                                       unsigned int* __restrict__ ticket, double* __restrict__ loss) {
+    __shared__ double wsum[kResT / 32];
+    __shared__ bool last;
+    const int i = blockIdx.x * kResT + threadIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     double s = 0.0;
-    for (int k = 0; k < 3; ++k) {
-        double r = (double)f[(size_t)k * n + i] - f_ref_aos[3 * (size_t)i + k];
-        g[(size_t)k * n + i] = (float)(c * r);
-        s += r * r;
+    if (i < n)
+        for (int k = 0; k < 3; ++k) {
+            double r = (double)f[(size_t)k * n + i] - f_ref_aos[3 * (size_t)i + k];
+            g[(size_t)k * n + i] = (float)(c * r);
+            s += r * r;
+        }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) wsum[w] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int k = 0; k < kResT / 32; ++k) t += wsum[k];
+        part[blockIdx.x] = t;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
-    sq[i] = s;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double t = 0.0;
+    for (int k = threadIdx.x; k < (int)gridDim.x; k += kResT) t += __ldcg(part + k);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    __syncthreads();
+    if (lane == 0) wsum[w] = t;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double u = 0.0;
+        for (int k = 0; k < kResT / 32; ++k) u += wsum[k];
+        *loss += 0.5 * c * u;
+        *ticket = 0u;
+    }
 }
 
 // ------------------------------------------------------------ edge tile (shared by both edge passes)
@@ -543,7 +576,7 @@ __global__ void __launch_bounds__(kAtomWarps * 32) k_fm_atom(PotArgs a, const fl
                                                               float* __restrict__ mbar_psi,
                                                               float* __restrict__ mdotbar_psi,
                                                               float* __restrict__ partial, int n_params,
-                                                              const double* __restrict__ c_energy) {
+                                                              const double* __restrict__ c_energy, int frame_atoms) {
     constexpr int F = 32;
     // U1, U2, R1 as W[k][f] (for x W), then padded copies U1T, U2T, R1T (for
     // x W^T); at the end the same array holds the block's gradient sums
@@ -565,8 +598,7 @@ __global__ void __launch_bounds__(kAtomWarps * 32) k_fm_atom(PotArgs a, const fl
     }
     __syncthreads();
     const float c1 = P[a.off.c1[0] + lane], d1 = P[a.off.d1 + lane], r2 = P[a.off.R2 + lane];
-    const float ce = c_energy ? (float)*c_energy : 0.f;        // dL/dE of this frame (energy term)
-    float n_here = 0.f, n_sp_here = 0.f;                       // atoms of this warp; of species `lane`
+    double ce_here = 0.0, ce_sp_here = 0.0;                    // sum of dL/dE over this warp's atoms; over those of species `lane`
     // per-lane gradient accumulators: column `lane` of dR1, dU2, dU1 (k = 0..31), and vectors
     float gR1[F], gU2[F], gU1[F];
 #pragma unroll
@@ -584,6 +616,7 @@ __global__ void __launch_bounds__(kAtomWarps * 32) k_fm_atom(PotArgs a, const fl
     auto slot = [&](int k) { return vs + k * F; };
     for (int i = blockIdx.x * kAtomWarps + w; i < a.n_atoms; i += gridDim.x * kAtomWarps) {
         const size_t o = (size_t)i * F + lane;
+        const float ce = c_energy ? (float)c_energy[i / frame_atoms] : 0.f;   // dL/dE of the atom's frame (energy term)
         const float mv = m[o], md = mdot[o], h1 = a.h[o];
         __syncwarp();                              // the previous atom's slots have been read
         slot(0)[lane] = mv;
@@ -635,8 +668,8 @@ __global__ void __launch_bounds__(kAtomWarps * 32) k_fm_atom(PotArgs a, const fl
 #pragma unroll
         for (int zz = 0; zz < 16; ++zz)
             if (zz == sp) gA[zz] += hb;               // residual h1 = h0 + ... with h0 = A[Z]
-        n_here += 1.f;
-        if (lane == sp) n_sp_here += 1.f;
+        ce_here += (double)ce;
+        if (lane == sp) ce_sp_here += (double)ce;
     }
     // the block's partials: the warps' sums added in warp order in shared
     // memory, then one row partial[blockIdx * n_params + param]
@@ -658,9 +691,9 @@ __global__ void __launch_bounds__(kAtomWarps * 32) k_fm_atom(PotArgs a, const fl
             put(sv + 2 * F + lane, gc2);
             put(sv + 3 * F + lane, gc1);
             for (int zz = 0; zz < n_sp && zz < 16; ++zz) put(sA + zz * F + lane, gA[zz]);
-            // every atom adds d2 and e0[Z_i] to the energy once (exact counts in FP32)
-            if (lane == 0) put(sE, -ce * n_here);
-            if (lane < n_sp) put(sE + 1 + lane, -ce * n_sp_here);
+            // every atom adds d2 and e0[Z_i] to the energy once
+            if (lane == 0) put(sE, (float)-ce_here);
+            if (lane < n_sp) put(sE + 1 + lane, (float)-ce_sp_here);
         }
         __syncthreads();
     }
@@ -1339,17 +1372,27 @@ __global__ void __launch_bounds__(kAtomWarps * 32) k_fm_input(PotArgs a, const f
     for (int t = tid; t < n_sp * F; t += blockDim.x) out[a.off.A + t] = sA[t];
 }
 
-// Energy term of one frame: E = sum over the systems of the model's energies,
-// r = (E - E_ref) / N; loss += lambda r^2 / M and c_E = dL/dE = 2 lambda r / (M N).
-__global__ void k_fm_energy_term(int n_sys, const double* __restrict__ E, const double* __restrict__ e_ref,
-                                 double lambda, int n_atoms, double inv_frames, double* __restrict__ c_energy,
-                                 double* __restrict__ loss) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double e = 0.0;
-    for (int k = 0; k < n_sys; ++k) e += E[k];
-    const double r = (e - *e_ref) / (double)n_atoms;
-    *loss += lambda * r * r * inv_frames;
-    *c_energy = 2.0 * lambda * r * inv_frames / (double)n_atoms;
+// Energy term of n_frames frames of n_sys systems each: per frame, E = sum
+// over its systems of the model's energies, r = (E - E_ref) / N; loss +=
+// lambda r^2 / M (in frame order) and c_E = dL/dE = 2 lambda r / (M N). One
+// warp, a frame per lane.
+__global__ void k_fm_energy_term(int n_frames, int n_sys, const double* __restrict__ E,
+                                 const double* __restrict__ e_ref, double lambda, int n_atoms, double inv_frames,
+                                 double* __restrict__ c_energy, double* __restrict__ loss) {
+    double sum = 0.0;
+    for (int f0 = 0; f0 < n_frames; f0 += 32) {
+        const int f = f0 + (int)threadIdx.x;
+        double term = 0.0;
+        if (f < n_frames) {
+            double e = 0.0;
+            for (int k = 0; k < n_sys; ++k) e += E[(size_t)f * n_sys + k];
+            const double r = (e - e_ref[f]) / (double)n_atoms;
+            term = lambda * r * r * inv_frames;
+            c_energy[f] = 2.0 * lambda * r * inv_frames / (double)n_atoms;
+        }
+        for (int k = 0; k < 32; ++k) sum += __shfl_sync(0xffffffffu, term, k);
+    }
+    if (threadIdx.x == 0) *loss += sum;
 }
 
 // grad[p] -= sum_c partial[c][p] for p in up to four ranges [p0, p1) of
@@ -1415,30 +1458,6 @@ void fm_reduce(const float* partial, int n_rows, int n_params, std::initializer_
     k_fm_reduce<<<blocks, kRedP * kRedG, 0, s>>>(partial, n_rows, n_params, rr, grad);
 }
 
-// out += scale * sum v (one block; each thread four interleaved FP64 sums,
-// so four loads are in flight, then a fixed-order tree).
-constexpr int kSumT = 1024;
-__global__ void __launch_bounds__(kSumT) k_sum_all(int n, const double* __restrict__ v, double scale,
-                                                   double* __restrict__ out) {
-    __shared__ double sh[kSumT];
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    int i = threadIdx.x;
-    for (; i + 3 * kSumT < n; i += 4 * kSumT) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) acc[u] += v[i + u * kSumT];
-    }
-#pragma unroll
-    for (int u = 0; u < 3; ++u)
-        if (i + u * kSumT < n) acc[u] += v[i + u * kSumT];
-    sh[threadIdx.x] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-    __syncthreads();
-    for (int w = kSumT / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *out += scale * sh[0];
-}
-
 template <int F, int K>
 size_t edge_smem() { return sizeof(EdgeSmem<F, K>); }
 
@@ -1488,20 +1507,28 @@ int device_sms() {
     return sms;
 }
 
-// Atoms per CTA of an edge pass that runs `per_sm` CTAs per SM: the atoms
-// shared by one wave of CTAs (no partial last wave, fewer ragged tiles), at
-// most kFmAtomsMax.
+// Atoms per CTA of an edge pass that runs `per_sm` CTAs per SM: at most
+// kFmAtomsMax, shared by whole waves of CTAs (no partial last wave).
 int fm_edge_atoms(int n_atoms, int per_sm) {
-    const int ctas = device_sms() * per_sm;
-    return std::max(1, std::min(kFmAtomsMax, (n_atoms + ctas - 1) / ctas));
+    const long long ctas = (long long)device_sms() * per_sm;
+    const long long waves = std::max(1ll, (n_atoms + kFmAtomsMax * ctas - 1) / (kFmAtomsMax * ctas));
+    return (int)std::max(1ll, (n_atoms + waves * ctas - 1) / (waves * ctas));
 }
-}  // namespace
 
 // The gradient edge pass (one CTA per SM, one partial row per CTA).
 int fm_edge_ctas(int n_atoms) {
     const int apc = fm_edge_atoms(n_atoms, 1);
     return (n_atoms + apc - 1) / apc;
 }
+}  // namespace
+
+// Partial rows of the gradient edge pass for at most n_atoms atoms.
+int fm_edge_rows(int n_atoms) {
+    const int sms = device_sms();
+    return sms * std::max(1, (n_atoms + kFmAtomsMax * sms - 1) / (kFmAtomsMax * sms));
+}
+
+int fm_residual_blocks(int n_atoms) { return (n_atoms + kResT - 1) / kResT; }
 
 // The per-atom adjoint pass: one block per SM (its registers allow one), one partial row per block.
 int fm_atom_ctas(int n_atoms) { return std::max(1, std::min(device_sms(), (n_atoms + kAtomWarps - 1) / kAtomWarps)); }
@@ -1516,22 +1543,25 @@ int fm_input_ctas(int n_atoms) {
 // Rows of the per-atom passes' partial buffer.
 int fm_atom_rows(int n_atoms) { return std::max(fm_atom_ctas(n_atoms), fm_input_ctas(n_atoms)); }
 
-// One frame's contribution: g from the forces already in p.force, then the
-// three passes; grad_out accumulates -dPsi/dtheta (+ c_E dE/dtheta with the
-// energy term), loss_out the loss. e_ref: this frame's reference energy on
-// the device, or null for force matching alone.
-void launch_fm_frame(const PotArgs& p, int K, const double* f_ref, double c_loss, float* g, double* sq,
-                     const float* m, float* mdot, float* mbar_psi, float* mdotbar_psi, float* ubar, float* partial_e,
-                     float* partial_a, int n_params, double* grad, double* loss, const FmEnergy& en,
-                     bool tensor_cores, int* status, cudaStream_t s) {
+// The contribution of p.n_atoms / frame_atoms frames, stored back to back as
+// systems of one batch: g from the forces already in p.force, then the three
+// passes; grad accumulates -dPsi/dtheta (+ c_E dE/dtheta with the energy
+// term), loss the loss.
+void launch_fm_frames(const PotArgs& p, int K, int frame_atoms, const double* f_ref, double c_loss, const FmBuffers& b,
+                      const float* m, int n_params, const FmEnergy& en, bool tensor_cores, int* status,
+                      cudaStream_t s) {
     const int n = p.n_atoms;
     if (n == 0) return;
-    k_fm_residual<<<(n + 255) / 256, 256, 0, s>>>(n, p.force, f_ref, c_loss, g, sq);
-    k_sum_all<<<1, kSumT, 0, s>>>(n, sq, 0.5 * c_loss, loss);
+    k_fm_residual<<<fm_residual_blocks(n), kResT, 0, s>>>(n, p.force, f_ref, c_loss, b.g, b.part, b.ticket, b.loss);
     if (en.e_ref) {
-        k_fm_energy_term<<<1, 32, 0, s>>>(en.n_sys, en.E, en.e_ref, en.lambda, n, en.inv_frames, en.c_energy, loss);
+        k_fm_energy_term<<<1, 32, 0, s>>>(n / frame_atoms, en.n_sys, en.E, en.e_ref, en.lambda, frame_atoms,
+                                          en.inv_frames, en.c_energy, b.loss);
         count_launch();
     }
+    float* const g = b.g;
+    float *const mdot = b.mdot, *const mbar_psi = b.mbar_psi, *const mdotbar_psi = b.mdotbar_psi, *const ubar = b.ubar;
+    float *const partial_e = b.partial_e, *const partial_a = b.partial_a;
+    double* const grad = b.grad;
     PotArgs a = p;
     a.atoms_per_cta = fm_edge_atoms(n, 2);               // the tangent pass: two CTAs per SM
     if (tensor_cores) {
@@ -1547,7 +1577,7 @@ void launch_fm_frame(const PotArgs& p, int K, const double* f_ref, double c_loss
     const int F = 32, S = (o.W_in[0] - o.A) / F;
     const int ga = fm_atom_ctas(n), ra = ga;             // one partial row per per-atom block
     k_fm_atom<<<ga, kAtomWarps * 32, 0, s>>>(a, m, mdot, mbar_psi, mdotbar_psi, partial_a, n_params,
-                                             en.e_ref ? en.c_energy : nullptr);
+                                             en.e_ref ? en.c_energy : nullptr, frame_atoms);
     fm_reduce(partial_a, ra, n_params, {{o.A, o.A + S * F},                      // A
                                         {o.U1[0], o.c2[0] + F},                 // U1, c1, U2, c2
                                         {o.R1, o.e0 + S}}, grad, s);            // R1, d1, R2, d2, e0
@@ -1565,7 +1595,7 @@ void launch_fm_frame(const PotArgs& p, int K, const double* f_ref, double c_loss
     k_fm_input<<<gi, kAtomWarps * 32, 0, s>>>(a, ubar, partial_a, n_params);
     fm_reduce(partial_a, gi, n_params, {{o.A, o.A + S * F},                      // A
                                         {o.W_in[0], o.W_in[0] + F * F}}, grad, s);   // W_in
-    count_launch(9);
+    count_launch(8);
 }
 
 }  // namespace dmts

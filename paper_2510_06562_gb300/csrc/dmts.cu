@@ -158,6 +158,7 @@ struct Model {
     float* erep = nullptr;
     size_t n_params = 0;
     std::vector<double> hp;            // the parameters as last uploaded (FP64, flat order)
+    long long version = 0;             // uploads so far
     ModelOffsets off{};
     float* P = nullptr;
     int nc = 0, n_cells = 0;
@@ -251,11 +252,15 @@ struct dmts_ctx {
     bool state_set = false, forces_valid = false;
     bool broken = false;
     bool autotune = true, tuned = false;
-    // force-matching buffers (allocated on first use)
-    float *fm_g = nullptr, *fm_m = nullptr, *fm_mdot = nullptr, *fm_mb = nullptr, *fm_mdb = nullptr,
-          *fm_ubar = nullptr, *fm_pe = nullptr, *fm_pa = nullptr;
-    double *fm_sq = nullptr, *fm_grad = nullptr, *fm_loss = nullptr, *fm_stage = nullptr;
-    double *fm_eref = nullptr, *fm_ce = nullptr;   // reference energies [fm_eref_cap], dL/dE scratch
+    // distillation: the frames of a call run in batches, as the systems of an
+    // inner context with the small model (its m[1]; the context itself when
+    // there is one frame or no memory for it), and the buffers of its passes
+    dmts_ctx* batch = nullptr;
+    int batch_frames = 0;                  // frames the inner context holds
+    long long batch_params = -1;           // m[0].version its weights were taken from
+    FmBuffers fm{};
+    int fm_atoms = 0;                      // atoms the buffers hold
+    double *fm_stage = nullptr, *fm_eref = nullptr, *fm_ce = nullptr;   // frames and forces; energies, dL/dE
     int fm_eref_cap = 0;
     cudaGraphExec_t graph = nullptr;
     int g_n_inner = 0;
@@ -492,6 +497,7 @@ std::vector<float> build_transposed(const Model& m, const std::vector<float>& pf
 
 int upload_params(dmts_ctx* c, Model& m, const double* params) {
     if (m.hp.data() != params) m.hp.assign(params, params + m.n_params);
+    ++m.version;
     std::vector<float> pf(m.n_params);
     for (size_t k = 0; k < m.n_params; ++k) pf[k] = (float)params[k];
     CUDA_TRY(cudaMemcpyAsync(m.P, pf.data(), pf.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream));
@@ -1252,6 +1258,17 @@ ModelOffsets model_offsets(int S, int F, int K, int L) {
 }
 }  // namespace dmts
 
+namespace {
+void free_fm(dmts_ctx* c) {
+    FmBuffers& b = c->fm;
+    dfree(b.g); dfree(b.mdot); dfree(b.mbar_psi); dfree(b.mdotbar_psi); dfree(b.ubar); dfree(b.partial_e);
+    dfree(b.partial_a); dfree(b.part); dfree(b.ticket); dfree(b.grad); dfree(b.loss); dfree(c->fm_stage);
+    b = FmBuffers{};
+    c->fm_stage = nullptr;
+    c->fm_atoms = 0;
+}
+}  // namespace
+
 extern "C" {
 
 const char* dmts_last_error(void) { return g_err.c_str(); }
@@ -1273,9 +1290,9 @@ void dmts_destroy(dmts_ctx* c) {
     if (c->s_big) cudaStreamDestroy(c->s_big);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
-    dfree(c->fm_g); dfree(c->fm_m); dfree(c->fm_mdot); dfree(c->fm_mb); dfree(c->fm_mdb); dfree(c->fm_ubar);
-    dfree(c->fm_pe); dfree(c->fm_pa); dfree(c->fm_sq); dfree(c->fm_grad); dfree(c->fm_loss); dfree(c->fm_stage);
+    free_fm(c);
     dfree(c->fm_eref); dfree(c->fm_ce);
+    dmts_destroy(c->batch);
     if (c->h_flags) cudaFreeHost(c->h_flags);
     if (c->stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -1682,79 +1699,172 @@ void* dmts_stream(dmts_ctx* c) { return c ? (void*)c->stream : nullptr; }
 
 namespace {
 
+// Atoms of one batch of distillation frames, about: enough to fill the GPU
+// while the batch's buffers stay below 1 GB. One frame at a time, its twenty
+// kernels of 3 to 120 us leave most SMs idle: 5 frames of 1,029 atoms (FP32)
+// 1.10 -> 0.40 ms in one batch, 8 of 12,288 (BF16) 3.09 -> 1.96 ms.
+constexpr int kFmBatchAtoms = 131072;
+
+// The inner context that evaluates `frames` frames of c's systems at once:
+// the systems repeated, the small model alone, its weights copied from c's.
+// Returns null if it cannot be created (no memory): one frame at a time then.
+dmts_ctx* batch_context(dmts_ctx* c, int frames) {
+    if (c->batch && c->batch_frames < frames) {
+        dmts_destroy(c->batch);
+        c->batch = nullptr;
+    }
+    const Model& m = c->m[0];
+    if (!c->batch) {
+        std::vector<int> off(1, 0), sp((size_t)c->N), spb;
+        std::vector<double> mass((size_t)frames * c->N, 1.0), box;
+        if (cudaMemcpy(sp.data(), c->d_species, sizeof(int) * c->N, cudaMemcpyDeviceToHost) != cudaSuccess) return nullptr;
+        for (int f = 0; f < frames; ++f) {
+            for (int k = 0; k < c->n_sys; ++k) off.push_back(f * c->N + c->h_off[k + 1]);
+            box.insert(box.end(), c->h_box.begin(), c->h_box.end());
+            spb.insert(spb.end(), sp.begin(), sp.end());
+        }
+        dmts_model_desc d{};
+        d.cutoff = m.rc; d.n_radial = m.K; d.n_layers = m.L; d.n_feat = m.F; d.n_species = m.S;
+        d.params = m.hp.data();
+        d.n_params = m.n_params;
+        d.precision = m.precision;
+        d.rep_a = m.rep_a; d.rep_rho = m.rep_rho; d.rep_cutoff = m.rep_rc;
+        const dmts_system_desc sys{frames * c->n_sys, off.data(), spb.data(), mass.data(), box.data()};
+        if (dmts_create(nullptr, &d, &sys, "{\"autotune\": 0}", &c->batch) != DMTS_OK) return nullptr;
+        c->batch_frames = frames;
+        c->batch_params = m.version;
+        c->batch->keep_msg = true;             // the second-order passes read every message row
+    }
+    return c->batch;
+}
+
+int alloc_fm(dmts_ctx* c, int atoms) {
+    if (c->fm_atoms >= atoms && c->fm.g) return DMTS_OK;
+    free_fm(c);
+    const Model& m = c->m[0];
+    const size_t nf = (size_t)atoms * m.F;
+    FmBuffers& b = c->fm;
+    cudaError_t e = dalloc(&b.g, (size_t)3 * atoms);
+    for (float** p : {&b.mdot, &b.mbar_psi, &b.mdotbar_psi, &b.ubar})
+        if (e == cudaSuccess) e = dalloc(p, nf);
+    if (e == cudaSuccess) e = dalloc(&b.partial_e, (size_t)fm_edge_rows(atoms) * m.n_params);
+    if (e == cudaSuccess) e = dalloc(&b.partial_a, (size_t)fm_atom_rows(atoms) * m.n_params);
+    if (e == cudaSuccess) e = dalloc(&b.part, (size_t)fm_residual_blocks(atoms));
+    if (e == cudaSuccess) e = dalloc(&b.ticket, 1);
+    if (e == cudaSuccess) e = cudaMemset(b.ticket, 0, sizeof(unsigned int));
+    if (e == cudaSuccess) e = dalloc(&b.grad, m.n_params);
+    if (e == cudaSuccess) e = dalloc(&b.loss, 1);
+    if (e == cudaSuccess) e = dalloc(&c->fm_stage, (size_t)6 * atoms);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        free_fm(c);
+        return fail(DMTS_ERR_OOM, "distillation buffers: %s", cudaGetErrorString(e));
+    }
+    c->fm_atoms = atoms;
+    return DMTS_OK;
+}
+
 // Distillation loss of the small model over n_frames frames and its
-// parameter gradient (e_ref null: force matching alone). Every frame is
-// enqueued without a host synchronisation; a neighbour overflow in any frame
-// grows the capacities and redoes the whole batch.
+// parameter gradient (e_ref null: force matching alone). The frames run in
+// batches of equal size, each batch as independent systems through one set of
+// launches, with no host synchronisation between batches; a neighbour
+// overflow in any frame grows the capacities and redoes the call.
 int distill_impl(dmts_ctx* c, int n_frames, const double* frames, const double* f_ref, const double* e_ref,
                  double lambda_e, double* loss_out, double* grad_out) {
     CTX_GUARD(c);
     Range nvtx_range("dmts_distill_grad");
-    Model& m = c->m[0];
-    if (!m.present) return fail(DMTS_ERR_ARG, "no small model in this context");
-    if (!fm_supported(m.F, m.K, m.L))
+    Model& m0 = c->m[0];
+    if (!m0.present) return fail(DMTS_ERR_ARG, "no small model in this context");
+    if (!fm_supported(m0.F, m0.K, m0.L))
         return fail(DMTS_ERR_ARG, "distillation needs a single-layer small model with n_feat 32, n_radial 8 or 16");
     if (n_frames < 1 || !frames || !f_ref || !loss_out || !grad_out) return fail(DMTS_ERR_ARG, "bad arguments");
     if (e_ref && !(lambda_e >= 0.0 && isfinite(lambda_e))) return fail(DMTS_ERR_ARG, "lambda_e must be >= 0");
-    LaunchScope ls(c);
     const int N = c->N;
-    const size_t n3 = (size_t)3 * N, nf = (size_t)N * m.F;
-    const int np = (int)m.n_params;
-    if (!c->fm_g) {
-        cudaError_t e = cudaSuccess;
-        if (e == cudaSuccess) e = dalloc(&c->fm_g, n3);
-        if (e == cudaSuccess) e = dalloc(&c->fm_m, nf);
-        if (e == cudaSuccess) e = dalloc(&c->fm_mdot, nf);
-        if (e == cudaSuccess) e = dalloc(&c->fm_mb, nf);
-        if (e == cudaSuccess) e = dalloc(&c->fm_mdb, nf);
-        if (e == cudaSuccess) e = dalloc(&c->fm_ubar, nf);
-        if (e == cudaSuccess) e = dalloc(&c->fm_pe, (size_t)fm_edge_ctas(N) * np);
-        if (e == cudaSuccess) e = dalloc(&c->fm_pa, (size_t)fm_atom_rows(N) * np);
-        if (e == cudaSuccess) e = dalloc(&c->fm_sq, N);
-        if (e == cudaSuccess) e = dalloc(&c->fm_grad, np);
-        if (e == cudaSuccess) e = dalloc(&c->fm_loss, 1);
-        if (e == cudaSuccess) e = dalloc(&c->fm_ce, 1);
-        if (e == cudaSuccess) e = dalloc(&c->fm_stage, 2 * n3);
-        if (e != cudaSuccess) return fail(DMTS_ERR_OOM, "distillation buffers: %s", cudaGetErrorString(e));
+    const size_t n3 = (size_t)3 * N;
+    const int np = (int)m0.n_params;
+    int rc;
+    // frames per batch: the number of batches that the target size asks for, evenly
+    const int most = (int)std::max<long long>(1, std::min<long long>(n_frames, kFmBatchAtoms / std::max(1, N)));
+    const int n_batches = (n_frames + most - 1) / most;
+    int per = (n_frames + n_batches - 1) / n_batches;
+    dmts_ctx* w = per > 1 ? batch_context(c, per) : nullptr;      // the context that evaluates the frames
+    if (w && alloc_fm(c, per * N) != DMTS_OK) w = nullptr;
+    if (!w) {
+        per = 1;
+        cudaGetLastError();
+        if ((rc = alloc_fm(c, N))) return rc;
+        w = c;
     }
+    const bool own = w == c;
+    const int which = own ? 0 : 1;
+    Model& m = w->m[which];
+    LaunchScope ls(c);
+    const cudaStream_t s = w->stream;
     if (e_ref && n_frames > c->fm_eref_cap) {
         dfree(c->fm_eref);
-        c->fm_eref = nullptr;
+        dfree(c->fm_ce);
+        c->fm_eref = c->fm_ce = nullptr;
         c->fm_eref_cap = 0;
         CUDA_TRY(dalloc(&c->fm_eref, (size_t)n_frames));
+        CUDA_TRY(dalloc(&c->fm_ce, (size_t)n_frames));
         c->fm_eref_cap = n_frames;
     }
-    int rc;
-    if (e_ref && (rc = copy_in(c, c->fm_eref, e_ref, (size_t)n_frames))) return rc;
-    // keep the dynamical state
-    CUDA_TRY(cudaMemcpyAsync(c->d_bx, c->d_x, n3 * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
-    CUDA_TRY(cudaMemcpyAsync(c->d_bv, c->d_v, n3 * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
-    // each frame's force and energy come from the model in its own precision
-    // (BF16 MLP operands on the tensor cores in DMTS_BF16_MLP mode); the
-    // second-order adjoint passes around them are FP32 and read every
-    // message row, so the split rows are written back (no fused fix-up)
-    struct KeepMsg {
-        dmts_ctx* c;
-        ~KeepMsg() { c->keep_msg = false; }
-    } keep_msg{c};
-    c->keep_msg = true;
+    if (e_ref && (rc = copy_in(w, c->fm_eref, e_ref, (size_t)n_frames))) return rc;
+    // After this call the context's state is what it was; the evaluations of a
+    // single frame at a time pass through it. In a batch, positions and
+    // velocities of the inner context are scratch.
+    struct Restore {
+        dmts_ctx *c, *w;
+        int N, n_sys, n_cells;
+        ~Restore() {
+            c->keep_msg = false;
+            if (w != c) {
+                w->N = N;
+                w->n_sys = n_sys;
+                w->m[1].n_cells = n_cells;
+            }
+        }
+    } restore{c, w, w->N, w->n_sys, m.n_cells};
+    if (own) {
+        CUDA_TRY(cudaMemcpyAsync(c->d_bx, c->d_x, n3 * sizeof(double), cudaMemcpyDeviceToDevice, s));
+        CUDA_TRY(cudaMemcpyAsync(c->d_bv, c->d_v, n3 * sizeof(double), cudaMemcpyDeviceToDevice, s));
+        c->keep_msg = true;                    // the second-order passes read every message row
+    } else {
+        m.apc_fwd = m0.apc_fwd; m.apc_bwd = m0.apc_bwd;
+        m.cps_fwd = m0.cps_fwd; m.cps_bwd = m0.cps_bwd;
+        m.bwd_tiles = m0.bwd_tiles;
+        if (c->batch_params != m0.version) {   // new weights since the last call
+            CUDA_TRY(cudaMemcpyAsync(m.P, m0.P, sizeof(float) * m.n_params, cudaMemcpyDeviceToDevice, s));
+            CUDA_TRY(cudaMemcpyAsync(m.wt, m0.wt, m.wt_layer_bytes * m.L, cudaMemcpyDeviceToDevice, s));
+            CUDA_TRY(cudaMemcpyAsync(m.PT, m0.PT, sizeof(float) * (3 * m.L + 1) * m.F * m.F, cudaMemcpyDeviceToDevice, s));
+            CUDA_TRY(cudaMemcpyAsync(m.at, m0.at, atom_tile_bytes(m.F, m.L), cudaMemcpyDeviceToDevice, s));
+            if ((rc = prepare_embedding(w, m))) return rc;
+            c->batch_params = m0.version;
+        }
+    }
     const double cl = 2.0 / (3.0 * (double)N * (double)n_frames);
-    for (int attempt = 0;; ++attempt) {
-        if ((rc = reset_flags(c))) return rc;
-        CUDA_TRY(cudaMemsetAsync(c->fm_grad, 0, sizeof(double) * np, c->stream));
-        CUDA_TRY(cudaMemsetAsync(c->fm_loss, 0, sizeof(double), c->stream));
-        for (int fr = 0; fr < n_frames && N > 0; ++fr) {
-            if ((rc = copy_in(c, c->fm_stage, frames + (size_t)fr * n3, n3))) return rc;
-            if ((rc = copy_in(c, c->fm_stage + n3, f_ref + (size_t)fr * n3, n3))) return rc;
-            // frame positions into x (velocities, saved above, are zeroed meanwhile)
-            launch_set_state(N, c->fm_stage, nullptr, c->d_sys, c->d_box, c->d_x, c->d_v, nullptr, c->stream);
-            enqueue_eval(c, 0, true, e_ref != nullptr);
-            CUDA_TRY(cudaMemcpyAsync(c->fm_m, m.msg, nf * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
-            PotArgs a = pot_args(c, m);
+    auto batches = [&]() -> int {
+        if ((rc = reset_flags(w))) return rc;
+        CUDA_TRY(cudaMemsetAsync(c->fm.grad, 0, sizeof(double) * np, s));
+        CUDA_TRY(cudaMemsetAsync(c->fm.loss, 0, sizeof(double), s));
+        for (int fr = 0; fr < n_frames && N > 0; fr += per) {
+            const int b = std::min(per, n_frames - fr), nb = b * N;
+            if (!own) {                        // the systems of this batch (the last may have fewer frames)
+                w->N = nb;
+                w->n_sys = b * c->n_sys;
+                m.n_cells = m.nc > 0 ? w->n_sys * m.nc * m.nc * m.nc : 0;
+            }
+            double* const xs = c->fm_stage;
+            double* const fs = c->fm_stage + (size_t)3 * nb;
+            if ((rc = copy_in(w, xs, frames + (size_t)fr * n3, b * n3))) return rc;
+            if ((rc = copy_in(w, fs, f_ref + (size_t)fr * n3, b * n3))) return rc;
+            launch_set_state(nb, xs, nullptr, w->d_sys, w->d_box, w->d_x, w->d_v, nullptr, s);
+            // each frame's force and energy come from the model in its own
+            // precision; the second-order passes follow
+            enqueue_eval(w, which, true, e_ref != nullptr);
+            PotArgs a = pot_args(w, m);
             a.layer = 0;
             a.u = m.u[0];                      // u^0 = h0 W_in (gathered per edge)
-            if (!a.u || !a.h || !a.force || !a.P || !a.row_ptr || !a.col || !a.recv || !a.q)
-                return fail(DMTS_ERR_STATE, "distillation: buffers missing");
             FmEnergy en;
             if (e_ref) {
                 en.e_ref = c->fm_eref + fr;
@@ -1764,21 +1874,35 @@ int distill_impl(dmts_ctx* c, int n_frames, const double* frames, const double* 
                 en.inv_frames = 1.0 / n_frames;
                 en.c_energy = c->fm_ce;
             }
-            launch_fm_frame(a, m.K, c->fm_stage + n3, cl, c->fm_g, c->fm_sq, c->fm_m, c->fm_mdot, c->fm_mb,
-                            c->fm_mdb, c->fm_ubar, c->fm_pe, c->fm_pa, np, c->fm_grad, c->fm_loss, en,
-                            m.precision == DMTS_BF16_MLP, c->d_flags + kFlagTimeout, c->stream);
+            // (the messages stay where the forward pass left them: a one-layer
+            // backward pass writes no per-atom vectors)
+            launch_fm_frames(a, m.K, N, fs, cl, c->fm, m.msg, np, en, m.precision == DMTS_BF16_MLP,
+                             w->d_flags + kFlagTimeout, s);
         }
-        if ((rc = sync_check(c))) return rc;
-        if (!c->h_flags[kFlagOverflow]) break;
+        return sync_check(w);
+    };
+    for (int attempt = 0;; ++attempt) {
+        if ((rc = batches())) {
+            c->broken = c->broken || w->broken;
+            return rc;
+        }
+        if (!w->h_flags[kFlagOverflow]) break;
         if (attempt == 3) return fail(DMTS_ERR_CAPACITY, "neighbour capacity overflow persists");
-        if ((rc = grow_capacity(c))) return rc;
+        if (!own) {                            // capacities for whole batches
+            w->N = restore.N;
+            w->n_sys = restore.n_sys;
+            m.n_cells = restore.n_cells;
+        }
+        if ((rc = grow_capacity(w))) return rc;
     }
-    CUDA_TRY(cudaMemcpyAsync(c->d_x, c->d_bx, n3 * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
-    CUDA_TRY(cudaMemcpyAsync(c->d_v, c->d_bv, n3 * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
+    if (own) {
+        CUDA_TRY(cudaMemcpyAsync(c->d_x, c->d_bx, n3 * sizeof(double), cudaMemcpyDeviceToDevice, s));
+        CUDA_TRY(cudaMemcpyAsync(c->d_v, c->d_bv, n3 * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    }
     c->forces_valid = false;
-    if ((rc = copy_out(c, grad_out, c->fm_grad, np))) return rc;
-    if ((rc = copy_out(c, loss_out, c->fm_loss, 1))) return rc;
-    return sync_check(c);
+    if ((rc = copy_out(w, grad_out, c->fm.grad, np))) return rc;
+    if ((rc = copy_out(w, loss_out, c->fm.loss, 1))) return rc;
+    return sync_check(w);
 }
 
 }  // namespace

@@ -350,21 +350,30 @@ int bf16_default_bwd_tiles(int F);
 
 // distill.cu: distillation (energy and force matching) gradient of a single-layer model
 bool fm_supported(int F, int K, int L);
-int fm_edge_ctas(int n_atoms);    // CTAs (= partial rows) of the gradient edge pass on the current device
+int fm_edge_rows(int n_atoms);    // partial rows of the gradient edge pass for up to n_atoms atoms
 int fm_atom_ctas(int n_atoms);    // blocks (= partial rows) of the per-atom adjoint pass
 int fm_atom_rows(int n_atoms);    // rows of the per-atom passes' partial buffer
-// Energy term of the distillation loss for one frame (e_ref null: none).
+int fm_residual_blocks(int n_atoms);
+// Energy term of the distillation loss (e_ref null: none).
 struct FmEnergy {
-    const double* e_ref = nullptr;   // device scalar: the frame's reference energy
-    const double* E = nullptr;       // device [n_sys]: the model's energies at the frame
+    const double* e_ref = nullptr;   // device: each frame's reference energy
+    const double* E = nullptr;       // device: the model's energies, n_sys per frame
     int n_sys = 0;
     double lambda = 0.0, inv_frames = 0.0;
-    double* c_energy = nullptr;      // device scalar scratch: dL/dE of the frame
+    double* c_energy = nullptr;      // device scratch: dL/dE of each frame
 };
-void launch_fm_frame(const PotArgs& p, int K, const double* f_ref, double c_loss, float* g, double* sq,
-                     const float* m, float* mdot, float* mbar_psi, float* mdotbar_psi, float* ubar, float* partial_e,
-                     float* partial_a, int n_params, double* grad, double* loss, const FmEnergy& en,
-                     bool tensor_cores, int* status, cudaStream_t s);
+// Buffers of the distillation passes for the atoms of one batch of frames.
+struct FmBuffers {
+    float *g = nullptr;                                      // [3][atoms] residual, dL/dF
+    float *mdot = nullptr, *mbar_psi = nullptr, *mdotbar_psi = nullptr, *ubar = nullptr;   // [atoms][F]
+    float *partial_e = nullptr, *partial_a = nullptr;        // partial gradient rows
+    double *part = nullptr;                                  // residual block sums
+    unsigned int* ticket = nullptr;                          // zero between launches
+    double *grad = nullptr, *loss = nullptr;
+};
+void launch_fm_frames(const PotArgs& p, int K, int frame_atoms, const double* f_ref, double c_loss, const FmBuffers& b,
+                      const float* m, int n_params, const FmEnergy& en, bool tensor_cores, int* status,
+                      cudaStream_t s);
 // (tensor_cores: the filter-weight gradient sums over pairs on tcgen05 with
 // BF16 operands; a bounded wait that gives up sets bit 0 of *status, bit 1
 // as well if the tensor-core work in flight did not drain)
@@ -381,7 +390,7 @@ size_t atom_tile_bytes(int F, int L);
 // few large systems are split over many CTAs; calls that may run at the same
 // time need separate scratch.
 constexpr int kSumChunks = 48;
-constexpr int kSumMaxSplit = 8;
+constexpr int kSumMaxSplit = 32;
 struct SumScratch {
     double* part;
     unsigned int* ctr;
