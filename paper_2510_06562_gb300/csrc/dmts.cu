@@ -199,7 +199,7 @@ struct Model {
 struct dmts_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
-    int N = 0, n_sys = 0;
+    int N = 0, n_sys = 0, max_sys = 0;     // atoms, systems, atoms of the largest system
     bool periodic = false;
     std::vector<int> h_off;
     std::vector<double> h_box;
@@ -770,6 +770,16 @@ void enqueue_rebuild(dmts_ctx* c, cudaStream_t s) {
     }
 }
 
+// Cells of model w for the kernel that writes the fixed-point positions to
+// fill (periodic systems with fresh lists); nc = 0: none.
+CellPlace cell_place(dmts_ctx* c, int w) {
+    const Model& m = c->m[w];
+    CellPlace p{};
+    if (c->periodic && c->skin <= 0 && m.present && m.nc > 0 && m.ccap > 0)
+        p = CellPlace{m.nc, m.ccap, m.cell_count, m.cell_atoms, m.cell_q, m.atom_pos, kFlagMaxCell0 + w};
+    return p;
+}
+
 enum class Check {
     None,     // positions unchanged since the last check: filter only
     Kernel,   // run the displacement check, then the (gated) rebuild
@@ -787,8 +797,16 @@ void enqueue_neighbors(dmts_ctx* c, int which, bool quantize, Check check = Chec
     Model& m = c->m[which];
     cudaStream_t s = c->stream;
     if (quantize) {
-        if (!c->periodic) launch_frames(c->n_sys, c->d_off, c->d_x, c->N, c->d_box, c->rc_max, c->d_frame, s);
-        launch_quantize(c->N, c->d_x, c->d_sys, c->d_frame, c->d_q, s);
+        // also places the atoms into the cells of a fresh periodic list
+        const CellPlace cp = cell_place(c, which);
+        if (c->periodic) launch_quantize(c->N, c->d_x, c->d_sys, c->d_frame, c->d_q, cp, c->d_flags, s);
+        else launch_frames(c->n_sys, c->max_sys, c->d_off, c->d_x, c->N, c->d_box, c->rc_max, c->d_frame, c->d_q, s);
+        if (cp.nc > 0) {
+            NbrArgs a = nbr_args(c, m, which);
+            a.placed = 1;
+            launch_neighbors(a, s);
+            return;
+        }
     }
     if (c->skin <= 0) {
         launch_neighbors(nbr_args(c, m, which), s);     // places the atoms into the cells first
@@ -1042,16 +1060,6 @@ cudaError_t capture_fallback_node(dmts_ctx* c, cudaGraphConditionalHandle h, int
     return cudaStreamUpdateCaptureDependencies(c->stream, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
 }
 
-// Cells of model w for the integrator kernel to fill (periodic systems with
-// fresh lists, whose fixed-point positions that kernel writes); nc = 0: none.
-CellPlace cell_place(dmts_ctx* c, int w) {
-    const Model& m = c->m[w];
-    CellPlace p{};
-    if (c->periodic && c->skin <= 0 && m.present && m.nc > 0 && m.ccap > 0)
-        p = CellPlace{m.nc, m.ccap, m.cell_count, m.cell_atoms, m.cell_q, m.atom_pos, kFlagMaxCell0 + w};
-    return p;
-}
-
 // F_small as the integrator kernels of a captured step read it (ForceFold).
 ForceFold small_fold(dmts_ctx* c) {
     const Model& m = c->m[0];
@@ -1112,8 +1120,8 @@ int capture_step_graph(dmts_ctx* c, int n_inner, double dt) {
             c->m[1].placed = last && cp1.nc > 0;
             if (fork && k == n_inner - 1) {
                 if (nonper) {                                  // frames and fixed-point positions for both
-                    launch_frames(c->n_sys, c->d_off, c->d_x, c->N, c->d_box, c->rc_max, c->d_frame, s);
-                    launch_quantize(c->N, c->d_x, c->d_sys, c->d_frame, c->d_q, s);
+                    launch_frames(c->n_sys, c->max_sys, c->d_off, c->d_x, c->N, c->d_box, c->rc_max, c->d_frame, c->d_q,
+                                  s);
                 }
                 CUDA_TRY(cudaEventRecord(c->ev_fork, s));
                 CUDA_TRY(cudaStreamWaitEvent(c->s_big, c->ev_fork, 0));
@@ -1347,6 +1355,7 @@ int dmts_create(const dmts_model_desc* small, const dmts_model_desc* big, const 
     c->N = N;
     c->n_sys = ns;
     c->periodic = n_per > 0;
+    for (int s = 0; s < ns; ++s) c->max_sys = std::max(c->max_sys, sys->atom_offset[s + 1] - sys->atom_offset[s]);
     c->h_off.assign(sys->atom_offset, sys->atom_offset + ns + 1);
     c->h_box.assign(sys->box, sys->box + ns);
     c->rc_max = rc_max;
@@ -1493,7 +1502,7 @@ int dmts_create(const dmts_model_desc* small, const dmts_model_desc* big, const 
     }
     if (c->periodic) {
         // constant frame; computed once on the device
-        launch_frames(ns, c->d_off, c->d_x, N, c->d_box, rc_max, c->d_frame, c->stream);
+        launch_frames(ns, c->max_sys, c->d_off, c->d_x, N, c->d_box, rc_max, c->d_frame, nullptr, c->stream);
         CREATE_TRY(cudaStreamSynchronize(c->stream));
     }
     CREATE_TRY(cudaGetLastError());

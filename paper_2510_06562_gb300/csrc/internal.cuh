@@ -309,10 +309,12 @@ struct PotArgs {
 
 // ---------------------------------------------------------------- launchers
 // neighbours.cu
-void launch_frames(int n_sys, const int* atom_offset, const double* x, int n_atoms,
-                   const double* box, double rc_max, Frame* frame, cudaStream_t s);
-void launch_quantize(int n_atoms, const double* x, const int* sys_of_atom, const Frame* frame,
-                     uint4* q, cudaStream_t s);
+// Frames of all systems (of at most max_atoms atoms each) and, with q, the
+// fixed-point positions.
+void launch_frames(int n_sys, int max_atoms, const int* atom_offset, const double* x, int n_atoms, const double* box,
+                   double rc_max, Frame* frame, uint4* q, cudaStream_t s);
+void launch_quantize(int n_atoms, const double* x, const int* sys_of_atom, const Frame* frame, uint4* q,
+                     const CellPlace& cp, int* flags, cudaStream_t s);
 void launch_neighbors(const NbrArgs& a, cudaStream_t s);
 // Fresh pair list with fixed-capacity cells (a.ccap > 0; a.cell_count zero on
 // entry, and again on exit): placement, row build, row scan, compaction.

@@ -34,12 +34,33 @@ namespace dmts {
 // Non-periodic systems: origin = lower corner of the bounding box, Q = the
 // smallest power of two >= 2 (extent + 2 rc_max + 1) so that every in-cutoff
 // difference stays far below Q/2. Periodic systems: origin 0, Q = L.
-__global__ void k_frames(int n_sys, const int* __restrict__ off, const double* __restrict__ x,
-                         int n, const double* __restrict__ box, double rc_max,
-                         Frame* __restrict__ frame) {
-    int s = blockIdx.x;
-    if (s >= n_sys) return;
-    double L = box[s];
+__device__ __forceinline__ unsigned int to_fixed(double v, double o, double inv) {
+    double t = floor((v - o) * inv);
+    long long k = (long long)t;
+    return (unsigned int)(k & 0xffffffffll);
+}
+
+__device__ __forceinline__ uint4 fixed_position(const double* __restrict__ x, int n, int i, int s, const Frame& f) {
+    uint4 r;
+    r.x = to_fixed(x[i], f.ox, f.inv);
+    r.y = to_fixed(x[(size_t)n + i], f.oy, f.inv);
+    r.z = to_fixed(x[2 * (size_t)n + i], f.oz, f.inv);
+    r.w = (unsigned int)s;
+    return r;
+}
+
+// One block per system: its frame and, with q, the fixed-point positions of
+// its atoms. The bounds are FP64 minima and maxima, which this GPU runs at
+// two lanes per SM and clock: a block of one warp for small molecules reduces
+// them once instead of in eight warps (512 molecules of 10 to 60 atoms:
+// frames and positions 21 -> 8 us; a 3 fs step of them 0.49 -> 0.455 ms).
+__global__ void __launch_bounds__(256) k_frames(int n_sys, const int* __restrict__ off, const double* __restrict__ x,
+                                                int n, const double* __restrict__ box, double rc_max,
+                                                Frame* __restrict__ frame, uint4* __restrict__ q) {
+    const int s = blockIdx.x;
+    const double L = box[s];
+    const int beg = off[s], end = off[s + 1];
+    __shared__ Frame sf;
     if (L > 0.0) {
         if (threadIdx.x == 0) {
             Frame f;
@@ -48,79 +69,82 @@ __global__ void k_frames(int n_sys, const int* __restrict__ off, const double* _
             f.qscale = (float)(L / 4294967296.0);
             f.pad = 0.f;
             frame[s] = f;
+            sf = f;
         }
-        return;
+    } else {
+        __shared__ double smin[3][8], smax[3][8];
+        double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
+        for (int i = beg + threadIdx.x; i < end; i += blockDim.x) {
+            for (int c = 0; c < 3; ++c) {
+                double v = x[(size_t)c * n + i];
+                lo[c] = fmin(lo[c], v);
+                hi[c] = fmax(hi[c], v);
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                lo[c] = fmin(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
+                hi[c] = fmax(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
+            }
+        const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+        if (lane == 0)
+            for (int c = 0; c < 3; ++c) { smin[c][w] = lo[c]; smax[c][w] = hi[c]; }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double ext = 0.0, o3[3];
+            for (int c = 0; c < 3; ++c) {
+                double a = 1e300, b = -1e300;
+                for (int k = 0; k < nw; ++k) { a = fmin(a, smin[c][k]); b = fmax(b, smax[c][k]); }
+                if (end == beg) { a = 0.0; b = 0.0; }
+                o3[c] = a;
+                ext = fmax(ext, b - a);
+            }
+            const double need = 2.0 * (ext + 2.0 * rc_max + 1.0);
+            // the smallest power of two >= max(need, 1), from need's exponent (NaN: 1)
+            const long long bits = __double_as_longlong(need);
+            int e = (int)((bits >> 52) & 0x7ff) - 1023 + ((bits & 0xfffffffffffffll) != 0 ? 1 : 0);
+            e = need >= 1.0 ? min(e, 1024) : 0;
+            const double Q = __longlong_as_double((long long)(e + 1023) << 52);
+            Frame f;
+            f.ox = o3[0]; f.oy = o3[1]; f.oz = o3[2];
+            f.inv = 4294967296.0 / Q;
+            f.qscale = (float)(Q / 4294967296.0);
+            f.pad = 0.f;
+            frame[s] = f;
+            sf = f;
+        }
     }
-    __shared__ double smin[3][32], smax[3][32];
-    double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
-    for (int i = off[s] + threadIdx.x; i < off[s + 1]; i += blockDim.x) {
-        for (int c = 0; c < 3; ++c) {
-            double v = x[(size_t)c * n + i];
-            lo[c] = fmin(lo[c], v);
-            hi[c] = fmax(hi[c], v);
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1)
-        for (int c = 0; c < 3; ++c) {
-            lo[c] = fmin(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
-            hi[c] = fmax(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
-        }
-    int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0)
-        for (int c = 0; c < 3; ++c) { smin[c][w] = lo[c]; smax[c][w] = hi[c]; }
+    if (!q) return;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int nw = blockDim.x >> 5;
-        double ext = 0.0, o3[3];
-        for (int c = 0; c < 3; ++c) {
-            double a = 1e300, b = -1e300;
-            for (int k = 0; k < nw; ++k) { a = fmin(a, smin[c][k]); b = fmax(b, smax[c][k]); }
-            if (off[s + 1] == off[s]) { a = 0.0; b = 0.0; }
-            o3[c] = a;
-            ext = fmax(ext, b - a);
-        }
-        double need = 2.0 * (ext + 2.0 * rc_max + 1.0);
-        double Q = 1.0;
-        while (Q < need) Q *= 2.0;
-        Frame f;
-        f.ox = o3[0]; f.oy = o3[1]; f.oz = o3[2];
-        f.inv = 4294967296.0 / Q;
-        f.qscale = (float)(Q / 4294967296.0);
-        f.pad = 0.f;
-        frame[s] = f;
-    }
+    const Frame f = sf;
+    for (int i = beg + threadIdx.x; i < end; i += blockDim.x) q[i] = fixed_position(x, n, i, s, f);
 }
 
-void launch_frames(int n_sys, const int* atom_offset, const double* x, int n_atoms,
-                   const double* box, double rc_max, Frame* frame, cudaStream_t s) {
-    k_frames<<<n_sys, 256, 0, s>>>(n_sys, atom_offset, x, n_atoms, box, rc_max, frame);
+void launch_frames(int n_sys, int max_atoms, const int* atom_offset, const double* x, int n_atoms, const double* box,
+                   double rc_max, Frame* frame, uint4* q, cudaStream_t s) {
+    k_frames<<<n_sys, max_atoms <= 128 ? 32 : 256, 0, s>>>(n_sys, atom_offset, x, n_atoms, box, rc_max, frame, q);
     count_launch();
 }
 
-__device__ __forceinline__ unsigned int to_fixed(double v, double o, double inv) {
-    double t = floor((v - o) * inv);
-    long long k = (long long)t;
-    return (unsigned int)(k & 0xffffffffll);
-}
-
+// Fixed-point positions of periodic systems; with cp.nc > 0 each atom also
+// takes its slot in those cells (the build then skips k_cell_place).
 __global__ void k_quantize(int n, const double* __restrict__ x, const int* __restrict__ sys,
-                           const Frame* __restrict__ frame, uint4* __restrict__ q) {
+                           const Frame* __restrict__ frame, uint4* __restrict__ q, CellPlace cp,
+                           int* __restrict__ flags) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int s = sys[i];
-    Frame f = frame[s];
-    uint4 r;
-    r.x = to_fixed(x[i], f.ox, f.inv);
-    r.y = to_fixed(x[(size_t)n + i], f.oy, f.inv);
-    r.z = to_fixed(x[2 * (size_t)n + i], f.oz, f.inv);
-    r.w = (unsigned int)s;
+    const uint4 r = fixed_position(x, n, i, s, frame[s]);
     q[i] = r;
+    if (cp.nc > 0) place_in_cell(cp, i, r, flags);
 }
 
-void launch_quantize(int n_atoms, const double* x, const int* sys_of_atom, const Frame* frame,
-                     uint4* q, cudaStream_t s) {
+void launch_quantize(int n_atoms, const double* x, const int* sys_of_atom, const Frame* frame, uint4* q,
+                     const CellPlace& cp, int* flags, cudaStream_t s) {
     if (n_atoms == 0) return;
-    k_quantize<<<(n_atoms + 255) / 256, 256, 0, s>>>(n_atoms, x, sys_of_atom, frame, q);
+    k_quantize<<<(n_atoms + 127) / 128, 128, 0, s>>>(n_atoms, x, sys_of_atom, frame, q, cp, flags);
     count_launch();
 }
 
