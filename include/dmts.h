@@ -197,7 +197,8 @@ DMTS_API int dmts_get_state(dmts_ctx* ctx, double* x, double* v);
 /* Evaluate one model (DMTS_SMALL or DMTS_BIG) at the current positions.
  * f_out [N*3] forces F = -dE/dx (or NULL); energy_out [n_systems] potential
  * energies (or NULL); virial_out [n_systems*9] row-major 3x3 virial
- * W_ab = -sum_pairs r_ij,a dE/dr_ij,b (or NULL). */
+ * W_ab = -sum_pairs r_ij,a dE/dr_ij,b (or NULL). If the call fails, their
+ * contents are unspecified. */
 DMTS_API int dmts_forces(dmts_ctx* ctx, int which, double* f_out, double* energy_out,
                 double* virial_out);
 

@@ -293,6 +293,17 @@ bool is_device_ptr(const void* p) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// Memory of the context's own device, which its kernels may read and write
+// directly (memory elsewhere goes through a staging buffer).
+bool is_own_device_ptr(const dmts_ctx* c, const void* p) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == c->device;
+}
+
 template <class T>
 cudaError_t dalloc(T** p, size_t n) {
     *p = nullptr;
@@ -1517,12 +1528,18 @@ int dmts_set_state(dmts_ctx* c, const double* x, const double* v, int n_atoms) {
     if (n_atoms != c->N) return fail(DMTS_ERR_ARG, "n_atoms %d != %d", n_atoms, c->N);
     LaunchScope ls(c);
     size_t n3 = (size_t)3 * c->N;
-    int rc = copy_in(c, c->d_stage, x, n3);
-    if (rc) return rc;
-    if (v && (rc = copy_in(c, c->d_stage + n3, v, n3))) return rc;
+    int rc;
+    const double *xs = x, *vs = v;
+    if (!is_own_device_ptr(c, x)) {
+        if ((rc = copy_in(c, c->d_stage, x, n3))) return rc;
+        xs = c->d_stage;
+    }
+    if (v && !is_own_device_ptr(c, v)) {
+        if ((rc = copy_in(c, c->d_stage + n3, v, n3))) return rc;
+        vs = c->d_stage + n3;
+    }
     CUDA_TRY(cudaMemsetAsync(c->d_flags + kFlagMoved, 0, sizeof(int), c->stream));
-    launch_set_state(c->N, c->d_stage, v ? c->d_stage + n3 : nullptr, c->d_sys, c->d_box, c->d_x, c->d_v,
-                     c->d_flags + kFlagMoved, c->stream);
+    launch_set_state(c->N, xs, vs, c->d_sys, c->d_box, c->d_x, c->d_v, c->d_flags + kFlagMoved, c->stream);
     CUDA_TRY(cudaMemsetAsync(c->d_rng, 0, sizeof(unsigned long long), c->stream));   // noise restarts at step 0
     if ((rc = sync_check(c))) return rc;
     // The forces depend on the positions only, and every evaluation of them is
@@ -1538,10 +1555,12 @@ int dmts_get_state(dmts_ctx* c, double* x, double* v) {
     Range nvtx_range("dmts_get_state");
     LaunchScope ls(c);
     size_t n3 = (size_t)3 * c->N;
-    launch_get_state(c->N, c->d_x, c->d_v, c->d_stage, c->d_stage + n3, c->stream);
+    const bool xd = x && is_own_device_ptr(c, x), vd = v && is_own_device_ptr(c, v);
+    launch_get_state(c->N, c->d_x, c->d_v, xd ? x : (x ? c->d_stage : nullptr),
+                     vd ? v : (v ? c->d_stage + n3 : nullptr), c->stream);
     int rc;
-    if (x && (rc = copy_out(c, x, c->d_stage, n3))) return rc;
-    if (v && (rc = copy_out(c, v, c->d_stage + n3, n3))) return rc;
+    if (x && !xd && (rc = copy_out(c, x, c->d_stage, n3))) return rc;
+    if (v && !vd && (rc = copy_out(c, v, c->d_stage + n3, n3))) return rc;
     return sync_check(c);
 }
 
@@ -1555,23 +1574,23 @@ int dmts_forces(dmts_ctx* c, int which, double* f_out, double* energy_out, doubl
     Model& m = c->m[which];
     int rc;
     if ((rc = autotune_models(c))) return rc;
+    const size_t n3 = (size_t)3 * c->N;
+    const bool fd = f_out && is_own_device_ptr(c, f_out);
+    // the outputs follow the evaluation on the stream (one wait); after an
+    // overflow they are written again
     for (int attempt = 0; attempt < 4; ++attempt) {
         if ((rc = reset_flags(c))) return rc;
         enqueue_eval(c, which, true, true, Check::Kernel, virial_out != nullptr);
         if (virial_out) launch_virial_sum(c->n_sys, c->d_off, m.vir6, m.W, c->stream);
+        if (f_out) launch_forces_out(c->N, m.force, fd ? f_out : c->d_stage, c->stream);
+        if (f_out && !fd && (rc = copy_out(c, f_out, c->d_stage, n3))) return rc;
+        if (energy_out && (rc = copy_out(c, energy_out, m.E, c->n_sys))) return rc;
+        if (virial_out && (rc = copy_out(c, virial_out, m.W, (size_t)9 * c->n_sys))) return rc;
         if ((rc = sync_check(c))) return rc;
-        if (!c->h_flags[kFlagOverflow]) break;
+        if (!c->h_flags[kFlagOverflow]) return DMTS_OK;
         if ((rc = grow_capacity(c))) return rc;
-        if (attempt == 3) return fail(DMTS_ERR_CAPACITY, "neighbour capacity overflow persists");
     }
-    size_t n3 = (size_t)3 * c->N;
-    if (f_out) {
-        launch_forces_out(c->N, m.force, c->d_stage, c->stream);
-        if ((rc = copy_out(c, f_out, c->d_stage, n3))) return rc;
-    }
-    if (energy_out && (rc = copy_out(c, energy_out, m.E, c->n_sys))) return rc;
-    if (virial_out && (rc = copy_out(c, virial_out, m.W, (size_t)9 * c->n_sys))) return rc;
-    return sync_check(c);
+    return fail(DMTS_ERR_CAPACITY, "neighbour capacity overflow persists");
 }
 
 int dmts_neighbors(dmts_ctx* c, int which, int* row_ptr, int* col, long long capacity, long long* n_pairs) {
