@@ -614,7 +614,7 @@ int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells) {
     CUDA_TRY(dalloc(&m.Ei, N));
     CUDA_TRY(dalloc(&m.erep, N));
     CUDA_TRY(dalloc(&m.E, c->n_sys));
-    CUDA_TRY(dalloc(&m.esum.part, (size_t)kSumMaxSplit * kSumChunks));
+    CUDA_TRY(dalloc(&m.esum.part, (size_t)kSumMaxSplit * kSumChunks * 6));
     CUDA_TRY(dalloc(&m.esum.ctr, kSumMaxSplit));
     CUDA_TRY(cudaMemset(m.esum.ctr, 0, sizeof(unsigned int) * kSumMaxSplit));
     CUDA_TRY(dalloc(&m.W, (size_t)9 * c->n_sys));
@@ -1581,7 +1581,7 @@ int dmts_forces(dmts_ctx* c, int which, double* f_out, double* energy_out, doubl
     for (int attempt = 0; attempt < 4; ++attempt) {
         if ((rc = reset_flags(c))) return rc;
         enqueue_eval(c, which, true, true, Check::Kernel, virial_out != nullptr);
-        if (virial_out) launch_virial_sum(c->n_sys, c->d_off, m.vir6, m.W, c->stream);
+        if (virial_out) launch_virial_sum(c->n_sys, c->d_off, m.vir6, m.W, m.esum, c->stream);
         if (f_out) launch_forces_out(c->N, m.force, fd ? f_out : c->d_stage, c->stream);
         if (f_out && !fd && (rc = copy_out(c, f_out, c->d_stage, n3))) return rc;
         if (energy_out && (rc = copy_out(c, energy_out, m.E, c->n_sys))) return rc;

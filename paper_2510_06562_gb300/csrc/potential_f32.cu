@@ -885,9 +885,62 @@ __global__ void k_virial_sum(int n_sys, const int* __restrict__ off, const float
     }
 }
 
-void launch_virial_sum(int n_sys, const int* atom_offset, const float* vir6, double* out,
+// A few large systems: as k_system_sum_split, for the six components at once
+// (FP64 additions run at two lanes per SM and clock: in one block, the virial of
+// 12,288 atoms made the call 752 -> 808 us).
+__global__ void __launch_bounds__(128) k_virial_split(const int* __restrict__ off, const float* __restrict__ v6,
+                                                      double* __restrict__ out, double* __restrict__ part,
+                                                      unsigned int* __restrict__ ctr) {
+    __shared__ double wsum[4][6];
+    __shared__ bool last;
+    const int s = blockIdx.y, b = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int begin = off[s], end = off[s + 1];
+    const int per = (end - begin + kSumChunks - 1) / kSumChunks;
+    const int lo = begin + b * per, hi = min(end, lo + per);
+    double acc[6] = {0, 0, 0, 0, 0, 0};
+    for (int i = lo + threadIdx.x; i < hi; i += 128)
+#pragma unroll
+        for (int c = 0; c < 6; ++c) acc[c] += (double)v6[(size_t)i * 6 + c];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_down_sync(0xffffffffu, acc[c], o);
+        if (lane == 0) wsum[w][c] = acc[c];
+    }
+    __syncthreads();
+    double* p = part + ((size_t)s * kSumChunks + b) * 6;
+    if (threadIdx.x < 6) {
+        p[threadIdx.x] = (wsum[0][threadIdx.x] + wsum[1][threadIdx.x]) + (wsum[2][threadIdx.x] + wsum[3][threadIdx.x]);
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&ctr[s], 1u) == (unsigned int)kSumChunks - 1u;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    __shared__ double tot[6];
+    if (threadIdx.x < 6) {
+        double t = 0.0;
+        for (int k = 0; k < kSumChunks; ++k) t += __ldcg(part + ((size_t)s * kSumChunks + k) * 6 + threadIdx.x);
+        tot[threadIdx.x] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double* o = out + (size_t)s * 9;
+        o[0] = tot[0]; o[4] = tot[1]; o[8] = tot[2];
+        o[1] = o[3] = tot[3];
+        o[2] = o[6] = tot[4];
+        o[5] = o[7] = tot[5];
+        ctr[s] = 0u;
+    }
+}
+
+void launch_virial_sum(int n_sys, const int* atom_offset, const float* vir6, double* out, const SumScratch& sc,
                        cudaStream_t s) {
-    k_virial_sum<<<n_sys, 128, 0, s>>>(n_sys, atom_offset, vir6, out);
+    if (n_sys <= kSumMaxSplit && sc.part)
+        k_virial_split<<<dim3(kSumChunks, n_sys), 128, 0, s>>>(atom_offset, vir6, out, sc.part, sc.ctr);
+    else
+        k_virial_sum<<<n_sys, 128, 0, s>>>(n_sys, atom_offset, vir6, out);
     count_launch();
 }
 
