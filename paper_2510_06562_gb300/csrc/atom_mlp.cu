@@ -115,6 +115,18 @@ __device__ __forceinline__ void gemm_blk(const float* X, const float* Ws, int a0
     }
 }
 
+// The same for species s of the [N][n_species][F] sums.
+template <int F>
+__device__ __forceinline__ void stage_species(float* X, const float* __restrict__ src, int s, int n_species, int base,
+                                              int n_atoms) {
+    using T = AtomTile<F>;
+    for (int t = threadIdx.x; t < T::A * F / 4; t += T::NT) {
+        const int a = t / (F / 4), c = (t % (F / 4)) * 4;
+        if (base + a < n_atoms) cp_async16(X + a * T::XS + c, src + ((size_t)(base + a) * n_species + s) * F + c);
+        else *reinterpret_cast<float4*>(X + a * T::XS + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+
 template <int F>
 __device__ __forceinline__ void put_rows(float* X, int a0, int f0,
                                          const float (&v)[AtomTile<F>::RA][AtomTile<F>::RF]) {
@@ -183,7 +195,54 @@ __device__ __forceinline__ const float* r1t_of(const PotArgs& p, int F) {
     return p.PT + (size_t)3 * p.n_layers * F * F;
 }
 
+__device__ __forceinline__ const float* w2t_of(const PotArgs& p, int F) {
+    return p.PT + ((size_t)3 * p.n_layers + 1) * F * F;
+}
+
+// Layer 0 by species, backward: from the block's mbar^0 (v) the rows
+// Y_is = W2 (mbar_i * u_s) and scalars B_is = b2 . (mbar_i * u_s) of every
+// species s, over the forward pass's sums. W holds W2^T; A0 and A1 are row
+// buffers, A0 free on entry, A1 read by the preceding product.
 template <int F>
+__device__ __forceinline__ void species_adjoint(const PotArgs& p, float* A0, float* A1, const float* W, int base, int a0,
+                                                int f0, const float (&v)[AtomTile<F>::RA][AtomTile<F>::RF]) {
+    using T = AtomTile<F>;
+    float b2[T::RF];
+#pragma unroll
+    for (int f = 0; f < T::RF; ++f) b2[f] = __ldg(p.P + p.off.b2[0] + f0 + f);
+    for (int s = 0; s < p.n_species; ++s) {
+        float x[T::RA][T::RF], y[T::RA][T::RF], part[T::RA];
+#pragma unroll
+        for (int a = 0; a < T::RA; ++a) part[a] = 0.f;
+#pragma unroll
+        for (int f = 0; f < T::RF; ++f) {
+            const float us = __ldg(p.u_spec + s * F + f0 + f);
+#pragma unroll
+            for (int a = 0; a < T::RA; ++a) {
+                x[a][f] = v[a][f] * us;
+                part[a] += x[a][f] * b2[f];
+            }
+        }
+        put_rows<F>(A0, a0, f0, x);
+#pragma unroll
+        for (int a = 0; a < T::RA; ++a)
+#pragma unroll
+            for (int o = T::FG / 2; o > 0; o >>= 1) part[a] += __shfl_xor_sync(0xffffffffu, part[a], o);
+        __syncthreads();
+        gemm_blk<F>(A0, W, a0, f0, y);
+#pragma unroll
+        for (int a = 0; a < T::RA; ++a) {
+            const int i = base + a0 + a;
+            if (i >= p.n_atoms) continue;
+            const size_t row = (size_t)i * p.n_species + s;
+            st_vec<T::RF>(p.spec_row + row * F + f0, y[a]);
+            if (f0 == 0) p.spec_sum[row] = part[a];
+        }
+        float* t = A0; A0 = A1; A1 = t;
+    }
+}
+
+template <int F, bool SPEC>
 __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_fwd(PotArgs p, const float* __restrict__ msg) {
     using T = AtomTile<F>;
     extern __shared__ float4 smem4[];
@@ -201,9 +260,15 @@ __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_fwd(PotArgs p, const f
     const bool last = (l == p.n_layers - 1);
     float z[T::RA][T::RF], v[T::RA][T::RF], h[T::RA][T::RF];
 
-    stage_rows<F>(X, msg, base, p.n_atoms);
+    const bool by_species = SPEC && l == 0;          // the messages are formed here (below)
+    if (by_species) {
+        stage_species<F>(X, p.spec_row, 0, p.n_species, base, p.n_atoms);
+        stage_w<F>(W1, P + p.off.W2[0]);                                 // group: first species' sums + W2
+    } else {
+        stage_rows<F>(X, msg, base, p.n_atoms);
+    }
     stage_w<F>(W0, P + p.off.U1[l]);                                     // group: message rows + U1
-    stage_w<F>(W1, P + p.off.U2[l]);                                     // group: U2
+    if (!by_species) stage_w<F>(W1, P + p.off.U2[l]);                    // group: U2
     load_rows<F>(h, p.h_in, base, p.n_atoms, a0, f0);
     // the small per-layer vectors and the per-atom energy constants, loaded while the copies run
     for (int t = tid; t < F; t += T::NT) {
@@ -243,6 +308,42 @@ __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_fwd(PotArgs p, const f
             erep = p.erep[i];
         }
         if (last) e_const = (double)__ldg(P + p.off.d2) + (double)__ldg(P + p.off.e0 + p.species[i]) + (double)erep;
+    }
+    if (by_species) {
+        // m_i = sum_s u_s * (T_is W2 + t_is b2)
+        float m[T::RA][T::RF];
+#pragma unroll
+        for (int a = 0; a < T::RA; ++a)
+#pragma unroll
+            for (int f = 0; f < T::RF; ++f) m[a][f] = 0.f;
+        float *cur = X, *nxt = Y;
+        for (int s = 0; s < p.n_species; ++s) {
+            if (s + 1 < p.n_species) {
+                stage_species<F>(nxt, p.spec_row, s + 1, p.n_species, base, p.n_atoms);
+                cp_commit();
+                if (s == 0) cp_wait<2>();                                // (U1 is in flight too)
+                else cp_wait<1>();
+            } else {
+                cp_wait<0>();
+            }
+            __syncthreads();
+            gemm_blk<F>(cur, W1, a0, f0, v);
+            float t[T::RA];
+#pragma unroll
+            for (int a = 0; a < T::RA; ++a)
+                t[a] = base + a0 + a < p.n_atoms ? p.spec_sum[(size_t)(base + a0 + a) * p.n_species + s] : 0.f;
+#pragma unroll
+            for (int f = 0; f < T::RF; ++f) {
+                const float us = __ldg(p.u_spec + s * F + f0 + f), b2 = __ldg(P + p.off.b2[0] + f0 + f);
+#pragma unroll
+                for (int a = 0; a < T::RA; ++a) m[a][f] += us * (v[a][f] + t[a] * b2);
+            }
+            __syncthreads();                                             // cur (and, at the end, W2) read
+            float* sw = cur; cur = nxt; nxt = sw;
+        }
+        stage_w<F>(W1, P + p.off.U2[l]);                                 // group: U2
+        put_rows<F>(X, a0, f0, m);
+        if (p.keep_msg) store_rows<F>(p.msg_out, base, p.n_atoms, a0, f0, m);
     }
     cp_wait<1>();
     __syncthreads();
@@ -356,13 +457,18 @@ __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_fwd(PotArgs p, const f
         }
     put_rows<F>(Y, a0, f0, v);
     cp_wait<0>();
-    __syncthreads();
+    __syncthreads();                                                     // W0 and X read, Y complete
+    if (by_species) stage_w<F>(W0, w2t_of(p, F));
     gemm_blk<F>(Y, W1, a0, f0, v);                                       // mbar = gz U1^T
     store_rows<F>(p.mbar_out, base, p.n_atoms, a0, f0, v);
     store_rows_bf16<F>(p.um_mbar_out, 1, base, p.n_atoms, a0, f0, v);
+    if (by_species) {
+        cp_wait<0>();                                                    // (visible after the first barrier inside)
+        species_adjoint<F>(p, X, Y, W0, base, a0, f0, v);
+    }
 }
 
-template <int F>
+template <int F, bool SPEC>
 __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_bwd(PotArgs p, const float* __restrict__ ubar) {
     using T = AtomTile<F>;
     extern __shared__ float4 smem4[];
@@ -403,39 +509,47 @@ __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_bwd(PotArgs p, const f
         }
     put_rows<F>(X, a0, f0, v);
     cp_wait<0>();
-    __syncthreads();
+    __syncthreads();                                                     // W1 and Y read, X complete
+    const bool by_species = SPEC && l == 1;
+    if (by_species) stage_w<F>(W1, w2t_of(p, F));
     gemm_blk<F>(X, W0, a0, f0, v);                                       // mbar^{l-1} = gz U1^T
     store_rows<F>(p.mbar_out, base, p.n_atoms, a0, f0, v);
     store_rows_bf16<F>(p.um_mbar_out, 1, base, p.n_atoms, a0, f0, v);
+    if (by_species) {
+        cp_wait<0>();
+        species_adjoint<F>(p, Y, X, W1, base, a0, f0, v);
+    }
 }
 
-template <int F>
+template <int F, bool SPEC>
 void atom_fwd_go(const PotArgs& p, const float* msg, cudaStream_t s) {
     using T = AtomTile<F>;
-    smem_opt_in((const void*)k_atom_fwd<F>, T::SMEM);
-    k_atom_fwd<F><<<(p.n_atoms + T::A - 1) / T::A, T::NT, T::SMEM, s>>>(p, msg);
+    smem_opt_in((const void*)k_atom_fwd<F, SPEC>, T::SMEM);
+    k_atom_fwd<F, SPEC><<<(p.n_atoms + T::A - 1) / T::A, T::NT, T::SMEM, s>>>(p, msg);
 }
 
-template <int F>
+template <int F, bool SPEC>
 void atom_bwd_go(const PotArgs& p, const float* ubar, cudaStream_t s) {
     using T = AtomTile<F>;
-    smem_opt_in((const void*)k_atom_bwd<F>, T::SMEM);
-    k_atom_bwd<F><<<(p.n_atoms + T::A - 1) / T::A, T::NT, T::SMEM, s>>>(p, ubar);
+    smem_opt_in((const void*)k_atom_bwd<F, SPEC>, T::SMEM);
+    k_atom_bwd<F, SPEC><<<(p.n_atoms + T::A - 1) / T::A, T::NT, T::SMEM, s>>>(p, ubar);
 }
 
 }  // namespace
 
 void launch_atom_fwd(const PotArgs& p, int F, const float* msg, cudaStream_t s) {
     if (p.n_atoms == 0) return;
-    if (F == 64) atom_fwd_go<64>(p, msg, s);
-    else atom_fwd_go<32>(p, msg, s);
+    const bool spec = p.spec_row && p.layer == 0;
+    if (F == 64) spec ? atom_fwd_go<64, true>(p, msg, s) : atom_fwd_go<64, false>(p, msg, s);
+    else spec ? atom_fwd_go<32, true>(p, msg, s) : atom_fwd_go<32, false>(p, msg, s);
     count_launch();
 }
 
 void launch_atom_bwd(const PotArgs& p, int F, const float* ubar, cudaStream_t s) {
     if (p.n_atoms == 0) return;
-    if (F == 64) atom_bwd_go<64>(p, ubar, s);
-    else atom_bwd_go<32>(p, ubar, s);
+    const bool spec = p.spec_row && p.layer == 1;
+    if (F == 64) spec ? atom_bwd_go<64, true>(p, ubar, s) : atom_bwd_go<64, false>(p, ubar, s);
+    else spec ? atom_bwd_go<32, true>(p, ubar, s) : atom_bwd_go<32, false>(p, ubar, s);
     count_launch();
 }
 

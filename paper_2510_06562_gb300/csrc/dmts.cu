@@ -182,6 +182,7 @@ struct Model {
     float* mbar[2] = {};
     unsigned char* um[kMaxLayers] = {};   // BF16 u^l | mbar^l rows for the tensor-core backward
     float* msg = nullptr;              // [N][F] per-atom sums between edge and atom kernels
+    float *spec_row = nullptr, *spec_sum = nullptr, *u_spec = nullptr;   // layer 0 by species (PotArgs)
     unsigned char* wt = nullptr;       // BF16 filter-weight operand tiles, per layer
     unsigned char* at = nullptr;       // BF16 hi/lo tiles of the per-atom MLP matrices (tensor-core path)
     size_t wt_layer_bytes = 0;
@@ -409,7 +410,8 @@ void free_model(Model& m) {
     dfree(m.h); dfree(m.gh); dfree(m.force); dfree(m.vir6); dfree(m.h0); dfree(m.PT);
     for (int l = 0; l < kMaxLayers; ++l) { dfree(m.u[l]); dfree(m.z[l]); dfree(m.um[l]); }
     dfree(m.mbar[0]); dfree(m.mbar[1]); dfree(m.esum.part); dfree(m.esum.ctr);
-    dfree(m.Ei); dfree(m.E); dfree(m.W); dfree(m.erep); dfree(m.msg); dfree(m.wt); dfree(m.at);
+    dfree(m.Ei); dfree(m.E); dfree(m.W); dfree(m.erep); dfree(m.msg); dfree(m.spec_row); dfree(m.spec_sum);
+    dfree(m.u_spec); dfree(m.wt); dfree(m.at);
     m = Model();
 }
 
@@ -488,11 +490,11 @@ std::vector<uint16_t> build_atom_tiles(const Model& m, const std::vector<float>&
 }
 
 // Transposed copies of the per-atom MLP matrices: W_in^T, U1^T, U2^T of each
-// layer, then R1^T (each F x F, row-major).
+// layer, then R1^T and layer 0's W2^T (each F x F, row-major).
 std::vector<float> build_transposed(const Model& m, const std::vector<float>& pf) {
     const int F = m.F;
     const size_t FF = (size_t)F * F;
-    std::vector<float> t((3 * (size_t)m.L + 1) * FF);
+    std::vector<float> t((3 * (size_t)m.L + 2) * FF);
     auto put = [&](size_t slot, int off) {
         for (int r = 0; r < F; ++r)
             for (int k = 0; k < F; ++k) t[slot * FF + (size_t)k * F + r] = pf[off + (size_t)r * F + k];
@@ -503,6 +505,7 @@ std::vector<float> build_transposed(const Model& m, const std::vector<float>& pf
         put(3 * l + 2, m.off.U2[l]);
     }
     put(3 * (size_t)m.L, m.off.R1);
+    put(3 * (size_t)m.L + 1, m.off.W2[0]);
     return t;
 }
 
@@ -536,7 +539,7 @@ int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells) {
     CUDA_TRY(dalloc(&m.P, m.n_params));
     m.wt_layer_bytes = bf16_weight_tile_bytes(m.F);
     CUDA_TRY(dalloc(&m.wt, m.wt_layer_bytes * m.L));
-    CUDA_TRY(dalloc(&m.PT, (3 * (size_t)m.L + 1) * m.F * m.F));
+    CUDA_TRY(dalloc(&m.PT, (3 * (size_t)m.L + 2) * m.F * m.F));
     CUDA_TRY(dalloc(&m.at, atom_tile_bytes(m.F, m.L)));
     int rc = upload_params(c, m, d->params);
     if (rc) return rc;
@@ -608,6 +611,11 @@ int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells) {
     CUDA_TRY(dalloc(&m.mbar[0], nf));
     CUDA_TRY(dalloc(&m.mbar[1], nf));
     CUDA_TRY(dalloc(&m.msg, nf));
+    if (m.precision == DMTS_FP32 && m.S <= kMaxFactorSpecies && c->periodic && N >= kMinFactorAtoms) {
+        CUDA_TRY(dalloc(&m.spec_row, nf * m.S));
+        CUDA_TRY(dalloc(&m.spec_sum, (size_t)N * m.S));
+        CUDA_TRY(dalloc(&m.u_spec, (size_t)2 * m.S * m.F));   // u^0 and h^0 of each species
+    }
     CUDA_TRY(dalloc(&m.force, (size_t)3 * N));
     CUDA_TRY(cudaMemset(m.force, 0, sizeof(float) * 3 * std::max(N, 1)));
     CUDA_TRY(dalloc(&m.vir6, (size_t)6 * N));
@@ -696,6 +704,11 @@ PotArgs pot_args(dmts_ctx* c, Model& m) {
     a.carry = m.carry;
     a.carry_w = m.F + 16;
     a.filter = m.filt;
+    a.spec_row = m.spec_row;
+    a.spec_sum = m.spec_sum;
+    a.u_spec = m.u_spec;
+    a.n_species = m.S;
+    a.keep_msg = c->keep_msg ? 1 : 0;
     a.h = m.h;
     a.h_in = m.h;
     a.gh = m.gh;
@@ -714,6 +727,14 @@ int prepare_embedding(dmts_ctx* c, Model& m) {
     a.u_next = m.u[0];
     a.um_u_out = m.um[0];
     launch_embed(a, m.F, c->stream);
+    if (m.u_spec) {                        // the same of each species
+        a.n_atoms = m.S;
+        a.species = nullptr;
+        a.h = m.u_spec + (size_t)m.S * m.F;
+        a.u_next = m.u_spec;
+        a.um_u_out = nullptr;
+        launch_embed(a, m.F, c->stream);
+    }
     CUDA_TRY(cudaGetLastError());
     return DMTS_OK;
 }
@@ -1864,7 +1885,7 @@ int distill_impl(dmts_ctx* c, int n_frames, const double* frames, const double* 
         if (c->batch_params != m0.version) {   // new weights since the last call
             CUDA_TRY(cudaMemcpyAsync(m.P, m0.P, sizeof(float) * m.n_params, cudaMemcpyDeviceToDevice, s));
             CUDA_TRY(cudaMemcpyAsync(m.wt, m0.wt, m.wt_layer_bytes * m.L, cudaMemcpyDeviceToDevice, s));
-            CUDA_TRY(cudaMemcpyAsync(m.PT, m0.PT, sizeof(float) * (3 * m.L + 1) * m.F * m.F, cudaMemcpyDeviceToDevice, s));
+            CUDA_TRY(cudaMemcpyAsync(m.PT, m0.PT, sizeof(float) * (3 * m.L + 2) * m.F * m.F, cudaMemcpyDeviceToDevice, s));
             CUDA_TRY(cudaMemcpyAsync(m.at, m0.at, atom_tile_bytes(m.F, m.L), cudaMemcpyDeviceToDevice, s));
             if ((rc = prepare_embedding(w, m))) return rc;
             c->batch_params = m0.version;
