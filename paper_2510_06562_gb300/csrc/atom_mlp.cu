@@ -12,12 +12,14 @@
 //                            mbar^{l-1} = ((gh U2^{l-1 T}) * SiLU'(z^{l-1})) U1^{l-1 T}
 //
 // Layer 0 reads h^0 = A[Z_i] from the per-atom copy built once per parameter
-// upload. A CTA takes A = 32 atoms; each stage is an [A x F] x [F x F]
-// product, each thread owning RA atoms x RF features (4 x 4 at F = 64; 4 x 2
+// upload. A CTA takes A = 8, 16 or 32 atoms; each stage is an [A x F] x [F x F]
+// product, each thread owning RA = A / 8 atoms x RF features (4 at F = 64; 2
 // at F = 32, so that the narrow model still has 4 warps per CTA). Inputs stay in their
-// natural [atom][k] layout in shared memory; the weight matrix of the next
-// stage (row-major; the transposed ones are copies prepared on the host)
-// streams in with cp.async while the current stage computes.
+// natural [atom][k] layout in shared memory. The weight matrices (row-major;
+// the transposed ones are copies prepared on the host) all stream in at the
+// start, or, at 32 atoms per CTA, where their shared memory costs residency
+// (3.5 % of a 3 fs step of 100,000 atoms), the next stage's while the current
+// one computes.
 #include <cuda_bf16.h>
 
 #include "internal.cuh"
@@ -26,16 +28,17 @@ namespace dmts {
 
 namespace {
 
-template <int F>
+template <int F, int RA_>
 struct AtomTile {
-    static constexpr int A = 32;            // atoms per CTA
-    static constexpr int RA = 4;            // atoms per thread
+    static constexpr int RA = RA_;          // atoms per thread
+    static constexpr int A = 8 * RA;        // atoms per CTA
     static constexpr int RF = F >= 64 ? 4 : 2;  // features per thread
     static constexpr int FG = F / RF;       // feature groups
     static constexpr int NT = (A / RA) * FG; // threads per CTA: 128
     static constexpr int XS = F + 4;        // row stride of per-atom rows [a][k]
     static constexpr int WS = F + 4;        // row stride of staged weights [k][f]
-    static constexpr int SMEM = (2 * A * XS + 2 * F * WS) * 4;
+    static constexpr bool PRE = RA < 4;     // every matrix in its own buffer, loaded at the start
+    static constexpr int smem(int slots) { return (2 * A * XS + (PRE ? slots : 2) * F * WS) * 4; }
     static_assert(FG <= 32 && 32 % FG == 0, "an atom's feature groups are lanes of one warp");
 };
 
@@ -66,22 +69,31 @@ __device__ __forceinline__ void st_vec(float* d, const float (&v)[RF]) {
     else *reinterpret_cast<float2*>(d) = make_float2(v[0], v[1]);
 }
 
-// Start copying the row-major F x F matrix W into Ws [F][WS] (closes a commit group).
-template <int F>
-__device__ __forceinline__ void stage_w(float* Ws, const float* __restrict__ W) {
-    using T = AtomTile<F>;
+// Weight buffers of the forward kernel: one each (PRE), or two in turn by the slot's parity.
+enum WSlot { kU1, kU2, kOut, kR1T, kU2T, kU1T, kSlotsPlain, kW2T = kSlotsPlain, kW2, kSlots };
+
+// Start copying the row-major F x F matrix W into Ws [F][WS]; joins the next commit group.
+template <int F, int RA>
+__device__ __forceinline__ void copy_w(float* Ws, const float* __restrict__ W) {
+    using T = AtomTile<F, RA>;
     for (int t = threadIdx.x; t < F * F / 4; t += T::NT) {
         const int r = t / (F / 4), c = (t % (F / 4)) * 4;
         cp_async16(Ws + r * T::WS + c, W + (size_t)r * F + c);
     }
+}
+
+// The same as a commit group of its own.
+template <int F, int RA>
+__device__ __forceinline__ void stage_w(float* Ws, const float* __restrict__ W) {
+    copy_w<F, RA>(Ws, W);
     cp_commit();
 }
 
 // Start copying rows base .. base + A - 1 of the [N][F] array src into X [A][XS]
 // (rows past N are zero); joins the next commit group.
-template <int F>
+template <int F, int RA>
 __device__ __forceinline__ void stage_rows(float* X, const float* __restrict__ src, int base, int n_atoms) {
-    using T = AtomTile<F>;
+    using T = AtomTile<F, RA>;
     for (int t = threadIdx.x; t < T::A * F / 4; t += T::NT) {
         const int a = t / (F / 4), c = (t % (F / 4)) * 4;
         if (base + a < n_atoms) cp_async16(X + a * T::XS + c, src + (size_t)(base + a) * F + c);
@@ -90,10 +102,10 @@ __device__ __forceinline__ void stage_rows(float* X, const float* __restrict__ s
 }
 
 // acc[a][f] = sum_k X[a0 + a][k] * Ws[k][f0 + f], k ascending.
-template <int F>
+template <int F, int RA>
 __device__ __forceinline__ void gemm_blk(const float* X, const float* Ws, int a0, int f0,
-                                         float (&acc)[AtomTile<F>::RA][AtomTile<F>::RF]) {
-    using T = AtomTile<F>;
+                                         float (&acc)[AtomTile<F, RA>::RA][AtomTile<F, RA>::RF]) {
+    using T = AtomTile<F, RA>;
 #pragma unroll
     for (int a = 0; a < T::RA; ++a)
 #pragma unroll
@@ -116,10 +128,10 @@ __device__ __forceinline__ void gemm_blk(const float* X, const float* Ws, int a0
 }
 
 // The same for species s of the [N][n_species][F] sums.
-template <int F>
+template <int F, int RA>
 __device__ __forceinline__ void stage_species(float* X, const float* __restrict__ src, int s, int n_species, int base,
                                               int n_atoms) {
-    using T = AtomTile<F>;
+    using T = AtomTile<F, RA>;
     for (int t = threadIdx.x; t < T::A * F / 4; t += T::NT) {
         const int a = t / (F / 4), c = (t % (F / 4)) * 4;
         if (base + a < n_atoms) cp_async16(X + a * T::XS + c, src + ((size_t)(base + a) * n_species + s) * F + c);
@@ -127,18 +139,18 @@ __device__ __forceinline__ void stage_species(float* X, const float* __restrict_
     }
 }
 
-template <int F>
+template <int F, int RA>
 __device__ __forceinline__ void put_rows(float* X, int a0, int f0,
-                                         const float (&v)[AtomTile<F>::RA][AtomTile<F>::RF]) {
-    using T = AtomTile<F>;
+                                         const float (&v)[AtomTile<F, RA>::RA][AtomTile<F, RA>::RF]) {
+    using T = AtomTile<F, RA>;
 #pragma unroll
     for (int a = 0; a < T::RA; ++a) st_vec<T::RF>(X + (a0 + a) * T::XS + f0, v[a]);
 }
 
-template <int F>
+template <int F, int RA>
 __device__ __forceinline__ void store_rows(float* __restrict__ dst, int base, int n_atoms, int a0, int f0,
-                                           const float (&v)[AtomTile<F>::RA][AtomTile<F>::RF]) {
-    using T = AtomTile<F>;
+                                           const float (&v)[AtomTile<F, RA>::RA][AtomTile<F, RA>::RF]) {
+    using T = AtomTile<F, RA>;
 #pragma unroll
     for (int a = 0; a < T::RA; ++a) {
         const int i = base + a0 + a;
@@ -148,10 +160,10 @@ __device__ __forceinline__ void store_rows(float* __restrict__ dst, int base, in
 
 // BF16 copy of the same block into interleaved rows (F * 4 bytes per atom;
 // per 16 features 16 u values then 16 mbar values, half 0 or 1).
-template <int F>
+template <int F, int RA>
 __device__ __forceinline__ void store_rows_bf16(unsigned char* __restrict__ dst, int half, int base, int n_atoms,
-                                                int a0, int f0, const float (&v)[AtomTile<F>::RA][AtomTile<F>::RF]) {
-    using T = AtomTile<F>;
+                                                int a0, int f0, const float (&v)[AtomTile<F, RA>::RA][AtomTile<F, RA>::RF]) {
+    using T = AtomTile<F, RA>;
     if (!dst) return;
 #pragma unroll
     for (int a = 0; a < T::RA; ++a) {
@@ -171,10 +183,10 @@ __device__ __forceinline__ void store_rows_bf16(unsigned char* __restrict__ dst,
     }
 }
 
-template <int F>
-__device__ __forceinline__ void load_rows(float (&v)[AtomTile<F>::RA][AtomTile<F>::RF], const float* __restrict__ src,
+template <int F, int RA>
+__device__ __forceinline__ void load_rows(float (&v)[AtomTile<F, RA>::RA][AtomTile<F, RA>::RF], const float* __restrict__ src,
                                           int base, int n_atoms, int a0, int f0) {
-    using T = AtomTile<F>;
+    using T = AtomTile<F, RA>;
 #pragma unroll
     for (int a = 0; a < T::RA; ++a) {
         const int i = base + a0 + a;
@@ -203,10 +215,10 @@ __device__ __forceinline__ const float* w2t_of(const PotArgs& p, int F) {
 // Y_is = W2 (mbar_i * u_s) and scalars B_is = b2 . (mbar_i * u_s) of every
 // species s, over the forward pass's sums. W holds W2^T; A0 and A1 are row
 // buffers, A0 free on entry, A1 read by the preceding product.
-template <int F>
+template <int F, int RA>
 __device__ __forceinline__ void species_adjoint(const PotArgs& p, float* A0, float* A1, const float* W, int base, int a0,
-                                                int f0, const float (&v)[AtomTile<F>::RA][AtomTile<F>::RF]) {
-    using T = AtomTile<F>;
+                                                int f0, const float (&v)[AtomTile<F, RA>::RA][AtomTile<F, RA>::RF]) {
+    using T = AtomTile<F, RA>;
     float b2[T::RF];
 #pragma unroll
     for (int f = 0; f < T::RF; ++f) b2[f] = __ldg(p.P + p.off.b2[0] + f0 + f);
@@ -223,13 +235,13 @@ __device__ __forceinline__ void species_adjoint(const PotArgs& p, float* A0, flo
                 part[a] += x[a][f] * b2[f];
             }
         }
-        put_rows<F>(A0, a0, f0, x);
+        put_rows<F, RA>(A0, a0, f0, x);
 #pragma unroll
         for (int a = 0; a < T::RA; ++a)
 #pragma unroll
             for (int o = T::FG / 2; o > 0; o >>= 1) part[a] += __shfl_xor_sync(0xffffffffu, part[a], o);
         __syncthreads();
-        gemm_blk<F>(A0, W, a0, f0, y);
+        gemm_blk<F, RA>(A0, W, a0, f0, y);
 #pragma unroll
         for (int a = 0; a < T::RA; ++a) {
             const int i = base + a0 + a;
@@ -242,14 +254,14 @@ __device__ __forceinline__ void species_adjoint(const PotArgs& p, float* A0, flo
     }
 }
 
-template <int F, bool SPEC>
-__global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_fwd(PotArgs p, const float* __restrict__ msg) {
-    using T = AtomTile<F>;
+template <int F, int RA, bool SPEC>
+__global__ void __launch_bounds__(AtomTile<F, RA>::NT) k_atom_fwd(PotArgs p, const float* __restrict__ msg) {
+    using T = AtomTile<F, RA>;
     extern __shared__ float4 smem4[];
     float* X = reinterpret_cast<float*>(smem4);      // [A][XS]
     float* Y = X + T::A * T::XS;                     // [A][XS]
-    float* W0 = Y + T::A * T::XS;                    // [F][WS]
-    float* W1 = W0 + F * T::WS;                      // [F][WS]
+    float* Wb = Y + T::A * T::XS;                    // weight buffers [F][WS]
+    auto W = [&](int slot) { return Wb + (T::PRE ? slot : slot & 1) * F * T::WS; };
     __shared__ float sE[T::A];
     __shared__ float sBias[4][F];                    // c1, c2 of this layer; d1, R2 (last layer)
     const int l = p.layer;
@@ -262,14 +274,28 @@ __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_fwd(PotArgs p, const f
 
     const bool by_species = SPEC && l == 0;          // the messages are formed here (below)
     if (by_species) {
-        stage_species<F>(X, p.spec_row, 0, p.n_species, base, p.n_atoms);
-        stage_w<F>(W1, P + p.off.W2[0]);                                 // group: first species' sums + W2
+        stage_species<F, RA>(X, p.spec_row, 0, p.n_species, base, p.n_atoms);
+        stage_w<F, RA>(W(kW2), P + p.off.W2[0]);                         // group: first species' sums + W2
     } else {
-        stage_rows<F>(X, msg, base, p.n_atoms);
+        stage_rows<F, RA>(X, msg, base, p.n_atoms);
+        stage_w<F, RA>(W(kU1), P + p.off.U1[l]);                         // group: message rows + U1
     }
-    stage_w<F>(W0, P + p.off.U1[l]);                                     // group: message rows + U1
-    if (!by_species) stage_w<F>(W1, P + p.off.U2[l]);                    // group: U2
-    load_rows<F>(h, p.h_in, base, p.n_atoms, a0, f0);
+    if constexpr (T::PRE) {                                              // group: all other matrices
+        if (by_species) copy_w<F, RA>(W(kU1), P + p.off.U1[l]);
+        copy_w<F, RA>(W(kU2), P + p.off.U2[l]);
+        copy_w<F, RA>(W(kOut), last ? P + p.off.R1 : P + p.off.W_in[l + 1]);
+        if (last) {
+            copy_w<F, RA>(W(kR1T), r1t_of(p, F));
+            copy_w<F, RA>(W(kU2T), wt_of(p, F, l, 2));
+            copy_w<F, RA>(W(kU1T), wt_of(p, F, l, 1));
+            if (by_species) copy_w<F, RA>(W(kW2T), w2t_of(p, F));
+        }
+        cp_commit();
+    } else {
+        if (by_species) stage_w<F, RA>(W(kU1), P + p.off.U1[l]);         // group: U1
+        else stage_w<F, RA>(W(kU2), P + p.off.U2[l]);                    // group: U2
+    }
+    load_rows<F, RA>(h, p.h_in, base, p.n_atoms, a0, f0);
     // the small per-layer vectors and the per-atom energy constants, loaded while the copies run
     for (int t = tid; t < F; t += T::NT) {
         sBias[0][t] = __ldg(P + p.off.c1[l] + t);
@@ -319,7 +345,7 @@ __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_fwd(PotArgs p, const f
         float *cur = X, *nxt = Y;
         for (int s = 0; s < p.n_species; ++s) {
             if (s + 1 < p.n_species) {
-                stage_species<F>(nxt, p.spec_row, s + 1, p.n_species, base, p.n_atoms);
+                stage_species<F, RA>(nxt, p.spec_row, s + 1, p.n_species, base, p.n_atoms);
                 cp_commit();
                 if (s == 0) cp_wait<2>();                                // (U1 is in flight too)
                 else cp_wait<1>();
@@ -327,7 +353,7 @@ __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_fwd(PotArgs p, const f
                 cp_wait<0>();
             }
             __syncthreads();
-            gemm_blk<F>(cur, W1, a0, f0, v);
+            gemm_blk<F, RA>(cur, W(kW2), a0, f0, v);
             float t[T::RA];
 #pragma unroll
             for (int a = 0; a < T::RA; ++a)
@@ -341,9 +367,9 @@ __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_fwd(PotArgs p, const f
             __syncthreads();                                             // cur (and, at the end, W2) read
             float* sw = cur; cur = nxt; nxt = sw;
         }
-        stage_w<F>(W1, P + p.off.U2[l]);                                 // group: U2
-        put_rows<F>(X, a0, f0, m);
-        if (p.keep_msg) store_rows<F>(p.msg_out, base, p.n_atoms, a0, f0, m);
+        if (!T::PRE) stage_w<F, RA>(W(kU2), P + p.off.U2[l]);            // group: U2
+        put_rows<F, RA>(X, a0, f0, m);
+        if (p.keep_msg) store_rows<F, RA>(p.msg_out, base, p.n_atoms, a0, f0, m);
     }
     cp_wait<1>();
     __syncthreads();
@@ -371,7 +397,7 @@ __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_fwd(PotArgs p, const f
         }
         __syncthreads();
     }
-    gemm_blk<F>(X, W0, a0, f0, z);                                       // z = m U1 + c1
+    gemm_blk<F, RA>(X, W(kU1), a0, f0, z);                               // z = m U1 + c1
 #pragma unroll
     for (int f = 0; f < T::RF; ++f) {
         const float c1 = sBias[0][f0 + f];
@@ -383,34 +409,36 @@ __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_fwd(PotArgs p, const f
     }
     // a one-layer model read only for its force needs z, h, dE/dh and E_i of no later kernel
     const bool keep = !(p.lean && p.n_layers == 1);
-    if (keep) store_rows<F>(p.z, base, p.n_atoms, a0, f0, z);
-    put_rows<F>(Y, a0, f0, v);
-    __syncthreads();                                                     // W0 read, Y complete
-    stage_w<F>(W0, last ? P + p.off.R1 : P + p.off.W_in[l + 1]);
-    cp_wait<1>();
+    if (keep) store_rows<F, RA>(p.z, base, p.n_atoms, a0, f0, z);
+    put_rows<F, RA>(Y, a0, f0, v);
+    __syncthreads();                                                     // U1 read, Y complete
+    if (!T::PRE) stage_w<F, RA>(W(kOut), last ? P + p.off.R1 : P + p.off.W_in[l + 1]);
+    cp_wait<T::PRE ? 0 : 1>();
     __syncthreads();
-    gemm_blk<F>(Y, W1, a0, f0, v);                                       // h += SiLU(z) U2 + c2
+    gemm_blk<F, RA>(Y, W(kU2), a0, f0, v);                               // h += SiLU(z) U2 + c2
 #pragma unroll
     for (int f = 0; f < T::RF; ++f) {
         const float c2 = sBias[1][f0 + f];
 #pragma unroll
         for (int a = 0; a < T::RA; ++a) h[a][f] += v[a][f] + c2;
     }
-    if (keep) store_rows<F>(p.h, base, p.n_atoms, a0, f0, h);
-    put_rows<F>(X, a0, f0, h);
-    __syncthreads();                                                     // W1 read, X complete
+    if (keep) store_rows<F, RA>(p.h, base, p.n_atoms, a0, f0, h);
+    put_rows<F, RA>(X, a0, f0, h);
+    __syncthreads();                                                     // U2 read, X complete
     if (!last) {
         cp_wait<0>();
         __syncthreads();
-        gemm_blk<F>(X, W0, a0, f0, v);                                   // u^{l+1} = h W_in^{l+1}
-        store_rows<F>(p.u_next, base, p.n_atoms, a0, f0, v);
-        store_rows_bf16<F>(p.um_u_out, 0, base, p.n_atoms, a0, f0, v);
+        gemm_blk<F, RA>(X, W(kOut), a0, f0, v);                          // u^{l+1} = h W_in^{l+1}
+        store_rows<F, RA>(p.u_next, base, p.n_atoms, a0, f0, v);
+        store_rows_bf16<F, RA>(p.um_u_out, 0, base, p.n_atoms, a0, f0, v);
         return;
     }
-    stage_w<F>(W1, r1t_of(p, F));
-    cp_wait<1>();
-    __syncthreads();
-    gemm_blk<F>(X, W0, a0, f0, v);                                       // q = h R1 + d1
+    if constexpr (!T::PRE) {
+        stage_w<F, RA>(W(kR1T), r1t_of(p, F));
+        cp_wait<1>();
+        __syncthreads();
+    }
+    gemm_blk<F, RA>(X, W(kOut), a0, f0, v);                              // q = h R1 + d1
     float e_part[T::RA];
 #pragma unroll
     for (int a = 0; a < T::RA; ++a) e_part[a] = 0.f;
@@ -433,21 +461,25 @@ __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_fwd(PotArgs p, const f
     if (fg == 0)
 #pragma unroll
         for (int a = 0; a < T::RA; ++a) sE[a0 + a] = e_part[a];
-    put_rows<F>(Y, a0, f0, v);
-    __syncthreads();                                                     // W0 read, Y and sE complete
-    stage_w<F>(W0, wt_of(p, F, l, 2));                                   // U2^T
+    put_rows<F, RA>(Y, a0, f0, v);
+    __syncthreads();                                                     // R1 read, Y and sE complete
+    if (!T::PRE) stage_w<F, RA>(W(kU2T), wt_of(p, F, l, 2));
     static_assert(T::NT >= T::A, "one thread per atom of the tile");
     if (keep && tid < T::A && base + tid < p.n_atoms) p.Ei[base + tid] = (double)sE[tid] + e_const;
-    cp_wait<1>();
-    __syncthreads();
-    gemm_blk<F>(Y, W1, a0, f0, v);                                       // gh = gq R1^T
-    if (keep) store_rows<F>(p.gh, base, p.n_atoms, a0, f0, v);
-    put_rows<F>(X, a0, f0, v);
-    __syncthreads();                                                     // W1 read, X complete
-    stage_w<F>(W1, wt_of(p, F, l, 1));                                   // U1^T
-    cp_wait<1>();
-    __syncthreads();
-    gemm_blk<F>(X, W0, a0, f0, v);                                       // gy = gh U2^T
+    if constexpr (!T::PRE) {
+        cp_wait<1>();
+        __syncthreads();
+    }
+    gemm_blk<F, RA>(Y, W(kR1T), a0, f0, v);                              // gh = gq R1^T
+    if (keep) store_rows<F, RA>(p.gh, base, p.n_atoms, a0, f0, v);
+    put_rows<F, RA>(X, a0, f0, v);
+    __syncthreads();                                                     // R1^T read, X complete
+    if constexpr (!T::PRE) {
+        stage_w<F, RA>(W(kU1T), wt_of(p, F, l, 1));
+        cp_wait<1>();
+        __syncthreads();
+    }
+    gemm_blk<F, RA>(X, W(kU2T), a0, f0, v);                              // gy = gh U2^T
 #pragma unroll
     for (int a = 0; a < T::RA; ++a)
 #pragma unroll
@@ -455,51 +487,61 @@ __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_fwd(PotArgs p, const f
             const float s = sig(z[a][f]);
             v[a][f] *= s * (1.f + z[a][f] * (1.f - s));
         }
-    put_rows<F>(Y, a0, f0, v);
+    put_rows<F, RA>(Y, a0, f0, v);
     cp_wait<0>();
-    __syncthreads();                                                     // W0 and X read, Y complete
-    if (by_species) stage_w<F>(W0, w2t_of(p, F));
-    gemm_blk<F>(Y, W1, a0, f0, v);                                       // mbar = gz U1^T
-    store_rows<F>(p.mbar_out, base, p.n_atoms, a0, f0, v);
-    store_rows_bf16<F>(p.um_mbar_out, 1, base, p.n_atoms, a0, f0, v);
+    __syncthreads();                                                     // U2^T and X read, Y complete
+    if (by_species && !T::PRE) stage_w<F, RA>(W(kW2T), w2t_of(p, F));
+    gemm_blk<F, RA>(Y, W(kU1T), a0, f0, v);                              // mbar = gz U1^T
+    store_rows<F, RA>(p.mbar_out, base, p.n_atoms, a0, f0, v);
+    store_rows_bf16<F, RA>(p.um_mbar_out, 1, base, p.n_atoms, a0, f0, v);
     if (by_species) {
         cp_wait<0>();                                                    // (visible after the first barrier inside)
-        species_adjoint<F>(p, X, Y, W0, base, a0, f0, v);
+        species_adjoint<F, RA>(p, X, Y, W(kW2T), base, a0, f0, v);
     }
 }
 
-template <int F, bool SPEC>
-__global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_bwd(PotArgs p, const float* __restrict__ ubar) {
-    using T = AtomTile<F>;
+template <int F, int RA, bool SPEC>
+__global__ void __launch_bounds__(AtomTile<F, RA>::NT) k_atom_bwd(PotArgs p, const float* __restrict__ ubar) {
+    using T = AtomTile<F, RA>;
     extern __shared__ float4 smem4[];
     float* X = reinterpret_cast<float*>(smem4);
     float* Y = X + T::A * T::XS;
-    float* W0 = Y + T::A * T::XS;
-    float* W1 = W0 + F * T::WS;
+    float* Wb = Y + T::A * T::XS;
+    auto W = [&](int slot) { return Wb + (T::PRE ? slot : slot & 1) * F * T::WS; };
     const int l = p.layer;   // >= 1
     const int base = blockIdx.x * T::A;
     const int tid = threadIdx.x, fg = tid % T::FG, ag = tid / T::FG;
     const int f0 = T::RF * fg, a0 = T::RA * ag;
     float v[T::RA][T::RF], g[T::RA][T::RF], z[T::RA][T::RF];
-    stage_rows<F>(X, ubar, base, p.n_atoms);
-    stage_w<F>(W0, wt_of(p, F, l, 0));                                   // group: ubar rows + W_in^{l T}
-    stage_w<F>(W1, wt_of(p, F, l - 1, 2));                               // group: U2^{l-1 T}
-    load_rows<F>(g, p.gh, base, p.n_atoms, a0, f0);
-    load_rows<F>(z, p.z_prev, base, p.n_atoms, a0, f0);
+    stage_rows<F, RA>(X, ubar, base, p.n_atoms);
+    const bool by_species = SPEC && l == 1;
+    stage_w<F, RA>(W(0), wt_of(p, F, l, 0));                             // group: ubar rows + W_in^{l T}
+    copy_w<F, RA>(W(1), wt_of(p, F, l - 1, 2));                          // group: U2^{l-1 T} (all other matrices)
+    if constexpr (T::PRE) {
+        copy_w<F, RA>(W(2), wt_of(p, F, l - 1, 1));
+        if (by_species) copy_w<F, RA>(W(3), w2t_of(p, F));
+    }
+    cp_commit();
+    load_rows<F, RA>(g, p.gh, base, p.n_atoms, a0, f0);
+    load_rows<F, RA>(z, p.z_prev, base, p.n_atoms, a0, f0);
     cp_wait<1>();
     __syncthreads();
-    gemm_blk<F>(X, W0, a0, f0, v);                                       // ubar W_in^T
+    gemm_blk<F, RA>(X, W(0), a0, f0, v);                                 // ubar W_in^T
 #pragma unroll
     for (int a = 0; a < T::RA; ++a)
 #pragma unroll
         for (int f = 0; f < T::RF; ++f) g[a][f] += v[a][f];
-    store_rows<F>(p.gh, base, p.n_atoms, a0, f0, g);
-    put_rows<F>(Y, a0, f0, g);
-    __syncthreads();                                                     // W0 read, Y complete
-    stage_w<F>(W0, wt_of(p, F, l - 1, 1));                               // U1^{l-1 T}
-    cp_wait<1>();
-    __syncthreads();
-    gemm_blk<F>(Y, W1, a0, f0, v);                                       // gy = gh U2^T
+    store_rows<F, RA>(p.gh, base, p.n_atoms, a0, f0, g);
+    put_rows<F, RA>(Y, a0, f0, g);
+    if constexpr (!T::PRE) {
+        __syncthreads();                                                 // W_in^T read
+        stage_w<F, RA>(W(2), wt_of(p, F, l - 1, 1));                     // U1^{l-1 T}
+        cp_wait<1>();
+    } else {
+        cp_wait<0>();
+    }
+    __syncthreads();                                                     // Y complete
+    gemm_blk<F, RA>(Y, W(1), a0, f0, v);                                       // gy = gh U2^T
 #pragma unroll
     for (int a = 0; a < T::RA; ++a)
 #pragma unroll
@@ -507,50 +549,67 @@ __global__ void __launch_bounds__(AtomTile<F>::NT) k_atom_bwd(PotArgs p, const f
             const float s = sig(z[a][f]);
             v[a][f] *= s * (1.f + z[a][f] * (1.f - s));
         }
-    put_rows<F>(X, a0, f0, v);
+    put_rows<F, RA>(X, a0, f0, v);
     cp_wait<0>();
-    __syncthreads();                                                     // W1 and Y read, X complete
-    const bool by_species = SPEC && l == 1;
-    if (by_species) stage_w<F>(W1, w2t_of(p, F));
-    gemm_blk<F>(X, W0, a0, f0, v);                                       // mbar^{l-1} = gz U1^T
-    store_rows<F>(p.mbar_out, base, p.n_atoms, a0, f0, v);
-    store_rows_bf16<F>(p.um_mbar_out, 1, base, p.n_atoms, a0, f0, v);
+    __syncthreads();                                                     // U2^T and Y read, X complete
+    if (by_species && !T::PRE) stage_w<F, RA>(W(3), w2t_of(p, F));
+    gemm_blk<F, RA>(X, W(2), a0, f0, v);                                 // mbar^{l-1} = gz U1^T
+    store_rows<F, RA>(p.mbar_out, base, p.n_atoms, a0, f0, v);
+    store_rows_bf16<F, RA>(p.um_mbar_out, 1, base, p.n_atoms, a0, f0, v);
     if (by_species) {
         cp_wait<0>();
-        species_adjoint<F>(p, Y, X, W1, base, a0, f0, v);
+        species_adjoint<F, RA>(p, Y, X, W(3), base, a0, f0, v);
     }
 }
 
-template <int F, bool SPEC>
+template <int F, int RA, bool SPEC>
 void atom_fwd_go(const PotArgs& p, const float* msg, cudaStream_t s) {
-    using T = AtomTile<F>;
-    smem_opt_in((const void*)k_atom_fwd<F, SPEC>, T::SMEM);
-    k_atom_fwd<F, SPEC><<<(p.n_atoms + T::A - 1) / T::A, T::NT, T::SMEM, s>>>(p, msg);
+    using T = AtomTile<F, RA>;
+    constexpr int bytes = T::smem(SPEC ? kSlots : kSlotsPlain);
+    smem_opt_in((const void*)k_atom_fwd<F, RA, SPEC>, bytes);
+    k_atom_fwd<F, RA, SPEC><<<(p.n_atoms + T::A - 1) / T::A, T::NT, bytes, s>>>(p, msg);
 }
 
-template <int F, bool SPEC>
+template <int F, int RA, bool SPEC>
 void atom_bwd_go(const PotArgs& p, const float* ubar, cudaStream_t s) {
-    using T = AtomTile<F>;
-    smem_opt_in((const void*)k_atom_bwd<F, SPEC>, T::SMEM);
-    k_atom_bwd<F, SPEC><<<(p.n_atoms + T::A - 1) / T::A, T::NT, T::SMEM, s>>>(p, ubar);
+    using T = AtomTile<F, RA>;
+    constexpr int bytes = T::smem(SPEC ? 4 : 3);
+    smem_opt_in((const void*)k_atom_bwd<F, RA, SPEC>, bytes);
+    k_atom_bwd<F, RA, SPEC><<<(p.n_atoms + T::A - 1) / T::A, T::NT, bytes, s>>>(p, ubar);
+}
+
+template <int F, int RA>
+void atom_go(const PotArgs& p, const float* x, bool fwd, cudaStream_t s) {
+    const bool spec = p.spec_row && p.layer == (fwd ? 0 : 1);
+    if (fwd) spec ? atom_fwd_go<F, RA, true>(p, x, s) : atom_fwd_go<F, RA, false>(p, x, s);
+    else spec ? atom_bwd_go<F, RA, true>(p, x, s) : atom_bwd_go<F, RA, false>(p, x, s);
+}
+
+// Atoms per thread: as few as leave one block per SM. The products are then a
+// chain of latencies, and a block of 8 atoms walks it in a third of the time
+// of one of 32. 3 fs step in BF16, blocks of 32 atoms (large model on tensor
+// cores) against these: 192 atoms 210 -> 181 us, 1,536 256 -> 233, 2,187
+// 265 -> 246; FP32 forces of 192 atoms 221 -> 206 us.
+template <int F>
+void atom_any(const PotArgs& p, const float* x, bool fwd, cudaStream_t s) {
+    if (p.n_atoms <= 8 * kSmCount) atom_go<F, 1>(p, x, fwd, s);
+    else if (p.n_atoms <= 16 * kSmCount) atom_go<F, 2>(p, x, fwd, s);
+    else atom_go<F, 4>(p, x, fwd, s);
+    count_launch();
 }
 
 }  // namespace
 
 void launch_atom_fwd(const PotArgs& p, int F, const float* msg, cudaStream_t s) {
     if (p.n_atoms == 0) return;
-    const bool spec = p.spec_row && p.layer == 0;
-    if (F == 64) spec ? atom_fwd_go<64, true>(p, msg, s) : atom_fwd_go<64, false>(p, msg, s);
-    else spec ? atom_fwd_go<32, true>(p, msg, s) : atom_fwd_go<32, false>(p, msg, s);
-    count_launch();
+    if (F == 64) atom_any<64>(p, msg, true, s);
+    else atom_any<32>(p, msg, true, s);
 }
 
 void launch_atom_bwd(const PotArgs& p, int F, const float* ubar, cudaStream_t s) {
     if (p.n_atoms == 0) return;
-    const bool spec = p.spec_row && p.layer == 1;
-    if (F == 64) spec ? atom_bwd_go<64, true>(p, ubar, s) : atom_bwd_go<64, false>(p, ubar, s);
-    else spec ? atom_bwd_go<32, true>(p, ubar, s) : atom_bwd_go<32, false>(p, ubar, s);
-    count_launch();
+    if (F == 64) atom_any<64>(p, ubar, false, s);
+    else atom_any<32>(p, ubar, false, s);
 }
 
 }  // namespace dmts
