@@ -162,10 +162,10 @@ struct Model {
     ModelOffsets off{};
     float* P = nullptr;
     int nc = 0, n_cells = 0;
-    int *cell_count = nullptr, *cell_start = nullptr, *cell_atoms = nullptr, *atom_cell = nullptr,
-        *atom_slot = nullptr, *atom_pos = nullptr;
+    int *cell_count = nullptr, *cell_start = nullptr, *atom_cell = nullptr,
+        *atom_slot = nullptr;
     uint4* cell_q = nullptr;
-    int ccap = 0;                      // skin 0: slots per cell ([n_cells][ccap] cell_atoms / cell_q)
+    int ccap = 0;                      // skin 0: slots per cell ([n_cells][ccap] cell_q)
     bool placed = false;               // while capturing: the integrator kernel fills the cells
     int row_cap = 0;
     long long e_cap = 0;
@@ -402,8 +402,8 @@ cudaError_t alloc_model_nbr(dmts_ctx* c, Model& m) {
 
 void free_model(Model& m) {
     dfree(m.P);
-    dfree(m.cell_count); dfree(m.cell_start); dfree(m.cell_atoms); dfree(m.atom_cell); dfree(m.atom_slot);
-    dfree(m.atom_pos); dfree(m.cell_q);
+    dfree(m.cell_count); dfree(m.cell_start); dfree(m.atom_cell); dfree(m.atom_slot);
+    dfree(m.cell_q);
     free_model_nbr(m);
     dfree(m.nbr_cnt); dfree(m.row_ptr); dfree(m.vl_cnt);
     dfree(m.block_sum); dfree(m.chunk_sum); dfree(m.ticket);
@@ -574,16 +574,13 @@ int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells) {
         m.n_cells = c->n_sys * m.nc * m.nc * m.nc;            // each system its own cells
         CUDA_TRY(dalloc(&m.cell_count, m.n_cells));
         CUDA_TRY(cudaMemset(m.cell_count, 0, sizeof(int) * m.n_cells));
-        CUDA_TRY(dalloc(&m.atom_pos, N));
         if (c->skin > 0) {                 // compact cells rebuilt by count, scan and fill
             CUDA_TRY(dalloc(&m.cell_start, m.n_cells + 1));
             CUDA_TRY(dalloc(&m.atom_cell, N));
             CUDA_TRY(dalloc(&m.atom_slot, N));
-            CUDA_TRY(dalloc(&m.cell_atoms, N));
             CUDA_TRY(dalloc(&m.cell_q, N));
         } else {                           // fixed-capacity cells: twice the mean occupancy plus 16, grown on overflow
             m.ccap = ((int)(2.0 * N / m.n_cells) + 16 + 7) / 8 * 8;
-            CUDA_TRY(dalloc(&m.cell_atoms, (size_t)m.n_cells * m.ccap));
             CUDA_TRY(dalloc(&m.cell_q, (size_t)m.n_cells * m.ccap));
         }
     }
@@ -646,9 +643,7 @@ NbrArgs nbr_args(dmts_ctx* c, Model& m, int which) {
     a.rc2_hi = (float)(rc2 * (1.0 + 1e-5));
     a.nc = m.nc;
     a.cell_start = m.cell_start;
-    a.cell_atoms = m.cell_atoms;
     a.cell_q = m.cell_q;
-    a.atom_pos = m.atom_pos;
     a.row_cap = m.row_cap;
     a.e_cap = m.e_cap;
     a.nbr_tmp = m.nbr_tmp;
@@ -789,8 +784,8 @@ void enqueue_rebuild(dmts_ctx* c, cudaStream_t s) {
     Model& src = c->m[w0];
     NbrArgs b = candidate_args(c, w0);
     if (src.nc > 0)
-        launch_cells_gated(c->N, c->d_q, src.nc, src.cell_count, src.cell_start, src.cell_atoms, src.atom_cell,
-                           src.atom_slot, src.cell_q, src.atom_pos, b.gate, s);
+        launch_cells_gated(c->N, c->d_q, src.nc, src.cell_count, src.cell_start, src.atom_cell,
+                           src.atom_slot, src.cell_q, b.gate, s);
     b.xref = c->d_xref;
     launch_vl_build(b, s);
     if (c->m[1 - w0].present) {
@@ -808,7 +803,7 @@ CellPlace cell_place(dmts_ctx* c, int w) {
     const Model& m = c->m[w];
     CellPlace p{};
     if (c->periodic && c->skin <= 0 && m.present && m.nc > 0 && m.ccap > 0)
-        p = CellPlace{m.nc, m.ccap, m.cell_count, m.cell_atoms, m.cell_q, m.atom_pos, kFlagMaxCell0 + w};
+        p = CellPlace{m.nc, m.ccap, m.cell_count, m.cell_q, kFlagMaxCell0 + w};
     return p;
 }
 
@@ -1001,12 +996,9 @@ int grow_capacity(dmts_ctx* c) {
         if (m.ccap > 0 && max_cell > m.ccap) {
             m.ccap = ((int)(max_cell * 1.25) + 8 + 7) / 8 * 8;
             CUDA_TRY(cudaStreamSynchronize(c->stream));
-            dfree(m.cell_atoms);
             dfree(m.cell_q);
-            m.cell_atoms = nullptr;
             m.cell_q = nullptr;
-            cudaError_t e = dalloc(&m.cell_atoms, (size_t)m.n_cells * m.ccap);
-            if (e == cudaSuccess) e = dalloc(&m.cell_q, (size_t)m.n_cells * m.ccap);
+            cudaError_t e = dalloc(&m.cell_q, (size_t)m.n_cells * m.ccap);
             if (e != cudaSuccess) return fail(DMTS_ERR_OOM, "growing cell capacity: %s", cudaGetErrorString(e));
         }
         if (grow) {
@@ -1520,11 +1512,8 @@ int dmts_create(const dmts_model_desc* small, const dmts_model_desc* big, const 
             // smaller initial cell capacity (exercises the overflow-and-retry path)
             Model& m = c->m[w];
             m.ccap = std::min(m.ccap, (int)opt_cell_cap);
-            dfree(m.cell_atoms);
             dfree(m.cell_q);
-            m.cell_atoms = nullptr;
             m.cell_q = nullptr;
-            CREATE_TRY(dalloc(&m.cell_atoms, (size_t)m.n_cells * m.ccap));
             CREATE_TRY(dalloc(&m.cell_q, (size_t)m.n_cells * m.ccap));
         }
         c->m[w].apc_fwd = std::max(8, c->m[w].apc_fwd);

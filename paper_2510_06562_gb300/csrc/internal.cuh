@@ -196,9 +196,7 @@ struct NbrArgs {
     float rc2_lo, rc2_hi;    // FP32 band around rc^2
     int nc;                  // cells per dimension (0: all pairs within system)
     const int* cell_start;   // [nc^3 + 1]
-    const int* cell_atoms;   // [N] atoms in cell order
-    const uint4* cell_q;     // [N] their fixed-point positions {qx, qy, qz, atom index}, in cell order
-    const int* atom_pos;     // [N] each atom's place in cell order
+    const uint4* cell_q;     // [N] fixed-point positions {qx, qy, qz, atom index}, in cell order
     int row_cap;
     long long e_cap;
     int* nbr_tmp;            // [N][row_cap]
@@ -217,7 +215,7 @@ struct NbrArgs {
     const int* src_cnt;      // [N]
     int src_cap;
     // fresh lists (skin 0): cells of fixed capacity ccap > 0, slots
-    // [n_cells][ccap] of cell_atoms / cell_q filled by atomic counters
+    // [n_cells][ccap] of cell_q filled by atomic counters
     // cell_count (zero between builds: the compaction clears them)
     int ccap;
     int n_cells;
@@ -237,9 +235,7 @@ struct NbrArgs {
 struct CellPlace {
     int nc, ccap;
     int* count;
-    int* atoms;
     uint4* q;
-    int* pos;
     int flag_cell;
 };
 
@@ -346,7 +342,7 @@ void launch_neighbors(const NbrArgs& a, cudaStream_t s);
 void launch_vl_check(int n_atoms, const double* x, const int* sys_of_atom, const double* box,
                      const VerletCheck& vc, cudaStream_t s);
 void launch_cells_gated(int n_atoms, const uint4* q, int nc, int* cell_count, int* cell_start,
-                        int* cell_atoms, int* atom_cell, int* atom_slot, uint4* cell_q, int* atom_pos,
+                        int* atom_cell, int* atom_slot, uint4* cell_q,
                         const int* gate, cudaStream_t s);
 void launch_vl_build(const NbrArgs& a, cudaStream_t s);
 void launch_row_filter(const NbrArgs& a, cudaStream_t s);
@@ -591,11 +587,8 @@ __device__ __forceinline__ void place_in_cell(const CellPlace& cp, int i, uint4 
     const int slot = atomicAdd(&cp.count[c], 1);
     if (slot < cp.ccap) {
         const int pos = c * cp.ccap + slot;
-        cp.atoms[pos] = i;
         cp.q[pos] = make_uint4(p.x, p.y, p.z, (unsigned int)i);   // the atom index beside its position
-        cp.pos[i] = pos;
     } else {
-        cp.pos[i] = -1;
         atomicMax(&flags[cp.flag_cell], slot + 1);
         atomicOr(&flags[kFlagOverflow], 1);
     }
