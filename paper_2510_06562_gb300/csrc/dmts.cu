@@ -608,10 +608,10 @@ int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells) {
     CUDA_TRY(dalloc(&m.mbar[0], nf));
     CUDA_TRY(dalloc(&m.mbar[1], nf));
     CUDA_TRY(dalloc(&m.msg, nf));
+    CUDA_TRY(dalloc(&m.u_spec, (size_t)2 * m.S * m.F));       // u^0 and h^0 of each species
     if (m.precision == DMTS_FP32 && m.S <= kMaxFactorSpecies && c->periodic && N >= kMinFactorAtoms) {
         CUDA_TRY(dalloc(&m.spec_row, nf * m.S));
         CUDA_TRY(dalloc(&m.spec_sum, (size_t)N * m.S));
-        CUDA_TRY(dalloc(&m.u_spec, (size_t)2 * m.S * m.F));   // u^0 and h^0 of each species
     }
     CUDA_TRY(dalloc(&m.force, (size_t)3 * N));
     CUDA_TRY(cudaMemset(m.force, 0, sizeof(float) * 3 * std::max(N, 1)));
@@ -722,14 +722,12 @@ int prepare_embedding(dmts_ctx* c, Model& m) {
     a.u_next = m.u[0];
     a.um_u_out = m.um[0];
     launch_embed(a, m.F, c->stream);
-    if (m.u_spec) {                        // the same of each species
-        a.n_atoms = m.S;
-        a.species = nullptr;
-        a.h = m.u_spec + (size_t)m.S * m.F;
-        a.u_next = m.u_spec;
-        a.um_u_out = nullptr;
-        launch_embed(a, m.F, c->stream);
-    }
+    a.n_atoms = m.S;                       // the same of each species
+    a.species = nullptr;
+    a.h = m.u_spec + (size_t)m.S * m.F;
+    a.u_next = m.u_spec;
+    a.um_u_out = nullptr;
+    launch_embed(a, m.F, c->stream);
     CUDA_TRY(cudaGetLastError());
     return DMTS_OK;
 }

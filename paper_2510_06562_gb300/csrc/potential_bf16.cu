@@ -118,6 +118,7 @@ __device__ __forceinline__ void gather_rows(float* buf, const float* __restrict_
 struct EdgeIn {
     int j, i, rp;
     uint4 qj, qi;
+    int zj, zi;                      // species (layer 0 with a species table)
 };
 
 __device__ __forceinline__ void load_idx(const PotArgs& a, long long e, long long e_end, EdgeIn& x) {
@@ -132,12 +133,41 @@ __device__ __forceinline__ void load_idx(const PotArgs& a, long long e, long lon
     }
 }
 
+template <bool SPECIES = false>
 __device__ __forceinline__ void load_pos(const PotArgs& a, EdgeIn& x) {
     if (x.j >= 0) {
         x.qj = __ldg(a.q + x.j);
         x.qi = __ldg(a.q + x.i);
+        if (SPECIES) {
+            x.zj = __ldg(a.species + x.j);
+            x.zi = __ldg(a.species + x.i);
+        }
     }
 }
+
+// Layer 0: u_j = A[Z_j] W_in is one row per species. With at most
+// kTableSpecies of them the layer-0 passes read it from a table in shared
+// memory (rows padded by 16 bytes: a warp's lanes read the same columns of
+// different rows from different banks) instead of gathering F floats per
+// directed pair through L2 (164 MB per pass of the big model on 12,288-atom
+// water). The values are those of the gathered rows, bit for bit.
+// 3 fs step: polymer of 100,000 atoms 4.09 -> 4.03 ms, 27,783-atom water 1.037 ->
+// 1.025, 12,288 atoms 0.539 -> 0.536; a small system's pass is a chain of
+// latencies that the table's copy lengthens (1,536 atoms 223.7 -> 225.0 us).
+constexpr int kTableSpecies = 8, kMinTableAtoms = 32 * kSmCount;
+inline bool species_table(const PotArgs& a) {
+    return a.layer == 0 && a.n_species <= kTableSpecies && a.n_atoms > kMinTableAtoms;
+}
+template <int F>
+struct SpeciesTable {
+    float u[kTableSpecies][F + 4];
+};
+template <int F>
+struct SpeciesTableBf {
+    float u[kTableSpecies][F + 4];
+    __nv_bfloat16 b[kTableSpecies][F + 8];      // as the backward pass gathers u_j
+};
+struct NoTable {};
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
@@ -491,10 +521,15 @@ struct FwdSmem {
     uint32_t taddr;
 };
 
-template <int F, int KC>
+// TAB: layer 0 with a species table (behind the other shared memory).
+template <int F, bool TAB>
+constexpr int fwd_smem() { return (int)((sizeof(FwdSmem<F>) + 15) / 16 * 16 + (TAB ? sizeof(SpeciesTable<F>) : 0)); }
+
+template <int F, int KC, bool TAB>
 __global__ void __launch_bounds__(kT, F == 32 ? 8 : 1) k_edge_fwd_bf16(PotArgs a, int K, int* status) {
     extern __shared__ __align__(1024) unsigned char smraw[];
     FwdSmem<F>& S = *reinterpret_cast<FwdSmem<F>*>(smraw);
+    SpeciesTable<F>& ST = *reinterpret_cast<SpeciesTable<F>*>(smraw + fwd_smem<F, false>());
     const int tid = threadIdx.x, warp = tid >> 5;
     const int l = a.layer;
     const bool rep_on = l == 0 && a.energy;                // the repulsion energy of layer 0, when read
@@ -509,6 +544,9 @@ __global__ void __launch_bounds__(kT, F == 32 ? 8 : 1) k_edge_fwd_bf16(PotArgs a
     const unsigned char* const wsrc = a.wt + (size_t)l * a.wt_layer_bytes;
     copy_weights(S.w1t, wsrc, F * kKP * 2, tid, kT);
     copy_weights(S.w2t, wsrc + F * kKP * 2, F * F * 2, tid, kT);
+    if (TAB)
+        for (int t = tid; t < a.n_species * (F / 4); t += kT)
+            cp_async16(&ST.u[t / (F / 4)][t % (F / 4) * 4], a.u_spec + 4 * t);
     cp_async_commit();
     EdgeIn nx;
     load_idx(a, (long long)blockIdx.x * kT + tid, E, nx);
@@ -516,7 +554,7 @@ __global__ void __launch_bounds__(kT, F == 32 ? 8 : 1) k_edge_fwd_bf16(PotArgs a
     const float bias2 = tid < F ? __ldg(a.P + a.off.b2[l] + tid) : 0.f;
     if (tid == 0) mbar_init(&S.mbar, 1);
     if (warp == 0) tmem_alloc(&S.taddr, 2 * F);
-    load_pos(a, nx);
+    load_pos<TAB>(a, nx);
     if (tid < F) {
         S.b1[tid] = bias1;
         S.b2[tid] = bias2;
@@ -553,9 +591,12 @@ __global__ void __launch_bounds__(kT, F == 32 ? 8 : 1) k_edge_fwd_bf16(PotArgs a
                     if (rep_on) a.erep[r] = 0.f;
                 });
             load_idx(a, (tile + gridDim.x) * kT + tid, E, nx);   // next tile's indices
-            // the message needs u_j: start copying the warp's rows into P now
-            gather_rows<F>(S.P, a.u, j, tid);
-            cp_async_commit();
+            const float* const uj = TAB ? ST.u[valid ? ex.zj : 0] : nullptr;
+            if (!TAB) {
+                // the message needs u_j: start copying the warp's rows into P now
+                gather_rows<F>(S.P, a.u, j, tid);
+                cp_async_commit();
+            }
             float fc = 0.f, rep = 0.f;
             {
                 float eb[kKP], dfc;
@@ -583,7 +624,7 @@ __global__ void __launch_bounds__(kT, F == 32 ? 8 : 1) k_edge_fwd_bf16(PotArgs a
                 mma_out = true;
                 pend = phase;
             }
-            load_pos(a, nx);                               // next tile's positions
+            load_pos<TAB>(a, nx);                               // next tile's positions
             ok = mbar_wait(&S.mbar, phase, kWaitIter);
             if (tid == 0 && ok) mma_out = false;
             phase ^= 1;
@@ -620,8 +661,10 @@ __global__ void __launch_bounds__(kT, F == 32 ? 8 : 1) k_edge_fwd_bf16(PotArgs a
             if (tid == 0 && ok) mma_out = false;
             phase ^= 1;
             fence_after_sync();
-            cp_async_wait();                               // the warp's u_j rows are in P
-            __syncwarp();
+            if (!TAB) {
+                cp_async_wait();                           // the warp's u_j rows are in P
+                __syncwarp();
+            }
             {
                 const f2::f32x2 fc2 = f2::splat(fc);
 #pragma unroll
@@ -631,7 +674,7 @@ __global__ void __launch_bounds__(kT, F == 32 ? 8 : 1) k_edge_fwd_bf16(PotArgs a
 #pragma unroll
                     for (int q = 0; q < 16; q += 4) {      // message fc (D2 + b2) u_j, two features per operation
                         float* p4 = S.P + prow<F>(tid, c + q);
-                        const float4 u4 = *reinterpret_cast<const float4*>(p4);
+                        const float4 u4 = *reinterpret_cast<const float4*>(TAB ? uj + c + q : p4);
                         const f2::f32x2* b2 = reinterpret_cast<const f2::f32x2*>(S.b2 + c + q);
                         const f2::f32x2 o01 = f2::mul(f2::mul(fc2, f2::add(f2::pack(v[q], v[q + 1]), b2[0])),
                                                       f2::pack(u4.x, u4.y));
@@ -694,6 +737,36 @@ struct BwdSmem {
     uint32_t taddr;
 };
 
+// The species table from u^0 per species, asynchronously (u) and rounded (b), thread t of nt.
+template <int F>
+__device__ __forceinline__ void load_table(SpeciesTableBf<F>& T, const PotArgs& a, int t, int nt) {
+    for (int k = t; k < a.n_species * (F / 4); k += nt) cp_async16(&T.u[k / (F / 4)][k % (F / 4) * 4], a.u_spec + 4 * k);
+    for (int k = t; k < a.n_species * F; k += nt) T.b[k / F][k % F] = __float2bfloat16_rn(__ldg(a.u_spec + k));
+}
+
+// Four floats of the receiving atom's row, from the table in shared memory or from global memory.
+template <bool TAB>
+__device__ __forceinline__ float4 ld_row4(const float* p) {
+    if (TAB) return *reinterpret_cast<const float4*>(p);
+    return __ldg(reinterpret_cast<const float4*>(p));
+}
+
+// gather_rows of the mbar halves only (16-byte chunks 2 and 3 of every 4) of
+// the interleaved BF16 rows, to the same places.
+template <int F>
+__device__ __forceinline__ void gather_mbar(float* buf, const unsigned char* __restrict__ um, int j, int tid) {
+    constexpr int TPR = F / 8;
+    constexpr int RPI = 32 / TPR;
+    const int lane = tid & 31, w0 = tid & ~31;
+    const int sub = lane / TPR, ch = (lane % TPR / 2) * 4 + 2 + (lane & 1);
+#pragma unroll
+    for (int rr = 0; rr < 32; rr += RPI) {
+        const int je = __shfl_sync(0xffffffffu, j, rr + sub);
+        const int e = w0 + rr + sub;
+        cp_async16(buf + e * F + ((ch ^ (e & 7)) << 2), um + (size_t)je * F * 4 + ch * 16);
+    }
+}
+
 template <int F>
 __host__ __device__ constexpr int scal_slot_offset() { return (int)((sizeof(VecSlots<F>) + 15) / 16 * 16); }
 
@@ -709,10 +782,16 @@ __device__ __forceinline__ void unpack_bf16x8(uint4 w, float* v) {
 
 // NV = 9: forces and the per-atom virial; NV = 3: forces only.
 // L0: the layer-0 pass (a.layer == 0), whose u does not depend on the positions.
-template <int F, int NV, int KC, bool L0>
+// TAB: with a species table (behind the other shared memory).
+template <int F, int NV, bool TAB>
+constexpr int bwd_smem() { return (int)((sizeof(BwdSmem<F, NV>) + 15) / 16 * 16 + (TAB ? sizeof(SpeciesTableBf<F>) : 0)); }
+
+template <int F, int NV, int KC, bool L0, bool TAB>
 __global__ void __launch_bounds__(kT) k_edge_bwd_bf16(PotArgs a, int K, int* status) {
+    static_assert(L0 || !TAB, "the species table is layer 0's");
     extern __shared__ __align__(1024) unsigned char smraw[];
     BwdSmem<F, NV>& S = *reinterpret_cast<BwdSmem<F, NV>*>(smraw);
+    SpeciesTableBf<F>& ST = *reinterpret_cast<SpeciesTableBf<F>*>(smraw + bwd_smem<F, NV, false>());
     static_assert(scal_slot_offset<F>() + sizeof(ScalSlots<NV>) <= sizeof(S.a14), "slots must fit the basis tiles");
     // the slots are written once the tile's first MMA (the only reader of the basis tiles) has completed
     VecSlots<F>* vs = reinterpret_cast<VecSlots<F>*>(S.a14);
@@ -732,6 +811,7 @@ __global__ void __launch_bounds__(kT) k_edge_bwd_bf16(PotArgs a, int K, int* sta
     copy_weights(S.w1t, wsrc, F * kKP * 2, tid, kT);
     if (!L0) copy_weights(S.w2t, wsrc + F * kKP * 2, F * F * 2, tid, kT);
     copy_weights(S.w2n, wsrc + F * kKP * 2 + F * F * 2, F * F * 2, tid, kT);
+    if (TAB) load_table(ST, a, tid, kT);
     cp_async_commit();
     EdgeIn nx;
     load_idx(a, (long long)blockIdx.x * kT + tid, E, nx);
@@ -739,7 +819,7 @@ __global__ void __launch_bounds__(kT) k_edge_bwd_bf16(PotArgs a, int K, int* sta
     const float bias2 = tid < F ? __ldg(a.P + a.off.b2[l] + tid) : 0.f;
     if (tid == 0) mbar_init(&S.mbar, 1);
     if (warp == 0) tmem_alloc(&S.taddr, TCOLS);
-    load_pos(a, nx);
+    load_pos<TAB>(a, nx);
     if (tid < F) {
         S.b1[tid] = bias1;
         S.b2[tid] = bias2;
@@ -777,10 +857,11 @@ __global__ void __launch_bounds__(kT) k_edge_bwd_bf16(PotArgs a, int K, int* sta
                                    [&](int r) { zero_force_row<NV>(a, r); });
             load_idx(a, (tile + gridDim.x) * kT + tid, E, nx);   // next tile's indices
             // g needs u_j and mbar_j, the ubar message mbar_j: start the warp's row copies now
-            gather_rows<F>(S.G, reinterpret_cast<const float*>(a.um), j, tid);
+            if (TAB) gather_mbar<F>(S.G, a.um, j, tid);
+            else gather_rows<F>(S.G, reinterpret_cast<const float*>(a.um), j, tid);
             cp_async_commit();
             if (valid) {                                   // the receiving atom's rows, read in the second epilogue
-                prefetch_row_l1<F>(a.u + (size_t)row * F);
+                if (!TAB) prefetch_row_l1<F>(a.u + (size_t)row * F);
                 prefetch_row_l1<F>(a.mbar + (size_t)row * F);
             }
             float fc = 0.f, dfc = 0.f, d = 1.f, rx = 0.f, ry = 0.f, rz = 0.f;
@@ -814,7 +895,7 @@ __global__ void __launch_bounds__(kT) k_edge_bwd_bf16(PotArgs a, int K, int* sta
                 mma_out = true;
                 pend = phase;
             }
-            load_pos(a, nx);                               // next tile's positions
+            load_pos<TAB>(a, nx);                               // next tile's positions
             float se;
             if constexpr (!need_ubar) {
                 // Layer 0: u does not depend on the positions, so the pass needs
@@ -828,14 +909,15 @@ __global__ void __launch_bounds__(kT) k_edge_bwd_bf16(PotArgs a, int K, int* sta
                 f2::f32x2 gb22 = 0ull;
                 {
                     const int i = valid ? row : 0;
-                    const float* ui = a.u + (size_t)i * F;
+                    const float* ui = TAB ? ST.u[valid ? ex.zi : 0] : a.u + (size_t)i * F;
+                    const __nv_bfloat16* ub = TAB ? ST.b[valid ? ex.zj : 0] : nullptr;
                     const float* mi = a.mbar + (size_t)i * F;
 #pragma unroll
                     for (int c = 0; c < F; c += 16) {
                         float4 ui16[4], mi16[4];
 #pragma unroll
                         for (int qq = 0; qq < 4; ++qq) {
-                            ui16[qq] = __ldg(reinterpret_cast<const float4*>(ui + c + 4 * qq));
+                            ui16[qq] = ld_row4<TAB>(ui + c + 4 * qq);
                             mi16[qq] = __ldg(reinterpret_cast<const float4*>(mi + c + 4 * qq));
                         }
                         float g[16], uj[16], mj[16];
@@ -843,7 +925,9 @@ __global__ void __launch_bounds__(kT) k_edge_bwd_bf16(PotArgs a, int K, int* sta
                             uint4 w[4];
 #pragma unroll
                             for (int k = 0; k < 4; ++k)
-                                w[k] = *reinterpret_cast<const uint4*>(S.G + prow<F>(tid, c + 4 * k));
+                                w[k] = *reinterpret_cast<const uint4*>(
+                                    TAB && k < 2 ? reinterpret_cast<const float*>(ub + c + 8 * k)
+                                                 : S.G + prow<F>(tid, c + 4 * k));
                             unpack_bf16x8(w[0], uj);
                             unpack_bf16x8(w[1], uj + 8);
                             unpack_bf16x8(w[2], mj);
@@ -1146,10 +1230,15 @@ __device__ __forceinline__ void unpack_bf16x16(const uint32_t* w, float* v) {
     }
 }
 
-template <int F, int NV, int NG, int KC, bool L0>
+template <int F, int NG, bool TAB>
+constexpr int bwd_grp_smem() { return (int)((sizeof(BwdGSmem<F, NG>) + 15) / 16 * 16 + (TAB ? sizeof(SpeciesTableBf<F>) : 0)); }
+
+template <int F, int NV, int NG, int KC, bool L0, bool TAB>
 __global__ void __launch_bounds__(kT * NG, 2) k_edge_bwd_grp(PotArgs a, int K, int* status) {
+    static_assert(L0 || !TAB, "the species table is layer 0's");
     extern __shared__ __align__(1024) unsigned char smraw[];
     BwdGSmem<F, NG>& S = *reinterpret_cast<BwdGSmem<F, NG>*>(smraw);
+    SpeciesTableBf<F>& ST = *reinterpret_cast<SpeciesTableBf<F>*>(smraw + bwd_grp_smem<F, NG, false>());
     constexpr int H = F / 2;
     const int g = threadIdx.x / kT;                    // this thread's group
     const int tid = threadIdx.x & (kT - 1), warp = tid >> 5;
@@ -1170,6 +1259,7 @@ __global__ void __launch_bounds__(kT * NG, 2) k_edge_bwd_grp(PotArgs a, int K, i
     copy_weights(S.w1t, wsrc, F * kKP * 2, threadIdx.x, kT * NG);
     if (!L0) copy_weights(S.w2t, wsrc + F * kKP * 2, F * F * 2, threadIdx.x, kT * NG);
     copy_weights(S.w2n, wsrc + F * kKP * 2 + F * F * 2, F * F * 2, threadIdx.x, kT * NG);
+    if (TAB) load_table(ST, a, threadIdx.x, kT * NG);
     cp_async_commit();
     const long long first = (long long)blockIdx.x * NG + g, step = (long long)gridDim.x * NG;
     EdgeIn nx;
@@ -1178,7 +1268,7 @@ __global__ void __launch_bounds__(kT * NG, 2) k_edge_bwd_grp(PotArgs a, int K, i
     const float bias2 = threadIdx.x < F ? __ldg(a.P + a.off.b2[l] + threadIdx.x) : 0.f;
     if (tid == 0) mbar_init(&T.mbar, 1);
     if (threadIdx.x < 32) tmem_alloc(&S.taddr, NG * 2 * F);
-    load_pos(a, nx);
+    load_pos<TAB>(a, nx);
     if (threadIdx.x < F) {
         S.b1[threadIdx.x] = bias1;
         S.b2[threadIdx.x] = bias2;
@@ -1213,10 +1303,11 @@ __global__ void __launch_bounds__(kT * NG, 2) k_edge_bwd_grp(PotArgs a, int K, i
             fill_empty_rows<F>(ex.rp, row, tb + tid == E - 1, a.n_atoms, need_ubar ? a.msg_out : nullptr,
                                [&](int r) { zero_force_row<NV>(a, r); });
         load_idx(a, (tile + step) * kT + tid, E, nx);      // this group's next tile's indices
-        gather_rows<F>(T.G, reinterpret_cast<const float*>(a.um), j, tid);
+        if (TAB) gather_mbar<F>(T.G, a.um, j, tid);
+        else gather_rows<F>(T.G, reinterpret_cast<const float*>(a.um), j, tid);
         cp_async_commit();
         if (valid) {                                       // the receiving atom's rows, read in the second epilogue
-            prefetch_row_l1<F>(a.u + (size_t)row * F);
+            if (!TAB) prefetch_row_l1<F>(a.u + (size_t)row * F);
             prefetch_row_l1<F>(a.mbar + (size_t)row * F);
         }
         float fc = 0.f, dfc = 0.f, d = 1.f, rx = 0.f, ry = 0.f, rz = 0.f;
@@ -1250,7 +1341,7 @@ __global__ void __launch_bounds__(kT * NG, 2) k_edge_bwd_grp(PotArgs a, int K, i
             mma_out = true;
             pend = phase;
         }
-        load_pos(a, nx);                                   // next tile's positions
+        load_pos<TAB>(a, nx);                                   // next tile's positions
         ok = mbar_wait(&T.mbar, phase, kWaitIter);
         if (tid == 0 && ok) mma_out = false;
         phase ^= 1;
@@ -1285,17 +1376,20 @@ __global__ void __launch_bounds__(kT * NG, 2) k_edge_bwd_grp(PotArgs a, int K, i
             f2::f32x2 gb22 = 0ull;
             {
                 const int i = valid ? row : 0;
-                const float* ui = a.u + (size_t)i * F;
+                const float* ui = TAB ? ST.u[valid ? ex.zi : 0] : a.u + (size_t)i * F;
+                const __nv_bfloat16* ub = TAB ? ST.b[valid ? ex.zj : 0] : nullptr;
                 const float* mi = a.mbar + (size_t)i * F;
 #pragma unroll
                 for (int c = 0; c < F; c += 16) {
                     uint4 w[4];                            // BF16 u_j (w[0], w[1]) and mbar_j (w[2], w[3])
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) w[k] = *reinterpret_cast<const uint4*>(T.G + prow<F>(tid, c + 4 * k));
+                    for (int k = 0; k < 4; ++k)
+                        w[k] = *reinterpret_cast<const uint4*>(TAB && k < 2 ? reinterpret_cast<const float*>(ub + c + 8 * k)
+                                                                            : T.G + prow<F>(tid, c + 4 * k));
                     uint32_t pg[8];
 #pragma unroll
                     for (int q = 0; q < 16; q += 4) {
-                        const float4 ui4 = __ldg(reinterpret_cast<const float4*>(ui + c + q));
+                        const float4 ui4 = ld_row4<TAB>(ui + c + q);
                         const float4 mi4 = __ldg(reinterpret_cast<const float4*>(mi + c + q));
                         const uint32_t u01 = q < 8 ? (q == 0 ? w[0].x : w[0].z) : (q == 8 ? w[1].x : w[1].z);
                         const uint32_t u23 = q < 8 ? (q == 0 ? w[0].y : w[0].w) : (q == 8 ? w[1].y : w[1].w);
@@ -1564,27 +1658,31 @@ constexpr int kSpecK = F == 64 ? 16 : 8;
 
 template <int F, int KC>
 void go_fwd(const PotArgs& a, int K, int* status, cudaStream_t s) {
-    launch_persistent(k_edge_fwd_bf16<F, KC>, (int)sizeof(FwdSmem<F>), 2 * F, kT, 1, a, K, status, s);
+    if (species_table(a))
+        launch_persistent(k_edge_fwd_bf16<F, KC, true>, fwd_smem<F, true>(), 2 * F, kT, 1, a, K, status, s);
+    else
+        launch_persistent(k_edge_fwd_bf16<F, KC, false>, fwd_smem<F, false>(), 2 * F, kT, 1, a, K, status, s);
     if (a.fused_fixup) return;                         // the per-atom kernel sums the split rows
     k_tile_fixup<F><<<fixup_blocks(a.e_cap), 256, 0, s>>>(a.n_atoms, a.row_ptr, a.recv, a.e_cap, a.carry,
                                                           a.carry_w, a.msg_out, a.layer == 0 ? 1 : 0, 0, a.erep,
                                                           nullptr, nullptr, 0, a.check);
 }
 
-template <int F, int NV, int KC, bool L0>
+template <int F, int NV, int KC, bool L0, bool TAB>
 void go_bwd_layer(const PotArgs& a, int K, int* status, cudaStream_t s) {
     const int tiles = a.bwd_tiles > 0 ? a.bwd_tiles : bf16_default_bwd_tiles(F);
     if (tiles == 2)
-        launch_persistent(k_edge_bwd_grp<F, NV, kBwdGroups, KC, L0>, (int)sizeof(BwdGSmem<F, kBwdGroups>),
+        launch_persistent(k_edge_bwd_grp<F, NV, kBwdGroups, KC, L0, TAB>, bwd_grp_smem<F, kBwdGroups, TAB>(),
                           kBwdGroups * 2 * F, kT * kBwdGroups, kBwdGroups, a, K, status, s);
     else
-        launch_persistent(k_edge_bwd_bf16<F, NV, KC, L0>, (int)sizeof(BwdSmem<F, NV>), 2 * F, kT, 1, a, K, status, s);
+        launch_persistent(k_edge_bwd_bf16<F, NV, KC, L0, TAB>, bwd_smem<F, NV, TAB>(), 2 * F, kT, 1, a, K, status, s);
 }
 
 template <int F, int NV, int KC>
 void go_bwd(const PotArgs& a, int K, int* status, cudaStream_t s) {
-    if (a.layer == 0) go_bwd_layer<F, NV, KC, true>(a, K, status, s);
-    else go_bwd_layer<F, NV, KC, false>(a, K, status, s);
+    if (species_table(a)) go_bwd_layer<F, NV, KC, true, true>(a, K, status, s);
+    else if (a.layer == 0) go_bwd_layer<F, NV, KC, true, false>(a, K, status, s);
+    else go_bwd_layer<F, NV, KC, false, false>(a, K, status, s);
     if (a.fold_fixup && a.layer == 0 && !a.accumulate && NV == 3) return;   // the integrator sums the split rows
     k_tile_fixup<F><<<fixup_blocks(a.e_cap), 256, 0, s>>>(a.n_atoms, a.row_ptr, a.recv, a.e_cap, a.carry,
                                                           a.carry_w, a.layer > 0 ? a.msg_out : nullptr, NV, 1,
@@ -1657,31 +1755,23 @@ void launch_edge_bwd_bf16(const PotArgs& a, int F, int K, int* status, cudaStrea
 // against 2 of 8 (28.6 vs 31.6 us measured on 12,288-atom water).
 int bf16_default_bwd_tiles(int F) { return F == 64 ? 2 : 1; }
 
+template <int F>
+int max_ctas(bool bwd, int tiles) {
+    constexpr int G = kBwdGroups, K = kSpecK<F>;
+    // the fewer of the layer variants
+    if (!bwd)
+        return std::min(ctas_per_sm_limit(k_edge_fwd_bf16<F, K, false>, fwd_smem<F, false>(), 2 * F, kT),
+                        ctas_per_sm_limit(k_edge_fwd_bf16<F, K, true>, fwd_smem<F, true>(), 2 * F, kT));
+    if (tiles == 2)
+        return std::min(ctas_per_sm_limit(k_edge_bwd_grp<F, 3, G, K, false, false>, bwd_grp_smem<F, G, false>(), G * 2 * F, kT * G),
+                        ctas_per_sm_limit(k_edge_bwd_grp<F, 3, G, K, true, true>, bwd_grp_smem<F, G, true>(), G * 2 * F, kT * G));
+    return std::min(ctas_per_sm_limit(k_edge_bwd_bf16<F, 3, K, false, false>, bwd_smem<F, 3, false>(), 2 * F, kT),
+                    ctas_per_sm_limit(k_edge_bwd_bf16<F, 3, K, true, true>, bwd_smem<F, 3, true>(), 2 * F, kT));
+}
+
 int bf16_max_ctas_per_sm(int F, bool bwd, int tiles) {
-    if (bwd) {
-        constexpr int G = kBwdGroups;
-        if (tiles <= 0) tiles = bf16_default_bwd_tiles(F);
-        // the fewer of the two layer variants
-        if (tiles == 2)
-            return F == 64 ? std::min(ctas_per_sm_limit(k_edge_bwd_grp<64, 3, G, kSpecK<64>, false>,
-                                                        (int)sizeof(BwdGSmem<64, G>), G * 128, kT * G),
-                                      ctas_per_sm_limit(k_edge_bwd_grp<64, 3, G, kSpecK<64>, true>,
-                                                        (int)sizeof(BwdGSmem<64, G>), G * 128, kT * G))
-                           : std::min(ctas_per_sm_limit(k_edge_bwd_grp<32, 3, G, kSpecK<32>, false>,
-                                                        (int)sizeof(BwdGSmem<32, G>), G * 64, kT * G),
-                                      ctas_per_sm_limit(k_edge_bwd_grp<32, 3, G, kSpecK<32>, true>,
-                                                        (int)sizeof(BwdGSmem<32, G>), G * 64, kT * G));
-        return F == 64 ? std::min(ctas_per_sm_limit(k_edge_bwd_bf16<64, 3, kSpecK<64>, false>,
-                                                    (int)sizeof(BwdSmem<64, 3>), 128, kT),
-                                  ctas_per_sm_limit(k_edge_bwd_bf16<64, 3, kSpecK<64>, true>,
-                                                    (int)sizeof(BwdSmem<64, 3>), 128, kT))
-                       : std::min(ctas_per_sm_limit(k_edge_bwd_bf16<32, 3, kSpecK<32>, false>,
-                                                    (int)sizeof(BwdSmem<32, 3>), 64, kT),
-                                  ctas_per_sm_limit(k_edge_bwd_bf16<32, 3, kSpecK<32>, true>,
-                                                    (int)sizeof(BwdSmem<32, 3>), 64, kT));
-    }
-    return F == 64 ? ctas_per_sm_limit(k_edge_fwd_bf16<64, kSpecK<64>>, (int)sizeof(FwdSmem<64>), 128, kT)
-                   : ctas_per_sm_limit(k_edge_fwd_bf16<32, kSpecK<32>>, (int)sizeof(FwdSmem<32>), 64, kT);
+    if (tiles <= 0) tiles = bf16_default_bwd_tiles(F);
+    return F == 64 ? max_ctas<64>(bwd, tiles) : max_ctas<32>(bwd, tiles);
 }
 
 size_t bf16_weight_tile_bytes(int F) {
