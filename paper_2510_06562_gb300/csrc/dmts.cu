@@ -294,9 +294,11 @@ bool is_device_ptr(const void* p) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-// Memory of the context's own device, which its kernels may read and write
-// directly (memory elsewhere goes through a staging buffer).
+// Doubles in memory of the context's own device, which its kernels may read
+// and write directly (memory elsewhere, or not on an 8-byte boundary, goes
+// through a staging buffer).
 bool is_own_device_ptr(const dmts_ctx* c, const void* p) {
+    if ((uintptr_t)p % sizeof(double) != 0) return false;
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
