@@ -860,12 +860,14 @@ void launch_edge_fwd(dmts_ctx* c, Model& m, const PotArgs& a) {
 }
 
 // Per-atom MLPs: tensor cores in the BF16 precision mode for F >= 64
-// (unless the option atom_tensor_cores is 0) and more atoms than the SIMT
-// kernels take in one block of 8 or 16 atoms per SM, FP32 SIMT otherwise. At F = 32
+// (unless the option atom_tensor_cores is 0), FP32 SIMT otherwise. (The SIMT
+// kernels for systems of up to 2,432 atoms, in blocks of 8 or 16 atoms: a
+// faster 3 fs step of 192 atoms, and the same distance from 64 bits, but after
+// ten steps the trajectory is 1e-3 from the tensor-core kernels'.) At F = 32
 // the SIMT kernels measured faster (16 vs 17 us for 12,288 atoms): the
 // tensor-core kernels' fixed cost is not repaid by their half-size products.
 bool atom_on_tc(const dmts_ctx* c, const Model& m) {
-    return m.precision == DMTS_BF16_MLP && c->atom_tc && m.F >= 64 && c->N > kMaxAtomsSimt;
+    return m.precision == DMTS_BF16_MLP && c->atom_tc && m.F >= 64;
 }
 
 void launch_atom_fwd_m(dmts_ctx* c, Model& m, const PotArgs& a) {

@@ -51,10 +51,6 @@ constexpr int kSmCount = 152;          // SMs of a GB300 (grid sizes only)
 // 192 atoms 217 -> 223 us; 1,536 atoms 1.7 % faster, 12,288 atoms 8 %).
 constexpr int kMaxFactorSpecies = 4;
 constexpr int kMinFactorAtoms = 1024;
-// BF16 mode, F >= 64: atoms up to which the per-atom MLPs run on FP32 SIMT
-// (blocks of 8 or 16 atoms, one per SM; the tensor-core kernel takes 128 atoms
-// per block and a fixed 11 to 19 us: 3 fs step of 2,187 atoms 265 -> 246 us)
-constexpr int kMaxAtomsSimt = 16 * kSmCount;
 constexpr int kMaxMolAtoms = 1024;     // atoms per non-periodic system
 
 // Offsets (in floats) of every parameter block inside the flat vector.

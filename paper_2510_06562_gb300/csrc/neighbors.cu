@@ -15,7 +15,7 @@
 // its pair count to per-block and per-chunk sums, and the compaction finds
 // each row's offset from those sums, writes the CSR arrays and clears the
 // cell counters for the next build. (One kernel that finds the offsets by a
-// chained scan with look-back: 1.6 % less for a 3 fs step of 192 atoms, but 2 %
+// chained scan with look-back: 3 us less per 3 fs step of 192 atoms, but 2 %
 // more at 1,536 and 11 % at 12,288, as blocks wait for earlier ones in their
 // place on the SM.)
 //
@@ -308,9 +308,10 @@ constexpr int kNbrDynSmemMax = 226 * 1024;
 // them, each cell that starts there sets its bit of a ballot-wide word, and a
 // candidate's cell is the count of bits at or below it (a search through the
 // 27 starts took five dependent shared loads). Both halves' positions are
-// loaded before either is tested. 3 fs step in BF16: 648 atoms 199 -> 195 us,
-// 1,536 234 -> 231, 3,993 316 -> 313, the same within 0.5 % from 12,288 on; at
-// five blocks per SM (48 registers) 0.5 % less for the largest than at four.
+// loaded before either is tested. Per 3 fs step in BF16 (three small lists and
+// a large one) 4 us less at 648 atoms, 3 at 1,536 and 3,993, the same within
+// 0.5 % from 12,288 on; at five blocks per SM (48 registers) 0.5 % less for the
+// largest than at four.
 __device__ __forceinline__ int nbr_candidates(const NbrArgs& a, int i, int* row, int* off) {
     const int lane = threadIdx.x & 31;
     const uint4 qi = a.q[i];
