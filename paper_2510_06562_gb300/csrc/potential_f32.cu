@@ -504,8 +504,10 @@ __global__ void __launch_bounds__(kThreads) k_gather(PotArgs a, PairFilter pf, c
 // m_i = sum_s u_s * (T_is W2 + t_is b2) with T_is = sum_{j of species s} fc SiLU(a_ij)
 // and t_is = sum_{j of species s} fc_ij, and the filter's second product runs
 // once per atom and species (in the per-atom kernel) instead of once per
-// pair: 2 F^2 flop of 17 to 26 pairs against 2 S F^2. One warp per atom, as
-// k_gather, without the rows of v.
+// pair: 2 F^2 flop of 9 to 26 unordered pairs against 2 S F^2. One warp per
+// atom, as k_gather, without the rows of v; the sums take selected values, as a
+// branch on the species splits the rows of one instruction (12,288 atoms,
+// forces with virial 683 -> 676 us).
 template <int F, int NS>
 __global__ void __launch_bounds__(kThreads) k_gather_species(PotArgs a, PairFilter pf, int a0, int a1) {
     constexpr int LPR = F / 4, RPI = 32 / LPR;
@@ -554,13 +556,12 @@ __global__ void __launch_bounds__(kThreads) k_gather_species(PotArgs a, PairFilt
                 const int zk = __shfl_sync(0xffffffffu, z, k + sub);
                 const float4 w = ld4(W, max(pk, 0), F);
 #pragma unroll
-                for (int s = 0; s < NS; ++s)
-                    if (zk == s) {
-                        acc[s].x += w.x;
-                        acc[s].y += w.y;
-                        acc[s].z += w.z;
-                        acc[s].w += w.w;
-                    }
+                for (int s = 0; s < NS; ++s) {           // (selected values: the rows of an instruction do not diverge)
+                    acc[s].x += zk == s ? w.x : 0.f;
+                    acc[s].y += zk == s ? w.y : 0.f;
+                    acc[s].z += zk == s ? w.z : 0.f;
+                    acc[s].w += zk == s ? w.w : 0.f;
+                }
             }
 #pragma unroll
             for (int s = 0; s < NS; ++s) fsum[s] += z == s ? fc : 0.f;
