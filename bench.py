@@ -210,13 +210,15 @@ def measure(D, I, torch, s, models_, prec, args, flush, dt, n_inner, seed):
 KERNEL_OF_STAGE = {
     # (precision is BF16, stage name or prefix) -> (kernel name in the ncu capture, source file);
     # the tensor-core backward pass has a layer-0 variant (two MMA groups per tile)
-    (True, "edge_bwd_l0"): ("k_edge_bwd_grp<64,3,2,16,1>", "potential_bf16.cu"),
-    (True, "edge_bwd"): ("k_edge_bwd_grp<64,3,2,16,0>", "potential_bf16.cu"),
-    (True, "edge_fwd"): ("k_edge_fwd_bf16<64,16>", "potential_bf16.cu"),
+    (True, "edge_bwd_l0"): ("k_edge_bwd_grp<64,3,2,16,1,1>", "potential_bf16.cu"),
+    (True, "edge_bwd"): ("k_edge_bwd_grp<64,3,2,16,0,0>", "potential_bf16.cu"),
+    (True, "edge_fwd_l0"): ("k_edge_fwd_bf16<64,16,1>", "potential_bf16.cu"),
+    (True, "edge_fwd"): ("k_edge_fwd_bf16<64,16,0>", "potential_bf16.cu"),
     # FP32: the layer-0 forward stage is the pair index, the filters of every layer and the layer's gather
-    (False, "edge_fwd_l0"): ("k_pair_filter<64,16>", "potential_f32.cu"),
-    (False, "edge_bwd"): ("k_gather_bwd<64,3,0>", "potential_f32.cu"),
-    (False, "edge_fwd"): ("k_gather_fwd<64>", "potential_f32.cu"),
+    (False, "edge_fwd_l0"): ("k_pair_filter<64,16,1>", "potential_f32.cu"),
+    (False, "edge_bwd_l0"): ("k_pair_dedd<64,1,1>", "potential_f32.cu"),
+    (False, "edge_bwd"): ("k_gather<64,0>", "potential_f32.cu"),
+    (False, "edge_fwd"): ("k_gather<64,1>", "potential_f32.cu"),
 }
 
 
@@ -249,9 +251,12 @@ def roofline_of(D, prec, stages_big, E_big, ba):
     dom = max((k for k in stages_big if k.startswith("edge_")), key=lambda k: stages_big[k])
     K, F = ba.n_radial, ba.n_feat
     if prec == D.FP32:
-        # w and dw/dd of every layer, 4 F (K + F) flop per unordered pair and layer; the other stages are
-        # gathers: g . dw/dd and w * mbar (8 F) or w * u (2 F) per directed pair
-        flop_edge = {"edge_fwd_l0": getattr(ba, "n_layers", 1) * 2 * F * (K + F)}.get(dom, 8 * F if dom.startswith("edge_bwd") else 2 * F)
+        # w and dw/dd of every layer, 4 F (K + F) flop per unordered pair and layer (deeper models of the
+        # periodic systems timed here leave out layer 0's second product, which runs per atom and species);
+        # the other stages are gathers: g . dw/dd and w * mbar (8 F) or w * u (2 F) per directed pair
+        layers = getattr(ba, "n_layers", 1)
+        filters = layers * 2 * F * (K + F) - (2 * F * F if layers > 1 else 0)
+        flop_edge = {"edge_fwd_l0": filters}.get(dom, 8 * F if dom.startswith("edge_bwd") else 2 * F)
         peak, bound, src, kind = FP32_SIMT_TFLOPS, "alu", "derived: 152 SMs x 128 FP32 lanes x 2 x 2.07 GHz", "FP32 SIMT"
     else:
         # the algorithmic edge-GEMM work per pair and layer, K padded to 16: one pass 2F(16 + F) forward,
