@@ -69,8 +69,9 @@ __device__ __forceinline__ void st_vec(float* d, const float (&v)[RF]) {
     else *reinterpret_cast<float2*>(d) = make_float2(v[0], v[1]);
 }
 
-// Weight buffers of the forward kernel: one each (PRE), or two in turn by the slot's parity.
-enum WSlot { kU1, kU2, kOut, kR1T, kU2T, kU1T, kSlotsPlain, kW2T = kSlotsPlain, kW2, kSlots };
+// Weight buffers of the forward kernel: one each (PRE), or two in turn by the slot's parity
+// (layer 0 by species, which is never the last layer, has W2 in the place of R1^T).
+enum WSlot { kU1, kU2, kOut, kR1T, kU2T, kU1T, kSlots, kW2 = kR1T };
 
 // Start copying the row-major F x F matrix W into Ws [F][WS]; joins the next commit group.
 template <int F, int RA>
@@ -288,7 +289,6 @@ __global__ void __launch_bounds__(AtomTile<F, RA>::NT) k_atom_fwd(PotArgs p, con
             copy_w<F, RA>(W(kR1T), r1t_of(p, F));
             copy_w<F, RA>(W(kU2T), wt_of(p, F, l, 2));
             copy_w<F, RA>(W(kU1T), wt_of(p, F, l, 1));
-            if (by_species) copy_w<F, RA>(W(kW2T), w2t_of(p, F));
         }
         cp_commit();
     } else {
@@ -490,14 +490,9 @@ __global__ void __launch_bounds__(AtomTile<F, RA>::NT) k_atom_fwd(PotArgs p, con
     put_rows<F, RA>(Y, a0, f0, v);
     cp_wait<0>();
     __syncthreads();                                                     // U2^T and X read, Y complete
-    if (by_species && !T::PRE) stage_w<F, RA>(W(kW2T), w2t_of(p, F));
     gemm_blk<F, RA>(Y, W(kU1T), a0, f0, v);                              // mbar = gz U1^T
     store_rows<F, RA>(p.mbar_out, base, p.n_atoms, a0, f0, v);
     store_rows_bf16<F, RA>(p.um_mbar_out, 1, base, p.n_atoms, a0, f0, v);
-    if (by_species) {
-        cp_wait<0>();                                                    // (visible after the first barrier inside)
-        species_adjoint<F, RA>(p, X, Y, W(kW2T), base, a0, f0, v);
-    }
 }
 
 template <int F, int RA, bool SPEC>
@@ -557,7 +552,7 @@ __global__ void __launch_bounds__(AtomTile<F, RA>::NT) k_atom_bwd(PotArgs p, con
     store_rows<F, RA>(p.mbar_out, base, p.n_atoms, a0, f0, v);
     store_rows_bf16<F, RA>(p.um_mbar_out, 1, base, p.n_atoms, a0, f0, v);
     if (by_species) {
-        cp_wait<0>();
+        cp_wait<0>();                                                    // (visible after the first barrier inside)
         species_adjoint<F, RA>(p, Y, X, W(3), base, a0, f0, v);
     }
 }
@@ -565,7 +560,7 @@ __global__ void __launch_bounds__(AtomTile<F, RA>::NT) k_atom_bwd(PotArgs p, con
 template <int F, int RA, bool SPEC>
 void atom_fwd_go(const PotArgs& p, const float* msg, cudaStream_t s) {
     using T = AtomTile<F, RA>;
-    constexpr int bytes = T::smem(SPEC ? kSlots : kSlotsPlain);
+    constexpr int bytes = T::smem(kSlots);
     smem_opt_in((const void*)k_atom_fwd<F, RA, SPEC>, bytes);
     k_atom_fwd<F, RA, SPEC><<<(p.n_atoms + T::A - 1) / T::A, T::NT, bytes, s>>>(p, msg);
 }

@@ -611,7 +611,7 @@ int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells) {
     CUDA_TRY(dalloc(&m.mbar[1], nf));
     CUDA_TRY(dalloc(&m.msg, nf));
     CUDA_TRY(dalloc(&m.u_spec, (size_t)2 * m.S * m.F));       // u^0 and h^0 of each species
-    if (m.precision == DMTS_FP32 && m.S <= kMaxFactorSpecies && c->periodic && N >= kMinFactorAtoms) {
+    if (m.precision == DMTS_FP32 && m.S <= kMaxFactorSpecies && m.L > 1 && c->periodic && N >= kMinFactorAtoms) {
         CUDA_TRY(dalloc(&m.spec_row, nf * m.S));
         CUDA_TRY(dalloc(&m.spec_sum, (size_t)N * m.S));
     }

@@ -44,7 +44,9 @@ constexpr int kThreads = 256;          // threads per CTA of the edge kernels
 constexpr int kSmCount = 152;          // SMs of a GB300 (grid sizes only)
 // FP32 mode: the first layer sums over neighbours by species before the
 // filter's second product (2 S F^2 products per atom and direction against
-// 2 F^2 per unordered pair) for up to kMaxFactorSpecies species, in periodic
+// 2 F^2 per unordered pair) in models of more than one layer (the small model
+// spends on the sums and their products what its pair kernel saves: 66 us per
+// evaluation of 12,288 atoms either way), for up to kMaxFactorSpecies species, in periodic
 // systems (9 to 26 unordered pairs per atom; molecules have 5 to 9 and lost
 // 2 % by it: 301 molecules 388 -> 397 us) of at least kMinFactorAtoms atoms (the
 // per-atom kernels' chain of products gets longer, the pairs' kernel shorter:

@@ -16,7 +16,7 @@
 // At layer 0, u_j is one row per species, and where that pays (kMinFactorAtoms)
 // the second product of the filter is taken out of the sums: rows fc SiLU(a)
 // are summed per atom and neighbour species, and multiplied by W2 once each
-// (k_gather_species; the adjoint alike in k_pair_dedd and k_row_force).
+// (k_gather_species; the adjoint alike in k_pair_dedd).
 // 12,288-atom water: forces with virial 748 -> 692 us, 3 fs step 1.00 -> 0.93 ms.
 //
 // Against recomputing the filter per directed pair in each pass (20,480 and
@@ -774,7 +774,7 @@ __global__ void __launch_bounds__(kThreads) k_pair_force(PotArgs a, PairFilter p
 // atom's row, every pair's dE/dd evaluated in both directions: at F = 32 that
 // costs no more than the two passes above (12,288-atom water, small model:
 // 18.5 against 18.9 us; 192 atoms: 8 against 14 us).
-template <int F, int NV, bool SPEC>
+template <int F, int NV>
 __global__ void __launch_bounds__(kThreads, NV == 3 ? 3 : 2) k_row_force(PotArgs a, PairFilter pf, int a0, int a1) {
     constexpr int LPR = F / 4, RPI = 32 / LPR;
     const int lane = threadIdx.x & 31, sub = lane / LPR, ch = lane % LPR;
@@ -782,7 +782,6 @@ __global__ void __launch_bounds__(kThreads, NV == 3 ? 3 : 2) k_row_force(PotArgs
     const float* DW = pf.w + (size_t)pf.cap * F + 4 * ch;
     const float* U = a.u + 4 * ch;
     const float* MB = a.mbar + 4 * ch;
-    const float* Y = a.spec_row + 4 * ch;
     const long long e_beg = min((long long)a.row_ptr[a0], a.e_cap);
     int first, last;
     gather_range(a.atoms_per_cta, a0, a1, first, last);
@@ -790,15 +789,13 @@ __global__ void __launch_bounds__(kThreads, NV == 3 ? 3 : 2) k_row_force(PotArgs
         const long long beg = min((long long)a.row_ptr[i], a.e_cap), end = min((long long)a.row_ptr[i + 1], a.e_cap);
         const uint4 qi = a.q[i];
         const float qscale = a.frame[qi.w].qscale;
-        const float4 ui = SPEC ? float4{} : ld4(U, i, F), mi = SPEC ? float4{} : ld4(MB, i, F);
-        const int zi = SPEC ? a.species[i] : 0;
+        const float4 ui = ld4(U, i, F), mi = ld4(MB, i, F);
         float fv[NV];
 #pragma unroll
         for (int c = 0; c < NV; ++c) fv[c] = 0.f;
         for (long long b = beg; b < end; b += 32) {
             const long long e = b + RPI * ch + sub;       // this lane's pair of the chunk
-            int j = i, ju = i, p = -1;                    // (SPEC: j and ju are rows of Y)
-            float fb = 0.f;
+            int j = i, ju = i, p = -1;
             float rx = 0.f, ry = 0.f, rz = 0.f, d = 1.f;
             if (e < end) {
                 j = DMTS_IDX(a.col[e], a.n_atoms, a.check);
@@ -807,13 +804,7 @@ __global__ void __launch_bounds__(kThreads, NV == 3 ? 3 : 2) k_row_force(PotArgs
                 d = sqrtf(r.x * r.x + r.y * r.y + r.z * r.z);
                 const float inv = 1.0f / d;
                 rx = r.x * inv; ry = r.y * inv; rz = r.z * inv;
-                if (SPEC) {
-                    ju = i * a.n_species + a.species[j];
-                    j = j * a.n_species + zi;
-                    fb = cutoff_deriv(d, a.pi_over_rc) * (a.spec_sum[ju] + a.spec_sum[j]);
-                } else {
-                    ju = a.first_of[j];
-                }
+                ju = a.first_of[j];
             }
             const int n = (int)min(32ll, end - b);
             float s[LPR];
@@ -824,17 +815,7 @@ __global__ void __launch_bounds__(kThreads, NV == 3 ? 3 : 2) k_row_force(PotArgs
                     const int src = sub * LPR + k;
                     const int pk = __shfl_sync(0xffffffffu, p, src), jk = __shfl_sync(0xffffffffu, j, src);
                     const int juk = __shfl_sync(0xffffffffu, ju, src);
-                    const float4 dw = ld4(DW, max(pk, 0), F);
-                    if constexpr (SPEC) {
-                        const float4 yi = ld4(Y, juk, F), yj = ld4(Y, jk, F);
-                        float t = (yi.x + yj.x) * dw.x;
-                        t += (yi.y + yj.y) * dw.y;
-                        t += (yi.z + yj.z) * dw.z;
-                        t += (yi.w + yj.w) * dw.w;
-                        s[k] = pk >= 0 ? t : 0.f;
-                        continue;
-                    }
-                    const float4 uj = ld4(U, juk, F), mj = ld4(MB, jk, F);
+                    const float4 dw = ld4(DW, max(pk, 0), F), uj = ld4(U, juk, F), mj = ld4(MB, jk, F);
                     float t = (mi.x * uj.x + mj.x * ui.x) * dw.x;
                     t += (mi.y * uj.y + mj.y * ui.y) * dw.y;
                     t += (mi.z * uj.z + mj.z * ui.z) * dw.z;
@@ -846,7 +827,7 @@ __global__ void __launch_bounds__(kThreads, NV == 3 ? 3 : 2) k_row_force(PotArgs
             if (e < end) {
                 float dphi;
                 (void)rep_phi(d, a.rep_a, a.rep_inv_rho, a.rep_rc, a.rep_pi_over_rc, &dphi);
-                add_force<NV>(fv, s[0] + fb + dphi, rx, ry, rz, d);
+                add_force<NV>(fv, s[0] + dphi, rx, ry, rz, d);
             }
         }
         store_force<NV>(a, i, fv, lane, a.accumulate);
@@ -927,13 +908,8 @@ void bwd_go(const PotArgs& a, int K, cudaStream_t s) {
         const int warps = (int)std::min<long long>((a.filter.cap + 31) / 32, (long long)kSmCount * 8 * (F == 64 ? 3 : 4));
         const int pgrid = (warps + kThreads / 32 - 1) / (kThreads / 32);
         if (a.n_layers == 1) {
-            if (a.spec_row) {
-                if (a.virial) k_row_force<F, 9, true><<<grid, kThreads, 0, s>>>(a, a.filter, a0, a1);
-                else k_row_force<F, 3, true><<<grid, kThreads, 0, s>>>(a, a.filter, a0, a1);
-            } else {
-                if (a.virial) k_row_force<F, 9, false><<<grid, kThreads, 0, s>>>(a, a.filter, a0, a1);
-                else k_row_force<F, 3, false><<<grid, kThreads, 0, s>>>(a, a.filter, a0, a1);
-            }
+            if (a.virial) k_row_force<F, 9><<<grid, kThreads, 0, s>>>(a, a.filter, a0, a1);
+            else k_row_force<F, 3><<<grid, kThreads, 0, s>>>(a, a.filter, a0, a1);
             count_launch();
             continue;
         }

@@ -1,6 +1,6 @@
 """Per-atom kernels at the atom counts where their blocks change: part of a
-block of 8, whole, one more; the most atoms in blocks of 8 and of 16 (one per
-SM) and one more; both models and both precisions against the FP64 oracle.
+block of 8, whole, one more; the most atoms in blocks of 8 and of 16 (at F = 32
+and 64) and one more; both models and both precisions against the FP64 oracle.
 Tolerances: those of the parity tests (1e-6 eV per atom and 1e-5 eV/A RMSE in
 FP32, 5e-3 eV per atom and eV/A in BF16) per unit of the largest |E| per atom
 or RMS force beyond 1.
@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("prec,tol_e,tol_f", [(D.FP32, 1e-6, 1e-5), (D.BF16_MLP, 5e-3, 5e-3)])
-@pytest.mark.parametrize("n", [3, 8, 9, 1215, 1216, 1217, 2432, 2433])
+@pytest.mark.parametrize("n", [3, 8, 9, 1215, 1216, 1217, 1824, 1825, 2432, 2433])
 def test_block_sizes(n, prec, tol_e, tol_f):
     s = I.make_water(10, 31.05, n)
     s.x, s.mass, s.species = s.x[:n], s.mass[:n], s.species[:n]

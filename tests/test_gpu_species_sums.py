@@ -1,7 +1,7 @@
 """FP32 mode, layer 0 summed by neighbour species before the filter's second
-product (periodic systems of at least 1,024 atoms and up to four species;
-others take the general passes): forces, energies and virial of one to five
-species, both widths, one to three layers, atom counts that are not multiples
+product (models of two layers and more, periodic systems of at least 1,024
+atoms, up to four species; others take the general passes): forces, energies
+and virial of one to five species, both widths, one to three layers, atom counts that are not multiples
 of the 32-atom blocks, species that no atom has, and the distillation
 gradient, against the FP64 oracle. Tolerances as in test_gpu_pair_filter.py,
 and of test_gpu_distill.py for the gradient.
