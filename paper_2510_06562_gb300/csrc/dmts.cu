@@ -200,6 +200,7 @@ struct Model {
 struct dmts_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
+    bool own_stream = true;                // the inner context of distillation batches runs on its outer one's
     int N = 0, n_sys = 0, max_sys = 0;     // atoms, systems, atoms of the largest system
     bool periodic = false;
     std::vector<int> h_off;
@@ -1329,13 +1330,18 @@ void dmts_destroy(dmts_ctx* c) {
     dfree(c->fm_eref); dfree(c->fm_ce);
     dmts_destroy(c->batch);
     if (c->h_flags) cudaFreeHost(c->h_flags);
-    if (c->stream) cudaStreamDestroy(c->stream);
+    if (c->stream && c->own_stream) cudaStreamDestroy(c->stream);
     delete c;
 }
 
-int dmts_create(const dmts_model_desc* small, const dmts_model_desc* big, const dmts_system_desc* sys,
-                const char* options, dmts_ctx** out) {
-    Range nvtx_range("dmts_create");
+}  // extern "C"
+
+namespace {
+
+// dmts_create, on a stream of its own (stream null) or on the caller's, which
+// has to outlive the context.
+int create_context(const dmts_model_desc* small, const dmts_model_desc* big, const dmts_system_desc* sys,
+                   const char* options, cudaStream_t stream, dmts_ctx** out) {
     g_err.clear();
     if (!out) return fail(DMTS_ERR_ARG, "out is NULL");
     *out = nullptr;
@@ -1424,7 +1430,9 @@ int dmts_create(const dmts_model_desc* small, const dmts_model_desc* big, const 
             return code_;                                                         \
         }                                                                         \
     } while (0)
-    CREATE_TRY(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
+    c->own_stream = !stream;
+    c->stream = stream;
+    if (!stream) CREATE_TRY(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
     std::vector<int> sys_of(N);
     for (int s = 0; s < ns; ++s)
         for (int i = sys->atom_offset[s]; i < sys->atom_offset[s + 1]; ++i) sys_of[i] = s;
@@ -1532,6 +1540,16 @@ int dmts_create(const dmts_model_desc* small, const dmts_model_desc* big, const 
     CREATE_TRY(cudaGetLastError());
     *out = c;
     return DMTS_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int dmts_create(const dmts_model_desc* small, const dmts_model_desc* big, const dmts_system_desc* sys,
+                const char* options, dmts_ctx** out) {
+    Range nvtx_range("dmts_create");
+    return create_context(small, big, sys, options, nullptr, out);
 }
 
 int dmts_set_state(dmts_ctx* c, const double* x, const double* v, int n_atoms) {
@@ -1748,7 +1766,9 @@ constexpr int kFmBatchAtoms = 131072;
 
 // The inner context that evaluates `frames` frames of c's systems at once:
 // the systems repeated, the small model alone, its weights copied from c's.
-// Returns null if it cannot be created (no memory): one frame at a time then.
+// It runs on c's stream: behind what the caller queued there, and before what
+// the caller queues there next. Returns null if it cannot be created (no
+// memory): one frame at a time then.
 dmts_ctx* batch_context(dmts_ctx* c, int frames) {
     if (c->batch && c->batch_frames < frames) {
         dmts_destroy(c->batch);
@@ -1771,7 +1791,7 @@ dmts_ctx* batch_context(dmts_ctx* c, int frames) {
         d.precision = m.precision;
         d.rep_a = m.rep_a; d.rep_rho = m.rep_rho; d.rep_cutoff = m.rep_rc;
         const dmts_system_desc sys{frames * c->n_sys, off.data(), spb.data(), mass.data(), box.data()};
-        if (dmts_create(nullptr, &d, &sys, "{\"autotune\": 0}", &c->batch) != DMTS_OK) return nullptr;
+        if (create_context(nullptr, &d, &sys, "{\"autotune\": 0}", c->stream, &c->batch) != DMTS_OK) return nullptr;
         c->batch_frames = frames;
         c->batch_params = m.version;
         c->batch->keep_msg = true;             // the second-order passes read every message row
