@@ -360,7 +360,7 @@ constexpr size_t kFilterBytes = (size_t)64 << 20, kFilterChunkBytes = (size_t)16
 constexpr size_t kFilterBytes = (size_t)32 << 30, kFilterChunkBytes = (size_t)8 << 30;
 #endif
 
-cudaError_t alloc_filters(Model& m) {
+cudaError_t alloc_filters(dmts_ctx* c, Model& m) {
     PairFilter& f = m.filt;
     const size_t row = 2 * sizeof(float) * m.F;               // w and dw/dd of one layer
     const long long half = m.e_cap / 2 + 1;
@@ -371,7 +371,7 @@ cudaError_t alloc_filters(Model& m) {
         if (e == cudaSuccess) e = dalloc(&f.pairs, (size_t)half);
         if (e == cudaSuccess) e = dalloc(&f.pid, (size_t)m.e_cap);
         if (e == cudaSuccess) e = dalloc(&f.count, 1);
-        if (e == cudaSuccess) e = cudaMemset(f.count, 0, sizeof(int));
+        if (e == cudaSuccess) e = cudaMemsetAsync(f.count, 0, sizeof(int), c->stream);
         f.cap = half;
         if (e == cudaSuccess) return e;
         cudaGetLastError();
@@ -399,7 +399,7 @@ cudaError_t alloc_model_nbr(dmts_ctx* c, Model& m) {
     if (c->skin > 0 && (e = dalloc(&m.vl_rows, (size_t)c->N * m.vl_cap)) != cudaSuccess) return e;
     const size_t tiles = (size_t)((m.e_cap + 127) / 128);
     if ((e = dalloc(&m.carry, tiles * 2 * (size_t)(m.F + 16))) != cudaSuccess) return e;
-    if (m.precision == DMTS_FP32 && (e = alloc_filters(m)) != cudaSuccess) return e;
+    if (m.precision == DMTS_FP32 && (e = alloc_filters(c, m)) != cudaSuccess) return e;
     return cudaSuccess;
 }
 
@@ -576,7 +576,7 @@ int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells) {
     if (m.nc > 0) {
         m.n_cells = c->n_sys * m.nc * m.nc * m.nc;            // each system its own cells
         CUDA_TRY(dalloc(&m.cell_count, m.n_cells));
-        CUDA_TRY(cudaMemset(m.cell_count, 0, sizeof(int) * m.n_cells));
+        CUDA_TRY(cudaMemsetAsync(m.cell_count, 0, sizeof(int) * m.n_cells, c->stream));
         if (c->skin > 0) {                 // compact cells rebuilt by count, scan and fill
             CUDA_TRY(dalloc(&m.cell_start, m.n_cells + 1));
             CUDA_TRY(dalloc(&m.atom_cell, N));
@@ -595,8 +595,8 @@ int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells) {
         CUDA_TRY(dalloc(&m.block_sum, nb));
         CUDA_TRY(dalloc(&m.chunk_sum, nch));
         CUDA_TRY(dalloc(&m.ticket, 1));
-        CUDA_TRY(cudaMemset(m.chunk_sum, 0, sizeof(int) * nch));
-        CUDA_TRY(cudaMemset(m.ticket, 0, sizeof(unsigned int)));
+        CUDA_TRY(cudaMemsetAsync(m.chunk_sum, 0, sizeof(int) * nch, c->stream));
+        CUDA_TRY(cudaMemsetAsync(m.ticket, 0, sizeof(unsigned int), c->stream));
     }
     CUDA_TRY(dalloc(&m.row_ptr, N + 1));
     size_t nf = (size_t)N * m.F;
@@ -617,14 +617,14 @@ int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells) {
         CUDA_TRY(dalloc(&m.spec_sum, (size_t)N * m.S));
     }
     CUDA_TRY(dalloc(&m.force, (size_t)3 * N));
-    CUDA_TRY(cudaMemset(m.force, 0, sizeof(float) * 3 * std::max(N, 1)));
+    CUDA_TRY(cudaMemsetAsync(m.force, 0, sizeof(float) * 3 * std::max(N, 1), c->stream));
     CUDA_TRY(dalloc(&m.vir6, (size_t)6 * N));
     CUDA_TRY(dalloc(&m.Ei, N));
     CUDA_TRY(dalloc(&m.erep, N));
     CUDA_TRY(dalloc(&m.E, c->n_sys));
     CUDA_TRY(dalloc(&m.esum.part, (size_t)kSumMaxSplit * kSumChunks * 6));
     CUDA_TRY(dalloc(&m.esum.ctr, kSumMaxSplit));
-    CUDA_TRY(cudaMemset(m.esum.ctr, 0, sizeof(unsigned int) * kSumMaxSplit));
+    CUDA_TRY(cudaMemsetAsync(m.esum.ctr, 0, sizeof(unsigned int) * kSumMaxSplit, c->stream));
     CUDA_TRY(dalloc(&m.W, (size_t)9 * c->n_sys));
     // FP32: atoms per CTA of the gathers (eight warps, one atom each at a time)
     m.apc_fwd = m.apc_bwd = 8;
@@ -1339,7 +1339,9 @@ void dmts_destroy(dmts_ctx* c) {
 namespace {
 
 // dmts_create, on a stream of its own (stream null) or on the caller's, which
-// has to outlive the context.
+// has to outlive the context. Uploads and clears go to that stream, as those
+// of buffers allocated later do: the streams are non-blocking, so nothing would
+// order a clear on the default stream before the kernels that read the buffer.
 int create_context(const dmts_model_desc* small, const dmts_model_desc* big, const dmts_system_desc* sys,
                    const char* options, cudaStream_t stream, dmts_ctx** out) {
     g_err.clear();
@@ -1461,23 +1463,23 @@ int create_context(const dmts_model_desc* small, const dmts_model_desc* big, con
     CREATE_TRY(dalloc(&c->d_ekin, ns));
     CREATE_TRY(dalloc(&c->d_epart, (size_t)2 * std::max(1, integrator_blocks(N))));
     CREATE_TRY(dalloc(&c->d_eticket, 1));
-    CREATE_TRY(cudaMemset(c->d_eticket, 0, sizeof(unsigned int)));
+    CREATE_TRY(cudaMemsetAsync(c->d_eticket, 0, sizeof(unsigned int), c->stream));
     CREATE_TRY(dalloc(&c->d_flags, kFlagCount));
     CREATE_TRY(dalloc(&c->d_bx, (size_t)3 * N));
     CREATE_TRY(dalloc(&c->d_bv, (size_t)3 * N));
     CREATE_TRY(cudaMallocHost((void**)&c->h_flags, sizeof(int) * kFlagCount));
     CREATE_TRY(dalloc(&c->kesum.part, (size_t)kSumMaxSplit * kSumChunks));
     CREATE_TRY(dalloc(&c->kesum.ctr, kSumMaxSplit));
-    CREATE_TRY(cudaMemset(c->kesum.ctr, 0, sizeof(unsigned int) * kSumMaxSplit));
+    CREATE_TRY(cudaMemsetAsync(c->kesum.ctr, 0, sizeof(unsigned int) * kSumMaxSplit, c->stream));
     CREATE_TRY(dalloc(&c->d_rng, 2));
-    CREATE_TRY(cudaMemset(c->d_rng, 0, 2 * sizeof(unsigned long long)));
+    CREATE_TRY(cudaMemsetAsync(c->d_rng, 0, 2 * sizeof(unsigned long long), c->stream));
     CREATE_TRY(cudaStreamCreateWithFlags(&c->s_big, cudaStreamNonBlocking));
     CREATE_TRY(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
     CREATE_TRY(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
     c->concurrent = opt.get("concurrent_models", 1.0) != 0.0;
     c->atom_tc = opt.get("atom_tensor_cores", 1.0) != 0.0;
     CREATE_TRY(dalloc(&c->d_mon, 1));
-    CREATE_TRY(cudaMemset(c->d_mon, 0, sizeof(ForceMonitor)));
+    CREATE_TRY(cudaMemsetAsync(c->d_mon, 0, sizeof(ForceMonitor), c->stream));
     if (c->fb_threshold > 0.0) {
         CREATE_TRY(dalloc(&c->d_sx, (size_t)3 * N));
         CREATE_TRY(dalloc(&c->d_sv, (size_t)3 * N));
@@ -1487,19 +1489,19 @@ int create_context(const dmts_model_desc* small, const dmts_model_desc* big, con
     if (c->skin > 0) {
         CREATE_TRY(dalloc(&c->d_xref, (size_t)3 * N));
         CREATE_TRY(dalloc(&c->d_vl, 1));
-        CREATE_TRY(cudaMemset(c->d_vl, 0, sizeof(VerletState)));
-        CREATE_TRY(cudaMemset(&c->d_vl->force, 1, sizeof(int)));
+        CREATE_TRY(cudaMemsetAsync(c->d_vl, 0, sizeof(VerletState), c->stream));
+        CREATE_TRY(cudaMemsetAsync(&c->d_vl->force, 1, sizeof(int), c->stream));
     }
-    CREATE_TRY(cudaMemcpy(c->d_off, sys->atom_offset, sizeof(int) * (ns + 1), cudaMemcpyHostToDevice));
-    CREATE_TRY(cudaMemcpy(c->d_species, sys->species, sizeof(int) * std::max(N, 0), cudaMemcpyHostToDevice));
-    CREATE_TRY(cudaMemcpy(c->d_first_of, first_of.data(), sizeof(int) * N, cudaMemcpyHostToDevice));
-    CREATE_TRY(cudaMemcpy(c->d_sys, sys_of.data(), sizeof(int) * N, cudaMemcpyHostToDevice));
-    CREATE_TRY(cudaMemcpy(c->d_box, sys->box, sizeof(double) * ns, cudaMemcpyHostToDevice));
-    CREATE_TRY(cudaMemcpy(c->d_mass, sys->mass, sizeof(double) * N, cudaMemcpyHostToDevice));
-    CREATE_TRY(cudaMemcpy(c->d_inv_m, inv_m.data(), sizeof(double) * N, cudaMemcpyHostToDevice));
-    CREATE_TRY(cudaMemset(c->d_x, 0, sizeof(double) * 3 * std::max(N, 1)));
-    CREATE_TRY(cudaMemset(c->d_v, 0, sizeof(double) * 3 * std::max(N, 1)));
-    CREATE_TRY(cudaMemset(c->d_flags, 0, sizeof(int) * kFlagCount));
+    CREATE_TRY(cudaMemcpyAsync(c->d_off, sys->atom_offset, sizeof(int) * (ns + 1), cudaMemcpyHostToDevice, c->stream));
+    CREATE_TRY(cudaMemcpyAsync(c->d_species, sys->species, sizeof(int) * std::max(N, 0), cudaMemcpyHostToDevice, c->stream));
+    CREATE_TRY(cudaMemcpyAsync(c->d_first_of, first_of.data(), sizeof(int) * N, cudaMemcpyHostToDevice, c->stream));
+    CREATE_TRY(cudaMemcpyAsync(c->d_sys, sys_of.data(), sizeof(int) * N, cudaMemcpyHostToDevice, c->stream));
+    CREATE_TRY(cudaMemcpyAsync(c->d_box, sys->box, sizeof(double) * ns, cudaMemcpyHostToDevice, c->stream));
+    CREATE_TRY(cudaMemcpyAsync(c->d_mass, sys->mass, sizeof(double) * N, cudaMemcpyHostToDevice, c->stream));
+    CREATE_TRY(cudaMemcpyAsync(c->d_inv_m, inv_m.data(), sizeof(double) * N, cudaMemcpyHostToDevice, c->stream));
+    CREATE_TRY(cudaMemsetAsync(c->d_x, 0, sizeof(double) * 3 * std::max(N, 1), c->stream));
+    CREATE_TRY(cudaMemsetAsync(c->d_v, 0, sizeof(double) * 3 * std::max(N, 1), c->stream));
+    CREATE_TRY(cudaMemsetAsync(c->d_flags, 0, sizeof(int) * kFlagCount, c->stream));
     if (small) {
         rc = init_model(c, c->m[0], small, c->skin <= 0 || c->vl_src == 0);
         if (rc) { std::string k = g_err; dmts_destroy(c); g_err = k; return rc; }
@@ -1535,9 +1537,9 @@ int create_context(const dmts_model_desc* small, const dmts_model_desc* big, con
     if (c->periodic) {
         // constant frame; computed once on the device
         launch_frames(ns, c->max_sys, c->d_off, c->d_x, N, c->d_box, rc_max, c->d_frame, nullptr, c->stream);
-        CREATE_TRY(cudaStreamSynchronize(c->stream));
     }
     CREATE_TRY(cudaGetLastError());
+    CREATE_TRY(cudaStreamSynchronize(c->stream));
     *out = c;
     return DMTS_OK;
 }
@@ -1778,7 +1780,9 @@ dmts_ctx* batch_context(dmts_ctx* c, int frames) {
     if (!c->batch) {
         std::vector<int> off(1, 0), sp((size_t)c->N), spb;
         std::vector<double> mass((size_t)frames * c->N, 1.0), box;
-        if (cudaMemcpy(sp.data(), c->d_species, sizeof(int) * c->N, cudaMemcpyDeviceToHost) != cudaSuccess) return nullptr;
+        if (cudaMemcpyAsync(sp.data(), c->d_species, sizeof(int) * c->N, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
+            cudaStreamSynchronize(c->stream) != cudaSuccess)
+            return nullptr;
         for (int f = 0; f < frames; ++f) {
             for (int k = 0; k < c->n_sys; ++k) off.push_back(f * c->N + c->h_off[k + 1]);
             box.insert(box.end(), c->h_box.begin(), c->h_box.end());
@@ -1812,7 +1816,7 @@ int alloc_fm(dmts_ctx* c, int atoms) {
     if (e == cudaSuccess) e = dalloc(&b.partial_a, (size_t)fm_atom_rows(atoms) * m.n_params);
     if (e == cudaSuccess) e = dalloc(&b.part, (size_t)fm_residual_blocks(atoms));
     if (e == cudaSuccess) e = dalloc(&b.ticket, 1);
-    if (e == cudaSuccess) e = cudaMemset(b.ticket, 0, sizeof(unsigned int));
+    if (e == cudaSuccess) e = cudaMemsetAsync(b.ticket, 0, sizeof(unsigned int), c->stream);
     if (e == cudaSuccess) e = dalloc(&b.grad, m.n_params);
     if (e == cudaSuccess) e = dalloc(&b.loss, 1);
     if (e == cudaSuccess) e = dalloc(&c->fm_stage, (size_t)6 * atoms);
