@@ -1218,6 +1218,7 @@ int autotune_models(dmts_ctx* c) {
         Model& m = c->m[w];
         if (!m.present) continue;
         const bool tc = m.precision == DMTS_BF16_MLP;
+        const PotArgs shape = pot_args(c, m);
         // tensor-core kernels: persistent CTAs per SM, and the backward
         // kernel's tiles in flight per CTA (one, or two sharing the weights);
         // FP32 kernels: atoms per CTA
@@ -1227,8 +1228,8 @@ int autotune_models(dmts_ctx* c) {
         double best_tf = 1e30, best_tb = 1e30;
         int best_f = gf, best_b = gb, best_t = m.bwd_tiles;
         for (int tiles : tiles_c) {
-            const int lim_f = tc ? bf16_max_ctas_per_sm(m.F, false) : kMaxAtomsPerCtaF32;
-            const int lim_b = tc ? bf16_max_ctas_per_sm(m.F, true, tiles) : kMaxAtomsPerCtaF32;
+            const int lim_f = tc ? bf16_max_ctas_per_sm(shape, m.F, false) : kMaxAtomsPerCtaF32;
+            const int lim_b = tc ? bf16_max_ctas_per_sm(shape, m.F, true, tiles) : kMaxAtomsPerCtaF32;
             std::vector<int> cand;
             if (tc) for (int k = 1; k <= std::max(lim_f, lim_b); ++k) cand.push_back(k);
             else cand = {8, 16};
@@ -2205,9 +2206,10 @@ int dmts_set_tuning(dmts_ctx* c, int which, int fwd, int bwd, int bwd_tiles) {
     if (fwd < 1 || bwd < 1) return fail(DMTS_ERR_ARG, "granularity must be >= 1");
     if (bwd_tiles < 0 || bwd_tiles > 2) return fail(DMTS_ERR_ARG, "bwd_tiles must be 0, 1 or 2");
     if (m.precision == DMTS_BF16_MLP) {
+        const PotArgs shape = pot_args(c, m);
         if (bwd_tiles > 0) m.bwd_tiles = bwd_tiles;
-        m.cps_fwd = std::min(fwd, bf16_max_ctas_per_sm(m.F, false));
-        m.cps_bwd = std::min(bwd, bf16_max_ctas_per_sm(m.F, true, m.bwd_tiles));
+        m.cps_fwd = std::min(fwd, bf16_max_ctas_per_sm(shape, m.F, false));
+        m.cps_bwd = std::min(bwd, bf16_max_ctas_per_sm(shape, m.F, true, m.bwd_tiles));
     } else {
         m.apc_fwd = std::min(fwd, kMaxAtomsPerCtaF32);
         m.apc_bwd = std::min(bwd, kMaxAtomsPerCtaF32);

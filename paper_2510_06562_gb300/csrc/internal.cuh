@@ -362,7 +362,7 @@ void launch_wait_selftest(int arrive, unsigned int polls, int* status, cudaStrea
 size_t bf16_weight_tile_bytes(int F);
 // CTAs per SM that fit for the forward (bwd = false) or backward kernel;
 // tiles: the backward kernel's tiles in flight per CTA (1 or 2).
-int bf16_max_ctas_per_sm(int F, bool bwd, int tiles = 0);
+int bf16_max_ctas_per_sm(const PotArgs& a, int F, bool bwd, int tiles = 0);   // of a's model (n_layers, n_species, n_atoms)
 int bf16_default_bwd_tiles(int F);
 
 // distill.cu: distillation (energy and force matching) gradient of a single-layer model

@@ -814,12 +814,15 @@ __global__ void __launch_bounds__(kT) k_edge_bwd_bf16(PotArgs a, int K, int* sta
     if (TAB) load_table(ST, a, tid, kT);
     cp_async_commit();
     EdgeIn nx;
-    load_idx(a, (long long)blockIdx.x * kT + tid, E, nx);
+    // (above layer 0 the first tile's loads wait for the weights: ahead of them
+    // they take the kernel from 95 to 128 registers at F = 32, and an SM from five
+    // CTAs to four)
+    if (L0) load_idx(a, (long long)blockIdx.x * kT + tid, E, nx);
     const float bias1 = tid < F ? __ldg(a.P + a.off.b1[l] + tid) : 0.f;
     const float bias2 = tid < F ? __ldg(a.P + a.off.b2[l] + tid) : 0.f;
     if (tid == 0) mbar_init(&S.mbar, 1);
     if (warp == 0) tmem_alloc(&S.taddr, TCOLS);
-    load_pos<TAB>(a, nx);
+    if (L0) load_pos<TAB>(a, nx);
     if (tid < F) {
         S.b1[tid] = bias1;
         S.b2[tid] = bias2;
@@ -840,6 +843,10 @@ __global__ void __launch_bounds__(kT) k_edge_bwd_bf16(PotArgs a, int K, int* sta
     uint32_t pend = 0;                                     // ... and the parity it completes
 
     const int cw = a.carry_w;
+    if (!L0) {
+        load_idx(a, (long long)blockIdx.x * kT + tid, E, nx);
+        load_pos<TAB>(a, nx);
+    }
     for (long long tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
         {
             const long long tb = tile * kT, te = min(tb + kT, E);
@@ -1752,26 +1759,33 @@ void launch_edge_bwd_bf16(const PotArgs& a, int F, int K, int* status, cudaStrea
 // The backward kernel's tiles in flight per CTA unless the tuner chooses:
 // two at F = 64 (two groups of 4 warps share one copy of the weights), one
 // at F = 32, where the one-tile kernel fits 5 CTAs of 4 warps per SM
-// against 2 of 8 (28.6 vs 31.6 us measured on 12,288-atom water).
+// against 2 of 8 (26.5 vs 27.4 us on 12,288-atom water, 117 vs 125 on the
+// 100,000-atom polymer).
 int bf16_default_bwd_tiles(int F) { return F == 64 ? 2 : 1; }
 
-template <int F>
-int max_ctas(bool bwd, int tiles) {
+// CTAs per SM of one pass: the most that a kernel of the model's layers runs at
+// (a launch takes no more than its own kernel can). Kernels that this model
+// does not launch have no say.
+template <int F, bool L0, bool TAB>
+int variant_ctas(bool bwd, int tiles) {
     constexpr int G = kBwdGroups, K = kSpecK<F>;
-    // the fewer of the layer variants
-    if (!bwd)
-        return std::min(ctas_per_sm_limit(k_edge_fwd_bf16<F, K, false>, fwd_smem<F, false>(), 2 * F, kT),
-                        ctas_per_sm_limit(k_edge_fwd_bf16<F, K, true>, fwd_smem<F, true>(), 2 * F, kT));
+    if (!bwd) return ctas_per_sm_limit(k_edge_fwd_bf16<F, K, TAB>, fwd_smem<F, TAB>(), 2 * F, kT);
     if (tiles == 2)
-        return std::min(ctas_per_sm_limit(k_edge_bwd_grp<F, 3, G, K, false, false>, bwd_grp_smem<F, G, false>(), G * 2 * F, kT * G),
-                        ctas_per_sm_limit(k_edge_bwd_grp<F, 3, G, K, true, true>, bwd_grp_smem<F, G, true>(), G * 2 * F, kT * G));
-    return std::min(ctas_per_sm_limit(k_edge_bwd_bf16<F, 3, K, false, false>, bwd_smem<F, 3, false>(), 2 * F, kT),
-                    ctas_per_sm_limit(k_edge_bwd_bf16<F, 3, K, true, true>, bwd_smem<F, 3, true>(), 2 * F, kT));
+        return ctas_per_sm_limit(k_edge_bwd_grp<F, 3, G, K, L0, TAB>, bwd_grp_smem<F, G, TAB>(), G * 2 * F, kT * G);
+    return ctas_per_sm_limit(k_edge_bwd_bf16<F, 3, K, L0, TAB>, bwd_smem<F, 3, TAB>(), 2 * F, kT);
 }
 
-int bf16_max_ctas_per_sm(int F, bool bwd, int tiles) {
+template <int F>
+int max_ctas(const PotArgs& a, bool bwd, int tiles) {
+    PotArgs l0 = a;
+    l0.layer = 0;
+    const int first = species_table(l0) ? variant_ctas<F, true, true>(bwd, tiles) : variant_ctas<F, true, false>(bwd, tiles);
+    return a.n_layers == 1 ? first : std::max(first, variant_ctas<F, false, false>(bwd, tiles));
+}
+
+int bf16_max_ctas_per_sm(const PotArgs& a, int F, bool bwd, int tiles) {
     if (tiles <= 0) tiles = bf16_default_bwd_tiles(F);
-    return F == 64 ? max_ctas<64>(bwd, tiles) : max_ctas<32>(bwd, tiles);
+    return F == 64 ? max_ctas<64>(a, bwd, tiles) : max_ctas<32>(a, bwd, tiles);
 }
 
 size_t bf16_weight_tile_bytes(int F) {
