@@ -66,9 +66,11 @@ int fail(int code, const char* fmt, ...) {
 #define CUDA_TRY(expr)                                                                   \
     do {                                                                                 \
         cudaError_t e_ = (expr);                                                         \
-        if (e_ != cudaSuccess)                                                           \
+        if (e_ != cudaSuccess) {                                                         \
+            cudaGetLastError();               /* reported here, not by the next call */  \
             return fail(e_ == cudaErrorMemoryAllocation ? DMTS_ERR_OOM : DMTS_ERR_CUDA,  \
                         "%s: %s", #expr, cudaGetErrorString(e_));                        \
+        }                                                                                \
     } while (0)
 
 // Context options: a flat JSON object whose values are numbers or booleans
@@ -340,20 +342,26 @@ int check_model(const dmts_model_desc* d, const char* name) {
     return DMTS_OK;
 }
 
+void free_filters(Model& m) {
+    dfree(m.filt.w); dfree(m.filt.se); dfree(m.filt.pairs); dfree(m.filt.pid); dfree(m.filt.count);
+    m.filt = PairFilter{};
+}
+
 void free_model_nbr(Model& m) {
     dfree(m.nbr_tmp); dfree(m.col); dfree(m.recv); dfree(m.vl_rows); dfree(m.carry);
-    dfree(m.filt.w); dfree(m.filt.se); dfree(m.filt.pairs); dfree(m.filt.pid); dfree(m.filt.count);
     m.nbr_tmp = m.col = m.recv = m.vl_rows = nullptr;
     m.carry = nullptr;
-    m.filt = PairFilter{};
+    free_filters(m);
 }
 
 // Filter rows of the FP32 mode (PairFilter): for every unordered pair and
 // layer if that takes at most kFilterBytes (about 800,000 atoms of water with
-// the big model; 0.5 GB at 12,288) and the memory is there, otherwise for the
-// directed pairs of as many atoms as fit in kFilterChunkBytes at a time,
-// halved until the allocation succeeds. Checked builds use small limits, so
-// that both forms run on small systems.
+// the big model; 0.5 GB at 12,288) and half of the free memory, otherwise for
+// the directed pairs of as many atoms as fit in kFilterChunkBytes and half of
+// the free memory at a time, halved until the allocation succeeds. They are
+// allocated behind every other buffer of the context, and what else needs
+// memory later takes it from them (with_room). Checked builds use small
+// limits, so that both forms run on small systems.
 #ifdef DMTS_CHECK
 constexpr size_t kFilterBytes = (size_t)64 << 20, kFilterChunkBytes = (size_t)16 << 20;
 #else
@@ -364,8 +372,11 @@ cudaError_t alloc_filters(dmts_ctx* c, Model& m) {
     PairFilter& f = m.filt;
     const size_t row = 2 * sizeof(float) * m.F;               // w and dw/dd of one layer
     const long long half = m.e_cap / 2 + 1;
-    cudaError_t e;
-    if (half * row * m.L <= kFilterBytes) {
+    size_t free_bytes = 0, total_bytes = 0;
+    cudaError_t e = cudaMemGetInfo(&free_bytes, &total_bytes);
+    if (e != cudaSuccess) return e;
+    if (half * (row * m.L + sizeof(float) + sizeof(int2)) + m.e_cap * sizeof(int) <=
+        std::min(kFilterBytes, free_bytes / 2)) {
         e = dalloc(&f.w, half * (row / sizeof(float)) * m.L);
         if (e == cudaSuccess) e = dalloc(&f.se, (size_t)half);
         if (e == cudaSuccess) e = dalloc(&f.pairs, (size_t)half);
@@ -375,20 +386,42 @@ cudaError_t alloc_filters(dmts_ctx* c, Model& m) {
         f.cap = half;
         if (e == cudaSuccess) return e;
         cudaGetLastError();
-        dfree(f.w); dfree(f.se); dfree(f.pairs); dfree(f.pid); dfree(f.count);
-        f = PairFilter{};
+        free_filters(m);
     }
-    long long atoms = std::max<long long>(1, (long long)(kFilterChunkBytes / row) / m.row_cap);
+    const size_t chunk = std::min(kFilterChunkBytes, free_bytes / 2);
+    long long atoms = std::max<long long>(1, (long long)(chunk / row) / m.row_cap);
     for (;; atoms /= 2) {
         f.chunk_atoms = (int)atoms;
         f.cap = atoms * m.row_cap;
         e = dalloc(&f.w, f.cap * (row / sizeof(float)));
         if (e == cudaSuccess) e = dalloc(&f.se, (size_t)f.cap);
-        if (e == cudaSuccess || atoms == 1) return e;
+        if (e == cudaSuccess) return e;
         cudaGetLastError();
-        dfree(f.w);
-        f.w = nullptr;
+        free_filters(m);
+        if (atoms == 1) return e;
     }
+}
+
+// Filter rows of the models that have none (at creation, or given up in with_room).
+cudaError_t ensure_filters(dmts_ctx* c) {
+    for (Model& m : c->m)
+        if (m.present && m.precision == DMTS_FP32 && !m.filt.w)
+            if (cudaError_t e = alloc_filters(c, m)) return e;
+    return cudaSuccess;
+}
+
+// An allocation that may take the memory of the filter rows: if it fails, they
+// are freed and it is tried again (ensure_filters then allocates what there is
+// room for). The caller drops the step graph, which holds their addresses.
+template <class Alloc>
+cudaError_t with_room(dmts_ctx* c, Alloc alloc) {
+    cudaError_t e = alloc();
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    for (Model& m : c->m) free_filters(m);
+    e = alloc();
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    return e;
 }
 
 cudaError_t alloc_model_nbr(dmts_ctx* c, Model& m) {
@@ -399,7 +432,6 @@ cudaError_t alloc_model_nbr(dmts_ctx* c, Model& m) {
     if (c->skin > 0 && (e = dalloc(&m.vl_rows, (size_t)c->N * m.vl_cap)) != cudaSuccess) return e;
     const size_t tiles = (size_t)((m.e_cap + 127) / 128);
     if ((e = dalloc(&m.carry, tiles * 2 * (size_t)(m.F + 16))) != cudaSuccess) return e;
-    if (m.precision == DMTS_FP32 && (e = alloc_filters(c, m)) != cudaSuccess) return e;
     return cudaSuccess;
 }
 
@@ -985,6 +1017,11 @@ int sync_check(dmts_ctx* c) {
 
 // Grow neighbour capacities from the maxima seen on the device.
 int grow_capacity(dmts_ctx* c) {
+    // buffers are missing then: no later call may use the context
+    auto out_of_memory = [c](const char* what, cudaError_t e) {
+        c->broken = true;
+        return fail(DMTS_ERR_OOM, "growing %s: %s", what, cudaGetErrorString(e));
+    };
     for (int w = 0; w < 2; ++w) {
         Model& m = c->m[w];
         if (!m.present) continue;
@@ -1001,18 +1038,21 @@ int grow_capacity(dmts_ctx* c) {
             CUDA_TRY(cudaStreamSynchronize(c->stream));
             dfree(m.cell_q);
             m.cell_q = nullptr;
-            cudaError_t e = dalloc(&m.cell_q, (size_t)m.n_cells * m.ccap);
-            if (e != cudaSuccess) return fail(DMTS_ERR_OOM, "growing cell capacity: %s", cudaGetErrorString(e));
+            cudaError_t e = with_room(c, [&] { return dalloc(&m.cell_q, (size_t)m.n_cells * m.ccap); });
+            if (e != cudaSuccess) return out_of_memory("cell capacity", e);
         }
         if (grow) {
             if (m.row_cap > 6000 || m.vl_cap > 6000)
                 return fail(DMTS_ERR_CAPACITY, "neighbour row capacity %d too large", std::max(m.row_cap, m.vl_cap));
             CUDA_TRY(cudaStreamSynchronize(c->stream));
-            free_model_nbr(m);
-            cudaError_t e = alloc_model_nbr(c, m);
-            if (e != cudaSuccess) return fail(DMTS_ERR_OOM, "growing neighbour capacity: %s", cudaGetErrorString(e));
+            cudaError_t e = with_room(c, [&] {
+                free_model_nbr(m);
+                return alloc_model_nbr(c, m);
+            });
+            if (e != cudaSuccess) return out_of_memory("neighbour capacity", e);
         }
     }
+    if (cudaError_t e = ensure_filters(c)) return out_of_memory("filter rows", e);
     if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
     return force_rebuild(c);                // rows reallocated, or truncated by the overflow
 }
@@ -1296,6 +1336,11 @@ ModelOffsets model_offsets(int S, int F, int K, int L) {
 }  // namespace dmts
 
 namespace {
+void free_batch(dmts_ctx* c) {
+    dmts_destroy(c->batch);
+    c->batch = nullptr;
+}
+
 void free_fm(dmts_ctx* c) {
     FmBuffers& b = c->fm;
     dfree(b.g); dfree(b.mdot); dfree(b.mbar_psi); dfree(b.mdotbar_psi); dfree(b.ubar); dfree(b.partial_e);
@@ -1329,7 +1374,7 @@ void dmts_destroy(dmts_ctx* c) {
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     free_fm(c);
     dfree(c->fm_eref); dfree(c->fm_ce);
-    dmts_destroy(c->batch);
+    free_batch(c);
     if (c->h_flags) cudaFreeHost(c->h_flags);
     if (c->stream && c->own_stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -1425,6 +1470,7 @@ int create_context(const dmts_model_desc* small, const dmts_model_desc* big, con
     do {                                                                          \
         cudaError_t e_ = (expr);                                                  \
         if (e_ != cudaSuccess) {                                                  \
+            cudaGetLastError();                                                   \
             int code_ = e_ == cudaErrorMemoryAllocation ? DMTS_ERR_OOM : DMTS_ERR_CUDA; \
             fail(code_, "%s: %s", #expr, cudaGetErrorString(e_));                 \
             std::string keep_ = g_err;                                            \
@@ -1532,6 +1578,7 @@ int create_context(const dmts_model_desc* small, const dmts_model_desc* big, con
         c->m[w].apc_fwd = std::max(8, c->m[w].apc_fwd);
         c->m[w].apc_bwd = std::max(8, c->m[w].apc_bwd);
     }
+    CREATE_TRY(ensure_filters(c));
     for (int w = 0; w < 2; ++w) {
         if ((rc = prepare_embedding(c, c->m[w]))) { std::string k = g_err; dmts_destroy(c); g_err = k; return rc; }
     }
@@ -1692,7 +1739,11 @@ int dmts_respa_step(dmts_ctx* c, int n_outer, double dt, int n_inner, double* en
         c->d_ring = nullptr;
         c->ring_len = 0;
         if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
-        cudaError_t e = dalloc(&c->d_ring, (size_t)n_outer * c->n_sys * 3);
+        cudaError_t e = with_room(c, [&] { return dalloc(&c->d_ring, (size_t)n_outer * c->n_sys * 3); });
+        if (cudaError_t ef = ensure_filters(c)) {
+            c->broken = true;
+            return fail(DMTS_ERR_OOM, "filter rows: %s", cudaGetErrorString(ef));
+        }
         if (e != cudaSuccess) return fail(DMTS_ERR_OOM, "energies ring: %s", cudaGetErrorString(e));
         c->ring_len = n_outer;
     }
@@ -1773,10 +1824,7 @@ constexpr int kFmBatchAtoms = 131072;
 // the caller queues there next. Returns null if it cannot be created (no
 // memory): one frame at a time then.
 dmts_ctx* batch_context(dmts_ctx* c, int frames) {
-    if (c->batch && c->batch_frames < frames) {
-        dmts_destroy(c->batch);
-        c->batch = nullptr;
-    }
+    if (c->batch && c->batch_frames < frames) free_batch(c);
     const Model& m = c->m[0];
     if (!c->batch) {
         std::vector<int> off(1, 0), sp((size_t)c->N), spb;
@@ -1831,35 +1879,30 @@ int alloc_fm(dmts_ctx* c, int atoms) {
 }
 
 // Distillation loss of the small model over n_frames frames and its
-// parameter gradient (e_ref null: force matching alone). The frames run in
-// batches of equal size, each batch as independent systems through one set of
-// launches, with no host synchronisation between batches; a neighbour
-// overflow in any frame grows the capacities and redoes the call.
-int distill_impl(dmts_ctx* c, int n_frames, const double* frames, const double* f_ref, const double* e_ref,
-                 double lambda_e, double* loss_out, double* grad_out) {
-    CTX_GUARD(c);
-    Range nvtx_range("dmts_distill_grad");
+// parameter gradient (e_ref null: force matching alone), per frames at a time:
+// the frames run in batches of equal size, each batch as independent systems
+// through one set of launches, with no host synchronisation between batches; a
+// neighbour overflow in any frame grows the capacities and redoes the call.
+int distill_frames(dmts_ctx* c, int per, int n_frames, const double* frames, const double* f_ref, const double* e_ref,
+                   double lambda_e, double* loss_out, double* grad_out) {
     Model& m0 = c->m[0];
-    if (!m0.present) return fail(DMTS_ERR_ARG, "no small model in this context");
-    if (!fm_supported(m0.F, m0.K, m0.L))
-        return fail(DMTS_ERR_ARG, "distillation needs a single-layer small model with n_feat 32, n_radial 8 or 16");
-    if (n_frames < 1 || !frames || !f_ref || !loss_out || !grad_out) return fail(DMTS_ERR_ARG, "bad arguments");
-    if (e_ref && !(lambda_e >= 0.0 && isfinite(lambda_e))) return fail(DMTS_ERR_ARG, "lambda_e must be >= 0");
     const int N = c->N;
     const size_t n3 = (size_t)3 * N;
     const int np = (int)m0.n_params;
     int rc;
-    // frames per batch: the number of batches that the target size asks for, evenly
-    const int most = (int)std::max<long long>(1, std::min<long long>(n_frames, kFmBatchAtoms / std::max(1, N)));
-    const int n_batches = (n_frames + most - 1) / most;
-    int per = (n_frames + n_batches - 1) / n_batches;
-    dmts_ctx* w = per > 1 ? batch_context(c, per) : nullptr;      // the context that evaluates the frames
-    if (w && alloc_fm(c, per * N) != DMTS_OK) w = nullptr;
-    if (!w) {
-        per = 1;
-        cudaGetLastError();
-        if ((rc = alloc_fm(c, N))) return rc;
-        w = c;
+    dmts_ctx* w = c;                                              // the context that evaluates the frames
+    if (per > 1) {
+        if (!(w = batch_context(c, per))) return DMTS_ERR_OOM;
+        if ((rc = alloc_fm(c, per * N))) return rc;
+    } else if ((rc = alloc_fm(c, N))) {
+        for (Model& m : c->m) free_filters(m);                    // (as with_room)
+        if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
+        rc = alloc_fm(c, N);
+        if (cudaError_t e = ensure_filters(c)) {
+            c->broken = true;
+            return fail(DMTS_ERR_OOM, "filter rows: %s", cudaGetErrorString(e));
+        }
+        if (rc) return rc;
     }
     const bool own = w == c;
     const int which = own ? 0 : 1;
@@ -1949,7 +1992,7 @@ int distill_impl(dmts_ctx* c, int n_frames, const double* frames, const double* 
     };
     for (int attempt = 0;; ++attempt) {
         if ((rc = batches())) {
-            c->broken = c->broken || w->broken;
+            c->broken = c->broken || w->broken;            // (a CUDA error: both contexts')
             return rc;
         }
         if (!w->h_flags[kFlagOverflow]) break;
@@ -1969,6 +2012,29 @@ int distill_impl(dmts_ctx* c, int n_frames, const double* frames, const double* 
     if ((rc = copy_out(w, grad_out, c->fm.grad, np))) return rc;
     if ((rc = copy_out(w, loss_out, c->fm.loss, 1))) return rc;
     return sync_check(w);
+}
+
+int distill_impl(dmts_ctx* c, int n_frames, const double* frames, const double* f_ref, const double* e_ref,
+                 double lambda_e, double* loss_out, double* grad_out) {
+    CTX_GUARD(c);
+    Range nvtx_range("dmts_distill_grad");
+    const Model& m = c->m[0];
+    if (!m.present) return fail(DMTS_ERR_ARG, "no small model in this context");
+    if (!fm_supported(m.F, m.K, m.L))
+        return fail(DMTS_ERR_ARG, "distillation needs a single-layer small model with n_feat 32, n_radial 8 or 16");
+    if (n_frames < 1 || !frames || !f_ref || !loss_out || !grad_out) return fail(DMTS_ERR_ARG, "bad arguments");
+    if (e_ref && !(lambda_e >= 0.0 && isfinite(lambda_e))) return fail(DMTS_ERR_ARG, "lambda_e must be >= 0");
+    // frames per batch: the number of batches that the target size asks for, evenly
+    const int most = (int)std::max<long long>(1, std::min<long long>(n_frames, kFmBatchAtoms / std::max(1, c->N)));
+    const int n_batches = (n_frames + most - 1) / most;
+    const int per = (n_frames + n_batches - 1) / n_batches;
+    int rc = distill_frames(c, per, n_frames, frames, f_ref, e_ref, lambda_e, loss_out, grad_out);
+    if (rc == DMTS_ERR_OOM && per > 1) {       // no memory for batches: given back, and one frame at a time
+        free_batch(c);
+        free_fm(c);
+        rc = distill_frames(c, 1, n_frames, frames, f_ref, e_ref, lambda_e, loss_out, grad_out);
+    }
+    return rc;
 }
 
 }  // namespace
