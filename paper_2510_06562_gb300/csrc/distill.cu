@@ -76,6 +76,28 @@ __device__ __forceinline__ void basis_pair(float d, float pi_over_rc, float pref
     dfc = -0.5f * pi_over_rc * s1;
 }
 
+// ------------------------------------------------------------ systems of a batch
+// blockIdx.x: the copy; its atoms and systems follow those of the copies before.
+__global__ void __launch_bounds__(256) k_fm_replicate(int n_atoms, int n_sys, const int* __restrict__ off,
+                                                      const int* __restrict__ species, const int* __restrict__ first_of,
+                                                      const int* __restrict__ sys, const double* __restrict__ box,
+                                                      int* __restrict__ off_out, int* __restrict__ species_out,
+                                                      int* __restrict__ first_of_out, int* __restrict__ sys_out,
+                                                      double* __restrict__ box_out) {
+    const int i = blockIdx.y * 256 + threadIdx.x, f = blockIdx.x;
+    if (i < n_atoms) {
+        const int o = f * n_atoms + i;
+        species_out[o] = species[i];
+        first_of_out[o] = first_of[i];
+        sys_out[o] = f * n_sys + sys[i];
+    }
+    if (i < n_sys) {
+        box_out[f * n_sys + i] = box[i];
+        off_out[f * n_sys + i + 1] = f * n_atoms + off[i + 1];
+    }
+    if (i == 0 && f == 0) off_out[0] = 0;
+}
+
 // ------------------------------------------------------------ residual g
 // g_i = c (F_i - F_ref,i) (SoA), c = 2 / (3 N M), and the force term of the
 // loss, c/2 sum |F_i - F_ref,i|^2 (FP64): every block leaves its sum in part,
@@ -1526,6 +1548,15 @@ int fm_edge_ctas(int n_atoms) {
 int fm_edge_rows(int n_atoms) {
     const int sms = device_sms();
     return sms * std::max(1, (n_atoms + kFmAtomsMax * sms - 1) / (kFmAtomsMax * sms));
+}
+
+void launch_fm_replicate(int frames, int n_atoms, int n_sys, const int* off, const int* species, const int* first_of,
+                         const int* sys, const double* box, int* off_out, int* species_out, int* first_of_out,
+                         int* sys_out, double* box_out, cudaStream_t s) {
+    const int n = std::max(n_atoms, n_sys);
+    k_fm_replicate<<<dim3(frames, (n + 255) / 256), 256, 0, s>>>(n_atoms, n_sys, off, species, first_of, sys, box, off_out,
+                                                                 species_out, first_of_out, sys_out, box_out);
+    count_launch();
 }
 
 int fm_residual_blocks(int n_atoms) { return (n_atoms + kResT - 1) / kResT; }

@@ -153,6 +153,7 @@ int parse_options(const char* js, Options& out) {
 }
 
 struct Model {
+    unsigned char* slab = nullptr;     // every buffer but the neighbour arrays, the filter rows and cell_q
     bool present = false;
     int F = 0, K = 0, L = 0, S = 0, precision = 0;
     double rc = 0;
@@ -202,7 +203,8 @@ struct Model {
 struct dmts_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
-    bool own_stream = true;                // the inner context of distillation batches runs on its outer one's
+    bool inner = false;                    // of distillation batches: stream and h_flags are the outer context's
+    unsigned char* slab = nullptr;         // every buffer of the context but d_ring and the distillation's
     int N = 0, n_sys = 0, max_sys = 0;     // atoms, systems, atoms of the largest system
     bool periodic = false;
     std::vector<int> h_off;
@@ -263,6 +265,7 @@ struct dmts_ctx {
     int batch_frames = 0;                  // frames the inner context holds
     long long batch_params = -1;           // m[0].version its weights were taken from
     FmBuffers fm{};
+    unsigned char* fm_slab = nullptr;      // the buffers of fm, and fm_stage
     int fm_atoms = 0;                      // atoms the buffers hold
     double *fm_stage = nullptr, *fm_eref = nullptr, *fm_ce = nullptr;   // frames and forces; energies, dL/dE
     int fm_eref_cap = 0;
@@ -320,6 +323,33 @@ cudaError_t dalloc(T** p, size_t n) {
 void dfree(void* p) {
     if (p) cudaFree(p);
 }
+
+// Buffers that live as long as their owner, from one allocation: each
+// cudaMalloc costs the host 5 to 60 us, and a context has some fifty.
+class Slab {
+public:
+    template <class T>
+    void add(T** p, size_t n) {
+        *p = nullptr;
+        want_.push_back({reinterpret_cast<void**>(p), (std::max<size_t>(n, 1) * sizeof(T) + 255) / 256 * 256});
+    }
+    cudaError_t commit(unsigned char** base) {
+        size_t total = 0;
+        for (const auto& w : want_) total += w.second;
+        cudaError_t e = dalloc(base, total);
+        if (e != cudaSuccess) return e;
+        unsigned char* q = *base;
+        for (const auto& w : want_) {
+            memcpy(w.first, &q, sizeof q);
+            q += w.second;
+        }
+        want_.clear();
+        return e;
+    }
+
+private:
+    std::vector<std::pair<void**, size_t>> want_;
+};
 
 int check_model(const dmts_model_desc* d, const char* name) {
     if (!d) return fail(DMTS_ERR_ARG, "%s model descriptor is NULL", name);
@@ -436,17 +466,9 @@ cudaError_t alloc_model_nbr(dmts_ctx* c, Model& m) {
 }
 
 void free_model(Model& m) {
-    dfree(m.P);
-    dfree(m.cell_count); dfree(m.cell_start); dfree(m.atom_cell); dfree(m.atom_slot);
-    dfree(m.cell_q);
     free_model_nbr(m);
-    dfree(m.nbr_cnt); dfree(m.row_ptr); dfree(m.vl_cnt);
-    dfree(m.block_sum); dfree(m.chunk_sum); dfree(m.ticket);
-    dfree(m.h); dfree(m.gh); dfree(m.force); dfree(m.vir6); dfree(m.h0); dfree(m.PT);
-    for (int l = 0; l < kMaxLayers; ++l) { dfree(m.u[l]); dfree(m.z[l]); dfree(m.um[l]); }
-    dfree(m.mbar[0]); dfree(m.mbar[1]); dfree(m.esum.part); dfree(m.esum.ctr);
-    dfree(m.Ei); dfree(m.E); dfree(m.W); dfree(m.erep); dfree(m.msg); dfree(m.spec_row); dfree(m.spec_sum);
-    dfree(m.u_spec); dfree(m.wt); dfree(m.at);
+    dfree(m.cell_q);
+    dfree(m.slab);
     m = Model();
 }
 
@@ -560,7 +582,19 @@ int upload_params(dmts_ctx* c, Model& m, const double* params) {
     return DMTS_OK;
 }
 
-int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells) {
+// The weights of another context's model of the same shape, on the same device.
+int copy_weights(dmts_ctx* c, Model& m, const Model& from) {
+    CUDA_TRY(cudaMemcpyAsync(m.P, from.P, sizeof(float) * m.n_params, cudaMemcpyDeviceToDevice, c->stream));
+    CUDA_TRY(cudaMemcpyAsync(m.wt, from.wt, m.wt_layer_bytes * m.L, cudaMemcpyDeviceToDevice, c->stream));
+    CUDA_TRY(cudaMemcpyAsync(m.PT, from.PT, sizeof(float) * (3 * m.L + 2) * m.F * m.F, cudaMemcpyDeviceToDevice,
+                             c->stream));
+    CUDA_TRY(cudaMemcpyAsync(m.at, from.at, atom_tile_bytes(m.F, m.L), cudaMemcpyDeviceToDevice, c->stream));
+    return DMTS_OK;
+}
+
+// One model's buffers for c's systems, and its weights: uploaded from d, or
+// copied on the device from another context's model of the same shape.
+int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells, const Model* from = nullptr) {
     m.present = true;
     m.F = d->n_feat; m.K = d->n_radial; m.L = d->n_layers; m.S = d->n_species;
     m.precision = d->precision;
@@ -571,13 +605,7 @@ int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells) {
     m.n_params = d->n_params;
     m.off = model_offsets(m.S, m.F, m.K, m.L);
     const int N = c->N;
-    CUDA_TRY(dalloc(&m.P, m.n_params));
     m.wt_layer_bytes = bf16_weight_tile_bytes(m.F);
-    CUDA_TRY(dalloc(&m.wt, m.wt_layer_bytes * m.L));
-    CUDA_TRY(dalloc(&m.PT, (3 * (size_t)m.L + 2) * m.F * m.F));
-    CUDA_TRY(dalloc(&m.at, atom_tile_bytes(m.F, m.L)));
-    int rc = upload_params(c, m, d->params);
-    if (rc) return rc;
     // cells (periodic) and capacity estimates; with a skin the cells and the
     // candidate rows use rc + skin
     double expected;
@@ -605,59 +633,67 @@ int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells) {
         m.vl_cap = m.row_cap;
         m.e_cap = std::max<long long>(1024, std::min<long long>(sq, (long long)(N * std::min(mx, 64) * c->cap_factor)) + 1024);
     }
+    Slab slab;
+    slab.add(&m.P, m.n_params);
+    slab.add(&m.wt, m.wt_layer_bytes * m.L);
+    slab.add(&m.PT, (3 * (size_t)m.L + 2) * m.F * m.F);
+    slab.add(&m.at, atom_tile_bytes(m.F, m.L));
     if (m.nc > 0) {
         m.n_cells = c->n_sys * m.nc * m.nc * m.nc;            // each system its own cells
-        CUDA_TRY(dalloc(&m.cell_count, m.n_cells));
-        CUDA_TRY(cudaMemsetAsync(m.cell_count, 0, sizeof(int) * m.n_cells, c->stream));
+        slab.add(&m.cell_count, m.n_cells);
         if (c->skin > 0) {                 // compact cells rebuilt by count, scan and fill
-            CUDA_TRY(dalloc(&m.cell_start, m.n_cells + 1));
-            CUDA_TRY(dalloc(&m.atom_cell, N));
-            CUDA_TRY(dalloc(&m.atom_slot, N));
-            CUDA_TRY(dalloc(&m.cell_q, N));
+            slab.add(&m.cell_start, m.n_cells + 1);
+            slab.add(&m.atom_cell, N);
+            slab.add(&m.atom_slot, N);
         } else {                           // fixed-capacity cells: twice the mean occupancy plus 16, grown on overflow
             m.ccap = ((int)(2.0 * N / m.n_cells) + 16 + 7) / 8 * 8;
-            CUDA_TRY(dalloc(&m.cell_q, (size_t)m.n_cells * m.ccap));
         }
     }
-    CUDA_TRY(alloc_model_nbr(c, m));
-    CUDA_TRY(dalloc(&m.nbr_cnt, N));
-    CUDA_TRY(dalloc(&m.vl_cnt, N));
-    {   // folded row scan: a pair count per build block of 8 atoms and per chunk of 32 blocks
-        const size_t nb = (size_t)(N + 7) / 8, nch = (nb + 31) / 32 + 1;
-        CUDA_TRY(dalloc(&m.block_sum, nb));
-        CUDA_TRY(dalloc(&m.chunk_sum, nch));
-        CUDA_TRY(dalloc(&m.ticket, 1));
-        CUDA_TRY(cudaMemsetAsync(m.chunk_sum, 0, sizeof(int) * nch, c->stream));
-        CUDA_TRY(cudaMemsetAsync(m.ticket, 0, sizeof(unsigned int), c->stream));
-    }
-    CUDA_TRY(dalloc(&m.row_ptr, N + 1));
-    size_t nf = (size_t)N * m.F;
-    CUDA_TRY(dalloc(&m.h, nf));
-    CUDA_TRY(dalloc(&m.h0, nf));
-    CUDA_TRY(dalloc(&m.gh, nf));
+    slab.add(&m.nbr_cnt, N);
+    slab.add(&m.vl_cnt, N);
+    // folded row scan: a pair count per build block of 8 atoms and per chunk of 32 blocks
+    const size_t nb = (size_t)(N + 7) / 8, nch = (nb + 31) / 32 + 1;
+    slab.add(&m.block_sum, nb);
+    slab.add(&m.chunk_sum, nch);
+    slab.add(&m.ticket, 1);
+    slab.add(&m.row_ptr, N + 1);
+    const size_t nf = (size_t)N * m.F;
+    slab.add(&m.h, nf);
+    slab.add(&m.h0, nf);
+    slab.add(&m.gh, nf);
     for (int l = 0; l < m.L; ++l) {
-        CUDA_TRY(dalloc(&m.u[l], nf));
-        CUDA_TRY(dalloc(&m.z[l], nf));
-        CUDA_TRY(dalloc(&m.um[l], nf * 4));
+        slab.add(&m.u[l], nf);
+        slab.add(&m.z[l], nf);
+        slab.add(&m.um[l], nf * 4);
     }
-    CUDA_TRY(dalloc(&m.mbar[0], nf));
-    CUDA_TRY(dalloc(&m.mbar[1], nf));
-    CUDA_TRY(dalloc(&m.msg, nf));
-    CUDA_TRY(dalloc(&m.u_spec, (size_t)2 * m.S * m.F));       // u^0 and h^0 of each species
+    slab.add(&m.mbar[0], nf);
+    slab.add(&m.mbar[1], nf);
+    slab.add(&m.msg, nf);
+    slab.add(&m.u_spec, (size_t)2 * m.S * m.F);               // u^0 and h^0 of each species
     if (m.precision == DMTS_FP32 && m.S <= kMaxFactorSpecies && m.L > 1 && c->periodic && N >= kMinFactorAtoms) {
-        CUDA_TRY(dalloc(&m.spec_row, nf * m.S));
-        CUDA_TRY(dalloc(&m.spec_sum, (size_t)N * m.S));
+        slab.add(&m.spec_row, nf * m.S);
+        slab.add(&m.spec_sum, (size_t)N * m.S);
     }
-    CUDA_TRY(dalloc(&m.force, (size_t)3 * N));
+    slab.add(&m.force, (size_t)3 * N);
+    slab.add(&m.vir6, (size_t)6 * N);
+    slab.add(&m.Ei, N);
+    slab.add(&m.erep, N);
+    slab.add(&m.E, c->n_sys);
+    slab.add(&m.esum.part, (size_t)kSumMaxSplit * kSumChunks * 6);
+    slab.add(&m.esum.ctr, kSumMaxSplit);
+    slab.add(&m.W, (size_t)9 * c->n_sys);
+    CUDA_TRY(slab.commit(&m.slab));
+    CUDA_TRY(alloc_model_nbr(c, m));
+    if (m.nc > 0) {
+        CUDA_TRY(dalloc(&m.cell_q, m.ccap > 0 ? (size_t)m.n_cells * m.ccap : (size_t)N));
+        CUDA_TRY(cudaMemsetAsync(m.cell_count, 0, sizeof(int) * m.n_cells, c->stream));
+    }
+    CUDA_TRY(cudaMemsetAsync(m.chunk_sum, 0, sizeof(int) * nch, c->stream));
+    CUDA_TRY(cudaMemsetAsync(m.ticket, 0, sizeof(unsigned int), c->stream));
     CUDA_TRY(cudaMemsetAsync(m.force, 0, sizeof(float) * 3 * std::max(N, 1), c->stream));
-    CUDA_TRY(dalloc(&m.vir6, (size_t)6 * N));
-    CUDA_TRY(dalloc(&m.Ei, N));
-    CUDA_TRY(dalloc(&m.erep, N));
-    CUDA_TRY(dalloc(&m.E, c->n_sys));
-    CUDA_TRY(dalloc(&m.esum.part, (size_t)kSumMaxSplit * kSumChunks * 6));
-    CUDA_TRY(dalloc(&m.esum.ctr, kSumMaxSplit));
     CUDA_TRY(cudaMemsetAsync(m.esum.ctr, 0, sizeof(unsigned int) * kSumMaxSplit, c->stream));
-    CUDA_TRY(dalloc(&m.W, (size_t)9 * c->n_sys));
+    const int rc = from ? copy_weights(c, m, *from) : upload_params(c, m, d->params);
+    if (rc) return rc;
     // FP32: atoms per CTA of the gathers (eight warps, one atom each at a time)
     m.apc_fwd = m.apc_bwd = 8;
     return DMTS_OK;
@@ -1342,10 +1378,9 @@ void free_batch(dmts_ctx* c) {
 }
 
 void free_fm(dmts_ctx* c) {
-    FmBuffers& b = c->fm;
-    dfree(b.g); dfree(b.mdot); dfree(b.mbar_psi); dfree(b.mdotbar_psi); dfree(b.ubar); dfree(b.partial_e);
-    dfree(b.partial_a); dfree(b.part); dfree(b.ticket); dfree(b.grad); dfree(b.loss); dfree(c->fm_stage);
-    b = FmBuffers{};
+    dfree(c->fm_slab);
+    c->fm_slab = nullptr;
+    c->fm = FmBuffers{};
     c->fm_stage = nullptr;
     c->fm_atoms = 0;
 }
@@ -1362,12 +1397,8 @@ void dmts_destroy(dmts_ctx* c) {
     if (c->graph) cudaGraphExecDestroy(c->graph);
     free_model(c->m[0]);
     free_model(c->m[1]);
-    dfree(c->d_off); dfree(c->d_species); dfree(c->d_first_of); dfree(c->d_sys); dfree(c->d_box); dfree(c->d_mass);
-    dfree(c->d_inv_m); dfree(c->d_x); dfree(c->d_v); dfree(c->d_q); dfree(c->d_frame); dfree(c->d_stage);
-    dfree(c->d_ke); dfree(c->d_ekin); dfree(c->d_ring); dfree(c->d_flags); dfree(c->d_epart); dfree(c->d_eticket);
-    dfree(c->d_bx); dfree(c->d_bv);
-    dfree(c->d_xref); dfree(c->d_vl); dfree(c->d_rng); dfree(c->kesum.part); dfree(c->kesum.ctr);
-    dfree(c->d_mon); dfree(c->d_sx); dfree(c->d_sv); dfree(c->d_sf);
+    dfree(c->slab);
+    dfree(c->d_ring);
     if (c->aux) cudaStreamDestroy(c->aux);
     if (c->s_big) cudaStreamDestroy(c->s_big);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
@@ -1375,21 +1406,19 @@ void dmts_destroy(dmts_ctx* c) {
     free_fm(c);
     dfree(c->fm_eref); dfree(c->fm_ce);
     free_batch(c);
-    if (c->h_flags) cudaFreeHost(c->h_flags);
-    if (c->stream && c->own_stream) cudaStreamDestroy(c->stream);
+    if (!c->inner) {
+        if (c->h_flags) cudaFreeHost(c->h_flags);
+        if (c->stream) cudaStreamDestroy(c->stream);
+    }
     delete c;
 }
 
-}  // extern "C"
-
-namespace {
-
-// dmts_create, on a stream of its own (stream null) or on the caller's, which
-// has to outlive the context. Uploads and clears go to that stream, as those
-// of buffers allocated later do: the streams are non-blocking, so nothing would
-// order a clear on the default stream before the kernels that read the buffer.
-int create_context(const dmts_model_desc* small, const dmts_model_desc* big, const dmts_system_desc* sys,
-                   const char* options, cudaStream_t stream, dmts_ctx** out) {
+// Uploads and clears go to the context's stream, as those of buffers allocated
+// later do: the stream is non-blocking, so nothing would order a clear on the
+// default stream before the kernels that read the buffer.
+int dmts_create(const dmts_model_desc* small, const dmts_model_desc* big, const dmts_system_desc* sys,
+                const char* options, dmts_ctx** out) {
+    Range nvtx_range("dmts_create");
     g_err.clear();
     if (!out) return fail(DMTS_ERR_ARG, "out is NULL");
     *out = nullptr;
@@ -1479,9 +1508,7 @@ int create_context(const dmts_model_desc* small, const dmts_model_desc* big, con
             return code_;                                                         \
         }                                                                         \
     } while (0)
-    c->own_stream = !stream;
-    c->stream = stream;
-    if (!stream) CREATE_TRY(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
+    CREATE_TRY(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
     std::vector<int> sys_of(N);
     for (int s = 0; s < ns; ++s)
         for (int i = sys->atom_offset[s]; i < sys->atom_offset[s + 1]; ++i) sys_of[i] = s;
@@ -1494,48 +1521,52 @@ int create_context(const dmts_model_desc* small, const dmts_model_desc* big, con
     }
     std::vector<double> inv_m(N);
     for (int i = 0; i < N; ++i) inv_m[i] = 1.0 / sys->mass[i];
-    CREATE_TRY(dalloc(&c->d_off, ns + 1));
-    CREATE_TRY(dalloc(&c->d_species, N));
-    CREATE_TRY(dalloc(&c->d_first_of, N));
-    CREATE_TRY(dalloc(&c->d_sys, N));
-    CREATE_TRY(dalloc(&c->d_box, ns));
-    CREATE_TRY(dalloc(&c->d_mass, N));
-    CREATE_TRY(dalloc(&c->d_inv_m, N));
-    CREATE_TRY(dalloc(&c->d_x, (size_t)3 * N));
-    CREATE_TRY(dalloc(&c->d_v, (size_t)3 * N));
-    CREATE_TRY(dalloc(&c->d_q, N));
-    CREATE_TRY(dalloc(&c->d_frame, ns));
-    CREATE_TRY(dalloc(&c->d_stage, (size_t)6 * N));
-    CREATE_TRY(dalloc(&c->d_ke, N));
-    CREATE_TRY(dalloc(&c->d_ekin, ns));
-    CREATE_TRY(dalloc(&c->d_epart, (size_t)2 * std::max(1, integrator_blocks(N))));
-    CREATE_TRY(dalloc(&c->d_eticket, 1));
+    Slab slab;
+    slab.add(&c->d_off, ns + 1);
+    slab.add(&c->d_species, N);
+    slab.add(&c->d_first_of, N);
+    slab.add(&c->d_sys, N);
+    slab.add(&c->d_box, ns);
+    slab.add(&c->d_mass, N);
+    slab.add(&c->d_inv_m, N);
+    slab.add(&c->d_x, (size_t)3 * N);
+    slab.add(&c->d_v, (size_t)3 * N);
+    slab.add(&c->d_q, N);
+    slab.add(&c->d_frame, ns);
+    slab.add(&c->d_stage, (size_t)6 * N);
+    slab.add(&c->d_ke, N);
+    slab.add(&c->d_ekin, ns);
+    slab.add(&c->d_epart, (size_t)2 * std::max(1, integrator_blocks(N)));
+    slab.add(&c->d_eticket, 1);
+    slab.add(&c->d_flags, kFlagCount);
+    slab.add(&c->d_bx, (size_t)3 * N);
+    slab.add(&c->d_bv, (size_t)3 * N);
+    slab.add(&c->kesum.part, (size_t)kSumMaxSplit * kSumChunks);
+    slab.add(&c->kesum.ctr, kSumMaxSplit);
+    slab.add(&c->d_rng, 2);
+    slab.add(&c->d_mon, 1);
+    if (c->fb_threshold > 0.0) {
+        slab.add(&c->d_sx, (size_t)3 * N);
+        slab.add(&c->d_sv, (size_t)3 * N);
+        slab.add(&c->d_sf, (size_t)3 * N);
+    }
+    if (c->skin > 0) {
+        slab.add(&c->d_xref, (size_t)3 * N);
+        slab.add(&c->d_vl, 1);
+    }
+    CREATE_TRY(slab.commit(&c->slab));
     CREATE_TRY(cudaMemsetAsync(c->d_eticket, 0, sizeof(unsigned int), c->stream));
-    CREATE_TRY(dalloc(&c->d_flags, kFlagCount));
-    CREATE_TRY(dalloc(&c->d_bx, (size_t)3 * N));
-    CREATE_TRY(dalloc(&c->d_bv, (size_t)3 * N));
     CREATE_TRY(cudaMallocHost((void**)&c->h_flags, sizeof(int) * kFlagCount));
-    CREATE_TRY(dalloc(&c->kesum.part, (size_t)kSumMaxSplit * kSumChunks));
-    CREATE_TRY(dalloc(&c->kesum.ctr, kSumMaxSplit));
     CREATE_TRY(cudaMemsetAsync(c->kesum.ctr, 0, sizeof(unsigned int) * kSumMaxSplit, c->stream));
-    CREATE_TRY(dalloc(&c->d_rng, 2));
     CREATE_TRY(cudaMemsetAsync(c->d_rng, 0, 2 * sizeof(unsigned long long), c->stream));
     CREATE_TRY(cudaStreamCreateWithFlags(&c->s_big, cudaStreamNonBlocking));
     CREATE_TRY(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
     CREATE_TRY(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
     c->concurrent = opt.get("concurrent_models", 1.0) != 0.0;
     c->atom_tc = opt.get("atom_tensor_cores", 1.0) != 0.0;
-    CREATE_TRY(dalloc(&c->d_mon, 1));
     CREATE_TRY(cudaMemsetAsync(c->d_mon, 0, sizeof(ForceMonitor), c->stream));
-    if (c->fb_threshold > 0.0) {
-        CREATE_TRY(dalloc(&c->d_sx, (size_t)3 * N));
-        CREATE_TRY(dalloc(&c->d_sv, (size_t)3 * N));
-        CREATE_TRY(dalloc(&c->d_sf, (size_t)3 * N));
-        CREATE_TRY(cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking));
-    }
+    if (c->fb_threshold > 0.0) CREATE_TRY(cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking));
     if (c->skin > 0) {
-        CREATE_TRY(dalloc(&c->d_xref, (size_t)3 * N));
-        CREATE_TRY(dalloc(&c->d_vl, 1));
         CREATE_TRY(cudaMemsetAsync(c->d_vl, 0, sizeof(VerletState), c->stream));
         CREATE_TRY(cudaMemsetAsync(&c->d_vl->force, 1, sizeof(int), c->stream));
     }
@@ -1590,16 +1621,6 @@ int create_context(const dmts_model_desc* small, const dmts_model_desc* big, con
     CREATE_TRY(cudaStreamSynchronize(c->stream));
     *out = c;
     return DMTS_OK;
-}
-
-}  // namespace
-
-extern "C" {
-
-int dmts_create(const dmts_model_desc* small, const dmts_model_desc* big, const dmts_system_desc* sys,
-                const char* options, dmts_ctx** out) {
-    Range nvtx_range("dmts_create");
-    return create_context(small, big, sys, options, nullptr, out);
 }
 
 int dmts_set_state(dmts_ctx* c, const double* x, const double* v, int n_atoms) {
@@ -1819,37 +1840,73 @@ namespace {
 constexpr int kFmBatchAtoms = 131072;
 
 // The inner context that evaluates `frames` frames of c's systems at once:
-// the systems repeated, the small model alone, its weights copied from c's.
-// It runs on c's stream: behind what the caller queued there, and before what
-// the caller queues there next. Returns null if it cannot be created (no
-// memory): one frame at a time then.
-dmts_ctx* batch_context(dmts_ctx* c, int frames) {
-    if (c->batch && c->batch_frames < frames) free_batch(c);
+// the systems repeated, the small model alone as its m[1], with what a force
+// evaluation needs and no more: a call with several frames pays for it when it
+// is the first one. The systems and the weights are copied on the device. It
+// runs on c's stream: behind what the caller queued there, and before what the
+// caller queues there next. Fails without leaving one behind.
+int batch_context(dmts_ctx* c, int frames) {
+    if (c->batch && c->batch_frames >= frames) return DMTS_OK;
+    free_batch(c);
     const Model& m = c->m[0];
-    if (!c->batch) {
-        std::vector<int> off(1, 0), sp((size_t)c->N), spb;
-        std::vector<double> mass((size_t)frames * c->N, 1.0), box;
-        if (cudaMemcpyAsync(sp.data(), c->d_species, sizeof(int) * c->N, cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
-            cudaStreamSynchronize(c->stream) != cudaSuccess)
-            return nullptr;
-        for (int f = 0; f < frames; ++f) {
-            for (int k = 0; k < c->n_sys; ++k) off.push_back(f * c->N + c->h_off[k + 1]);
-            box.insert(box.end(), c->h_box.begin(), c->h_box.end());
-            spb.insert(spb.end(), sp.begin(), sp.end());
-        }
+    dmts_ctx* b = c->batch = new dmts_ctx();
+    b->inner = true;
+    b->device = c->device;
+    b->stream = c->stream;
+    b->h_flags = c->h_flags;
+    b->N = frames * c->N;
+    b->n_sys = frames * c->n_sys;
+    b->max_sys = c->max_sys;
+    b->periodic = c->periodic;
+    b->h_off.assign(1, 0);
+    for (int f = 0; f < frames; ++f) {
+        for (int k = 0; k < c->n_sys; ++k) b->h_off.push_back(f * c->N + c->h_off[k + 1]);
+        b->h_box.insert(b->h_box.end(), c->h_box.begin(), c->h_box.end());
+    }
+    b->rc_max = m.rc;
+    b->vl_src = 1;
+    b->atom_tc = c->atom_tc;
+    b->keep_msg = true;                        // the second-order passes read every message row
+    LaunchScope ls(c);
+    auto fill = [&]() -> int {
+        Slab slab;
+        slab.add(&b->d_off, b->n_sys + 1);
+        slab.add(&b->d_species, b->N);
+        slab.add(&b->d_first_of, b->N);
+        slab.add(&b->d_sys, b->N);
+        slab.add(&b->d_box, b->n_sys);
+        slab.add(&b->d_x, (size_t)3 * b->N);
+        slab.add(&b->d_v, (size_t)3 * b->N);
+        slab.add(&b->d_q, b->N);
+        slab.add(&b->d_frame, b->n_sys);
+        slab.add(&b->d_flags, kFlagCount);
+        CUDA_TRY(slab.commit(&b->slab));
+        CUDA_TRY(cudaMemsetAsync(b->d_flags, 0, sizeof(int) * kFlagCount, b->stream));
+        launch_fm_replicate(frames, c->N, c->n_sys, c->d_off, c->d_species, c->d_first_of, c->d_sys, c->d_box, b->d_off,
+                            b->d_species, b->d_first_of, b->d_sys, b->d_box, b->stream);
         dmts_model_desc d{};
         d.cutoff = m.rc; d.n_radial = m.K; d.n_layers = m.L; d.n_feat = m.F; d.n_species = m.S;
-        d.params = m.hp.data();
         d.n_params = m.n_params;
         d.precision = m.precision;
         d.rep_a = m.rep_a; d.rep_rho = m.rep_rho; d.rep_cutoff = m.rep_rc;
-        const dmts_system_desc sys{frames * c->n_sys, off.data(), spb.data(), mass.data(), box.data()};
-        if (create_context(nullptr, &d, &sys, "{\"autotune\": 0}", c->stream, &c->batch) != DMTS_OK) return nullptr;
-        c->batch_frames = frames;
-        c->batch_params = m.version;
-        c->batch->keep_msg = true;             // the second-order passes read every message row
+        int rc = init_model(b, b->m[1], &d, true, &m);
+        if (rc) return rc;
+        CUDA_TRY(ensure_filters(b));
+        if ((rc = prepare_embedding(b, b->m[1]))) return rc;
+        if (b->periodic)                       // the constant frames
+            launch_frames(b->n_sys, b->max_sys, b->d_off, b->d_x, b->N, b->d_box, b->rc_max, b->d_frame, nullptr,
+                          b->stream);
+        CUDA_TRY(cudaGetLastError());
+        return DMTS_OK;
+    };
+    const int rc = fill();
+    if (rc) {
+        free_batch(c);
+        return rc;
     }
-    return c->batch;
+    c->batch_frames = frames;
+    c->batch_params = m.version;
+    return DMTS_OK;
 }
 
 int alloc_fm(dmts_ctx* c, int atoms) {
@@ -1858,17 +1915,18 @@ int alloc_fm(dmts_ctx* c, int atoms) {
     const Model& m = c->m[0];
     const size_t nf = (size_t)atoms * m.F;
     FmBuffers& b = c->fm;
-    cudaError_t e = dalloc(&b.g, (size_t)3 * atoms);
-    for (float** p : {&b.mdot, &b.mbar_psi, &b.mdotbar_psi, &b.ubar})
-        if (e == cudaSuccess) e = dalloc(p, nf);
-    if (e == cudaSuccess) e = dalloc(&b.partial_e, (size_t)fm_edge_rows(atoms) * m.n_params);
-    if (e == cudaSuccess) e = dalloc(&b.partial_a, (size_t)fm_atom_rows(atoms) * m.n_params);
-    if (e == cudaSuccess) e = dalloc(&b.part, (size_t)fm_residual_blocks(atoms));
-    if (e == cudaSuccess) e = dalloc(&b.ticket, 1);
+    Slab slab;
+    slab.add(&b.g, (size_t)3 * atoms);
+    for (float** p : {&b.mdot, &b.mbar_psi, &b.mdotbar_psi, &b.ubar}) slab.add(p, nf);
+    slab.add(&b.partial_e, (size_t)fm_edge_rows(atoms) * m.n_params);
+    slab.add(&b.partial_a, (size_t)fm_atom_rows(atoms) * m.n_params);
+    slab.add(&b.part, (size_t)fm_residual_blocks(atoms));
+    slab.add(&b.ticket, 1);
+    slab.add(&b.grad, m.n_params);
+    slab.add(&b.loss, 1);
+    slab.add(&c->fm_stage, (size_t)6 * atoms);
+    cudaError_t e = slab.commit(&c->fm_slab);
     if (e == cudaSuccess) e = cudaMemsetAsync(b.ticket, 0, sizeof(unsigned int), c->stream);
-    if (e == cudaSuccess) e = dalloc(&b.grad, m.n_params);
-    if (e == cudaSuccess) e = dalloc(&b.loss, 1);
-    if (e == cudaSuccess) e = dalloc(&c->fm_stage, (size_t)6 * atoms);
     if (e != cudaSuccess) {
         cudaGetLastError();
         free_fm(c);
@@ -1892,8 +1950,8 @@ int distill_frames(dmts_ctx* c, int per, int n_frames, const double* frames, con
     int rc;
     dmts_ctx* w = c;                                              // the context that evaluates the frames
     if (per > 1) {
-        if (!(w = batch_context(c, per))) return DMTS_ERR_OOM;
-        if ((rc = alloc_fm(c, per * N))) return rc;
+        if ((rc = batch_context(c, per)) || (rc = alloc_fm(c, per * N))) return rc;
+        w = c->batch;
     } else if ((rc = alloc_fm(c, N))) {
         for (Model& m : c->m) free_filters(m);                    // (as with_room)
         if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
@@ -1943,10 +2001,7 @@ int distill_frames(dmts_ctx* c, int per, int n_frames, const double* frames, con
         m.cps_fwd = m0.cps_fwd; m.cps_bwd = m0.cps_bwd;
         m.bwd_tiles = m0.bwd_tiles;
         if (c->batch_params != m0.version) {   // new weights since the last call
-            CUDA_TRY(cudaMemcpyAsync(m.P, m0.P, sizeof(float) * m.n_params, cudaMemcpyDeviceToDevice, s));
-            CUDA_TRY(cudaMemcpyAsync(m.wt, m0.wt, m.wt_layer_bytes * m.L, cudaMemcpyDeviceToDevice, s));
-            CUDA_TRY(cudaMemcpyAsync(m.PT, m0.PT, sizeof(float) * (3 * m.L + 2) * m.F * m.F, cudaMemcpyDeviceToDevice, s));
-            CUDA_TRY(cudaMemcpyAsync(m.at, m0.at, atom_tile_bytes(m.F, m.L), cudaMemcpyDeviceToDevice, s));
+            if ((rc = copy_weights(w, m, m0))) return rc;
             if ((rc = prepare_embedding(w, m))) return rc;
             c->batch_params = m0.version;
         }

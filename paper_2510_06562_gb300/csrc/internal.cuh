@@ -371,6 +371,11 @@ int fm_edge_rows(int n_atoms);    // partial rows of the gradient edge pass for 
 int fm_atom_ctas(int n_atoms);    // blocks (= partial rows) of the per-atom adjoint pass
 int fm_atom_rows(int n_atoms);    // rows of the per-atom passes' partial buffer
 int fm_residual_blocks(int n_atoms);
+// frames copies of n_sys systems of n_atoms atoms in all, one behind the other
+// (first_of names atoms of the first copy)
+void launch_fm_replicate(int frames, int n_atoms, int n_sys, const int* off, const int* species, const int* first_of,
+                         const int* sys, const double* box, int* off_out, int* species_out, int* first_of_out,
+                         int* sys_out, double* box_out, cudaStream_t s);
 // Energy term of the distillation loss (e_ref null: none).
 struct FmEnergy {
     const double* e_ref = nullptr;   // device: each frame's reference energy
