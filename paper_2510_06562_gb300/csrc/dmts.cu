@@ -254,7 +254,8 @@ struct dmts_ctx {
     bool atom_tc = true;                   // BF16 mode: per-atom MLPs on the tensor cores
     bool keep_msg = false;                 // every message row stays in memory (the distillation reads them)
     long long body_launches = 0, fallback_seen = 0;
-    double cap_factor = 1.5;
+    double cap_factor = 1.5;               // options edge_capacity_factor, row_capacity and cell_capacity
+    double row_cap0 = 0, cell_cap0 = 0;    // (below 1: none)
     bool state_set = false, forces_valid = false;
     bool broken = false;
     bool autotune = true, tuned = false;
@@ -633,6 +634,12 @@ int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells, cons
         m.vl_cap = m.row_cap;
         m.e_cap = std::max<long long>(1024, std::min<long long>(sq, (long long)(N * std::min(mx, 64) * c->cap_factor)) + 1024);
     }
+    // smaller initial capacities (the overflow-and-retry path grows them)
+    auto at_most = [](int& cap, double option) {
+        if (option >= 1.0 && option < cap) cap = (int)option;
+    };
+    at_most(m.row_cap, c->row_cap0);
+    at_most(m.vl_cap, c->row_cap0);
     Slab slab;
     slab.add(&m.P, m.n_params);
     slab.add(&m.wt, m.wt_layer_bytes * m.L);
@@ -647,6 +654,7 @@ int init_model(dmts_ctx* c, Model& m, const dmts_model_desc* d, bool cells, cons
             slab.add(&m.atom_slot, N);
         } else {                           // fixed-capacity cells: twice the mean occupancy plus 16, grown on overflow
             m.ccap = ((int)(2.0 * N / m.n_cells) + 16 + 7) / 8 * 8;
+            at_most(m.ccap, c->cell_cap0);
         }
     }
     slab.add(&m.nbr_cnt, N);
@@ -1472,8 +1480,8 @@ int dmts_create(const dmts_model_desc* small, const dmts_model_desc* big, const 
     c->autotune = opt.get("autotune", 1.0) != 0.0;
     c->cap_factor = opt.get("edge_capacity_factor", 1.5);
     if (!(c->cap_factor > 0.0)) c->cap_factor = 1.5;
-    const double opt_row_cap = opt.get("row_capacity", 0.0);
-    const double opt_cell_cap = opt.get("cell_capacity", 0.0);
+    c->row_cap0 = opt.get("row_capacity", 0.0);
+    c->cell_cap0 = opt.get("cell_capacity", 0.0);
     c->skin = opt.get("skin", 0.0);
     if (!(c->skin >= 0.0) || c->skin > 10.0) {
         delete c;
@@ -1591,21 +1599,6 @@ int dmts_create(const dmts_model_desc* small, const dmts_model_desc* big, const 
     c->m[1].apc_fwd = std::min(kMaxAtomsPerCtaF32, (int)opt.get("atoms_per_cta_big", c->m[1].apc_fwd));
     c->m[1].apc_bwd = std::min(kMaxAtomsPerCtaF32, (int)opt.get("atoms_per_cta_big", c->m[1].apc_bwd));
     for (int w = 0; w < 2; ++w) {
-        if (c->m[w].present && opt_row_cap >= 1.0) {
-            // smaller initial row capacity (exercises the overflow-and-retry path)
-            c->m[w].row_cap = std::min(c->m[w].row_cap, (int)opt_row_cap);
-            c->m[w].vl_cap = std::min(c->m[w].vl_cap, (int)opt_row_cap);
-            free_model_nbr(c->m[w]);
-            CREATE_TRY(alloc_model_nbr(c, c->m[w]));
-        }
-        if (c->m[w].present && c->m[w].ccap > 0 && opt_cell_cap >= 1.0) {
-            // smaller initial cell capacity (exercises the overflow-and-retry path)
-            Model& m = c->m[w];
-            m.ccap = std::min(m.ccap, (int)opt_cell_cap);
-            dfree(m.cell_q);
-            m.cell_q = nullptr;
-            CREATE_TRY(dalloc(&m.cell_q, (size_t)m.n_cells * m.ccap));
-        }
         c->m[w].apc_fwd = std::max(8, c->m[w].apc_fwd);
         c->m[w].apc_bwd = std::max(8, c->m[w].apc_bwd);
     }
@@ -1864,6 +1857,9 @@ int batch_context(dmts_ctx* c, int frames) {
         b->h_box.insert(b->h_box.end(), c->h_box.begin(), c->h_box.end());
     }
     b->rc_max = m.rc;
+    b->cap_factor = c->cap_factor;
+    b->row_cap0 = c->row_cap0;
+    b->cell_cap0 = c->cell_cap0;
     b->vl_src = 1;
     b->atom_tc = c->atom_tc;
     b->keep_msg = true;                        // the second-order passes read every message row
