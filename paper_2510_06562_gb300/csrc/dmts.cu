@@ -392,9 +392,9 @@ void free_model_nbr(Model& m) {
 // the free memory at a time, halved until the allocation succeeds. They are
 // allocated behind every other buffer of the context, and what else needs
 // memory later takes it from them (with_room). Checked builds use small
-// limits, so that both forms run on small systems.
+// limits, so that both forms run on small systems, for one layer and for two.
 #ifdef DMTS_CHECK
-constexpr size_t kFilterBytes = (size_t)64 << 20, kFilterChunkBytes = (size_t)16 << 20;
+constexpr size_t kFilterBytes = (size_t)16 << 20, kFilterChunkBytes = (size_t)4 << 20;
 #else
 constexpr size_t kFilterBytes = (size_t)32 << 30, kFilterChunkBytes = (size_t)8 << 30;
 #endif
