@@ -369,7 +369,6 @@ __global__ void __launch_bounds__(AtomTile<F, RA>::NT) k_atom_fwd(PotArgs p, con
         }
         if (!T::PRE) stage_w<F, RA>(W(kU2), P + p.off.U2[l]);            // group: U2
         put_rows<F, RA>(X, a0, f0, m);
-        if (p.keep_msg) store_rows<F, RA>(p.msg_out, base, p.n_atoms, a0, f0, m);
     }
     cp_wait<1>();
     __syncthreads();

@@ -782,7 +782,6 @@ PotArgs pot_args(dmts_ctx* c, Model& m) {
     a.spec_sum = m.spec_sum;
     a.u_spec = m.u_spec;
     a.n_species = m.S;
-    a.keep_msg = c->keep_msg ? 1 : 0;
     a.h = m.h;
     a.h_in = m.h;
     a.gh = m.gh;

@@ -41,7 +41,7 @@ __device__ __forceinline__ I checked_index(I i, long long n, int* flags, int lin
 
 constexpr int kMaxLayers = 4;
 constexpr int kThreads = 256;          // threads per CTA of the edge kernels
-constexpr int kSmCount = 152;          // SMs of a GB300 (grid sizes only)
+constexpr int kSmCount = 152;          // SMs of a GB300 (grid sizes, and the atom counts at which kernels take over)
 // FP32 mode: the first layer sums over neighbours by species before the
 // filter's second product (2 S F^2 products per atom and direction against
 // 2 F^2 per unordered pair) in models of more than one layer (the small model
@@ -49,8 +49,9 @@ constexpr int kSmCount = 152;          // SMs of a GB300 (grid sizes only)
 // evaluation of 12,288 atoms either way), for up to kMaxFactorSpecies species, in periodic
 // systems (9 to 26 unordered pairs per atom; molecules have 5 to 9 and lost
 // 2 % by it: 301 molecules 388 -> 397 us) of at least kMinFactorAtoms atoms (the
-// per-atom kernels' chain of products gets longer, the pairs' kernel shorter:
-// 192 atoms 217 -> 223 us; 1,536 atoms 1.7 % faster, 12,288 atoms 8 %).
+// per-atom kernels' chain of products gets longer, the pairs' kernel shorter.
+// Forces of the big model without and with it, us: 192 atoms 156 and 161, 648 atoms
+// 168 and 170, 1,029 atoms 188 and 185, 1,536 atoms 204 and 200, 3,993 atoms 306 and 283).
 constexpr int kMaxFactorSpecies = 4;
 constexpr int kMinFactorAtoms = 1024;
 constexpr int kMaxMolAtoms = 1024;     // atoms per non-periodic system
@@ -288,7 +289,6 @@ struct PotArgs {
     float* spec_sum;         // [N][n_species]
     const float* u_spec;     // [n_species][F]: u^0 of each species
     int n_species;
-    int keep_msg;            // the per-atom kernel writes the messages it forms from them to msg_out
     // features
     const float* h_in;       // h entering the per-atom MLP of this layer (h^0 table for layer 0)
     float* h;
@@ -309,7 +309,7 @@ struct PotArgs {
     float* force;            // SoA [3][N]
     float* vir6;             // [N][6]
     int accumulate;          // backward: add to force/vir6 instead of overwrite
-    int virial;              // backward: also the per-atom virial vir6 (tensor-core path; FP32 always)
+    int virial;              // backward: also the per-atom virial vir6
     // tensor-core path: 128-pair tiles
     float* carry;            // [tiles][2][carry_w] partial sums of rows split across tiles
     int carry_w;             // F + 16

@@ -86,32 +86,25 @@ __global__ void k_embed(PotArgs a) {
 // The unordered pairs of the list, one entry (i, j), j > i, each, and for
 // every directed pair e the number pid[e] of its entry. A row's columns
 // ascend, so its pairs with j > i are a suffix. A block takes a range of
-// entries for its 32 atoms with one atomic (the order of the ranges varies
-// from run to run and no result depends on it); the entry's number goes to
-// its own directed pair and, found by bisection in row j, to the reverse one.
-constexpr int kIdxWarps = 8, kIdxRows = 1;     // rows per warp
+// entries for its 8 atoms, one per warp, with one atomic (the order of the
+// ranges varies from run to run and no result depends on it); the entry's
+// number goes to its own directed pair and, found by bisection in row j, to the
+// reverse one.
+constexpr int kIdxWarps = 8;
 
 __global__ void __launch_bounds__(kIdxWarps * 32) k_pair_index(PotArgs a, PairFilter pf) {
     __shared__ int w_sum[kIdxWarps];
     __shared__ int blk;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r0 = (blockIdx.x * kIdxWarps + w) * kIdxRows;
-    int first[kIdxRows], cnt[kIdxRows], total = 0;       // first pair with j > i, and their number
-#pragma unroll
-    for (int q = 0; q < kIdxRows; ++q) {
-        const int i = r0 + q;
-        int n_up = 0;
-        long long end = 0;
-        if (i < a.n_atoms) {
-            const long long beg = min((long long)a.row_ptr[i], a.e_cap);
-            end = min((long long)a.row_ptr[i + 1], a.e_cap);
-            for (long long e = beg + lane; e < end; e += 32) n_up += a.col[e] > i ? 1 : 0;
-        }
-        n_up = __reduce_add_sync(0xffffffffu, n_up);
-        first[q] = (int)end - n_up;
-        cnt[q] = n_up;
-        total += n_up;
+    const int i = blockIdx.x * kIdxWarps + w;
+    int total = 0;                                       // pairs with j > i, and the end of the row
+    long long end = 0;
+    if (i < a.n_atoms) {
+        const long long beg = min((long long)a.row_ptr[i], a.e_cap);
+        end = min((long long)a.row_ptr[i + 1], a.e_cap);
+        for (long long e = beg + lane; e < end; e += 32) total += a.col[e] > i ? 1 : 0;
     }
+    total = __reduce_add_sync(0xffffffffu, total);
     if (lane == 0) w_sum[w] = total;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -123,15 +116,8 @@ __global__ void __launch_bounds__(kIdxWarps * 32) k_pair_index(PotArgs a, PairFi
     int base = blk;
     for (int k = 0; k < w; ++k) base += w_sum[k];
     for (int t = lane; t < total; t += 32) {
-        int q = 0, o = t;
-#pragma unroll
-        for (int k = 0; k < kIdxRows - 1; ++k)
-            if (q == k && o >= cnt[k]) { o -= cnt[k]; ++q; }
-        int e = 0;
-#pragma unroll
-        for (int k = 0; k < kIdxRows; ++k)
-            if (q == k) e = first[k] + o;
-        const int i = r0 + q, j = DMTS_IDX(a.col[e], a.n_atoms, a.check), p = base + t;
+        const int e = (int)end - total + t;
+        const int j = DMTS_IDX(a.col[e], a.n_atoms, a.check), p = base + t;
         if (p >= pf.cap) continue;                       // a truncated (overflowed) list: the call is redone
         pf.pairs[p] = make_int2(i, j);
         pf.pid[e] = p;
@@ -883,8 +869,7 @@ template <int F>
 void fwd_go(const PotArgs& a, int K, cudaStream_t s) {
     if (!a.filter.chunk_atoms) {
         if (a.layer == 0) {                              // the filters of every layer at once
-            k_pair_index<<<(a.n_atoms + kIdxWarps * kIdxRows - 1) / (kIdxWarps * kIdxRows), kIdxWarps * 32, 0, s>>>(
-                a, a.filter);
+            k_pair_index<<<(a.n_atoms + kIdxWarps - 1) / kIdxWarps, kIdxWarps * 32, 0, s>>>(a, a.filter);
             count_launch();
             filters<F>(a, K, 0, a.n_layers, 0, a.n_atoms, s);
         }
