@@ -860,7 +860,7 @@ void enqueue_rebuild(dmts_ctx* c, cudaStream_t s) {
     Model& src = c->m[w0];
     NbrArgs b = candidate_args(c, w0);
     if (src.nc > 0)
-        launch_cells_gated(c->N, c->d_q, src.nc, src.cell_count, src.cell_start, src.atom_cell,
+        launch_cells_gated(c->N, c->d_q, src.nc, src.n_cells, src.cell_count, src.cell_start, src.atom_cell,
                            src.atom_slot, src.cell_q, b.gate, s);
     b.xref = c->d_xref;
     launch_vl_build(b, s);

@@ -339,7 +339,8 @@ void launch_neighbors(const NbrArgs& a, cudaStream_t s);
 // of candidate rows into the CSR.
 void launch_vl_check(int n_atoms, const double* x, const int* sys_of_atom, const double* box,
                      const VerletCheck& vc, cudaStream_t s);
-void launch_cells_gated(int n_atoms, const uint4* q, int nc, int* cell_count, int* cell_start,
+// (nc cells per dimension of each system, n_cells of all systems)
+void launch_cells_gated(int n_atoms, const uint4* q, int nc, int n_cells, int* cell_count, int* cell_start,
                         int* atom_cell, int* atom_slot, uint4* cell_q,
                         const int* gate, cudaStream_t s);
 void launch_vl_build(const NbrArgs& a, cudaStream_t s);

@@ -263,10 +263,9 @@ __global__ void k_cell_fill(int n, const int* __restrict__ atom_cell, const int*
     cell_q[pos] = make_uint4(qi.x, qi.y, qi.z, (unsigned int)i);
 }
 
-void launch_cells_gated(int n_atoms, const uint4* q, int nc, int* cell_count, int* cell_start,
+void launch_cells_gated(int n_atoms, const uint4* q, int nc, int n_cells, int* cell_count, int* cell_start,
                         int* atom_cell, int* atom_slot, uint4* cell_q,
                         const int* gate, cudaStream_t s) {
-    int n_cells = nc * nc * nc;
     if (n_atoms == 0) return;
     k_cell_clear<<<std::min(152, (n_cells + 255) / 256), 256, 0, s>>>(n_cells, cell_count, gate);
     int g = (n_atoms + 255) / 256;
