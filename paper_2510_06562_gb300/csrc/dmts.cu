@@ -791,21 +791,15 @@ PotArgs pot_args(dmts_ctx* c, Model& m) {
     return a;
 }
 
-// Position-independent per-atom inputs of one model: h^0 = A[Z_i] and
-// u^0 = h^0 W_in^0. Run after every parameter upload.
+// Position-independent inputs of one model: h^0 = A[Z_i] and u^0 = h^0 W_in^0 of
+// every atom and of each species. Run after every parameter upload.
 int prepare_embedding(dmts_ctx* c, Model& m) {
     if (!m.present || c->N == 0) return DMTS_OK;
     PotArgs a = pot_args(c, m);
     a.h = m.h0;
     a.u_next = m.u[0];
     a.um_u_out = m.um[0];
-    launch_embed(a, m.F, c->stream);
-    a.n_atoms = m.S;                       // the same of each species
-    a.species = nullptr;
-    a.h = m.u_spec + (size_t)m.S * m.F;
-    a.u_next = m.u_spec;
-    a.um_u_out = nullptr;
-    launch_embed(a, m.F, c->stream);
+    launch_embed(a, m.F, m.u_spec + (size_t)m.S * m.F, m.u_spec, c->stream);
     CUDA_TRY(cudaGetLastError());
     return DMTS_OK;
 }

@@ -348,7 +348,7 @@ void launch_row_filter(const NbrArgs& a, cudaStream_t s);
 void launch_vl_filter(const NbrArgs& a, cudaStream_t s);
 
 // potential_f32.cu
-void launch_embed(const PotArgs& a, int F, cudaStream_t s);
+void launch_embed(const PotArgs& a, int F, float* h_spec, float* u_spec, cudaStream_t s);   // h_spec, u_spec: [n_species][F]
 // (the forward launch of layer 0 also computes the pairs' filters of every layer)
 void launch_edge_fwd_f32(const PotArgs& a, int F, int K, cudaStream_t s);
 void launch_edge_bwd_f32(const PotArgs& a, int F, int K, cudaStream_t s);

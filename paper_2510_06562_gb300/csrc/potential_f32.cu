@@ -65,16 +65,24 @@ __device__ __forceinline__ float cutoff_deriv(float d, float pi_over_rc) {
 }
 
 // ------------------------------------------------------------ embedding
+// h^0 = A[Z_i] and u^0 = h^0 W_in^0 of every atom and, behind them, the same
+// of each species, to h_spec and u_spec.
 template <int F>
-__global__ void k_embed(PotArgs a) {
+__global__ void k_embed(PotArgs a, float* __restrict__ h_spec, float* __restrict__ u_spec) {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     int i = t / F, f = t % F;
-    if (i >= a.n_atoms) return;
-    int z = a.species ? a.species[i] : i;
+    if (i >= a.n_atoms + a.n_species) return;
+    const bool atom = i < a.n_atoms;
+    int z = atom ? a.species[i] : i - a.n_atoms;
     const float* A = a.P + a.off.A + z * F;
     const float* W = a.P + a.off.W_in[0];
     float acc = 0.f;
     for (int k = 0; k < F; ++k) acc += __ldg(A + k) * __ldg(W + k * F + f);
+    if (!atom) {
+        h_spec[z * F + f] = __ldg(A + f);
+        u_spec[z * F + f] = acc;
+        return;
+    }
     a.h[(size_t)i * F + f] = __ldg(A + f);
     a.u_next[(size_t)i * F + f] = acc;
     if (a.um_u_out)
@@ -920,11 +928,11 @@ void bwd_go(const PotArgs& a, int K, cudaStream_t s) {
 
 }  // namespace
 
-void launch_embed(const PotArgs& a, int F, cudaStream_t s) {
+void launch_embed(const PotArgs& a, int F, float* h_spec, float* u_spec, cudaStream_t s) {
     if (a.n_atoms == 0) return;
-    int total = a.n_atoms * F;
-    if (F == 64) k_embed<64><<<(total + 255) / 256, 256, 0, s>>>(a);
-    else k_embed<32><<<(total + 255) / 256, 256, 0, s>>>(a);
+    int total = (a.n_atoms + a.n_species) * F;
+    if (F == 64) k_embed<64><<<(total + 255) / 256, 256, 0, s>>>(a, h_spec, u_spec);
+    else k_embed<32><<<(total + 255) / 256, 256, 0, s>>>(a, h_spec, u_spec);
     count_launch();
 }
 
