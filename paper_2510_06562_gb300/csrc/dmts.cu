@@ -291,6 +291,24 @@ struct Range {
     ~Range() { nvtxRangePop(); }
 };
 
+// Where a caller's buffer lies. own: doubles in memory of the context's own
+// device, which its kernels read and write directly (memory elsewhere, or not
+// on an 8-byte boundary, goes through a staging buffer).
+struct Place {
+    bool device, own;
+};
+
+Place place_of(const dmts_ctx* c, const void* p) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return {false, false};
+    }
+    const bool mem = at.type == cudaMemoryTypeDevice;
+    return {mem || at.type == cudaMemoryTypeManaged,
+            mem && at.device == c->device && (uintptr_t)p % sizeof(double) == 0};
+}
+
 bool is_device_ptr(const void* p) {
     cudaPointerAttributes at;
     cudaError_t e = cudaPointerGetAttributes(&at, p);
@@ -299,19 +317,6 @@ bool is_device_ptr(const void* p) {
         return false;
     }
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
-}
-
-// Doubles in memory of the context's own device, which its kernels may read
-// and write directly (memory elsewhere, or not on an 8-byte boundary, goes
-// through a staging buffer).
-bool is_own_device_ptr(const dmts_ctx* c, const void* p) {
-    if ((uintptr_t)p % sizeof(double) != 0) return false;
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return at.type == cudaMemoryTypeDevice && at.device == c->device;
 }
 
 template <class T>
@@ -1099,17 +1104,21 @@ int reset_flags(dmts_ctx* c) {
     return DMTS_OK;
 }
 
-int copy_in(dmts_ctx* c, double* dst, const double* src, size_t n) {
-    cudaMemcpyKind k = is_device_ptr(src) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+int copy_in(dmts_ctx* c, double* dst, const double* src, size_t n, Place p) {
+    cudaMemcpyKind k = p.device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     CUDA_TRY(cudaMemcpyAsync(dst, src, n * sizeof(double), k, c->stream));
     return DMTS_OK;
 }
 
-int copy_out(dmts_ctx* c, double* dst, const double* src, size_t n) {
-    cudaMemcpyKind k = is_device_ptr(dst) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+int copy_in(dmts_ctx* c, double* dst, const double* src, size_t n) { return copy_in(c, dst, src, n, place_of(c, src)); }
+
+int copy_out(dmts_ctx* c, double* dst, const double* src, size_t n, Place p) {
+    cudaMemcpyKind k = p.device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     CUDA_TRY(cudaMemcpyAsync(dst, src, n * sizeof(double), k, c->stream));
     return DMTS_OK;
 }
+
+int copy_out(dmts_ctx* c, double* dst, const double* src, size_t n) { return copy_out(c, dst, src, n, place_of(c, dst)); }
 
 // The single-time-step fallback of one outer step (body of the IF node):
 // restore x, v and the large-model force saved at the start of the step, take
@@ -1618,12 +1627,13 @@ int dmts_set_state(dmts_ctx* c, const double* x, const double* v, int n_atoms) {
     size_t n3 = (size_t)3 * c->N;
     int rc;
     const double *xs = x, *vs = v;
-    if (!is_own_device_ptr(c, x)) {
-        if ((rc = copy_in(c, c->d_stage, x, n3))) return rc;
+    const Place px = place_of(c, x), pv = v ? place_of(c, v) : Place{};
+    if (!px.own) {
+        if ((rc = copy_in(c, c->d_stage, x, n3, px))) return rc;
         xs = c->d_stage;
     }
-    if (v && !is_own_device_ptr(c, v)) {
-        if ((rc = copy_in(c, c->d_stage + n3, v, n3))) return rc;
+    if (v && !pv.own) {
+        if ((rc = copy_in(c, c->d_stage + n3, v, n3, pv))) return rc;
         vs = c->d_stage + n3;
     }
     CUDA_TRY(cudaMemsetAsync(c->d_flags + kFlagMoved, 0, sizeof(int), c->stream));
@@ -1643,12 +1653,12 @@ int dmts_get_state(dmts_ctx* c, double* x, double* v) {
     Range nvtx_range("dmts_get_state");
     LaunchScope ls(c);
     size_t n3 = (size_t)3 * c->N;
-    const bool xd = x && is_own_device_ptr(c, x), vd = v && is_own_device_ptr(c, v);
-    launch_get_state(c->N, c->d_x, c->d_v, xd ? x : (x ? c->d_stage : nullptr),
-                     vd ? v : (v ? c->d_stage + n3 : nullptr), c->stream);
+    const Place px = x ? place_of(c, x) : Place{}, pv = v ? place_of(c, v) : Place{};
+    launch_get_state(c->N, c->d_x, c->d_v, px.own ? x : (x ? c->d_stage : nullptr),
+                     pv.own ? v : (v ? c->d_stage + n3 : nullptr), c->stream);
     int rc;
-    if (x && !xd && (rc = copy_out(c, x, c->d_stage, n3))) return rc;
-    if (v && !vd && (rc = copy_out(c, v, c->d_stage + n3, n3))) return rc;
+    if (x && !px.own && (rc = copy_out(c, x, c->d_stage, n3, px))) return rc;
+    if (v && !pv.own && (rc = copy_out(c, v, c->d_stage + n3, n3, pv))) return rc;
     return sync_check(c);
 }
 
@@ -1663,15 +1673,15 @@ int dmts_forces(dmts_ctx* c, int which, double* f_out, double* energy_out, doubl
     int rc;
     if ((rc = autotune_models(c))) return rc;
     const size_t n3 = (size_t)3 * c->N;
-    const bool fd = f_out && is_own_device_ptr(c, f_out);
+    const Place pf = f_out ? place_of(c, f_out) : Place{};
     // the outputs follow the evaluation on the stream (one wait); after an
     // overflow they are written again
     for (int attempt = 0; attempt < 4; ++attempt) {
         if ((rc = reset_flags(c))) return rc;
         enqueue_eval(c, which, true, true, Check::Kernel, virial_out != nullptr);
         if (virial_out) launch_virial_sum(c->n_sys, c->d_off, m.vir6, m.W, m.esum, c->stream);
-        if (f_out) launch_forces_out(c->N, m.force, fd ? f_out : c->d_stage, c->stream);
-        if (f_out && !fd && (rc = copy_out(c, f_out, c->d_stage, n3))) return rc;
+        if (f_out) launch_forces_out(c->N, m.force, pf.own ? f_out : c->d_stage, c->stream);
+        if (f_out && !pf.own && (rc = copy_out(c, f_out, c->d_stage, n3, pf))) return rc;
         if (energy_out && (rc = copy_out(c, energy_out, m.E, c->n_sys))) return rc;
         if (virial_out && (rc = copy_out(c, virial_out, m.W, (size_t)9 * c->n_sys))) return rc;
         if ((rc = sync_check(c))) return rc;
