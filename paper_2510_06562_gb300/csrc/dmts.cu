@@ -9,6 +9,7 @@
 // replayed once per outer step. Neighbour capacity overflow is detected on
 // the device; the host restores the state saved at the start of the call,
 // grows the capacity, re-captures the graph and runs the call again.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdarg.h>
@@ -307,6 +308,38 @@ Place place_of(const dmts_ctx* c, const void* p) {
     const bool mem = at.type == cudaMemoryTypeDevice;
     return {mem || at.type == cudaMemoryTypeManaged,
             mem && at.device == c->device && (uintptr_t)p % sizeof(double) == 0};
+}
+
+// Whether bytes at the device address p lie inside allocations (one, or several
+// mapped one behind the other). Known false only: true where the driver cannot
+// tell. A copy checks its range itself; a kernel does not.
+bool is_allocated(const void* p, size_t bytes) {
+    using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const Range range = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &r) != cudaSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<Range>(f);
+    }();
+    CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p), end = at + bytes, base = 0;
+    size_t size = 0;
+    if (!range || range(&base, &size, at) != CUDA_SUCCESS) return true;
+    while (base + size < end) {
+        at = base + size;
+        if (range(&base, &size, at) != CUDA_SUCCESS || base != at) return false;
+    }
+    return true;
+}
+
+// The place of a buffer of n doubles that may be read or written in place.
+int place_in(const dmts_ctx* c, const void* p, size_t n, const char* name, Place& out) {
+    out = place_of(c, p);
+    if (out.own && !is_allocated(p, n * sizeof(double)))
+        return fail(DMTS_ERR_ARG, "%s: the device buffer is smaller than %zu doubles", name, n);
+    return DMTS_OK;
 }
 
 bool is_device_ptr(const void* p) {
@@ -1627,7 +1660,9 @@ int dmts_set_state(dmts_ctx* c, const double* x, const double* v, int n_atoms) {
     size_t n3 = (size_t)3 * c->N;
     int rc;
     const double *xs = x, *vs = v;
-    const Place px = place_of(c, x), pv = v ? place_of(c, v) : Place{};
+    Place px{}, pv{};
+    if ((rc = place_in(c, x, n3, "x", px))) return rc;
+    if (v && (rc = place_in(c, v, n3, "v", pv))) return rc;
     if (!px.own) {
         if ((rc = copy_in(c, c->d_stage, x, n3, px))) return rc;
         xs = c->d_stage;
@@ -1653,10 +1688,12 @@ int dmts_get_state(dmts_ctx* c, double* x, double* v) {
     Range nvtx_range("dmts_get_state");
     LaunchScope ls(c);
     size_t n3 = (size_t)3 * c->N;
-    const Place px = x ? place_of(c, x) : Place{}, pv = v ? place_of(c, v) : Place{};
+    Place px{}, pv{};
+    int rc;
+    if (x && (rc = place_in(c, x, n3, "x", px))) return rc;
+    if (v && (rc = place_in(c, v, n3, "v", pv))) return rc;
     launch_get_state(c->N, c->d_x, c->d_v, px.own ? x : (x ? c->d_stage : nullptr),
                      pv.own ? v : (v ? c->d_stage + n3 : nullptr), c->stream);
-    int rc;
     if (x && !px.own && (rc = copy_out(c, x, c->d_stage, n3, px))) return rc;
     if (v && !pv.own && (rc = copy_out(c, v, c->d_stage + n3, n3, pv))) return rc;
     return sync_check(c);
@@ -1670,10 +1707,11 @@ int dmts_forces(dmts_ctx* c, int which, double* f_out, double* energy_out, doubl
     if (!c->state_set) return fail(DMTS_ERR_STATE, "no state set");
     LaunchScope ls(c);
     Model& m = c->m[which];
-    int rc;
-    if ((rc = autotune_models(c))) return rc;
     const size_t n3 = (size_t)3 * c->N;
-    const Place pf = f_out ? place_of(c, f_out) : Place{};
+    Place pf{};
+    int rc;
+    if (f_out && (rc = place_in(c, f_out, n3, "f_out", pf))) return rc;
+    if ((rc = autotune_models(c))) return rc;
     // the outputs follow the evaluation on the stream (one wait); after an
     // overflow they are written again
     for (int attempt = 0; attempt < 4; ++attempt) {
