@@ -458,10 +458,10 @@ cudaError_t alloc_filters(dmts_ctx* c, Model& m) {
         free_filters(m);
     }
     const size_t chunk = std::min(kFilterChunkBytes, free_bytes / 2);
-    long long atoms = std::max<long long>(1, (long long)(chunk / row) / m.row_cap);
+    long long atoms = std::max<long long>(1, (long long)(chunk / row) / std::max(1, m.row_cap));
     for (;; atoms /= 2) {
         f.chunk_atoms = (int)atoms;
-        f.cap = atoms * m.row_cap;
+        f.cap = atoms * std::max(1, m.row_cap);
         e = dalloc(&f.w, f.cap * (row / sizeof(float)));
         if (e == cudaSuccess) e = dalloc(&f.se, (size_t)f.cap);
         if (e == cudaSuccess) return e;
