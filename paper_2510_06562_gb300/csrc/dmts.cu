@@ -1090,36 +1090,46 @@ int sync_check(dmts_ctx* c) {
     return DMTS_OK;
 }
 
-// Grow neighbour capacities from the maxima seen on the device.
+// Grow neighbour capacities from the maxima seen on the device. Capacities that
+// are too large for the kernels are refused before anything is changed.
 int grow_capacity(dmts_ctx* c) {
     // buffers are missing then: no later call may use the context
     auto out_of_memory = [c](const char* what, cudaError_t e) {
         c->broken = true;
         return fail(DMTS_ERR_OOM, "growing %s: %s", what, cudaGetErrorString(e));
     };
+    int rc = force_rebuild(c);              // candidate rows truncated by the overflow, or reallocated below
+    if (rc) return rc;
+    int row_cap[2], vl_cap[2];
+    long long e_cap[2];
+    for (int w = 0; w < 2; ++w) {
+        const Model& m = c->m[w];
+        if (!m.present) continue;
+        const int max_row = c->h_flags[kFlagMaxRow0 + w], max_vl = c->h_flags[kFlagMaxVl0 + w];
+        const long long max_e = (long long)(unsigned int)c->h_flags[kFlagMaxE0 + w];
+        row_cap[w] = max_row > m.row_cap ? std::min(c->N, ((int)(max_row * 1.25) + 63) / 32 * 32) : m.row_cap;
+        e_cap[w] = max_e > m.e_cap ? (long long)(max_e * 1.25) + 1024 : m.e_cap;
+        vl_cap[w] = c->skin > 0 && max_vl > m.vl_cap ? std::min(c->N, ((int)(max_vl * 1.25) + 63) / 32 * 32) : m.vl_cap;
+        if (row_cap[w] > 6000 || vl_cap[w] > 6000)
+            return fail(DMTS_ERR_CAPACITY, "neighbour row capacity %d too large", std::max(row_cap[w], vl_cap[w]));
+    }
+    if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
+    CUDA_TRY(cudaStreamSynchronize(c->stream));
     for (int w = 0; w < 2; ++w) {
         Model& m = c->m[w];
         if (!m.present) continue;
-        int max_row = c->h_flags[kFlagMaxRow0 + w];
-        long long max_e = (long long)(unsigned int)c->h_flags[kFlagMaxE0 + w];
-        bool grow = false;
-        int max_vl = c->h_flags[kFlagMaxVl0 + w];
-        if (max_row > m.row_cap) { m.row_cap = std::min(c->N, ((int)(max_row * 1.25) + 63) / 32 * 32); grow = true; }
-        if (max_e > m.e_cap) { m.e_cap = (long long)(max_e * 1.25) + 1024; grow = true; }
-        if (c->skin > 0 && max_vl > m.vl_cap) { m.vl_cap = std::min(c->N, ((int)(max_vl * 1.25) + 63) / 32 * 32); grow = true; }
         const int max_cell = c->h_flags[kFlagMaxCell0 + w];
         if (m.ccap > 0 && max_cell > m.ccap) {
             m.ccap = ((int)(max_cell * 1.25) + 8 + 7) / 8 * 8;
-            CUDA_TRY(cudaStreamSynchronize(c->stream));
             dfree(m.cell_q);
             m.cell_q = nullptr;
             cudaError_t e = with_room(c, [&] { return dalloc(&m.cell_q, (size_t)m.n_cells * m.ccap); });
             if (e != cudaSuccess) return out_of_memory("cell capacity", e);
         }
-        if (grow) {
-            if (m.row_cap > 6000 || m.vl_cap > 6000)
-                return fail(DMTS_ERR_CAPACITY, "neighbour row capacity %d too large", std::max(m.row_cap, m.vl_cap));
-            CUDA_TRY(cudaStreamSynchronize(c->stream));
+        if (row_cap[w] > m.row_cap || e_cap[w] > m.e_cap || vl_cap[w] > m.vl_cap) {
+            m.row_cap = row_cap[w];
+            m.e_cap = e_cap[w];
+            m.vl_cap = vl_cap[w];
             cudaError_t e = with_room(c, [&] {
                 free_model_nbr(m);
                 return alloc_model_nbr(c, m);
@@ -1128,8 +1138,7 @@ int grow_capacity(dmts_ctx* c) {
         }
     }
     if (cudaError_t e = ensure_filters(c)) return out_of_memory("filter rows", e);
-    if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
-    return force_rebuild(c);                // rows reallocated, or truncated by the overflow
+    return DMTS_OK;
 }
 
 int reset_flags(dmts_ctx* c) {
@@ -1851,10 +1860,10 @@ int dmts_respa_step(dmts_ctx* c, int n_outer, double dt, int n_inner, double* en
             c->fallback_seen = (long long)nf;
         }
         if (!c->h_flags[kFlagOverflow]) break;
-        if (attempt >= 3) return fail(DMTS_ERR_CAPACITY, "neighbour capacity overflow persists");
         // restore and retry with grown capacity
         if ((rc = restore())) return rc;
         if ((rc = grow_capacity(c))) return rc;
+        if (attempt >= 3) return fail(DMTS_ERR_CAPACITY, "neighbour capacity overflow persists");
     }
     c->forces_valid = true;
     if (c->h_flags[kFlagNonfinite]) return fail(DMTS_ERR_NONFINITE, "non-finite position or velocity");
@@ -2082,28 +2091,35 @@ int distill_frames(dmts_ctx* c, int per, int n_frames, const double* frames, con
         }
         return sync_check(w);
     };
-    for (int attempt = 0;; ++attempt) {
-        if ((rc = batches())) {
-            c->broken = c->broken || w->broken;            // (a CUDA error: both contexts')
-            return rc;
+    auto until_it_fits = [&]() -> int {
+        for (int attempt = 0;; ++attempt) {
+            if ((rc = batches())) {
+                c->broken = c->broken || w->broken;        // (a CUDA error: both contexts')
+                return rc;
+            }
+            if (!w->h_flags[kFlagOverflow]) return DMTS_OK;
+            if (!own) {                        // capacities for whole batches
+                w->N = restore.N;
+                w->n_sys = restore.n_sys;
+                m.n_cells = restore.n_cells;
+            }
+            if ((rc = grow_capacity(w))) return rc;
+            if (attempt == 3) return fail(DMTS_ERR_CAPACITY, "neighbour capacity overflow persists");
         }
-        if (!w->h_flags[kFlagOverflow]) break;
-        if (attempt == 3) return fail(DMTS_ERR_CAPACITY, "neighbour capacity overflow persists");
-        if (!own) {                            // capacities for whole batches
-            w->N = restore.N;
-            w->n_sys = restore.n_sys;
-            m.n_cells = restore.n_cells;
-        }
-        if ((rc = grow_capacity(w))) return rc;
-    }
-    if (own) {
+    };
+    const int result = until_it_fits();
+    c->forces_valid = false;
+    if (own && !c->broken) {                   // also after a failure
         CUDA_TRY(cudaMemcpyAsync(c->d_x, c->d_bx, n3 * sizeof(double), cudaMemcpyDeviceToDevice, s));
         CUDA_TRY(cudaMemcpyAsync(c->d_v, c->d_bv, n3 * sizeof(double), cudaMemcpyDeviceToDevice, s));
+        if (result) CUDA_TRY(cudaStreamSynchronize(s));
     }
-    c->forces_valid = false;
+    if (result) return result;
     if ((rc = copy_out(w, grad_out, c->fm.grad, np))) return rc;
     if ((rc = copy_out(w, loss_out, c->fm.loss, 1))) return rc;
-    return sync_check(w);
+    rc = sync_check(w);
+    c->broken = c->broken || w->broken;
+    return rc;
 }
 
 int distill_impl(dmts_ctx* c, int n_frames, const double* frames, const double* f_ref, const double* e_ref,
