@@ -582,9 +582,10 @@ void atom_go(const PotArgs& p, const float* x, bool fwd, cudaStream_t s) {
 // Atoms per thread: as few as leave one block per SM. The products are then a
 // chain of latencies, and a block of 8 atoms walks it in a third of the time
 // of one of 32. Blocks of 32 atoms against these, us: FP32 forces of 192 atoms
-// 213 -> 199, of 1,536 263 -> 249, 1 fs step of 1,536 183 -> 173; 3 fs step in
-// BF16 (the small model's kernels) of 192 atoms 197 -> 192, of 1,536 246 -> 240.
-// At F = 32 the line is 1,824 atoms: at 2,187 blocks of 16 take 256 against 254.
+// 171 -> 158, of 1,536 209 -> 199, of 2,187 230 -> 221, 1 fs step of 1,536
+// 164 -> 155; 3 fs step in BF16 (the small model's kernels; steps back to back) of
+// 192 atoms 174 -> 170, of 1,536 220 -> 217. At F = 32 the line is 1,824 atoms: at
+// 2,187 that step takes 256 in blocks of 16 against 254.
 template <int F>
 void atom_any(const PotArgs& p, const float* x, bool fwd, cudaStream_t s) {
     if (p.n_atoms <= 8 * kSmCount) atom_go<F, 1>(p, x, fwd, s);

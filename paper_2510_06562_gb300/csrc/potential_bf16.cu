@@ -539,8 +539,10 @@ __global__ void __launch_bounds__(kT, F == 32 ? 8 : 1) k_edge_fwd_bf16(PotArgs a
 
     // The weights (pre-converted BF16 operand tiles and the biases) travel while
     // the first tile's indices and positions, two dependent loads, are fetched:
-    // a small system's pass is one tile and mostly this chain (8 us less per 3 fs
-    // step of 192 atoms, 9 of 547 us of 12,288; the backward kernels alike).
+    // a small system's pass is one tile and mostly this chain. Against copies that
+    // the threads wait for, 8 us less per 3 fs step of 192 atoms and 6 of 550 us of
+    // 12,288, of which the loads ahead of the weights are 1.5 and 2 (the backward
+    // kernels alike).
     const unsigned char* const wsrc = a.wt + (size_t)l * a.wt_layer_bytes;
     copy_weights(S.w1t, wsrc, F * kKP * 2, tid, kT);
     copy_weights(S.w2t, wsrc + F * kKP * 2, F * F * 2, tid, kT);

@@ -17,14 +17,15 @@
 // the second product of the filter is taken out of the sums: rows fc SiLU(a)
 // are summed per atom and neighbour species, and multiplied by W2 once each
 // (k_gather_species; the adjoint alike in k_pair_dedd).
-// 12,288-atom water: forces with virial 748 -> 692 us, 3 fs step 1.00 -> 0.93 ms.
+// 12,288-atom water, when it came: forces with virial 748 -> 692 us, 3 fs step
+// 1.00 -> 0.93 ms (701 us and 0.95 ms now).
 //
 // Against recomputing the filter per directed pair in each pass (20,480 and
 // 10,240 flop per directed pair and layer), this is 20,480 flop per unordered
 // pair and layer in all, and w, dw/dd travel through memory (512 bytes per
 // unordered pair and layer at F = 64, written once, w read four times and
-// dw/dd once). Big model, 12,288-atom water, one evaluation: 3.48 -> 0.62 ms
-// (edge passes 3.36 -> 0.50 ms); 192 atoms: 0.61 -> 0.155 ms.
+// dw/dd once). Big model, 12,288-atom water, one evaluation: 3.48 -> 0.57 ms
+// (edge passes 3.36 -> 0.43 ms); 192 atoms: 0.61 -> 0.158 ms.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -146,8 +147,9 @@ __global__ void __launch_bounds__(kIdxWarps * 32) k_pair_index(PotArgs a, PairFi
 // a = e W1 + b1 and phi = SiLU(a) W2 + b2, for tiles of 128 pairs.
 //
 // Bound by FP32 FMA issue: 2 (2 KP F + 2 F F) flop per pair and layer against
-// 512 bytes written (F = 64): 639,638 directed pairs, two layers, 13.1 GFLOP in
-// 296 us (ncu: FMA pipe 63 %, DRAM 12 %). Each thread owns 8 pairs x 4 features of both
+// 512 bytes written (F = 64): 639,638 directed pairs, two layers, the first one
+// without its second product, 7.9 GFLOP in 215 us (cold, ncu: FMA pipe 57 %, issue
+// 52 %, 279 MB written). Each thread owns 8 pairs x 4 features of both
 // products that share a weight matrix (64 accumulators), as packed f32x2
 // operations over two pairs: one FFMA2 for two FMAs leaves issue slots for the
 // operand loads (five 16-byte shared loads per 64 FMAs). The hidden layer is
