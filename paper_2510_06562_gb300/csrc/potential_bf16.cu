@@ -816,15 +816,15 @@ __global__ void __launch_bounds__(kT) k_edge_bwd_bf16(PotArgs a, int K, int* sta
     if (TAB) load_table(ST, a, tid, kT);
     cp_async_commit();
     EdgeIn nx;
-    // (above layer 0 the first tile's loads wait for the weights: ahead of them
-    // they take the kernel from 95 to 128 registers at F = 32, and an SM from five
-    // CTAs to four)
-    if (L0) load_idx(a, (long long)blockIdx.x * kT + tid, E, nx);
+    // (above layer 0 at F = 32 the first tile's loads wait for the weights: ahead of
+    // them they take the kernel from 95 to 128 registers, and an SM from five CTAs to four)
+    constexpr bool kAhead = L0 || F == 64;
+    if (kAhead) load_idx(a, (long long)blockIdx.x * kT + tid, E, nx);
     const float bias1 = tid < F ? __ldg(a.P + a.off.b1[l] + tid) : 0.f;
     const float bias2 = tid < F ? __ldg(a.P + a.off.b2[l] + tid) : 0.f;
     if (tid == 0) mbar_init(&S.mbar, 1);
     if (warp == 0) tmem_alloc(&S.taddr, TCOLS);
-    if (L0) load_pos<TAB>(a, nx);
+    if (kAhead) load_pos<TAB>(a, nx);
     if (tid < F) {
         S.b1[tid] = bias1;
         S.b2[tid] = bias2;
@@ -845,7 +845,7 @@ __global__ void __launch_bounds__(kT) k_edge_bwd_bf16(PotArgs a, int K, int* sta
     uint32_t pend = 0;                                     // ... and the parity it completes
 
     const int cw = a.carry_w;
-    if (!L0) {
+    if (!kAhead) {
         load_idx(a, (long long)blockIdx.x * kT + tid, E, nx);
         load_pos<TAB>(a, nx);
     }
