@@ -31,6 +31,8 @@
  *  - All arrays are owned by the caller; the library copies what it needs.
  *    A pointer may point to host memory or to CUDA device memory of the
  *    context's device; the library tells them apart itself.
+ *    Positions, velocities and forces in device memory are read and written in
+ *    place; a device buffer too small for them is an argument error.
  *  - Per-atom 3-vectors are arrays of N*3 doubles, atom-major
  *    (x[3*i + 0..2]), i.e. a C-contiguous [N][3] array.
  *  - Every call returns DMTS_OK (0) or a negative dmts_status and throws
